@@ -10,7 +10,7 @@
 // per-query references in every pass.  Instead the reference of column c, R[c] (a bf16 number in units of raw scores),
 // is subtracted by the tensor core: a ninth K-step multiplies a column of ones (A) by a row holding -R[c] (B, 2 KB,
 // written by the softmax group), so the accumulator holds s - R[c] and a pass is p = 2^(scale * x) with no per-column
-// operand: half the TMEM reads of a pass and no reference registers.  R[c] sits 2^7 above the largest score its column
+// operand: half the TMEM reads of a pass and no reference registers.  R[c] sits 2^32 above the largest score its column
 // had when it was taken; a tile whose entries all stay below 2 (seen on the packed bf16 words) needs no cross-thread
 // reduction.  Otherwise, and on the first tile of a work item, the group rebases: exact column maxima, new R, row sums
 // and O^T rescaled, the -R row rewritten.  The (at most two) S^T tiles already computed with the old row are corrected in
@@ -38,8 +38,15 @@ namespace tc {
 using namespace tcc;
 
 constexpr int kThreads = 512;
-constexpr float kRefShift = 7.f;   // softmax references are kept this far (log2) above the column maxima they were taken from
-constexpr float kFirstShift = 12.f; // ... and this far above the score of the single key an item's first references are taken from
+// Softmax references are kept this far (log2) above the scores they were taken from.  P is bf16 and its sums are fp32, so
+// a common factor 2^-32 costs no precision, and a column's scores may rise by 2^33 before its references have to move;
+// a rebase costs as much as several tiles.  With 2^7 (and 2^12 above the one key an item's first references came from)
+// layers with a sink key and stripes lost a third to a half of the attention to rebases: 32k tokens at one block in ten
+// 2.29 -> 1.68 ms, a batch of 24 short prompts 0.71 -> 0.38 ms; 2^24 and 2^40 measured the same within 7 %.
+constexpr float kRefShift = 32.f;
+// A reference that rose by more than this factor (60 + kRefShift): the largest score of the tile was 2^60 above its old
+// reference, everything accumulated before is negligible, and the value taken out again may not have been finite.
+constexpr float kAlphaGone = 2.0195e-28f;   // 2^-92
 constexpr float kNoRef = -32768.f; // reference of a column that has not seen a key yet: the first visible score overflows it
 constexpr int kHelperRegs = 56, kSoftmaxRegs = 200;   // (2 * 56 + 2 * 200) * 128 = 65536
 constexpr int kGroupThreads = 128;
@@ -582,16 +589,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         const bool masked = !row_live || diag || ragged_q;   // uniform per warp (a warp lies in one block half)
         const uint32_t s_addr = tmem + lane_addr + col_s(s, sbuf);
         uint32_t pk[32];
-        // First tile of an item: the references are still those of another item.  Column c takes the score of the
-        // tile's first key (visible to every query of the block: it is the first key of a block not later than the
-        // query block) plus kFirstShift as its reference: no reduction over the keys.  A reference taken from a key of
-        // the column itself can never be too high (what it would flush to zero is negligible next to that key), and
-        // if it is too low the pass below says so and the group rebases on exact maxima.
+        // First tile of an item: the references are still those of another item.  Column c takes the largest of the
+        // scores of four of the tile's keys (rows 0, 32, 64, 96 where it sees them; it sees row 0, the first key of a
+        // block not later than the query block) plus kRefShift as its reference: no reduction over all the keys.  A
+        // reference taken from keys of the column itself can never be too high (what it would flush to zero is
+        // negligible next to those keys), and if it is too low the pass below says so and the group rebases on exact
+        // maxima.  (One key alone is often an outlier: the sink of a long prompt.)
         bool have_ref = t >= 1;
         if (t == 0 && ja >= 0) {
           if (!fail && it.ntiles > 1) fail = !mbar_wait(sh, bb + S_FULL + (int)(sbuf ^ 1u), ((cnt + 1) >> 1) & 1u, status);
           tc_fence_after();
-          if (!fail && gw == 0) {                         // (the TMEM load is a warp-wide instruction; lane 0 holds key row 0)
+          if (!fail) {                                    // (the TMEM load is a warp-wide instruction; lane 0 holds key row 32 * quad)
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {
               uint32_t sv[16];
@@ -599,8 +607,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
               tc_wait_ld(sv);
               if (lane == 0) {
 #pragma unroll
-                for (int e = 0; e < 16; e += 4)
-                  *reinterpret_cast<uint4*>(&lsum[ch * 16 + e]) = make_uint4(sv[e], sv[e + 1], sv[e + 2], sv[e + 3]);
+                for (int e = 0; e < 16; e += 4) {
+                  const int c = ch * 16 + e;
+                  const uint32_t hidden = 0xff800000u;    // -inf: a rejected block, or a key later than the query
+                  *reinterpret_cast<uint4*>(&lsum[quad * 64 + c]) =
+                      make_uint4(!row_live || (diag && key_local > c) ? hidden : sv[e], !row_live || (diag && key_local > c + 1) ? hidden : sv[e + 1],
+                                 !row_live || (diag && key_local > c + 2) ? hidden : sv[e + 2], !row_live || (diag && key_local > c + 3) ? hidden : sv[e + 3]);
+                }
               }
             }
           }
@@ -608,7 +621,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           if (named_bar_or(bar_vote, kGroupThreads, fail)) { ok = false; break; }
           if (gt < 64) {
             const float old = 0.f;                       // the first two S^T tiles of an item hold the raw scores
-            float nr = bf16_ceil(lsum[gt] + kFirstShift / sl2);
+            float nr = bf16_ceil(fmaxf(fmaxf(lsum[gt], lsum[64 + gt]), fmaxf(lsum[128 + gt], lsum[192 + gt])) + shift_raw);
             if (gt >= it.q_valid || !(fabsf(nr) < 3.0e38f)) nr = old;   // not a column of this block / not a finite score
             const float d = old - nr;
             rcur[gt] = nr;
@@ -732,15 +745,14 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             tc_commit(sh.bar(bb + FIXED));
           }
           if (have_ref) {                                // row sums (and, after the first tile, O^T) accumulated so far
-            // a reference that moved by more than 2^30 makes everything accumulated so far negligible (and the value
-            // taken out above may not have been finite): start the column afresh
+            // (beyond kAlphaGone the column starts afresh)
 #pragma unroll
             for (int c = 0; c < 64; c += 4) {
               const float4 a = *reinterpret_cast<const float4*>(&alpha[c]);
-              l_part[c] = a.x < 9.3e-10f ? 0.f : l_part[c] * a.x;
-              l_part[c + 1] = a.y < 9.3e-10f ? 0.f : l_part[c + 1] * a.y;
-              l_part[c + 2] = a.z < 9.3e-10f ? 0.f : l_part[c + 2] * a.z;
-              l_part[c + 3] = a.w < 9.3e-10f ? 0.f : l_part[c + 3] * a.w;
+              l_part[c] = a.x < kAlphaGone ? 0.f : l_part[c] * a.x;
+              l_part[c + 1] = a.y < kAlphaGone ? 0.f : l_part[c + 1] * a.y;
+              l_part[c + 2] = a.z < kAlphaGone ? 0.f : l_part[c + 2] * a.z;
+              l_part[c + 3] = a.w < kAlphaGone ? 0.f : l_part[c + 3] * a.w;
             }
 #pragma unroll 1
             for (int ch = 0; ch < (t >= 1 ? 4 : 0); ++ch) {
