@@ -208,7 +208,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   sh.abort_addr = sh.base + kOffMisc + 8;
   sh.limit_ns = (unsigned long long)m.wait_limit_us * 1000ull;
   unsigned char* smem = smem_raw + (sh.base - smem_u32(smem_raw));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // (warp-uniform for the compiler)
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
 
   if (threadIdx.x == 0) {
@@ -279,7 +279,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     // ========================================================================================== producers (TMA)
     // warps 0 / 2: Q and K of stream 0 / 1; warps 12 / 13: V of stream 0 / 1
     if (warp == 0 || warp == 2 || warp == 12 || warp == 13) {
-      if (lane == 0 && !(kBlockMax && warp >= 12)) {       // (no V in the block-maximum pass)
+      if (!(kBlockMax && warp >= 12)) if (elect_one()) {   // (no V in the block-maximum pass)
         const bool is_v = warp >= 12;
         const int s = is_v ? warp - 12 : warp >> 1, bb = s * kBarsPerStream;
         const uint32_t sbase = sh.base + (uint32_t)s * kStreamBytes;
@@ -344,7 +344,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     }
     // ========================================================================================== MMA issuer of a stream
     else if (warp == 1 || warp == 3) {
-      if (lane == 0) {
+      if (elect_one()) {
         const int s = warp >> 1, bb = s * kBarsPerStream;
         const uint32_t sbase = sh.base + (uint32_t)s * kStreamBytes;
         Tracer<kTrace> tr; tr.init(trace, s == 0 ? 1 : 3, smem + kOffTrace);

@@ -94,7 +94,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   }
   const uint32_t bar0 = base + kOffBar, abort_addr = base + kOffMisc + 4;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   const int row_tiles = (band.blk_hi - band.blk_lo + kRows - 1) / kRows;
   const int tile = row_tiles - 1 - (int)(blockIdx.x / band.heads);
@@ -165,7 +165,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
     // ------------------------------------------------------------------------------------------ MMAs
     // (the issuing threads copy nothing: a thread that waits for its own copies between two batches of MMAs leaves
     // the pipe idle for the latency of a copy, which was 40 % of the kernel)
-    if (lane == 0) {
+    if (elect_one()) {
       const int part = warp - 4;                          // 0: small terms, 1: large terms
       // (A plane, B plane): small = (hi, lo), (lo, hi), (mid, mid); large = (hi, mid), (mid, hi), (hi, hi)
       const int pa[3] = {0, part ? 1 : 2, part ? 0 : 1}, pb[3] = {part ? 1 : 2, 0, part ? 0 : 1};
