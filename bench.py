@@ -192,13 +192,11 @@ def cpu_oracle_sample(w, spec, rp, col, budget_rows=None):
             "mask_ms": 1e3 * mask_s}
 
 
-TIMELINE_TAGS = {1: "loop", 2: "wait for an empty K / V buffer", 10: "before S^T", 11: "wait K_FULL", 12: "S^T MMAs + commits",
-                 13: "before P V", 14: "wait V_FULL", 15: "wait P_FULL", 16: "P V MMAs + commits",
-                 29: "item start (decode, first list entries)", 30: "tile loop of an item (all tiles)", 31: "epilogue",
-                 32: "wait S_FULL", 33: "softmax pass (incl. first-tile references)", 34: "next list entries",
-                 35: "wait PV_DONE", 36: "vote (the group's barrier)", 37: "(branch)", 38: "P^T stores", 39: "proxy fence, arrive P_FULL",
-                 40: "rebase: wait next S^T + vote", 41: "rebase: TMEM reads", 42: "rebase: column maxima (shuffles)",
-                 43: "rebase: new references", 44: "rebase: fix MMAs, rescale", 45: "rebase: wait FIXED", 46: "rebase: pass + stores", 47: "next S_FULL test (waits behind the P^T stores)"}
+TIMELINE_TAGS = {1: "loop", 2: "copies of a tile (waits for empty units)", 10: "to the next S", 12: "S: wait K units, MMAs, commits",
+                 13: "to the next P V", 15: "wait P_FULL", 16: "P V: wait V units, MMAs, commits", 31: "list entry",
+                 32: "wait S_FULL", 33: "softmax pass (incl. first-tile reference)", 34: "store P, arrive P_FULL",
+                 36: "item start / end of the tile loop", 37: "epilogue: wait the last P V", 38: "epilogue: merge and store",
+                 40: "pass with a moved reference"}
 TIMELINE_ROLES = ["producer K+Q, stream 0", "issuer, stream 0", "producer V, stream 0", "issuer, stream 1",
                   "softmax group, stream 0", "softmax group, stream 1"]
 

@@ -35,7 +35,7 @@ struct Shared {
   uint32_t base;         // 1024-aligned shared address
   uint32_t bar0;         // shared address of mbarrier 0
   uint32_t abort_addr;   // shared address of the abort flag
-  unsigned long long limit_ns;   // a wait that lasts this long is declared lost (2 s unless a test shortens it)
+  uint32_t limit_us;     // a wait that lasts this long is declared lost (2 s unless a test shortens it)
   __device__ __forceinline__ uint32_t bar(int i) const { return bar0 + 8u * (uint32_t)i; }
   __device__ __forceinline__ uint32_t abort_flag() const { return abort_addr; }
 };
@@ -47,6 +47,23 @@ __device__ __forceinline__ uint32_t ld_shared_u32(uint32_t a) {
 }
 __device__ __forceinline__ void st_shared_u32(uint32_t a, uint32_t v) {
   asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void st_shared_v2(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.u32 [%0], {%1,%2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void st_shared_v4(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared_v4(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_shared_f32(uint32_t a) { return __uint_as_float(ld_shared_u32(a)); }
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t a) {
+  const uint4 v = ld_shared_v4(a);
+  return make_float4(__uint_as_float(v.x), __uint_as_float(v.y), __uint_as_float(v.z), __uint_as_float(v.w));
 }
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -72,7 +89,7 @@ __device__ __forceinline__ bool mbar_wait(const Shared& sh, int bar, uint32_t pa
     if (kSleepNs > 0) __nanosleep(kSleepNs);   // a waiting helper must not take issue slots from the softmax warps of its scheduler
     if ((it & 255u) == 0u) {
       if (ld_shared_u32(sh.abort_flag()) != 0u) return false;
-      if (global_ns() - t0 > sh.limit_ns) break;
+      if (global_ns() - t0 > (unsigned long long)sh.limit_us * 1000ull) break;
     }
   }
   st_shared_u32(sh.abort_flag(), 1u);
@@ -107,6 +124,17 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_
                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
                ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// Weight-stationary form, A from shared memory / from tensor memory (M = 64: see attn_tc.cu)
+__device__ __forceinline__ void tc_mma_ws(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+               "tcgen05.mma.ws.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+               ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tc_mma_ws_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+               "tcgen05.mma.ws.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+               ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
 __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
@@ -135,17 +163,16 @@ __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&r)[16])
                ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
                  "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
 }
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+                 "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+                 "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+                 "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]) : "memory");
+}
 // Same wait, with the loaded registers as in/out operands so that no use of them can be scheduled above it.
 __device__ __forceinline__ void tc_wait_ld(uint32_t (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :: "memory");
-}
-// No instruction: makes the registers of a load issued before the last wait depend on that wait.
-__device__ __forceinline__ void tc_tie(uint32_t (&r)[16]) {
-  asm volatile(""
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
                  "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
                :: "memory");
@@ -219,142 +246,44 @@ __device__ __forceinline__ int list_block(const Item& it, const int32_t* __restr
   return (j < 0 || j > it.i) ? -2 : j;
 }
 
-// The same in two steps, so that the load can be issued long before its result is looked at.
-__device__ __forceinline__ int list_fetch(const Item& it, const int32_t* __restrict__ col_idx, int p) {
-  return p < it.nlist ? __ldg(col_idx + it.l0 + p) : -1;
-}
-__device__ __forceinline__ int list_check(const Item& it, int p, int raw) {
-  if (p >= it.nlist) return -1;
-  return (raw < 0 || raw > it.i) ? -2 : raw;
-}
-
-// Maximum of each of 16 columns over the 32 lanes of a warp; lanes l and l ^ 1 end with column l >> 1.
-__device__ __forceinline__ float warp_colmax16(const float (&x)[16], int lane) {
-  float a[8], b[4], c[2];
-  {
-    const bool up = (lane & 16) != 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) a[i] = fmaxf(up ? x[i + 8] : x[i], __shfl_xor_sync(0xffffffffu, up ? x[i] : x[i + 8], 16));
-  }
-  {
-    const bool up = (lane & 8) != 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = fmaxf(up ? a[i + 4] : a[i], __shfl_xor_sync(0xffffffffu, up ? a[i] : a[i + 4], 8));
-  }
-  {
-    const bool up = (lane & 4) != 0;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) c[i] = fmaxf(up ? b[i + 2] : b[i], __shfl_xor_sync(0xffffffffu, up ? b[i] : b[i + 2], 4));
-  }
-  const bool up = (lane & 2) != 0;
-  const float d = fmaxf(up ? c[1] : c[0], __shfl_xor_sync(0xffffffffu, up ? c[0] : c[1], 2));
-  return fmaxf(d, __shfl_xor_sync(0xffffffffu, d, 1));
-}
-
-// Sums l[0..63] over the 32 lanes of a warp; lane ends with the totals of columns (2*bitrev-ish) base, base+1
-// where base = 32*b4 + 16*b3 + 8*b2 + 4*b1 + 2*b0 (b_i = bit i of the lane id).
-__device__ __forceinline__ void warp_colsum(float (&l)[64], int lane, float& out0, float& out1, int& base) {
-  float a[32];
-  {
-    const bool up = (lane & 16) != 0;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const float send = up ? l[i] : l[i + 32];
-      const float recv = __shfl_xor_sync(0xffffffffu, send, 16);
-      a[i] = (up ? l[i + 32] : l[i]) + recv;
-    }
-  }
-  float b[16];
-  {
-    const bool up = (lane & 8) != 0;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const float send = up ? a[i] : a[i + 16];
-      const float recv = __shfl_xor_sync(0xffffffffu, send, 8);
-      b[i] = (up ? a[i + 16] : a[i]) + recv;
-    }
-  }
-  float c[8];
-  {
-    const bool up = (lane & 4) != 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float send = up ? b[i] : b[i + 8];
-      const float recv = __shfl_xor_sync(0xffffffffu, send, 4);
-      c[i] = (up ? b[i + 8] : b[i]) + recv;
-    }
-  }
-  float d[4];
-  {
-    const bool up = (lane & 2) != 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float send = up ? c[i] : c[i + 4];
-      const float recv = __shfl_xor_sync(0xffffffffu, send, 2);
-      d[i] = (up ? c[i + 4] : c[i]) + recv;
-    }
-  }
-  {
-    const bool up = (lane & 1) != 0;
-    const float s0 = up ? d[0] : d[2], s1 = up ? d[1] : d[3];
-    const float r0 = __shfl_xor_sync(0xffffffffu, s0, 1), r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
-    out0 = (up ? d[2] : d[0]) + r0;
-    out1 = (up ? d[3] : d[1]) + r1;
-  }
-  base = ((lane >> 4) & 1) * 32 + ((lane >> 3) & 1) * 16 + ((lane >> 2) & 1) * 8 + ((lane >> 1) & 1) * 4 + (lane & 1) * 2;
-}
-
 // Optional cycle accounting of CTA 0 (diagnostics): every role attributes the clocks between two consecutive marks to the
-// tag of the later mark, accumulates per tag in shared memory, and writes the sums and mark counts to
-// trace[role * 8192 + tag * 2 ...] when it ends.
-constexpr int kTraceTags = 48;
+// tag of the later mark and adds them, and the mark, to trace[role * 8192 + tag * 2 ...] (reductions: nothing is waited for).
 template <bool ON>
 struct Tracer {
   unsigned long long* p;      // global destination (nullptr: off)
-  unsigned long long* acc;    // shared accumulators of this role: [tag][sum, count]
   long long last;
   bool on;
-  // Only every 8th tile is timed: the bookkeeping of a timed tile (~100 clocks per event) would otherwise slow the
-  // traced CTA by a quarter and distort what it measures.
+  // Only every 8th tile is timed, so that the bookkeeping does not distort what it measures.
   __device__ __forceinline__ void sample(uint32_t ordinal) {
     const bool was = on;
     on = p != nullptr && (ordinal & 7u) == 0u;
     if (on && !was) last = clock64();
   }
-  __device__ __forceinline__ void init(unsigned long long* base, int role, unsigned char* smem_trace) {
+  __device__ __forceinline__ void init(unsigned long long* base, int role) {
     p = (base != nullptr && blockIdx.x == 0) ? base + (size_t)role * 8192 : nullptr;
-    acc = reinterpret_cast<unsigned long long*>(smem_trace) + role * kTraceTags * 2;
-    if (p != nullptr) {
-      for (int i = 0; i < kTraceTags * 2; ++i) acc[i] = 0;
-      last = clock64();
-    }
+    last = 0;
     on = false;
   }
-  __device__ __forceinline__ void ev(uint32_t tag, uint32_t) {
+  __device__ __forceinline__ void ev(uint32_t tag) {
     if (on) {
       const long long now = clock64();
-      acc[2 * tag] += (unsigned long long)(now - last);
-      acc[2 * tag + 1] += 1;
+      asm volatile("red.global.add.u64 [%0], %1;" ::"l"(p + 2 * tag), "l"((unsigned long long)(now - last)) : "memory");
+      asm volatile("red.global.add.u64 [%0], %1;" ::"l"(p + 2 * tag + 1), "l"(1ull) : "memory");
       last = clock64();
     }
-  }
-  __device__ __forceinline__ void flush() {
-    if (p != nullptr)
-      for (int i = 0; i < kTraceTags * 2; ++i) p[i] = acc[i];
   }
 };
 template <>
 struct Tracer<false> {   // the production instantiation carries no state and no code
   __device__ __forceinline__ void sample(uint32_t) {}
-  __device__ __forceinline__ void init(unsigned long long*, int, unsigned char*) {}
-  __device__ __forceinline__ void ev(uint32_t, uint32_t) {}
-  __device__ __forceinline__ void flush() {}
+  __device__ __forceinline__ void init(unsigned long long*, int) {}
+  __device__ __forceinline__ void ev(uint32_t) {}
 };
 
-// kind::f16 instruction descriptor: fp32 accumulate, bf16 x bf16, M = 128, N = n
-constexpr uint32_t make_idesc(bool a_mn_major, bool b_mn_major, uint32_t n = 64u) {
+// kind::f16 instruction descriptor: fp32 accumulate, bf16 x bf16
+constexpr uint32_t make_idesc(bool a_mn_major, bool b_mn_major, uint32_t n = 64u, uint32_t m = 128u) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn_major ? 1u : 0u) << 15) | ((b_mn_major ? 1u : 0u) << 16) |
-         ((n >> 3) << 17) | ((128u >> 4) << 24);
+         ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 
 
