@@ -18,18 +18,23 @@ namespace seer {
 
 // ----------------------------------------------------------------------------------------------- kernel 1
 constexpr int kPoolThreads = 256;
+constexpr int kPoolChunkEx = 16;            // blocks per CTA of the variants' kernel
+constexpr unsigned kBigChunkFrom = 600;   // CTAs of 16 blocks from which the large chunk is taken
 
-// x = hi + mid + lo, each part the bf16 (round-to-nearest-even) of the remainder; the three planes of a tensor lie
-// `plane` elements apart.
-__device__ __forceinline__ void store_split3(uint16_t* __restrict__ dst, size_t plane, float x) {
+// Element o of the projected vector of block gb (numbered over the batch) as x = hi + mid + lo, each part the bf16
+// (round-to-nearest-even) of the remainder, into the tile layout of the head's planes.
+__device__ __forceinline__ void store_split3(char* __restrict__ head, int total_blocks, int gb, int o, float x) {
   const __nv_bfloat16 hi = __float2bfloat16_rn(x);
   const float r1 = x - __bfloat162float(hi);
   const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
   const float r2 = r1 - __bfloat162float(mid);
   const __nv_bfloat16 lo = __float2bfloat16_rn(r2);
-  dst[0] = __bfloat16_as_ushort(hi);
-  dst[plane] = __bfloat16_as_ushort(mid);
-  dst[2 * plane] = __bfloat16_as_ushort(lo);
+  const GateTile t(gb >> 6, total_blocks);
+  const int plane = t.rows * 256;
+  char* dst = head + t.base + (size_t)((o >> 6) * t.rows * 128 + (gb & 63) * 128 + ((((o >> 3) & 7) ^ (gb & 7)) << 4) + (o & 7) * 2);
+  *reinterpret_cast<uint16_t*>(dst) = __bfloat16_as_ushort(hi);
+  *reinterpret_cast<uint16_t*>(dst + plane) = __bfloat16_as_ushort(mid);
+  *reinterpret_cast<uint16_t*>(dst + 2 * plane) = __bfloat16_as_ushort(lo);
 }
 
 __device__ __forceinline__ uint4 ld_stream_16(const void* p) {
@@ -46,14 +51,25 @@ __device__ __forceinline__ void acc_bf16x8(float (&a)[8], const uint4& u) {
   a[6] += __uint_as_float(u.w << 16); a[7] += __uint_as_float(u.w & 0xffff0000u);
 }
 
-// grid.x = total_chunks * (Hq + Hkv); the head varies fastest so that CTAs running together read
-// neighbouring 256-byte segments of the same token rows.  A chunk is 16 consecutive blocks of the packed batch, whatever
-// sequences they belong to (a chunk per sequence would leave most of a CTA idle on batches of short sequences).
-__global__ void __launch_bounds__(kPoolThreads)
+// One CTA pools and projects kChunk consecutive blocks of the packed batch (whatever sequences they belong to: a chunk per
+// sequence would leave most of a CTA idle on batches of short ones) for one head.  grid.x = chunks * (Hq + Hkv); the head
+// varies fastest so that CTAs running together read neighbouring 256-byte segments of the same token rows.
+//
+// What bounds it: the bytes of Q and K in a large batch; in a small one the latency of a CTA's loads, one after the other,
+// because there are too few CTAs.  So a chunk is 16 blocks where that still makes more than a wave of CTAs (the head's 64 KB
+// matrix, read once per CTA from L2, is then a fifth of its traffic) and 2 blocks otherwise, with four warps per block.
+// The sums are formed in the same order for every chunk size (16 rows at a time; the two halves of the matrix's rows apart),
+// so the result does not depend on it.
+template <int kChunk>
+__global__ void __launch_bounds__(kPoolThreads, kChunk == 16 ? 3 : 1)
 pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
-                    const float* __restrict__ Wq, const float* __restrict__ Wk, uint16_t* __restrict__ gq,
-                    uint16_t* __restrict__ gk) {
-  __shared__ __align__(16) float pooled[kPoolChunk][kHeadDim];
+                    const float* __restrict__ Wq, const float* __restrict__ Wk, char* __restrict__ gq,
+                    char* __restrict__ gk) {
+  constexpr int kWarps = kPoolThreads / 32;
+  constexpr int kSplit = kChunk < kWarps ? kWarps / kChunk : 1;      // warps per block
+  constexpr int kMaxSteps = 8;                                       // groups of 16 rows in a block of 128 tokens
+  __shared__ __align__(16) float pooled[kChunk][kHeadDim];
+  __shared__ __align__(16) float part[kSplit > 1 ? kChunk * kMaxSteps * 2 * kHeadDim : kChunk * kHeadDim];
 
   const int heads_total = m.num_q_heads + m.num_kv_heads;
   const int chunk = blockIdx.x / heads_total;
@@ -63,18 +79,18 @@ pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* _
   const int h = is_q ? hh : hh - m.num_q_heads;
   const uint16_t* __restrict__ x = is_q ? q : k;
   const float* __restrict__ W = (is_q ? Wq : Wk) + (size_t)h * kHeadDim * kGateDim;
-  uint16_t* __restrict__ out = is_q ? gq : gk;
-  const size_t plane = (size_t)H * m.total_blocks * kGateDim;   // elements between the hi / mid / lo planes
+  char* __restrict__ out = (is_q ? gq : gk) + (size_t)h * m.total_blocks * kGatePairBytes;
 
-  const int g0 = chunk * kPoolChunk;                            // first block of the chunk, numbered over the batch
-  const int nblk = min(kPoolChunk, m.total_blocks - g0);
+  const int g0 = chunk * kChunk;                                // first block of the chunk, numbered over the batch
+  const int nblk = min(kChunk, m.total_blocks - g0);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int half = lane >> 4, cchunk = lane & 15;
   const size_t row_stride = (size_t)H * kHeadDim;  // elements between consecutive tokens
+  const int steps = m.block / 16;
   bool any = false;
 
-  for (int bi = warp; bi < nblk; bi += kPoolThreads / 32) {
+  for (int bi = warp / kSplit; bi < nblk; bi += kWarps / kSplit) {
     const int b = find_sequence(m.blk_off, m.batch, g0 + bi);
     const int i = g0 + bi - m.blk_off[b];
     const int s0 = m.cu_seqlens[b], s1 = m.cu_seqlens[b + 1];
@@ -87,46 +103,83 @@ pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* _
     const uint16_t* base = x + ((ptrdiff_t)t0 + q_shift) * (ptrdiff_t)row_stride + (size_t)h * kHeadDim + cchunk * 8;
     float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 1
-    for (int it = 0; it < m.block / 2; it += 8) {
+    for (int st = warp % kSplit; st < steps; st += kSplit) {
       uint4 u[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const int row = 2 * (it + j) + half;
+        const int row = 16 * st + 2 * j + half;
         u[j] = row < cnt ? ld_stream_16(base + (size_t)row * row_stride) : make_uint4(0, 0, 0, 0);
       }
+      float t[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc_bf16x8(a, u[j]);
-    }
-    const float inv = cnt > 0 ? 1.0f / (float)cnt : 0.f;
+      for (int j = 0; j < 8; ++j) acc_bf16x8(t, u[j]);
+      if (kSplit > 1) {
+        float4* dst = reinterpret_cast<float4*>(&part[((bi * kMaxSteps + st) * 2 + half) * kHeadDim + cchunk * 8]);
+        dst[0] = make_float4(t[0], t[1], t[2], t[3]);
+        dst[1] = make_float4(t[4], t[5], t[6], t[7]);
+      } else {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      a[j] += __shfl_xor_sync(0xffffffffu, a[j], 16);
-      a[j] *= inv;
+        for (int j = 0; j < 8; ++j) a[j] = __fadd_rn(a[j], t[j]);
+      }
     }
-    if (half == 0) {
-      float4* dst = reinterpret_cast<float4*>(&pooled[bi][cchunk * 8]);
-      dst[0] = make_float4(a[0], a[1], a[2], a[3]);
-      dst[1] = make_float4(a[4], a[5], a[6], a[7]);
-    }
+    if (kSplit == 1) {
+      const float inv = cnt > 0 ? 1.0f / (float)cnt : 0.f;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) a[j] = __fmul_rn(__fadd_rn(a[j], __shfl_xor_sync(0xffffffffu, a[j], 16)), inv);
+      if (half == 0) {
+        float4* dst = reinterpret_cast<float4*>(&pooled[bi][cchunk * 8]);
+        dst[0] = make_float4(a[0], a[1], a[2], a[3]);
+        dst[1] = make_float4(a[4], a[5], a[6], a[7]);
+      }
+    } else if (lane == 0 && warp % kSplit == 0) pooled[bi][0] = cnt > 0 ? 1.0f / (float)cnt : 0.f;   // (until the sums are combined)
   }
   if (!__syncthreads_or(any ? 1 : 0)) return;                   // every block of the chunk lies before its queries
+  if (kSplit > 1) {
+    float v[(kChunk * kHeadDim + kPoolThreads - 1) / kPoolThreads];
+    int e = 0;
+#pragma unroll
+    for (int idx = threadIdx.x; idx < kChunk * kHeadDim; idx += kPoolThreads, ++e) {
+      const int bi = idx / kHeadDim, c = idx % kHeadDim;
+      float s0 = 0.f, s1 = 0.f;
+      for (int st = 0; st < steps; ++st) {
+        s0 = __fadd_rn(s0, part[((bi * kMaxSteps + st) * 2) * kHeadDim + c]);
+        s1 = __fadd_rn(s1, part[((bi * kMaxSteps + st) * 2 + 1) * kHeadDim + c]);
+      }
+      v[e] = __fmul_rn(__fadd_rn(s0, s1), pooled[bi][0]);
+    }
+    __syncthreads();
+    e = 0;
+#pragma unroll
+    for (int idx = threadIdx.x; idx < kChunk * kHeadDim; idx += kPoolThreads, ++e) pooled[idx / kHeadDim][idx % kHeadDim] = v[e];
+    __syncthreads();
+  }
 
-  // projection: thread -> output column o, 8 of the 16 blocks
+  // projection: a thread takes output column o, one half of the matrix's rows and all blocks of the chunk
   const int o = threadIdx.x & (kGateDim - 1);
-  const int grp = threadIdx.x >> 7;  // 0 or 1
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-  for (int c = 0; c < kHeadDim; ++c) {
-    const float w = __ldg(W + (size_t)c * kGateDim + o);
+  const int ch = threadIdx.x >> 7;
+  float acc[kChunk];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = fmaf(pooled[grp * 8 + j][c], w, acc[j]);
-  }
-  const size_t obase = ((size_t)h * m.total_blocks + g0) * kGateDim;
+  for (int j = 0; j < kChunk; ++j) acc[j] = 0.f;
+  const float* __restrict__ Wh = W + (size_t)ch * 64 * kGateDim + o;
+#pragma unroll 2
+  for (int c = 0; c < 64; c += 8) {
+    float w[8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int bi = grp * 8 + j;
-    if (bi < nblk) store_split3(out + obase + (size_t)bi * kGateDim + o, plane, acc[j]);
+    for (int e = 0; e < 8; ++e) w[e] = __ldg(Wh + (size_t)(c + e) * kGateDim);
+#pragma unroll
+    for (int j = 0; j < kChunk; ++j) {
+      const float4 p0 = *reinterpret_cast<const float4*>(&pooled[j][ch * 64 + c]), p1 = *reinterpret_cast<const float4*>(&pooled[j][ch * 64 + c + 4]);
+      acc[j] = fmaf(p0.x, w[0], acc[j]); acc[j] = fmaf(p0.y, w[1], acc[j]); acc[j] = fmaf(p0.z, w[2], acc[j]); acc[j] = fmaf(p0.w, w[3], acc[j]);
+      acc[j] = fmaf(p1.x, w[4], acc[j]); acc[j] = fmaf(p1.y, w[5], acc[j]); acc[j] = fmaf(p1.z, w[6], acc[j]); acc[j] = fmaf(p1.w, w[7], acc[j]);
+    }
   }
+  // the halves are added by the thread that stores: the first half of the threads the first half of the blocks
+#pragma unroll
+  for (int j = 0; j < kChunk; ++j) if ((j >= kChunk / 2) != (ch == 1)) part[j * kGateDim + o] = acc[j];
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kChunk; ++j)
+    if ((j >= kChunk / 2) == (ch == 1) && j < nblk) store_split3(out, m.total_blocks, g0 + j, o, __fadd_rn(acc[j], part[j * kGateDim + o]));
 }
 
 
@@ -154,10 +207,11 @@ __device__ __forceinline__ void min_bf16x8(float (&a)[8], const uint4& u) {
 
 __global__ void __launch_bounds__(kPoolThreads)
 pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
-                       const float* __restrict__ Wq, const float* __restrict__ Wk, uint16_t* __restrict__ gq,
-                       uint16_t* __restrict__ gk, uint32_t pool_q, uint32_t pool_k, float rope_theta) {
-  __shared__ __align__(16) float pooled[kPoolChunk][3 * kHeadDim];
-  __shared__ int block_pos[kPoolChunk];                        // position of each block in its sequence (block RoPE)
+                       const float* __restrict__ Wq, const float* __restrict__ Wk, char* __restrict__ gq,
+                       char* __restrict__ gk, uint32_t pool_q, uint32_t pool_k, float rope_theta) {
+  constexpr int kChunk = kPoolChunkEx;
+  __shared__ __align__(16) float pooled[kChunk][3 * kHeadDim];
+  __shared__ int block_pos[kChunk];                        // position of each block in its sequence (block RoPE)
 
   const int heads_total = m.num_q_heads + m.num_kv_heads;
   const int chunk = blockIdx.x / heads_total;
@@ -170,15 +224,14 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
   const int width = nparts * kHeadDim;                       // rows of the head's gate matrix
   const uint16_t* __restrict__ x = is_q ? q : k;
   const float* __restrict__ W = (is_q ? Wq : Wk) + (size_t)h * width * kGateDim;
-  uint16_t* __restrict__ out = is_q ? gq : gk;
-  const size_t plane = (size_t)H * m.total_blocks * kGateDim;   // elements between the hi / mid / lo planes
+  char* __restrict__ out = (is_q ? gq : gk) + (size_t)h * m.total_blocks * kGatePairBytes;
   // offsets of the parts inside the concatenated vector (order: average, max, min)
   const int off_avg = 0;
   const int off_max = (methods & SEER_POOL_AVG) ? kHeadDim : 0;
   const int off_min = off_max + ((methods & SEER_POOL_MAX) ? kHeadDim : 0);
 
-  const int g0 = chunk * kPoolChunk;                            // first block of the chunk, numbered over the batch
-  const int nblk = min(kPoolChunk, m.total_blocks - g0);
+  const int g0 = chunk * kChunk;                            // first block of the chunk, numbered over the batch
+  const int nblk = min(kChunk, m.total_blocks - g0);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int half = lane >> 4, cchunk = lane & 15;
@@ -245,11 +298,17 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
   const int o = threadIdx.x & (kGateDim - 1);
   const int grp = threadIdx.x >> 7;  // 0 or 1
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-  for (int c = 0; c < width; ++c) {
-    const float w = __ldg(W + (size_t)c * kGateDim + o);
+#pragma unroll 2
+  for (int c = 0; c < width; c += 8) {
+    float w[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = fmaf(pooled[grp * 8 + j][c], w, acc[j]);
+    for (int e = 0; e < 8; ++e) w[e] = __ldg(W + (size_t)(c + e) * kGateDim + o);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float4 p0 = *reinterpret_cast<const float4*>(&pooled[grp * 8 + j][c]), p1 = *reinterpret_cast<const float4*>(&pooled[grp * 8 + j][c + 4]);
+      acc[j] = fmaf(p0.x, w[0], acc[j]); acc[j] = fmaf(p0.y, w[1], acc[j]); acc[j] = fmaf(p0.z, w[2], acc[j]); acc[j] = fmaf(p0.w, w[3], acc[j]);
+      acc[j] = fmaf(p1.x, w[4], acc[j]); acc[j] = fmaf(p1.y, w[5], acc[j]); acc[j] = fmaf(p1.z, w[6], acc[j]); acc[j] = fmaf(p1.w, w[7], acc[j]);
+    }
   }
   if (rope_theta > 0.f) {
     // rotate (o, o + dg/2) pairs: the partner's value goes through shared memory (the pooled vectors are no longer needed)
@@ -270,63 +329,89 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
                                   : (float)((double)acc[j] * cs + (double)partner * sn);
     }
   }
-  const size_t obase = ((size_t)h * m.total_blocks + g0) * kGateDim;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const int bi = grp * 8 + j;
-    if (bi < nblk) store_split3(out + obase + (size_t)bi * kGateDim + o, plane, acc[j]);
+    if (bi < nblk) store_split3(out, m.total_blocks, g0 + bi, o, acc[j]);
   }
 }
 
 // ----------------------------------------------------------------------------------------------- kernel 2
 // gate_scores_kernel (tcgen05) lives in gate_scores.cu.
+int launch_gate_stats(const SeqMeta& m, const uint16_t* gq, const uint16_t* gk, float2* stats, int* status, cudaStream_t stream);
 int launch_gate_scores(const SeqMeta& m, const ScoreBand& band, const uint16_t* gq, const uint16_t* gk, float* scores,
-                       int* status, cudaStream_t stream);
+                       float2* stats, int* status, int num_sms, cudaStream_t stream);
 bool init_gate_scores();
+
+namespace {
+// The workspace: planes of gq, of gk, statistics.
+struct GateWs {
+  char *gq, *gk;
+  float2* stats;
+  GateWs(const SeqMeta& m, void* ws) {
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    gq = (char*)ws;
+    gk = gq + up((size_t)m.num_q_heads * m.total_blocks * kGatePairBytes);
+    stats = (float2*)(gk + up((size_t)m.num_kv_heads * m.total_blocks * kGatePairBytes));
+  }
+};
+
+int launch_scores_whole(seer_ctx* ctx, const SeqMeta& m, const GateWs& w, float* scores, cudaStream_t stream) {
+  // (the fixed scratch of the allocation-free variant, which has no context, has no room for the statistics)
+  int* status = ctx ? ctx->d_status : nullptr;
+  float2* stats = ctx && gate_split(m, ctx->num_sms) ? w.stats : nullptr;
+  const int n1 = stats ? launch_gate_stats(m, (const uint16_t*)w.gq, (const uint16_t*)w.gk, stats, status, stream) : 0;
+  if (n1 < 0) return n1;
+  const ScoreBand all = {m.first_q_block, m.total_blocks, 0, m.num_q_heads, 0, 0, 0};
+  const int n2 = launch_gate_scores(m, all, (const uint16_t*)w.gq, (const uint16_t*)w.gk, scores, stats, status, ctx ? ctx->num_sms : 0, stream);
+  return n2 < 0 ? n2 : n1 + n2;
+}
+}  // namespace
 
 int launch_gate(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const float* Wq, const float* Wk,
                 float* scores, void* ws, cudaStream_t stream) {
-  // three bf16 planes per tensor (hi, mid, lo of the fp32 value)
-  size_t gq_bytes = ((size_t)m.num_q_heads * m.total_blocks * kGateDim * 6 + 255) / 256 * 256;
-  uint16_t* gq = (uint16_t*)ws;
-  uint16_t* gk = (uint16_t*)((char*)ws + gq_bytes);
-  const unsigned grid1 = (unsigned)m.total_chunks * (unsigned)(m.num_q_heads + m.num_kv_heads);
-  pool_project_kernel<<<grid1, kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, gq, gk);
-  if (scores == nullptr) {                             // projection only: the scores follow band by band
-    cudaError_t e0 = cudaGetLastError();
-    return e0 == cudaSuccess ? 1 : -(int)e0;
-  }
-  const ScoreBand all = {0, m.total_blocks, 0, m.num_q_heads, 0};
-  const int n2 = launch_gate_scores(m, all, gq, gk, scores, ctx ? ctx->d_status : nullptr, stream);
+  const GateWs w(m, ws);
+  const unsigned heads = (unsigned)(m.num_q_heads + m.num_kv_heads);
+  const unsigned big = (unsigned)((m.total_blocks + 15) / 16) * heads;
+  if (big > kBigChunkFrom)
+    pool_project_kernel<16><<<big, kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk);
+  else
+    pool_project_kernel<2><<<(unsigned)((m.total_blocks + 1) / 2) * heads, kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk);
+  cudaError_t e0 = cudaGetLastError();
+  if (e0 != cudaSuccess) return -(int)e0;
+  if (scores == nullptr) return 1;                     // projection only: the scores follow band by band
+  const int n2 = launch_scores_whole(ctx, m, w, scores, stream);
   return n2 < 0 ? n2 : 1 + n2;
 }
 
 int launch_gate_ex(seer_ctx* ctx, const SeqMeta& m, const seer_gate_options& opt, const void* q, const void* k,
                    const float* Wq, const float* Wk, float* scores, void* ws, cudaStream_t stream) {
-  (void)ctx;
-  // three bf16 planes per tensor (hi, mid, lo of the fp32 value)
-  size_t gq_bytes = ((size_t)m.num_q_heads * m.total_blocks * kGateDim * 6 + 255) / 256 * 256;
-  uint16_t* gq = (uint16_t*)ws;
-  uint16_t* gk = (uint16_t*)((char*)ws + gq_bytes);
-  const unsigned grid1 = (unsigned)m.total_chunks * (unsigned)(m.num_q_heads + m.num_kv_heads);
-  pool_project_ex_kernel<<<grid1, kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, gq, gk,
+  // averages alone and no rotation: the plain gate
+  if (opt.pool_q == SEER_POOL_AVG && opt.pool_k == SEER_POOL_AVG && opt.rope_theta == 0.f) return launch_gate(ctx, m, q, k, Wq, Wk, scores, ws, stream);
+  const GateWs w(m, ws);
+  const unsigned grid1 = (unsigned)((m.total_blocks + kPoolChunkEx - 1) / kPoolChunkEx) * (unsigned)(m.num_q_heads + m.num_kv_heads);
+  pool_project_ex_kernel<<<grid1, kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk,
                                                               opt.pool_q, opt.pool_k, opt.rope_theta);
-  if (scores == nullptr) {                             // projection only: the scores follow band by band
-    cudaError_t e0 = cudaGetLastError();
-    return e0 == cudaSuccess ? 1 : -(int)e0;
-  }
-  const ScoreBand all = {0, m.total_blocks, 0, m.num_q_heads, 0};
-  const int n2 = launch_gate_scores(m, all, gq, gk, scores, ctx ? ctx->d_status : nullptr, stream);
+  cudaError_t e0 = cudaGetLastError();
+  if (e0 != cudaSuccess) return -(int)e0;
+  if (scores == nullptr) return 1;
+  const int n2 = launch_scores_whole(ctx, m, w, scores, stream);
   return n2 < 0 ? n2 : 1 + n2;
 }
 
-// Scores of one band from the projected vectors launch_gate_ex(scores = nullptr) left in `ws`.
-int launch_gate_scores_band(const SeqMeta& m, const ScoreBand& band, const void* ws, float* scores, cudaStream_t stream) {
-  size_t gq_bytes = ((size_t)m.num_q_heads * m.total_blocks * kGateDim * 6 + 255) / 256 * 256;
-  const uint16_t* gq = (const uint16_t*)ws;
-  const uint16_t* gk = (const uint16_t*)((const char*)ws + gq_bytes);
-  return launch_gate_scores(m, band, gq, gk, scores, nullptr, stream);
+int launch_gate_stats_all(seer_ctx* ctx, const SeqMeta& m, void* ws, cudaStream_t stream) {
+  const GateWs w(m, ws);
+  return launch_gate_stats(m, (const uint16_t*)w.gq, (const uint16_t*)w.gk, w.stats, ctx->d_status, stream);
 }
+
+int launch_gate_scores_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& band, void* ws, float* scores, bool with_stats,
+                            cudaStream_t stream) {
+  const GateWs w(m, ws);
+  return launch_gate_scores(m, band, (const uint16_t*)w.gq, (const uint16_t*)w.gk, scores, with_stats ? w.stats : nullptr, ctx->d_status,
+                            ctx->num_sms, stream);
+}
+
+const float2* gate_stats(const SeqMeta& m, void* ws) { return GateWs(m, ws).stats; }
 
 // ----------------------------------------------------------------------------------------------- allocation-free variant
 // Scratch for seer_gate_scores_static lives in the library image: every GPU that loads the library carries these
@@ -366,7 +451,7 @@ seer_status gate_scores_static(const seer_shape* shape, const void* q, const voi
   if (t.total_blocks == 0) return SEER_OK;
   if (!q || !k || !Wq || !Wk || !scores) return SEER_ERR_INVALID_ARG;
   // sizes beyond the built-in scratch are refused, never truncated
-  if (shape->batch > kStaticMaxBatch || gate_workspace_bytes(t, shape) > kStaticScratchBytes) return SEER_ERR_WORKSPACE;
+  if (shape->batch > kStaticMaxBatch || gate_planes_bytes(t, shape) > kStaticScratchBytes) return SEER_ERR_WORKSPACE;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kStaticMaxDevices) return SEER_ERR_CUDA;
   unsigned char* base = nullptr;
@@ -405,7 +490,6 @@ seer_status gate_scores_static(const seer_shape* shape, const void* q, const voi
   m.group = shape->num_q_heads / shape->num_kv_heads;
   m.total_tokens = (int32_t)t.total_tokens;
   m.total_blocks = (int32_t)t.total_blocks;
-  m.total_chunks = (int32_t)t.total_chunks;
   m.max_nb = t.max_nb;
   m.rows = t.rows;
   m.score_elems = t.score_elems;
@@ -414,6 +498,7 @@ seer_status gate_scores_static(const seer_shape* shape, const void* q, const voi
   m.qoff = nullptr; m.qdelta = nullptr; m.chunked = 0;
   m.total_q_tokens = (int32_t)t.total_tokens;
   m.wait_limit_us = 0u; m.lose_v_copy = -1;   // unused by the gate
+  m.score_tiles = 0; m.first_q_block = 0;
   // The two kernels below are the ones seer_gate_scores launches; only the scratch pointer differs.  Nothing in the
   // scratch has to start at zero: the first kernel writes every projected vector the second one reads.
   const int n = launch_gate(nullptr, m, q, k, Wq, Wk, scores, base + kStaticMetaBytes, stream);

@@ -1,22 +1,30 @@
-// AttnGate, second kernel (Sec. 3.1, Eq. 1): logits = gq gk^T / sqrt(dg) over the causal blocks, row softmax -> scores.
+// AttnGate, second stage (Sec. 3.1, Eq. 1): logits = gq gk^T / sqrt(dg) over the causal blocks, row softmax -> scores.
 //
 // The logits need fp32-grade products (bf16 or tf32 inputs would not hold the 1e-3 relative bound on softmax outputs
 // when logits reach tens), so gq and gk arrive as three bf16 planes each, x = hi + mid + lo, and the product is the six
 // terms hi*lo + lo*hi + mid*mid (small) and hi*mid + mid*hi + hi*hi (large) (what is dropped is below 2^-24 of the
 // product), accumulated in fp32 TMEM accumulators by tcgen05.mma: 6 x 8 K-steps of M = 128, N = 64, K = 16 per tile.
 //
-// One CTA = 128 consecutive block rows of one head (rows of the packed batch, whatever sequences they belong to), walked
-// over the causal column tiles of 64 blocks twice: the first sweep keeps the running maximum and sum of every row (a
-// thread owns a row: TMEM lane = row, so neither needs a shuffle), the second recomputes the logits and writes
-// exp(x - m) / l: every score is written once and never read back.  The finished tile goes through shared memory so
-// that a warp writes whole 256-byte row segments (a thread storing its own row scatters 16-byte pieces over 32 rows
-// per instruction: measured three times slower).
+// What bounds it: the MMAs.  The rows' planes are the A operand in tensor memory (192 columns, written once per CTA):
+// an MMA then reads 2 KB of shared memory instead of 6 and takes 34 clocks instead of 48.
 //
-// Roles (320 threads): warps 0-3 own the rows (epilogue), warps 6-9 copy the operand tiles (cp.async into the 128-byte
-// swizzled K-major layout the MMA descriptors expect); one thread of warp 4 and one of warp 5 issue the MMAs, one the
-// three small terms, the other the three large ones, each into its own accumulator (one thread starts an MMA about every 100 clocks, two
-// keep the pipe at the 48 clocks an N = 64 instruction occupies it); the rows add the two.  Two accumulator pairs and
-// two B buffers: the MMAs of tile n + 1 run while the rows work on tile n.
+// One CTA = 128 consecutive block rows of one head (rows of the packed batch, whatever sequences they belong to) times a
+// range of column tiles of 64 blocks (tiles of the packed batch, aligned to 64).  A score needs the softmax statistics of
+// its whole row first, so every tile is computed twice and every score is written once:
+//   kBoth   one CTA walks all causal tiles of its rows twice (short sequences: one launch)
+//   kStats  a CTA walks one segment of up to SegTiles tiles and leaves the rows' (maximum, sum) of that segment
+//   kWrite  a CTA walks part_tiles tiles, after combining its rows' statistics, and writes exp(x - m) / l
+// With long sequences the first form has few CTAs of very unequal length (one head of a 262 144-token prompt: 32 CTAs, 245 us
+// a launch).  Statistics are always formed per segment of the batch's column grid and combined in segment order, so the
+// scores are the same bit for bit whichever form computes them and however the rows are grouped into calls.
+//
+// Roles (608 threads): warps 0-15 own the rows in two groups, one for the even, one for the odd tiles of the column grid, each
+// with an accumulator pair of its own (a warp takes 32 rows x 32 of a tile's 64 columns: TMEM lane = row, so maxima and sums
+// need no shuffle; one group took 2900 clocks per tile, the MMAs 1650); one thread of warp 16 issues the small terms, one of
+// warp 17 the large ones, each into its own accumulator (the rows add the two), one of warp 18 copies the column tiles (one
+// 48 KB bulk copy each: the first stage stores the planes in the swizzled tile layout).  A finished tile goes through shared
+// memory so that a warp writes whole 128-byte row segments (a thread storing its own row scatters 16-byte pieces over 32 rows:
+// three times slower).
 #include <cuda_bf16.h>
 #include <math_constants.h>
 
@@ -30,62 +38,59 @@ using namespace tcc;
 namespace gs {
 constexpr int kRows = 128;                         // score rows per CTA
 constexpr int kCols = kScoreTile;                  // columns per tile (64)
-constexpr int kThreads = 320;
-constexpr uint32_t kAPlane = kRows * kGateDim * 2;   // 32 KB: one plane of the 128 x 128 A tile, [2 k halves][128 rows][128 B]
-constexpr uint32_t kBPlane = kCols * kGateDim * 2;   // 16 KB: one plane of a 64 x 128 B tile
-constexpr uint32_t kOffA = 0;
-constexpr uint32_t kOffB = 3 * kAPlane;              // two buffers of three planes
+constexpr int kRowThreads = 512;                   // two groups of eight warps
+constexpr int kThreads = kRowThreads + 96;
+constexpr uint32_t kBPlane = kCols * kGateDim * 2;   // 16 KB: one plane of a column tile, [2 k halves][64 rows][128 B]
 constexpr uint32_t kBBuf = 3 * kBPlane;
-constexpr uint32_t kOffStage = kOffB + 2 * kBBuf;    // [128 rows][64 columns] fp32, 16-byte chunks XOR (row % 16): 32 KB
-constexpr uint32_t kOffMeta = kOffStage + kRows * kCols * 4;   // per row: element offset of column 0 (int64), first and last causal block
-constexpr uint32_t kOffBar = kOffMeta + kRows * 16;  // mbarriers: ACC_FULL[2], ACC_EMPTY[2], B_FULL[2]
-constexpr uint32_t kOffMisc = kOffBar + 64;          // tmem base, abort flag
+constexpr uint32_t kBBufs = 3;
+constexpr uint32_t kOffStage = kBBufs * kBBuf;       // 16 warps x [32 rows][32 columns] fp32; in the first sweep: (m, l) of the parts
+constexpr uint32_t kOffMeta = kOffStage + 16 * 4096;   // per row: element offset of column 0 (int64), first and last causal block
+constexpr uint32_t kOffBar = kOffMeta + kRows * 16;
+constexpr uint32_t kOffMisc = kOffBar + 128;         // tmem base, abort flag
 constexpr uint32_t kSmemBytes = kOffMisc + 64;
 static_assert(kSmemBytes <= 232448, "shared memory budget of one CTA");
-enum Bar { ACC_FULL = 0, ACC_EMPTY = 2, B_FULL = 4 };
-constexpr int kLoaders = 128;                       // threads of the four copying warps
-constexpr uint32_t kTmemCols = 256;                  // two buffers x (small terms, large terms) x 64 columns
+enum Bar { ACC_FULL = 0 /* + acc */, ACC_EMPTY = 2, B_FULL = 4 /* + buf */, B_EMPTY = 4 + kBBufs, A_FULL = 4 + 2 * kBBufs, kBars = A_FULL + 1 };
+constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kColA = 256;                      // columns 0..255: two accumulator pairs; 256..447: the A planes
 constexpr uint32_t kIdesc = make_idesc(false, false, kCols);
-constexpr uint32_t kWaitSpins = 1u << 24;          // a wait that lasts this many polls (seconds) is declared lost
+constexpr uint32_t kWaitSpins = 1u << 24;            // a wait that lasts this many polls (seconds) is declared lost
+enum Mode { kBoth = 0, kStats = 1, kWrite = 2 };
 
 // Bounded wait that never changes the control flow: after the limit the error is recorded and the wait counts as
 // satisfied, so every role still reaches its barriers and the CTA ends normally (with a wrong result and a status).
 __device__ __forceinline__ void wait_bar(uint32_t bar, uint32_t parity, uint32_t abort_addr, int* status) {
-  for (uint32_t it = 0; it < kWaitSpins; ++it)
+  for (uint32_t it = 0; it < kWaitSpins; ++it) {
     if (mbar_try(bar, parity)) return;
+    if ((it & 255u) == 255u && ld_shared_u32(abort_addr) != 0u) return;
+  }
   st_shared_u32(abort_addr, 1u);
   if (status != nullptr) atomicCAS(status, 0, (int)SEER_ERR_TIMEOUT);
 }
 
-// Rows r0 .. r0 + rows - 1 of the three planes of src ([blocks][128] bf16 each, `plane` elements apart) into the
-// swizzled K-major tile layout: k half (64 elements = 128 bytes per row) -> 8-row group (1024 bytes) -> row -> 16-byte
-// chunk XOR (row % 8).  Rows at or beyond rows_valid are zero-filled.
-template <int ROWS>
-__device__ __forceinline__ void load_planes(uint32_t dst, uint32_t plane_bytes, const uint16_t* __restrict__ src, size_t plane,
-                                            int r0, int rows_valid, int tid, int nthreads) {
-  for (int idx = tid; idx < 3 * ROWS * 16; idx += nthreads) {
-    const int pl = idx / (ROWS * 16), rem = idx - pl * (ROWS * 16);
-    const int row = rem >> 4, chunk = rem & 15;
-    const bool ok = row < rows_valid;
-    const uint16_t* g = src + (size_t)pl * plane + (size_t)(r0 + (ok ? row : 0)) * kGateDim + chunk * 8;
-    const uint32_t at = dst + (uint32_t)pl * plane_bytes + (uint32_t)(chunk >> 3) * (ROWS * 128u) + (uint32_t)(row >> 3) * 1024u +
-                        (uint32_t)(row & 7) * 128u + (uint32_t)(((chunk & 7) ^ (row & 7)) << 4);
-    const int sz = ok ? 16 : 0;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(at), "l"(g), "r"(sz) : "memory");
-  }
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+
+// (m, l) of two disjoint sets of a row's columns, in units of log2: l counts 2^(x - m); m = -inf: empty
+__device__ __forceinline__ void combine(float& m, float& l, float m2, float l2) {
+  const float nm = fmaxf(m, m2);
+  const float f = m == -CUDART_INF_F ? 0.f : ex2f(m - nm), f2 = m2 == -CUDART_INF_F ? 0.f : ex2f(m2 - nm);
+  l = __fadd_rn(__fmul_rn(l, f), __fmul_rn(l2, f2));
+  m = nm;
 }
 }  // namespace gs
 
-// grid.x = row tiles * band.heads (head fastest; row tiles are visited from the last rows to the first).  Row r of a
-// tile is query block i_r of sequence b_r; its causal columns are that sequence's blocks 0 .. i_r, i.e. the blocks
-// seq_start_r .. r of the batch.  The CTA walks the column tiles from the sequence start of its first row to its last
-// row; entries of other sequences are masked.  The whole problem is the band (0, total_blocks, 0, Hq, 0).  Scores are
-// written at their offset in the full matrix minus band.score_base.
+// grid.x = row tiles * band.heads (head fastest; row tiles are visited from the last rows to the first), grid.y = parts of
+// part_tiles column tiles (1 for kBoth; for kStats a part is a segment).  Row r of a tile is query block i_r of sequence b_r; its causal columns are the blocks seq_start_r .. r of
+// the batch.  The whole problem is the band (0, total_blocks, 0, Hq, 0).  Scores are written at their offset in the full
+// matrix minus band.score_base.  stats: [head][block of the batch][stat_segs] (m, l).
+template <int kMode>
 __global__ void __launch_bounds__(gs::kThreads, 1)
 gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, const uint16_t* __restrict__ gk,
-                   float* __restrict__ scores, int* __restrict__ status) {
+                   float* __restrict__ scores, float2* __restrict__ stats, int* __restrict__ status, int part_tiles) {
   using namespace gs;
-  extern __shared__ __align__(1024) unsigned char gs_raw[];   // (the swizzled tiles need 1024-byte alignment; no slack is left to round up)
+  extern __shared__ __align__(1024) unsigned char gs_raw[];   // (the swizzled tiles need 1024-byte alignment)
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(gs_raw);
   unsigned char* smem = gs_raw;
   if ((base & 1023u) != 0u) {
@@ -102,33 +107,45 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   const int g = h / m.group;
   const int r0 = band.blk_lo + tile * kRows;                              // first block row of the tile
   const int rows_valid = min(kRows, band.blk_hi - r0);
+  const int seg_cols = gate_seg_tiles(m.max_nb) * kCols;
+  const int stat_segs = gate_stat_segs(m.max_nb);
 
-  // this thread's row (threads 0..127); the helpers only need the tile's column range
+  const int first_col = m.blk_off[find_sequence(m.blk_off, m.batch, r0)]; // rows ascend, so do their sequence starts
+  const int last_col = r0 + rows_valid - 1;
+  int col_lo = first_col, col_hi = last_col;                              // columns of this CTA
+  if (kMode != kBoth) {
+    const int part_cols = part_tiles * kCols, part = first_col / part_cols + (int)blockIdx.y;
+    col_lo = max(col_lo, part * part_cols);
+    col_hi = min(col_hi, (part + 1) * part_cols - 1);
+    if (col_lo > col_hi) return;
+  }
+
+  // this thread's row (threads t, t + 128, .. share row t; the helpers only need the tile's column range)
+  const int row = (warp & 3) * 32 + lane;
   int my_start = 0, my_last = -1;
-  long long my_off = 0;
-  if (threadIdx.x < kRows && (int)threadIdx.x < rows_valid) {
-    const int gb = r0 + (int)threadIdx.x;
+  if (threadIdx.x < kRowThreads && row < rows_valid) {
+    const int gb = r0 + row;
     const int b = find_sequence(m.blk_off, m.batch, gb);
     const int nb = m.blk_off[b + 1] - m.blk_off[b];
     const int i = gb - m.blk_off[b];
     my_start = m.blk_off[b];
-    my_off = m.score_off[b] + ((long long)h * nb + i) * nb - band.score_base;
     if (!(m.chunked && i < m.qoff[b])) my_last = gb;                      // chunked prefill: rows before the chunk are skipped
-  }
-  if (threadIdx.x < kRows) {
-    *reinterpret_cast<long long*>(smem + kOffMeta + threadIdx.x * 16) = my_off - my_start;   // + j = element of column j
-    *reinterpret_cast<int2*>(smem + kOffMeta + threadIdx.x * 16 + 8) = make_int2(my_start, my_last);
+    if (threadIdx.x < kRows) {
+      const long long off = score_row_offset(m, band, b, nb, h, i) - my_start;   // + j = element of column j
+      *reinterpret_cast<long long*>(smem + kOffMeta + row * 16) = off;
+      *reinterpret_cast<int2*>(smem + kOffMeta + row * 16 + 8) = make_int2(my_start, my_last);
+    }
+  } else if (threadIdx.x < kRows) {
+    *reinterpret_cast<int2*>(smem + kOffMeta + row * 16 + 8) = make_int2(0, -1);
   }
   if (!__syncthreads_or(my_last >= 0 ? 1 : 0)) return;                    // a tile of query blocks before their chunks
-  const int first_col = m.blk_off[find_sequence(m.blk_off, m.batch, r0)];  // rows ascend, so do their sequence starts
-  const int last_col = r0 + rows_valid - 1;
-  const int ntiles = (last_col - first_col) / kCols + 1;                  // column tiles of one sweep
-  const int total = 2 * ntiles;                                           // both sweeps
+  const int tile_lo = col_lo / kCols;
+  const int ntiles = col_hi / kCols - tile_lo + 1;                        // column tiles of one sweep
+  const int total = kMode == kBoth ? 2 * ntiles : ntiles;
 
   if (threadIdx.x == 0) {
-    mbar_init(bar0 + 8 * (ACC_FULL + 0), 2); mbar_init(bar0 + 8 * (ACC_FULL + 1), 2);   // one commit per issuing thread
-    mbar_init(bar0 + 8 * (ACC_EMPTY + 0), kRows); mbar_init(bar0 + 8 * (ACC_EMPTY + 1), kRows);
-    mbar_init(bar0 + 8 * (B_FULL + 0), kLoaders); mbar_init(bar0 + 8 * (B_FULL + 1), kLoaders);
+    for (int i = 0; i < (int)kBars; ++i)                                  // one commit per issuing thread; one arrival per row warp
+      mbar_init(bar0 + 8 * i, i < ACC_EMPTY ? 2 : i < B_FULL ? 8 : i < (int)B_EMPTY ? 1 : i < (int)A_FULL ? 2 : kRowThreads / 32);
     st_shared_u32(abort_addr, 0u);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -140,117 +157,152 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
+  const int half = (warp >> 2) & 1;                                       // which 32 columns of a tile this row warp takes
+  const int grp = (warp >> 3) & 1;                                        // ... and of which tiles: even or odd ones
 
-  const size_t plane_q = (size_t)m.num_q_heads * m.total_blocks * kGateDim;
-  const size_t plane_k = (size_t)m.num_kv_heads * m.total_blocks * kGateDim;
-  const uint16_t* gq_h = gq + (size_t)h * m.total_blocks * kGateDim;
-  const uint16_t* gk_g = gk + (size_t)g * m.total_blocks * kGateDim;
+  // A: the rows' planes, lane = row, two bf16 per column; each of a row's four threads copies a quarter
+  if (warp < 16) {
+    const int gb = min(r0 + row, m.total_blocks - 1);
+    const GateTile at(gb >> 6, m.total_blocks);
+    const char* src = reinterpret_cast<const char*>(gq) + (size_t)h * m.total_blocks * kGatePairBytes + at.base + (size_t)half * at.rows * 128 + (size_t)(gb & 63) * 128;
+    uint32_t w[3][16];
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (my_last >= 0) v = *reinterpret_cast<const uint4*>(src + (size_t)pl * at.rows * 256 + (((grp * 4 + c) ^ (gb & 7)) << 4));
+        w[pl][4 * c] = v.x; w[pl][4 * c + 1] = v.y; w[pl][4 * c + 2] = v.z; w[pl][4 * c + 3] = v.w;
+      }
+#pragma unroll
+    for (int pl = 0; pl < 3; ++pl) tc_st16(tmem + lane_addr + kColA + (uint32_t)pl * 64u + (uint32_t)half * 32u + (uint32_t)grp * 16u, w[pl]);
+    tc_wait_st();
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar0 + 8 * A_FULL);
+  }
 
-  if (warp >= 6) {
+  if (warp == 18) {
     // ------------------------------------------------------------------------------------------ copies
-    const int tid = threadIdx.x - 192;                    // warps 6..9
-    load_planes<kRows>(base + kOffA, kAPlane, gq_h, plane_q, r0, rows_valid, tid, kLoaders);
-    for (int n = 0; n < total; ++n) {
-      const int buf = n & 1;
-      const int j0 = first_col + (n % ntiles) * kCols;
-      // the MMAs of tile n - 2 read this B buffer: their completion is ACC_FULL of that tile
-      if (n >= 2) wait_bar(bar0 + 8 * (ACC_FULL + buf), ((n - 2) >> 1) & 1u, abort_addr, status);
-      load_planes<kCols>(base + kOffB + (uint32_t)buf * kBBuf, kBPlane, gk_g, plane_k, j0, min(kCols, last_col + 1 - j0), tid, kLoaders);
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      fence_async_smem();                                 // the copies (generic proxy) before the MMAs' reads (async proxy)
-      mbar_arrive(bar0 + 8 * (B_FULL + buf));
+    if (elect_one()) {
+      const char* src = reinterpret_cast<const char*>(gk) + (size_t)g * m.total_blocks * kGatePairBytes;
+      uint32_t buf = 0, ph = 1;
+      for (int n = 0; n < total; ++n) {
+        wait_bar(bar0 + 8 * (B_EMPTY + buf), ph, abort_addr, status);
+        const GateTile bt(tile_lo + (n >= ntiles ? n - ntiles : n), m.total_blocks);
+        const uint32_t full = bar0 + 8 * (B_FULL + buf), dst = base + buf * kBBuf;
+        mbar_expect_tx(full, (uint32_t)bt.rows * kGatePairBytes);
+        if (bt.rows == 64) bulk_copy(dst, src + bt.base, kBBuf, full);
+        else                                              // the batch's last tile: shorter planes (what lies behind them is masked)
+          for (int p = 0; p < 6; ++p) bulk_copy(dst + (uint32_t)p * 8192u, src + bt.base + (size_t)p * bt.rows * 128, (uint32_t)bt.rows * 128u, full);
+        if (++buf == kBBufs) { buf = 0; ph ^= 1u; }
+      }
     }
-  } else if (warp >= 4) {
+  } else if (warp >= 16) {
     // ------------------------------------------------------------------------------------------ MMAs
     // (the issuing threads copy nothing: a thread that waits for its own copies between two batches of MMAs leaves
     // the pipe idle for the latency of a copy, which was 40 % of the kernel)
     if (elect_one()) {
-      const int part = warp - 4;                          // 0: small terms, 1: large terms
+      const int part = warp - 16;                          // 0: small terms, 1: large terms
       // (A plane, B plane): small = (hi, lo), (lo, hi), (mid, mid); large = (hi, mid), (mid, hi), (hi, hi)
-      const int pa[3] = {0, part ? 1 : 2, part ? 0 : 1}, pb[3] = {part ? 1 : 2, 0, part ? 0 : 1};
+      const uint32_t pa[3] = {0u, part ? 1u : 2u, part ? 0u : 1u}, pb[3] = {part ? 1u : 2u, 0u, part ? 0u : 1u};
+      uint32_t buf = 0, ph = 0, uses[2] = {0u, 0u};
+      wait_bar(bar0 + 8 * A_FULL, 0u, abort_addr, status);
       for (int n = 0; n < total; ++n) {
-        const int buf = n & 1;
-        wait_bar(bar0 + 8 * (B_FULL + buf), (n >> 1) & 1u, abort_addr, status);
-        // the rows have taken tile n - 2 out of this accumulator pair
-        if (n >= 2) wait_bar(bar0 + 8 * (ACC_EMPTY + buf), ((n - 2) >> 1) & 1u, abort_addr, status);
+        const int acc = (tile_lo + (n >= ntiles ? n - ntiles : n)) & 1;
+        wait_bar(bar0 + 8 * (B_FULL + buf), ph, abort_addr, status);
+        // the rows have taken the previous tile out of this accumulator pair
+        const uint32_t use = acc ? uses[1]++ : uses[0]++;
+        wait_bar(bar0 + 8 * (ACC_EMPTY + acc), (use & 1u) ^ 1u, abort_addr, status);
         tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)buf * 2u * kCols + (uint32_t)part * kCols;
-        const uint32_t sa = base + kOffA, sb = base + kOffB + (uint32_t)buf * kBBuf;
+        const uint32_t d = tmem + (uint32_t)acc * 2u * kCols + (uint32_t)part * kCols;
+        const uint32_t sb = base + buf * kBBuf;
 #pragma unroll
         for (int t = 0; t < 3; ++t)
 #pragma unroll
-          for (int kk = 0; kk < 8; ++kk) {
-            const uint64_t ad = make_desc(sa + (uint32_t)pa[t] * kAPlane + (uint32_t)(kk >> 2) * (kRows * 128u) + (uint32_t)(kk & 3) * 32u, 16, 1024);
-            const uint64_t bd = make_desc(sb + (uint32_t)pb[t] * kBPlane + (uint32_t)(kk >> 2) * (kCols * 128u) + (uint32_t)(kk & 3) * 32u, 16, 1024);
-            tc_mma(d, ad, bd, kIdesc, (t | kk) != 0 ? 1u : 0u);
-          }
-        tc_commit(bar0 + 8 * (ACC_FULL + buf));
+          for (int kk = 0; kk < 8; ++kk)
+            tc_mma_ts(d, tmem + kColA + pa[t] * 64u + (uint32_t)kk * 8u,
+                      make_desc(sb + pb[t] * kBPlane + (uint32_t)(kk >> 2) * (kCols * 128u) + (uint32_t)(kk & 3) * 32u, 16, 1024), kIdesc, (t | kk) != 0 ? 1u : 0u);
+        tc_commit(bar0 + 8 * (B_EMPTY + buf));
+        tc_commit(bar0 + 8 * (ACC_FULL + acc));
+        if (++buf == kBBufs) { buf = 0; ph ^= 1u; }
       }
     }
   } else {
     // ------------------------------------------------------------------------------------------ rows
-    // everything in units of log2: x2 = logit * log2(e); m2 the running maximum of x2; p = 2^(x2 - m2) / l
+    // everything in units of log2: x2 = logit * log2(e); m the running maximum of x2; p = 2^(x2 - m) / l
     const float scale2 = rsqrtf((float)kGateDim) * 1.4426950408889634f;
-    const uint32_t lane_addr = (uint32_t)(warp * 32) << 16;
-    float run_m = -CUDART_INF_F, run_l = 0.f, inv_l = 0.f;
+    float seg_m = -CUDART_INF_F, seg_l = 0.f;             // this thread's columns of the current segment
+    float row_m = -CUDART_INF_F, row_l = 0.f, inv_l = 0.f;   // the whole row
+    float2* ml = reinterpret_cast<float2*>(smem + kOffStage);   // [segment parity][group][half][row]
+    int nseg = 0;
+    uint32_t uses = 0;                                    // tiles this group has worked on
+    if (kMode == kWrite && my_last >= 0) {
+      const int s_lo = my_start / seg_cols, s_hi = my_last / seg_cols;
+      const float2* st = stats + ((size_t)h * m.total_blocks + r0 + row) * stat_segs;
+      for (int s = 0; s <= s_hi - s_lo; ++s) { const float2 v = st[s]; combine(row_m, row_l, v.x, v.y); }
+      inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
+    }
     for (int n = 0; n < total; ++n) {
-      const int buf = n & 1;
-      const int sweep = n / ntiles;
-      const int j0 = first_col + (n - sweep * ntiles) * kCols;
-      if (n == ntiles) inv_l = run_l > 0.f ? 1.0f / run_l : 0.f;
-      wait_bar(bar0 + 8 * (ACC_FULL + buf), (n >> 1) & 1u, abort_addr, status);
-      tc_fence_after();
-      const uint32_t acc = tmem + lane_addr + (uint32_t)buf * 2u * kCols;
-      // columns of this tile that are causal for this row: j in [my_start, my_last]
-      const int lo = max(my_start - j0, 0), hi = min(my_last - j0, kCols - 1);   // hi < lo: nothing (also my_last = -1)
-#pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        uint32_t vs[32], vl[32];
-        tc_ld32(acc + half * 32, vs);
-        tc_ld32(acc + kCols + half * 32, vl);
-        tc_wait_ld32(vs);
-        tc_wait_ld32(vl);
-        const int c0 = half * 32;
-        if (hi < c0 || lo > c0 + 31) continue;
-        const bool whole = lo <= c0 && hi >= c0 + 31;     // no column of this half is masked
-        float x[32];
-#pragma unroll
-        for (int c = 0; c < 32; ++c) x[c] = (__uint_as_float(vs[c]) + __uint_as_float(vl[c])) * scale2;
-        if (sweep == 0) {
-          if (!whole) {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) if (c0 + c < lo || c0 + c > hi) x[c] = -CUDART_INF_F;
-          }
-          float tmax = x[0];
-#pragma unroll
-          for (int c = 1; c < 32; ++c) tmax = fmaxf(tmax, x[c]);
-          const float nm = fmaxf(run_m, tmax);            // finite: the half holds a causal column
-          float sum = 0.f;
-#pragma unroll
-          for (int c = 0; c < 32; ++c) sum += ex2f(x[c] - nm);   // 2^(-inf) = 0 for the masked columns
-          run_l = run_l * ex2f(run_m - nm) + sum;         // 2^(-inf) = 0 on the first contribution
-          run_m = nm;
-        } else {
-#pragma unroll
-          for (int c = 0; c < 32; ++c) x[c] = ex2f(x[c] - run_m) * inv_l;
-          float* srow = reinterpret_cast<float*>(smem + kOffStage) + threadIdx.x * kCols;
-#pragma unroll
-          for (int c = 0; c < 32; c += 4)
-            *reinterpret_cast<float4*>(srow + ((((c0 + c) >> 2) ^ (threadIdx.x & 15)) << 2)) = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
-        }
+      const bool write = kMode == kWrite || (kMode == kBoth && n >= ntiles);
+      const int ct = tile_lo + (kMode == kBoth && n >= ntiles ? n - ntiles : n);
+      const int j0 = ct * kCols + half * 32;              // first column of this thread
+      if (kMode == kBoth && n == ntiles) {
+        inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
+        named_bar_sync(1, kRowThreads);                   // (the staging area held the segments' statistics)
       }
-      if (sweep == 1) {
-        // the warp's 32 rows, two rows per step: a half-warp takes a row, a lane four consecutive columns of it
+      if ((ct & 1) == grp) {
+      wait_bar(bar0 + 8 * (ACC_FULL + grp), uses & 1u, abort_addr, status);
+      ++uses;
+      tc_fence_after();
+      const uint32_t a = tmem + lane_addr + (uint32_t)grp * 2u * kCols + (uint32_t)half * 32u;
+      uint32_t vs[32], vl[32];
+      tc_ld32(a, vs);
+      tc_ld32(a + kCols, vl);
+      tc_wait_ld32(vs);
+      tc_wait_ld32(vl);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar0 + 8 * (ACC_EMPTY + grp));
+      float x[32];
+#pragma unroll
+      for (int c = 0; c < 32; ++c) x[c] = __fmul_rn(__fadd_rn(__uint_as_float(vs[c]), __uint_as_float(vl[c])), scale2);
+      // columns that are causal for this row: j in [my_start, my_last]
+      const int lo = my_start - j0, hi = my_last - j0;
+      if (!write) {
+        if (hi >= 0 && lo <= 31) {
+          if (lo > 0 || hi < 31) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) if (c < lo || c > hi) x[c] = -CUDART_INF_F;
+          }
+          float mx[4] = {x[0], x[1], x[2], x[3]};
+#pragma unroll
+          for (int c = 4; c < 32; ++c) mx[c & 3] = fmaxf(mx[c & 3], x[c]);
+          const float nm = fmaxf(seg_m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])));   // finite: there is a causal column
+          float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int c = 0; c < 32; ++c) sum[c & 3] = __fadd_rn(sum[c & 3], ex2f(__fsub_rn(x[c], nm)));   // 2^(-inf) = 0 for the masked columns
+          const float s4 = __fadd_rn(__fadd_rn(sum[0], sum[1]), __fadd_rn(sum[2], sum[3]));
+          seg_l = __fadd_rn(__fmul_rn(seg_l, ex2f(__fsub_rn(seg_m, nm))), s4);              // 2^(-inf) = 0 on the first contribution
+          seg_m = nm;
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) x[c] = __fmul_rn(ex2f(__fsub_rn(x[c], row_m)), inv_l);
+        float* stage = reinterpret_cast<float*>(smem + kOffStage) + warp * 1024;
+#pragma unroll
+        for (int c = 0; c < 32; c += 4)
+          *reinterpret_cast<float4*>(stage + lane * 32 + (((c >> 2) ^ (lane & 7)) << 2)) = make_float4(x[c], x[c + 1], x[c + 2], x[c + 3]);
         __syncwarp();
+        // the warp's 32 rows, four rows per step: eight lanes take a row, a lane four consecutive columns of it
 #pragma unroll 4
-        for (int rr = 0; rr < 32; rr += 2) {
-          const int row = warp * 32 + rr + (lane >> 4);
-          const long long off = *reinterpret_cast<const long long*>(smem + kOffMeta + row * 16);
-          const int2 se = *reinterpret_cast<const int2*>(smem + kOffMeta + row * 16 + 8);
-          const int c = 4 * (lane & 15), j = j0 + c;
-          const float4 v = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(smem + kOffStage) + row * kCols +
-                                                            (((c >> 2) ^ (row & 15)) << 2));
+        for (int rr = 0; rr < 32; rr += 4) {
+          const int lr = rr + (lane >> 3), mr = (warp & 3) * 32 + lr;
+          const long long off = *reinterpret_cast<const long long*>(smem + kOffMeta + mr * 16);
+          const int2 se = *reinterpret_cast<const int2*>(smem + kOffMeta + mr * 16 + 8);
+          const int j = j0 + 4 * (lane & 7);
+          const float4 v = *reinterpret_cast<const float4*>(stage + lr * 32 + (((lane & 7) ^ (lr & 7)) << 2));
           float* dst = scores + (off + j);
           if (j >= se.x && j + 3 <= se.y && ((off + j) & 3) == 0) *reinterpret_cast<float4*>(dst) = v;
           else {
@@ -262,8 +314,23 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
         }
         __syncwarp();                                    // the staging rows are free again
       }
-      tc_fence_before();
-      mbar_arrive(bar0 + 8 * (ACC_EMPTY + buf));
+      }
+      if (!write && (n == ntiles - 1 || ((ct + 1) * kCols) % seg_cols == 0)) {
+        // end of a segment: the four threads of a row combine their columns
+        float2* buf = ml + (nseg & 1) * 4 * kRows;
+        buf[(grp * 2 + half) * kRows + row] = make_float2(seg_m, seg_l);
+        named_bar_sync(1, kRowThreads);
+        float sm = -CUDART_INF_F, sl = 0.f;
+#pragma unroll
+        for (int p = 0; p < 4; ++p) { const float2 v = buf[p * kRows + row]; combine(sm, sl, v.x, v.y); }
+        const int seg = ct * kCols / seg_cols, s_lo = my_start / seg_cols;
+        const bool mine = my_last >= 0 && seg >= s_lo && seg <= my_last / seg_cols;
+        if (kMode == kStats) {
+          if (mine && half == 0 && grp == 0) stats[((size_t)h * m.total_blocks + r0 + row) * stat_segs + (seg - s_lo)] = make_float2(sm, sl);
+        } else if (mine) combine(row_m, row_l, sm, sl);
+        seg_m = -CUDART_INF_F; seg_l = 0.f;
+        ++nseg;
+      }
     }
   }
   tc_fence_before();
@@ -274,18 +341,57 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   }
 }
 
-int launch_gate_scores(const SeqMeta& m, const ScoreBand& band, const uint16_t* gq, const uint16_t* gk, float* scores,
-                       int* status, cudaStream_t stream) {
-  const unsigned grid = (unsigned)((band.blk_hi - band.blk_lo + gs::kRows - 1) / gs::kRows) * (unsigned)band.heads;
-  if (grid == 0) return 0;
-  gate_scores_kernel<<<grid, gs::kThreads, gs::kSmemBytes, stream>>>(m, band, gq, gk, scores, status);
+// part_tiles == 0: one CTA per row tile and head
+static dim3 score_grid(const SeqMeta& m, const ScoreBand& band, int part_tiles) {
+  const unsigned x = (unsigned)((band.blk_hi - band.blk_lo + gs::kRows - 1) / gs::kRows) * (unsigned)band.heads;
+  // a row tile that starts in one sequence and ends in another may touch a tile's worth of columns more than the longest one
+  const int cols = part_tiles * gs::kCols;
+  return dim3(x, part_tiles ? (unsigned)((m.max_nb + gs::kRows + cols - 1) / cols + 1) : 1u);
+}
+
+// Whether the whole problem takes two launches (statistics, then scores) rather than one.  In units of a tile (about 1 us): one
+// launch lasts as long as its longest CTA (both sweeps of the longest row) or its share of all tiles; two launches even that
+// out but pay a CTA's start (about three tiles) per segment, twice.
+bool gate_split(const SeqMeta& m, int num_sms) {
+  const int64_t tiles = m.score_tiles;
+  const int64_t longest = (m.max_nb + gs::kCols - 1) / gs::kCols, share = tiles / num_sms;
+  const int seg = gate_seg_tiles(m.max_nb);
+  const int64_t starts = 1 + tiles / seg / num_sms;
+  const int64_t one = 2 * (longest > share ? longest : share), two = 2 * ((seg > share ? seg : share) + 3 * starts) + 3;
+  return two < one;
+}
+
+// Statistics of all rows.
+int launch_gate_stats(const SeqMeta& m, const uint16_t* gq, const uint16_t* gk, float2* stats, int* status, cudaStream_t stream) {
+  const ScoreBand all = {m.first_q_block, m.total_blocks, 0, m.num_q_heads, 0, 0, 0};
+  const int part = gate_seg_tiles(m.max_nb);
+  const dim3 grid = score_grid(m, all, part);
+  if (grid.x == 0) return 0;
+  gate_scores_kernel<gs::kStats><<<grid, gs::kThreads, gs::kSmemBytes, stream>>>(m, all, gq, gk, nullptr, stats, status, part);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? 1 : -(int)e;
 }
 
-// Lifts the kernel's shared-memory limit on the current device (no allocation).
+// Scores of a band; with `stats` launch_gate_stats has run, without the rows' statistics are formed by the same launch.
+int launch_gate_scores(const SeqMeta& m, const ScoreBand& band, const uint16_t* gq, const uint16_t* gk, float* scores,
+                       float2* stats, int* status, int num_sms, cudaStream_t stream) {
+  // parts of 4 to 16 tiles, so that the band's tiles make about one wave of CTAs (a 4096-block head: 16 tiles a CTA 30 us, 8: 17)
+  const int64_t tiles = (int64_t)((band.blk_hi - band.blk_lo + gs::kRows - 1) / gs::kRows) * band.heads * (m.max_nb / gs::kCols / 2 + 1);
+  int part = 4;
+  while (part < 16 && tiles / part > num_sms) part *= 2;
+  const dim3 grid = score_grid(m, band, stats != nullptr ? part : 0);
+  if (grid.x == 0) return 0;
+  if (stats != nullptr) gate_scores_kernel<gs::kWrite><<<grid, gs::kThreads, gs::kSmemBytes, stream>>>(m, band, gq, gk, scores, stats, status, part);
+  else gate_scores_kernel<gs::kBoth><<<grid, gs::kThreads, gs::kSmemBytes, stream>>>(m, band, gq, gk, scores, nullptr, status, 0);
+  cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? 1 : -(int)e;
+}
+
+// Lifts the kernels' shared-memory limit on the current device (no allocation).
 bool init_gate_scores() {
-  return cudaFuncSetAttribute(gate_scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess;
+  return cudaFuncSetAttribute(gate_scores_kernel<gs::kBoth>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess &&
+         cudaFuncSetAttribute(gate_scores_kernel<gs::kStats>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess &&
+         cudaFuncSetAttribute(gate_scores_kernel<gs::kWrite>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess;
 }
 
 }  // namespace seer

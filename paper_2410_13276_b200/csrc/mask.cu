@@ -1,21 +1,19 @@
 // Binary block mask (Sec. 3.3, Eq. 3 TopK / Eq. 4 threshold) as CSR index lists.
 //   count_kernel : one warp per (sequence, head, query-block) row -> number of kept blocks
 //   scan_kernel  : exclusive prefix sum of the counts -> row_ptr, nnz, capacity check
-//   fill_kernel  : one warp per row repeats the selection and writes the ascending list by ballot compaction
+//   topk_kernel / fill_kernel : repeat the selection and write the ascending lists
 // Selection order in the TopK modes is (score descending, block index ascending): scores become order-preserving
-// 32-bit keys, the key of the last kept candidate is found by a radix select over the row held in shared memory (at most
-// four 8-bit passes with warp-private histograms; batches with rows too long to stage re-read the scores in every pass), and ties
-// at that key are resolved by rank in index order.
+// 32-bit keys, the key of the last kept candidate is found by a radix select (at most four 8-bit passes), and ties at that
+// key are resolved by rank in index order.
+#include <math_constants.h>
+
 #include "seer_internal.cuh"
 
 namespace seer {
 
 constexpr int kMaskWarps = 4;
-// Rows are staged in shared memory when the longest row of the batch has at most this many blocks (16 bytes of shared
-// memory per block and CTA).  Beyond that the staging buffer would cost more in occupancy than it saves in reads
-// (measured: 4096 blocks 4.6 ms staged, 3.1 ms not; 10240 blocks 103 ms against 27 ms), and every pass re-reads the
-// scores, which stay in L1 / L2 between the passes of a row.
-constexpr int kMaskSmemRowMax = 2048;
+// TopK rows of up to this many blocks are held in shared memory (topk_kernel); longer ones re-read their scores in every pass.
+constexpr int kTopkRowMax = 16384;
 
 struct RowInfo {
   const float* s;   // scores of this row
@@ -23,11 +21,13 @@ struct RowInfo {
   bool valid;
   bool skip;        // chunked prefill: a query block before the chunk, its list is empty
   int nb;           // blocks of the row's sequence
+  int h, gb;        // head; block row, numbered over the batch
 };
 
-// Rows [row_lo, row_hi) of the CSR structure whose scores sit at (offset in the full matrix - score_base) in `scores`.
+// Rows [row_lo, row_hi) of the CSR structure and where their scores are (ScoreBand).
 struct RowBand {
-  int64_t row_lo, row_hi, score_base;
+  int64_t row_lo, row_hi;
+  ScoreBand sb;
 };
 
 __device__ __forceinline__ RowInfo decode_row(const SeqMeta& m, const RowBand& band, const float* __restrict__ scores, int64_t r) {
@@ -42,9 +42,11 @@ __device__ __forceinline__ RowInfo decode_row(const SeqMeta& m, const RowBand& b
   const uint32_t local = (uint32_t)r - (uint32_t)m.num_q_heads * (uint32_t)m.blk_off[b];
   const int h = (int)(local / (uint32_t)nb);
   ri.i = (int)(local - (uint32_t)h * (uint32_t)nb);
-  ri.s = scores + (m.score_off[b] + ((int64_t)h * nb + ri.i) * nb - band.score_base);
+  ri.s = scores + score_row_offset(m, band.sb, b, nb, h, ri.i);   // (not looked at for a skipped row)
   ri.skip = m.chunked && ri.i < m.qoff[b];
   ri.nb = nb;
+  ri.h = h;
+  ri.gb = m.blk_off[b] + ri.i;
   return ri;
 }
 
@@ -131,59 +133,90 @@ count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mas
 }
 
 // Single CTA: in-place inclusive scan of row_ptr[1..rows].  `first`: row_ptr[0] = 0; otherwise the scan continues from
-// row_ptr[0], the last entry of the rows scanned before.  Tiles of 4096 counts go through shared memory (coalesced loads
-// and stores), four consecutive counts per thread, warp shuffles inside a warp, one carry per tile.
+// row_ptr[0], the last entry of the rows scanned before.  Tiles of 8192 counts go through shared memory (coalesced loads and
+// stores, the next tile's loads in flight meanwhile), eight consecutive counts per thread, warp shuffles inside a warp; every
+// warp adds up the warp totals for itself.  It is bound by the latency of a tile's three barriers (65 536 rows: 33 us with
+// tiles of 4096 and their loads exposed).  All sums fit 32 bits (the host refuses shapes with 2^31 causal blocks).
+//
+// kCounts (TopK of scores whose softmax statistics are at hand): the counts come from here as well.  A row whose maximum and sum
+// are finite has no NaN among its scores, so its length follows from n and the parameters and no score is read (4096 rows of
+// 4096: 20 us for the two kernels, 6 us); a row that has not is counted by its thread.
+struct CountArgs {
+  SeqMeta m;
+  RowBand band;
+  const float* scores;
+  const float2* stats;
+  seer_mask_params p;
+};
+__device__ __forceinline__ int topk_count(const CountArgs& a, int64_t r) {
+  const RowInfo ri = decode_row(a.m, a.band, a.scores, r);
+  if (ri.skip) return 0;
+  const int n = ri.i + 1;
+  if (ri.i >= ri.nb - a.p.dense_tail_blocks) return n;
+  const int nf = num_forced(ri.i, a.p.flags), take = max(keep_count(n, a.p) - nf, 0);
+  const int seg_cols = gate_seg_tiles(a.m.max_nb) * kScoreTile, segs = (ri.gb / seg_cols) - (ri.gb - ri.i) / seg_cols + 1;
+  const float2* st = a.stats + ((size_t)ri.h * a.m.total_blocks + ri.gb) * gate_stat_segs(a.m.max_nb);
+  bool finite = true;
+  for (int s = 0; s < segs; ++s) { const float2 v = st[s]; finite = finite && fabsf(v.x) < 3.0e38f && v.y > 0.f && v.y < 3.0e38f; }
+  int ncand = n - nf;
+  if (!finite) {
+    ncand = 0;
+    for (int j = 0; j < n; ++j) ncand += (!is_forced(j, ri.i, a.p.flags) && score_key(ri.s[j]) != 0u) ? 1 : 0;
+  }
+  return nf + min(take, ncand);
+}
+
+constexpr int kScanPer = 8, kScanTile = 1024 * kScanPer;
+template <bool kCounts>
 __global__ void __launch_bounds__(1024)
 scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_capacity, int64_t* __restrict__ nnz_out,
-            int* __restrict__ status) {
-  __shared__ int32_t tile[4096];
-  __shared__ long long warp_tot[32];
-  __shared__ long long carry_s;
+            int* __restrict__ status, CountArgs args) {
+  __shared__ int32_t tile[kScanTile + kScanTile / 32];     // (one word of padding per 32: eight consecutive words per thread)
+  __shared__ int32_t warp_tot[2][32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  long long carry = first ? 0 : row_ptr[0];
-  for (int64_t base = 0; base < rows; base += 4096) {
-    const int n = (int)min((int64_t)4096, rows - base);
+  int carry = first ? 0 : row_ptr[0];
+  int32_t next[kScanPer];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int idx = t + k * 1024;
-      tile[idx] = idx < n ? row_ptr[base + idx + 1] : 0;
-    }
+  for (int k = 0; k < kScanPer; ++k) next[k] = t + k * 1024 < rows ? (kCounts ? topk_count(args, args.band.row_lo + t + k * 1024) : row_ptr[t + k * 1024 + 1]) : 0;
+  int par = 0;
+  for (int64_t base = 0; base < rows; base += kScanTile, par ^= 1) {
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) { const int idx = t + k * 1024; tile[idx + (idx >> 5)] = next[k]; }
     __syncthreads();
-    long long v[4];
-    v[0] = tile[4 * t];
-    v[1] = v[0] + tile[4 * t + 1];
-    v[2] = v[1] + tile[4 * t + 2];
-    v[3] = v[2] + tile[4 * t + 3];
-    long long incl = v[3];
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) {
+      const int64_t idx = base + kScanTile + t + k * 1024;
+      next[k] = idx < rows ? (kCounts ? topk_count(args, args.band.row_lo + idx) : row_ptr[idx + 1]) : 0;
+    }
+    int v[kScanPer];
+#pragma unroll
+    for (int k = 0; k < kScanPer; ++k) { const int idx = kScanPer * t + k; v[k] = tile[idx + (idx >> 5)] + (k > 0 ? v[k - 1] : 0); }
+    int incl = v[kScanPer - 1];
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-      const long long o = __shfl_up_sync(0xffffffffu, incl, off);
+      const int o = __shfl_up_sync(0xffffffffu, incl, off);
       if (lane >= off) incl += o;
     }
-    if (lane == 31) warp_tot[warp] = incl;
+    if (lane == 31) warp_tot[par][warp] = incl;
     __syncthreads();
-    if (warp == 0) {
-      long long w = warp_tot[lane];
+    int w = warp_tot[par][lane];
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const long long o = __shfl_up_sync(0xffffffffu, w, off);
-        if (lane >= off) w += o;
-      }
-      warp_tot[lane] = w;                              // inclusive over warps
-      if (lane == 31) carry_s = w;                     // total of the tile
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, w, off);
+      if (lane >= off) w += o;
     }
-    __syncthreads();
-    const long long before = carry + (warp > 0 ? warp_tot[warp - 1] : 0) + (incl - v[3]);
+    const int before_warp = __shfl_sync(0xffffffffu, w, (warp + 31) & 31), total = __shfl_sync(0xffffffffu, w, 31);
+    const int before = carry + (warp > 0 ? before_warp : 0) + (incl - v[kScanPer - 1]);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) tile[4 * t + k] = (int32_t)(before + v[k]);
-    carry += carry_s;
+    for (int k = 0; k < kScanPer; ++k) { const int idx = kScanPer * t + k; tile[idx + (idx >> 5)] = before + v[k]; }
+    carry += total;
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kScanPer; ++k) {
       const int idx = t + k * 1024;
-      if (idx < n) row_ptr[base + idx + 1] = tile[idx];
+      if (base + idx < rows) row_ptr[base + idx + 1] = tile[idx + (idx >> 5)];
     }
-    __syncthreads();
+    // (a thread's stores of the next tile go to the words it has just read)
   }
   if (t == 0) {
     if (first) row_ptr[0] = 0;
@@ -192,11 +225,280 @@ scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_
   }
 }
 
+// The key a TopK row is ranked by, in fewer instructions than score_key (the loops are bound by instruction issue).
+__device__ __forceinline__ uint32_t lean_key(float sc) {
+  const float z = sc + 0.0f;                                     // -0 -> +0
+  const uint32_t u = __float_as_uint(z);
+  const uint32_t kk = u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
+  return z != z ? 0u : kk;                                       // NaN: never a candidate
+}
+
+// TopK lists, W warps per row, the row's keys in shared memory (`cap` of them, a multiple of 128 W; step k of a row is the
+// columns 128 W k + 4 t + u of thread t, u < 4).
+//
+// It is bound by instruction issue, so the loops are short and rolled: with the keys in registers and the loops unrolled the
+// kernel waited for instructions (a row of 2048 keys took 2300 instructions and 20 000 clocks, and more warps did not help).
+// A row gets one warp up to 2048 blocks, and as many as keep it at 2048 keys per warp beyond.  Measured: 65 536 rows of up to
+// 2048 blocks 251 -> 183 us, 4096 rows of up to 4096 blocks (which re-read their scores in every pass) 158 -> 34 us.
+template <int W>
+__global__ void __launch_bounds__(W < 4 ? 128 : W * 32)
+topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask_params p, const int32_t* __restrict__ row_ptr,
+            int32_t* __restrict__ col_idx, int64_t col_capacity, int cap) {
+  constexpr int kWarps = W < 4 ? 4 : W, kRows = kWarps / W, kStep = 128 * W;
+  constexpr int kMaxSteps = 16, kEntries = kMaxSteps * W;        // (the launcher keeps cap <= 16 steps)
+  extern __shared__ __align__(16) uint32_t key_smem[];
+  __shared__ __align__(16) uint32_t s_hist[kRows][256];
+  __shared__ uint32_t s_red[kRows][3][W];
+  __shared__ uint32_t s_list[kRows][32];
+  __shared__ uint32_t s_found[kRows];
+  __shared__ int s_cnt[kRows][2][W > 1 ? kEntries : 1];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rr = warp / W, w = warp % W, t = w * 32 + lane;      // row of the CTA, warp and thread within the row's group
+  auto meet = [&]() {                                            // the warps of a row
+    if (W == 1) __syncwarp();
+    else if (W < 4) asm volatile("bar.sync %0, %1;" ::"r"(1 + rr), "n"(W * 32) : "memory");
+    else __syncthreads();
+  };
+  const int64_t r = band.row_lo + (int64_t)blockIdx.x * kRows + rr;
+  const RowInfo ri = decode_row(m, band, scores, r);
+  if (!ri.valid || ri.skip) return;                              // (uniform in a row's group)
+  const int n = ri.i + 1;
+  const int32_t out0 = row_ptr[r], out1 = row_ptr[r + 1];
+  if ((int64_t)out1 > col_capacity) return;   // this row (and all later ones) do not fit; status already raised
+  int32_t* __restrict__ out = col_idx + out0;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  if (ri.i >= ri.nb - p.dense_tail_blocks) {           // a dense row at the end of the sequence: every causal block
+    for (int j = t; j < n; j += W * 32) out[j] = j;
+    return;
+  }
+  uint32_t* keys = key_smem + (size_t)rr * cap;
+  uint32_t* hist = s_hist[rr];
+  const bool sink_f = (p.flags & SEER_FORCE_SINK) != 0u;
+  const bool diag_f = (p.flags & SEER_FORCE_DIAG) != 0u && !(sink_f && ri.i == 0);
+  const int take = max(keep_count(n, p) - num_forced(ri.i, p.flags), 0);
+
+  // ---- keys (0: not a candidate: past the row, NaN, or forced, which the writer puts in its place by itself)
+  uint32_t c = 0, k_min = 0xffffffffu, k_max = 0u;               // over the candidates
+  const uint32_t nan_bits = 0x7fffffffu;
+  const uint32_t* __restrict__ src = reinterpret_cast<const uint32_t*>(ri.s);
+  const bool vec = (reinterpret_cast<uintptr_t>(ri.s) & 15) == 0;
+  for (int j0 = 4 * t; j0 - 4 * t < n; j0 += 4 * kStep) {
+    uint4 v[4];                                                  // four loads in flight per lane
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = j0 + q * kStep;
+      v[q] = make_uint4(nan_bits, nan_bits, nan_bits, nan_bits);
+      if (vec && j + 3 < n) v[q] = __ldg(reinterpret_cast<const uint4*>(src + j));
+      else if (j < n) {
+        v[q].x = __ldg(src + j);
+        if (j + 1 < n) v[q].y = __ldg(src + j + 1);
+        if (j + 2 < n) v[q].z = __ldg(src + j + 2);
+        if (j + 3 < n) v[q].w = __ldg(src + j + 3);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int j = j0 + q * kStep;
+      if (j - 4 * t >= n) break;                                 // (uniform)
+      uint4 kq = make_uint4(lean_key(__uint_as_float(v[q].x)), lean_key(__uint_as_float(v[q].y)), lean_key(__uint_as_float(v[q].z)), lean_key(__uint_as_float(v[q].w)));
+      if (sink_f && j == 0) kq.x = 0u;
+      if (diag_f && (uint32_t)(ri.i - j) < 4u) {
+        if (j == ri.i) kq.x = 0u;
+        if (j + 1 == ri.i) kq.y = 0u;
+        if (j + 2 == ri.i) kq.z = 0u;
+        if (j + 3 == ri.i) kq.w = 0u;
+      }
+      *reinterpret_cast<uint4*>(keys + j) = kq;
+      c += (kq.x != 0u) + (kq.y != 0u) + (kq.z != 0u) + (kq.w != 0u);
+      k_max = max(max(k_max, max(kq.x, kq.y)), max(kq.z, kq.w));
+      k_min = min(min(k_min, min(kq.x - 1u, kq.y - 1u)), min(kq.z - 1u, kq.w - 1u));   // (0, not a candidate, wraps to the largest)
+    }
+  }
+  *reinterpret_cast<uint4*>(hist + (t & 31) * 8) = make_uint4(0u, 0u, 0u, 0u);
+  *reinterpret_cast<uint4*>(hist + (t & 31) * 8 + 4) = make_uint4(0u, 0u, 0u, 0u);
+  if (t == 0) s_found[rr] = 0u;
+  uint32_t ncand = __reduce_add_sync(0xffffffffu, c);
+  k_min = __reduce_min_sync(0xffffffffu, k_min);
+  k_max = __reduce_max_sync(0xffffffffu, k_max);
+  if (W > 1) {
+    if (lane == 0) { s_red[rr][0][w] = ncand; s_red[rr][1][w] = k_min; s_red[rr][2][w] = k_max; }
+    meet();
+    ncand = __reduce_add_sync(0xffffffffu, lane < W ? s_red[rr][0][lane % W] : 0u);
+    k_min = __reduce_min_sync(0xffffffffu, lane < W ? s_red[rr][1][lane % W] : 0xffffffffu);
+    k_max = __reduce_max_sync(0xffffffffu, lane < W ? s_red[rr][2][lane % W] : 0u);
+  } else meet();
+
+  // ---- T: kept are the candidates with key >= T, of those with key == T only the first need_eq of n_eq
+  uint32_t T = 1u;
+  int need_eq = 0, n_eq = 0;
+  if (take >= (int)ncand) {
+    // every candidate is kept
+  } else if (take == 0) {
+    T = 0xffffffffu;                // nothing beyond the forced blocks (no key is that large: it would be a NaN's)
+  } else {
+    // The scores of a row are close together (probabilities of one softmax), often on both sides of a power of two.  So the
+    // first pass bins the distance from the smallest key, scaled to 128..256 bins: binning the keys' own leading bits put a
+    // flat row into a dozen bins, 32 lanes adding to a few shared-memory words, and took another pass.  Every warp of the row
+    // walks the bins for itself.
+    uint32_t lo = k_min + 1u, span = k_max - lo;                          // the class: keys lo .. lo + span
+    int shift = max(24 - __clz(span | 1u), 0);
+    int remaining = take;           // rank (1-based, from the top) still to locate inside the current class
+    for (;;) {
+      for (int j = 4 * t; j - 4 * t < n; j += kStep) {
+        const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
+        if (kq.x - lo <= span) atomicAdd(&hist[(kq.x - lo) >> shift], 1u);
+        if (kq.y - lo <= span) atomicAdd(&hist[(kq.y - lo) >> shift], 1u);
+        if (kq.z - lo <= span) atomicAdd(&hist[(kq.z - lo) >> shift], 1u);
+        if (kq.w - lo <= span) atomicAdd(&hist[(kq.w - lo) >> shift], 1u);
+      }
+      meet();
+      // lane l owns digits 8l .. 8l+7; suffix sums over lanes give the number of keys with a larger digit
+      uint32_t b[8], lane_total = 0u;
+      {
+        const uint4 h0 = *reinterpret_cast<const uint4*>(hist + lane * 8), h1 = *reinterpret_cast<const uint4*>(hist + lane * 8 + 4);
+        b[0] = h0.x; b[1] = h0.y; b[2] = h0.z; b[3] = h0.w; b[4] = h1.x; b[5] = h1.y; b[6] = h1.z; b[7] = h1.w;
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) lane_total += b[e];
+      uint32_t above = lane_total;                       // inclusive suffix sum over lanes >= this lane
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_down_sync(0xffffffffu, above, o);
+        if (lane + o < 32) above += x;
+      }
+      above -= lane_total;                               // keys in lanes with larger digits
+      // the digit holding rank `remaining` lies in the lane where above < remaining <= above + lane_total
+      const bool mine = (int)above < remaining && remaining <= (int)(above + lane_total);
+      uint32_t found = 0u;                               // digit, its keys and the rank within them
+      int cls = 0, rank = 0;
+      if (mine) {
+        uint32_t acc = above;
+#pragma unroll
+        for (int e = 7; e >= 0; --e) {
+          if ((int)acc < remaining && remaining <= (int)(acc + b[e])) { found = (uint32_t)(lane * 8 + e); rank = remaining - (int)acc; cls = (int)b[e]; }
+          acc += b[e];
+        }
+      }
+      const int at = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
+      found = __shfl_sync(0xffffffffu, found, at);
+      remaining = __shfl_sync(0xffffffffu, rank, at);
+      cls = __shfl_sync(0xffffffffu, cls, at);
+      lo += found << shift;
+      span = (1u << shift) - 1u;
+      if (shift == 0) { T = lo; need_eq = remaining; n_eq = cls; break; }
+      // A class of at most 32 keys (the usual case after one pass) is finished by rank: its keys are gathered, every lane of
+      // every warp ranks one of them against the others.
+      if (cls <= 32) {
+        for (int j = 4 * t; j - 4 * t < n; j += kStep) {
+          const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
+          const bool a0 = kq.x - lo <= span, a1 = kq.y - lo <= span, a2 = kq.z - lo <= span, a3 = kq.w - lo <= span;
+          if (a0 | a1 | a2 | a3) {
+            int to = (int)atomicAdd(&s_found[rr], (uint32_t)a0 + (uint32_t)a1 + (uint32_t)a2 + (uint32_t)a3);
+            if (a0) s_list[rr][to++] = kq.x;
+            if (a1) s_list[rr][to++] = kq.y;
+            if (a2) s_list[rr][to++] = kq.z;
+            if (a3) s_list[rr][to] = kq.w;
+          }
+        }
+        meet();
+        const uint32_t x = lane < cls ? s_list[rr][lane] : 0u;
+        int G = 0, E = 0;                                // keys of the class larger than / equal to this lane's
+#pragma unroll 4
+        for (int l = 0; l < cls; ++l) {
+          const uint32_t y = __shfl_sync(0xffffffffu, x, l);
+          G += y > x; E += y == x;
+        }
+        const int ts = __ffs(__ballot_sync(0xffffffffu, x != 0u && G < remaining && remaining <= G + E)) - 1;
+        T = __shfl_sync(0xffffffffu, x, ts);
+        need_eq = remaining - __shfl_sync(0xffffffffu, G, ts);
+        n_eq = __shfl_sync(0xffffffffu, E, ts);
+        break;
+      }
+      shift = max(shift - 8, 0);
+      meet();                                            // every warp has walked the bins
+      *reinterpret_cast<uint4*>(hist + (t & 31) * 8) = make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(hist + (t & 31) * 8 + 4) = make_uint4(0u, 0u, 0u, 0u);
+      meet();
+    }
+  }
+  // ---- the list: kept columns in ascending order.  With several warps the counts of all (step, warp) meet first: `excl` and
+  // `ent` are the exclusive sums a lane holds of them, before(k) the columns that precede this warp's in step k.
+  constexpr int kPer = (kEntries + 31) / 32;             // (step, warp) entries per lane, in order
+  int run = 0, ent[kPer], excl = 0;
+  auto publish = [&](int which, uint32_t limit, bool equal) {   // columns with key >= limit, or == limit
+    run = 0;
+    if (W == 1) return;
+    for (int k = 0; k < kMaxSteps; ++k) {
+      int cnt = 0;
+      if (k * kStep < n) {
+        const uint4 kq = *reinterpret_cast<const uint4*>(keys + k * kStep + 4 * t);
+        cnt = (equal ? kq.x == limit : kq.x >= limit) + (equal ? kq.y == limit : kq.y >= limit) + (equal ? kq.z == limit : kq.z >= limit) +
+              (equal ? kq.w == limit : kq.w >= limit);
+        cnt = (int)__reduce_add_sync(0xffffffffu, (uint32_t)cnt);
+      }
+      if (lane == 0) s_cnt[rr][which][k * W + w] = cnt;
+    }
+    meet();
+    int tot = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) { const int idx = lane * kPer + q; ent[q] = idx < kEntries ? s_cnt[rr][which][idx] : 0; tot += ent[q]; }
+    int incl = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    excl = incl - tot;
+  };
+  auto before = [&](int k, int cnt) -> int {
+    if (W == 1) { const int x = run; run += cnt; return x; }
+    const int idx = k * W + w;
+    int x = excl;
+#pragma unroll
+    for (int q = 0; q + 1 < kPer; ++q) if (q < idx % kPer) x += ent[q];
+    return __shfl_sync(0xffffffffu, x, idx / kPer);
+  };
+  if (need_eq < n_eq) {              // ties at T that are not all kept: the later ones are struck out (rare)
+    publish(1, T, true);
+    for (int k = 0; k * kStep < n; ++k) {
+      uint32_t* at = keys + k * kStep + 4 * t;
+      int cnt = 0, rank = 0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const uint32_t bal = __ballot_sync(0xffffffffu, at[u] == T);
+        cnt += __popc(bal); rank += __popc(bal & lt_mask);
+      }
+      rank += before(k, cnt);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (at[u] == T) { if (rank >= need_eq) at[u] = 0u; ++rank; }
+    }
+  }
+  publish(0, T, false);
+  const int base = sink_f ? 1 : 0;
+  for (int k = 0; k * kStep < n; ++k) {
+    const int j = k * kStep + 4 * t;
+    const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
+    const uint32_t b0 = __ballot_sync(0xffffffffu, kq.x >= T), b1 = __ballot_sync(0xffffffffu, kq.y >= T);
+    const uint32_t b2 = __ballot_sync(0xffffffffu, kq.z >= T), b3 = __ballot_sync(0xffffffffu, kq.w >= T);
+    int at = base + before(k, __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3)) +
+             __popc(b0 & lt_mask) + __popc(b1 & lt_mask) + __popc(b2 & lt_mask) + __popc(b3 & lt_mask);
+    if (kq.x >= T) out[at++] = j;
+    if (kq.y >= T) out[at++] = j + 1;
+    if (kq.z >= T) out[at++] = j + 2;
+    if (kq.w >= T) out[at] = j + 3;
+  }
+  if (t == 0) {
+    if (sink_f) out[0] = 0;
+    if (diag_f) out[out1 - out0 - 1] = ri.i;
+  }
+}
+
+// Threshold lists, and TopK lists of rows beyond kTopkRowMax: a warp per row.
 __global__ void __launch_bounds__(kMaskWarps * 32)
 fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask_params p, const int32_t* __restrict__ row_ptr,
-            int32_t* __restrict__ col_idx, int64_t col_capacity, int stage_cap) {
-  extern __shared__ __align__(16) uint32_t key_smem[];
-  uint32_t* hist_smem = key_smem + (size_t)kMaskWarps * stage_cap;   // 256 bins per warp
+            int32_t* __restrict__ col_idx, int64_t col_capacity) {
+  __shared__ __align__(16) uint32_t hist_smem[kMaskWarps * 256];      // 256 bins per warp
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * kMaskWarps + warp;
   const RowInfo ri = decode_row(m, band, scores, r);
@@ -250,68 +552,21 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   // ---- TopK
   const int nf = num_forced(ri.i, p.flags);
   const int take = max(keep_count(n, p) - nf, 0);
-  uint32_t* keys = key_smem + (size_t)warp * stage_cap;
-  const bool staged = n <= stage_cap;
+  auto key_at = [&](int j) -> uint32_t {
+    return is_forced(j, ri.i, p.flags) ? 0u : score_key(ri.s[j]);
+  };
   int c = 0;
   uint32_t k_and = 0xffffffffu, k_or = 0u;     // over the candidates' keys: the bits all of them share are k_and | ~k_or
-  // The same key as score_key in fewer instructions (this loop is bound by instruction issue); forced blocks are not
-  // told apart here: they are taken out again below.  (Their keys stay in k_and / k_or: the bits a superset shares are
-  // shared by the candidates too.)
-  auto lean_key = [](float sc) -> uint32_t {
-    const float z = sc + 0.0f;                                   // -0 -> +0
-    const uint32_t u = __float_as_uint(z);
-    const uint32_t kk = u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
-    return z != z ? 0u : kk;                                     // NaN: never a candidate
-  };
-  auto make_key = [&](int, float sc) -> uint32_t {
-    const uint32_t kk = lean_key(sc);
+#pragma unroll 4
+  for (int j = lane; j < n; j += 32) {
+    const uint32_t kk = key_at(j);
     c += kk != 0u;
     k_or |= kk;
     k_and &= kk != 0u ? kk : 0xffffffffu;
-    return kk;
-  };
-  // four scores per lane and load where the row is 16-byte aligned (the loop is bound by the latency of its loads);
-  // the staged row is padded with zero keys (never candidates) to a multiple of 128
-  const bool vec = (reinterpret_cast<uintptr_t>(ri.s) & 15) == 0;
-  const int head = vec ? (n & ~3) : 0;
-  // (four loads in flight per lane: one load per step left the loop waiting a memory latency per 128 columns, 45 % of
-  // the kernel)
-  for (int j0 = lane * 4; j0 < head; j0 += 512) {
-    float4 v[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      v[u] = j0 + u * 128 < head ? *reinterpret_cast<const float4*>(ri.s + j0 + u * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int j = j0 + u * 128;
-      if (j < head) {
-        const uint4 kq = make_uint4(make_key(j, v[u].x), make_key(j + 1, v[u].y), make_key(j + 2, v[u].z), make_key(j + 3, v[u].w));
-        if (staged) *reinterpret_cast<uint4*>(keys + j) = kq;
-      }
-    }
-  }
-  for (int j = head + lane; j < n; j += 32) {
-    const uint32_t kk = make_key(j, ri.s[j]);
-    if (staged) keys[j] = kk;
-  }
-  const int n_pad = (n + 127) & ~127;
-  if (staged) for (int j = n + lane; j < n_pad; j += 32) keys[j] = 0u;
-  // forced blocks are not candidates: out of the count, and their staged keys blanked (a zero key is never kept by the
-  // selection; the list writer below puts the forced blocks in their places: block 0 first, block i last)
-  const bool sink_f = (p.flags & SEER_FORCE_SINK) != 0u;
-  const bool diag_f = (p.flags & SEER_FORCE_DIAG) != 0u && !(sink_f && ri.i == 0);
-  __syncwarp();
-  if (lane == 0) {                                  // (the staged key where there is one: a global load here costs a memory latency per row)
-    if (sink_f) { c -= (staged ? keys[0] : lean_key(ri.s[0])) != 0u; if (staged) keys[0] = 0u; }
-    if (diag_f) { c -= (staged ? keys[ri.i] : lean_key(ri.s[ri.i])) != 0u; if (staged) keys[ri.i] = 0u; }
   }
   const int ncand = warp_sum(c);
   k_and = __reduce_and_sync(0xffffffffu, k_and);
   k_or = __reduce_or_sync(0xffffffffu, k_or);
-  __syncwarp();
-  auto key_at = [&](int j) -> uint32_t {
-    return is_forced(j, ri.i, p.flags) ? 0u : score_key(ri.s[j]);
-  };
 
   uint32_t T = 0u;      // key of the last kept candidate; kept: key > T, plus the first need_eq with key == T
   int need_eq = 0;
@@ -320,14 +575,8 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   } else if (take == 0) {
     T = 0xffffffffu; need_eq = 0;   // nothing beyond the forced blocks
   } else {
-    // Radix select, up to 8 bits per pass from the top (rows too long to stage re-read their scores in every pass):
-    // histogram the current digit of the keys that match the prefix found so far (warp-private shared-memory bins), walk
-    // the bins from the largest digit down until `remaining` is covered.
+    // radix select as in topk_kernel, the scores re-read in every pass
     uint32_t* hist = hist_smem + warp * 256;
-    // The scores of a row are close together (probabilities of one softmax): the leading bits all candidate keys share
-    // need no pass, and the first digit starts at the highest bit in which two keys differ, so that it spreads the keys
-    // over all 256 bins (a byte-aligned first digit put a whole row into two or three bins: 32 lanes adding to one
-    // shared-memory word).
     const uint32_t differ = k_and ^ k_or;                                 // bit set: not all keys agree there
     int hi_bit = differ == 0u ? 0 : 31 - __clz(differ);                   // highest differing bit
     uint32_t prefix_mask = hi_bit >= 31 ? 0u : ~((2u << hi_bit) - 1u);    // the shared leading bits
@@ -338,19 +587,9 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
       const uint32_t dmask = (2u << (top - shift)) - 1u;
       for (int b = lane; b < 256; b += 32) hist[b] = 0u;
       __syncwarp();
-      if (staged) {
-        for (int j = lane * 4; j < n_pad; j += 128) {
-          const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
-          if (kq.x != 0u && (kq.x & prefix_mask) == prefix) atomicAdd(&hist[(kq.x >> shift) & dmask], 1u);
-          if (kq.y != 0u && (kq.y & prefix_mask) == prefix) atomicAdd(&hist[(kq.y >> shift) & dmask], 1u);
-          if (kq.z != 0u && (kq.z & prefix_mask) == prefix) atomicAdd(&hist[(kq.z >> shift) & dmask], 1u);
-          if (kq.w != 0u && (kq.w & prefix_mask) == prefix) atomicAdd(&hist[(kq.w >> shift) & dmask], 1u);
-        }
-      } else {
-        for (int j = lane; j < n; j += 32) {
-          const uint32_t kk = key_at(j);
-          if (kk != 0u && (kk & prefix_mask) == prefix) atomicAdd(&hist[(kk >> shift) & dmask], 1u);
-        }
+      for (int j = lane; j < n; j += 32) {
+        const uint32_t kk = key_at(j);
+        if (kk != 0u && (kk & prefix_mask) == prefix) atomicAdd(&hist[(kk >> shift) & dmask], 1u);
       }
       __syncwarp();
       // lane l owns digits 8l .. 8l+7; suffix sums over lanes give the number of keys with a larger digit
@@ -370,12 +609,12 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
       above -= lane_total;                               // keys in lanes with larger digits
       // the digit holding rank `remaining` lies in the lane where above < remaining <= above + lane_total
       const bool mine = (int)above < remaining && remaining <= (int)(above + lane_total);
-      uint32_t digit = 0u, sel_cnt = 0u; int new_remaining = 0;
+      uint32_t digit = 0u; int new_remaining = 0;
       if (mine) {
         uint32_t acc = above;
 #pragma unroll
         for (int e = 7; e >= 0; --e) {
-          if ((int)acc < remaining && remaining <= (int)(acc + c[e])) { digit = (uint32_t)(lane * 8 + e); new_remaining = remaining - (int)acc; sel_cnt = c[e]; }
+          if ((int)acc < remaining && remaining <= (int)(acc + c[e])) { digit = (uint32_t)(lane * 8 + e); new_remaining = remaining - (int)acc; }
           acc += c[e];
         }
       }
@@ -383,82 +622,14 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
       const int src = __ffs(owner) - 1;
       digit = __shfl_sync(0xffffffffu, digit, src);
       remaining = __shfl_sync(0xffffffffu, new_remaining, src);
-      const uint32_t class_cnt = __shfl_sync(0xffffffffu, sel_cnt, src);   // keys that share the prefix found so far
       prefix |= digit << shift;
       prefix_mask |= dmask << shift;
       __syncwarp();
-      // A class of at most 32 keys (the usual case after one pass: a row of <= 2048 keys over 256 bins) is finished in
-      // registers: one sweep gathers its keys, every lane ranks one of them against the others.
-      if (staged && shift > 0 && class_cnt <= 32u) {
-        int found = 0;
-        for (int j = lane * 4; j < n_pad; j += 128) {
-          const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
-          const uint32_t kk[4] = {kq.x, kq.y, kq.z, kq.w};
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const bool mt = kk[u] != 0u && (kk[u] & prefix_mask) == prefix;
-            const uint32_t bal = __ballot_sync(0xffffffffu, mt);
-            if (mt) hist[found + __popc(bal & lt_mask)] = kk[u];
-            found += __popc(bal);
-          }
-        }
-        __syncwarp();
-        const uint32_t x = lane < (int)class_cnt ? hist[lane] : 0u;
-        int G = 0, E = 0;                              // keys of the class larger than / equal to this lane's
-#pragma unroll
-        for (int l = 0; l < 32; ++l) {
-          const uint32_t y = __shfl_sync(0xffffffffu, x, l);
-          G += y > x; E += y == x;
-        }
-        const bool is_t = x != 0u && G < remaining && remaining <= G + E;
-        const int ts = __ffs(__ballot_sync(0xffffffffu, is_t)) - 1;
-        prefix = __shfl_sync(0xffffffffu, x, ts);
-        remaining -= __shfl_sync(0xffffffffu, G, ts);
-        __syncwarp();
-        break;
-      }
     }
     T = prefix;                      // the take-th largest key; `remaining` of the keys equal to it are kept
     need_eq = remaining;
   }
   int written = 0, eq_seen = 0;
-  if (staged) {
-    if (sink_f) { if (lane == 0) out[0] = 0; written = 1; }
-    // 128 columns at a time, four consecutive ones per lane: a lane's kept columns follow those of the lanes below it
-    for (int base = 0; base < n_pad; base += 128) {
-      const int j = base + 4 * lane;
-      const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
-      const uint32_t kk[4] = {kq.x, kq.y, kq.z, kq.w};
-      bool eq[4], keep[4];
-      int my_eq = 0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) { eq[u] = kk[u] != 0u && kk[u] == T; my_eq += (int)eq[u]; }
-      int eq_incl = my_eq;
-      if (__any_sync(0xffffffffu, my_eq != 0)) {          // ties at the selection key are rare
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int u = __shfl_up_sync(0xffffffffu, eq_incl, o);
-          if (lane >= o) eq_incl += u;
-        }
-      }
-      int eq_rank = eq_seen + eq_incl - my_eq;            // ties before this lane's first column
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        keep[u] = (kk[u] != 0u && kk[u] > T) || (eq[u] && eq_rank < need_eq);
-        eq_rank += (int)eq[u];
-      }
-      // kept columns of the lanes below this one: four independent ballots instead of a five-step scan
-      const uint32_t b0 = __ballot_sync(0xffffffffu, keep[0]), b1 = __ballot_sync(0xffffffffu, keep[1]);
-      const uint32_t b2 = __ballot_sync(0xffffffffu, keep[2]), b3 = __ballot_sync(0xffffffffu, keep[3]);
-      int at = written + __popc(b0 & lt_mask) + __popc(b1 & lt_mask) + __popc(b2 & lt_mask) + __popc(b3 & lt_mask);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) if (keep[u]) out[at++] = j + u;
-      written += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
-      eq_seen += __shfl_sync(0xffffffffu, eq_incl, 31);
-    }
-    if (diag_f && lane == 0) out[written] = ri.i;
-    return;
-  }
   for (int base = 0; base < n; base += 32) {
     const int j = base + lane;
     const uint32_t kk = j < n ? key_at(j) : 0u;
@@ -473,19 +644,43 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   }
 }
 
-int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, int64_t score_base, int64_t row_lo,
+// Beyond this many rows one CTA's counting takes longer than a launch of its own.
+constexpr int64_t kCountRowsMax = 16384;
+
+template <int W>
+static void launch_topk_w(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
+                          int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
+  constexpr int kRows = W < 4 ? 4 / W : 1, kThreads = W < 4 ? 128 : W * 32;
+  const int cap = (m.max_nb + 128 * W - 1) / (128 * W) * (128 * W);
+  topk_kernel<W><<<(unsigned)((band.row_hi - band.row_lo + kRows - 1) / kRows), kThreads, (size_t)kRows * cap * 4, stream>>>(
+      m, band, scores, p, row_ptr, col_idx, col_capacity, cap);
+}
+// At most 2048 keys per warp (4096-block rows: two warps 4 % slower than four); kTopkRowMax = 8 warps' worth.
+static void launch_topk(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
+                        int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
+  if (m.max_nb <= 2048) launch_topk_w<1>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
+  else if (m.max_nb <= 8192) launch_topk_w<4>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
+  else launch_topk_w<8>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
+}
+
+int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const float2* stats, const ScoreBand& sb, int64_t row_lo,
                      int64_t row_hi, bool first, const seer_mask_params& p, int32_t* row_ptr, int32_t* col_idx,
                      int64_t col_capacity, int64_t* nnz_out, cudaStream_t stream) {
   if (row_hi <= row_lo) return 0;
-  const RowBand band = {row_lo, row_hi, score_base};
+  const RowBand band = {row_lo, row_hi, sb};
   const unsigned grid = (unsigned)((row_hi - row_lo + kMaskWarps - 1) / kMaskWarps);
-  count_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr);
-  scan_kernel<<<1, 1024, 0, stream>>>(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status);
-  const int stage_cap = m.max_nb <= kMaskSmemRowMax ? (m.max_nb + 127) & ~127 : 0;   // long rows re-read their scores instead
-  const size_t smem = (size_t)kMaskWarps * (stage_cap + 256) * sizeof(uint32_t);
-  fill_kernel<<<grid, kMaskWarps * 32, smem, stream>>>(m, band, scores, p, row_ptr, col_idx, col_capacity, stage_cap);
+  int launches = 2;
+  if (stats != nullptr && p.mode != SEER_THRESHOLD && row_hi - row_lo <= kCountRowsMax) {
+    scan_kernel<true><<<1, 1024, 0, stream>>>(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status, CountArgs{m, band, scores, stats, p});
+  } else {
+    count_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr);
+    scan_kernel<false><<<1, 1024, 0, stream>>>(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status, CountArgs{});
+    ++launches;
+  }
+  if (p.mode != SEER_THRESHOLD && m.max_nb <= kTopkRowMax) launch_topk(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
+  else fill_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr, col_idx, col_capacity);
   cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? 3 : -(int)e;
+  return e == cudaSuccess ? launches : -(int)e;
 }
 
 int launch_mask(seer_ctx* ctx, const SeqMeta& m, const float* scores, const seer_mask_params& p, int32_t* row_ptr,
@@ -495,7 +690,8 @@ int launch_mask(seer_ctx* ctx, const SeqMeta& m, const float* scores, const seer
     if (nnz_out) cudaMemsetAsync(nnz_out, 0, sizeof(int64_t), stream);
     return 0;
   }
-  return launch_mask_band(ctx, m, scores, 0, 0, m.rows, true, p, row_ptr, col_idx, col_capacity, nnz_out, stream);
+  const ScoreBand all = {0, m.total_blocks, 0, m.num_q_heads, 0, 0, 0};
+  return launch_mask_band(ctx, m, scores, nullptr, all, 0, m.rows, true, p, row_ptr, col_idx, col_capacity, nnz_out, stream);
 }
 
 // ----------------------------------------------------------------------------------------------- 128-token lists -> 64-token lists
@@ -556,7 +752,7 @@ int launch_expand_lists(seer_ctx* ctx, const SeqMeta& m128, const SeqMeta& m64, 
   }
   const unsigned grid = (unsigned)((m64.rows + kMaskWarps - 1) / kMaskWarps);
   expand_kernel<false><<<grid, kMaskWarps * 32, 0, stream>>>(m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
-  scan_kernel<<<1, 1024, 0, stream>>>(m64.rows, row_ptr64, 1, col_capacity64, nnz_out, ctx->d_status);
+  scan_kernel<false><<<1, 1024, 0, stream>>>(m64.rows, row_ptr64, 1, col_capacity64, nnz_out, ctx->d_status, CountArgs{});
   expand_kernel<true><<<grid, kMaskWarps * 32, 0, stream>>>(m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? 3 : -(int)e;
@@ -564,8 +760,7 @@ int launch_expand_lists(seer_ctx* ctx, const SeqMeta& m128, const SeqMeta& m64, 
 
 seer_status init_mask(seer_ctx* ctx) {
   (void)ctx;
-  cudaError_t e = cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       kMaskWarps * (kMaskSmemRowMax + 256) * (int)sizeof(uint32_t));
+  const cudaError_t e = cudaFuncSetAttribute(topk_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkRowMax * 4);
   return e == cudaSuccess ? SEER_OK : SEER_ERR_CUDA;
 }
 

@@ -47,7 +47,6 @@ seer_status shape_totals(const seer_shape* s, ShapeTotals* t) {
   t->total_tokens = cu[s->batch];
   t->total_q_tokens = s->cu_seqlens_q_host ? s->cu_seqlens_q_host[s->batch] : cu[s->batch];
   t->total_blocks = blocks;
-  t->total_chunks = (blocks + kPoolChunk - 1) / kPoolChunk;   // chunks of the gate's first kernel run over the whole batch
   t->rows = blocks * s->num_q_heads;
   t->score_elems = sq * s->num_q_heads;
   t->causal_blocks = causal * s->num_q_heads;
@@ -58,11 +57,15 @@ seer_status shape_totals(const seer_shape* s, ShapeTotals* t) {
   return SEER_OK;
 }
 
-size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* s) {
-  // projected pooled Q [Hq, blocks, dg] and K [Hkv, blocks, dg], each as three bf16 planes (hi, mid, lo of the fp32 value)
-  size_t gq = align_up((size_t)s->num_q_heads * t.total_blocks * kGateDim * 6, 256);
-  size_t gk = align_up((size_t)s->num_kv_heads * t.total_blocks * kGateDim * 6, 256);
+size_t gate_planes_bytes(const ShapeTotals& t, const seer_shape* s) {
+  // projected pooled Q [Hq, blocks] and K [Hkv, blocks], three bf16 planes (hi, mid, lo of the fp32 value) each
+  size_t gq = align_up((size_t)s->num_q_heads * t.total_blocks * kGatePairBytes, 256);
+  size_t gk = align_up((size_t)s->num_kv_heads * t.total_blocks * kGatePairBytes, 256);
   return gq + gk;
+}
+
+size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* s) {
+  return gate_planes_bytes(t, s) + align_up((size_t)s->num_q_heads * t.total_blocks * gate_stat_segs(t.max_nb) * sizeof(float2), 256);
 }
 
 seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream, SeqMeta* m, int* slot_out) {
@@ -138,7 +141,6 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
   m->group = shape->num_q_heads / shape->num_kv_heads;
   m->total_tokens = (int32_t)t.total_tokens;
   m->total_blocks = (int32_t)t.total_blocks;
-  m->total_chunks = (int32_t)t.total_chunks;
   m->max_nb = t.max_nb;
   m->rows = t.rows;
   m->score_elems = t.score_elems;
@@ -148,6 +150,17 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
   m->qdelta = (const int32_t*)(d + kOffQdelta);
   m->total_q_tokens = (int32_t)t.total_q_tokens;
   m->chunked = shape->cu_seqlens_q_host ? 1 : 0;
+  double tiles = 0;
+  for (int b = 0; b < shape->batch; ++b) {
+    const double nb = (shape->cu_seqlens_host[b + 1] - shape->cu_seqlens_host[b] + shape->block - 1) / shape->block;
+    double before = 0;                                 // blocks before the chunk
+    if (const int32_t* cq = shape->cu_seqlens_q_host)
+      before = ((shape->cu_seqlens_host[b + 1] - shape->cu_seqlens_host[b]) - (cq[b + 1] - cq[b])) / shape->block;
+    tiles += (nb * nb - before * before) / 2 / (128.0 * kScoreTile);
+    if (shape->batch == 1) m->first_q_block = (int32_t)before;
+  }
+  if (shape->batch != 1) m->first_q_block = 0;
+  m->score_tiles = (int64_t)(tiles * shape->num_q_heads);
   m->wait_limit_us = ctx->wait_limit_us;
   m->lose_v_copy = ctx->lose_v_copy;
   *slot_out = slot;
@@ -453,20 +466,25 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
   const int64_t cap = (int64_t)((ws_bytes - gate_bytes) / sizeof(float)) - (int64_t)kBandSlackElems;   // elements per band
   int64_t launched = 0;
   bool bad = false, first = true;
+  // several bands: the statistics of all rows by one launch that fills the GPU
+  const bool with_stats = t.score_elems > cap || gate_split(m, ctx->num_sms);
   {
     int n = opt ? launch_gate_ex(ctx, m, *opt, q, k, Wq, Wk, nullptr, ws, stream)
                 : launch_gate(ctx, m, q, k, Wq, Wk, nullptr, ws, stream);
     if (n < 0) bad = true; else launched += n;
+    if (!bad && with_stats) {
+      n = launch_gate_stats_all(ctx, m, ws, stream);
+      if (n < 0) bad = true; else launched += n;
+    }
   }
   // One band after the other, in CSR row order: scores of the band -> counts -> row_ptr (continued) -> lists.
-  auto run_band = [&](int64_t blk_lo, int64_t blk_hi, int head_lo, int heads, int64_t base, int64_t row_lo, int64_t row_hi) {
+  auto run_band = [&](ScoreBand band, int64_t row_lo, int64_t row_hi) {
     if (bad || row_hi <= row_lo) return;
-    const ScoreBand band = {(int32_t)blk_lo, (int32_t)blk_hi, head_lo, heads, base & ~(int64_t)3};
-    int n = launch_gate_scores_band(m, band, ws, band_buf, stream);
+    band.score_base &= ~(int64_t)3;
+    int n = band.blk_hi > band.blk_lo ? launch_gate_scores_band(ctx, m, band, ws, band_buf, with_stats, stream) : 0;
     if (n >= 0) {
       launched += n;
-      n = launch_mask_band(ctx, m, band_buf, band.score_base, row_lo, row_hi, first, *p, row_ptr, col_idx, col_capacity,
-                           nnz_out, stream);
+      n = launch_mask_band(ctx, m, band_buf, with_stats ? gate_stats(m, ws) : nullptr, band, row_lo, row_hi, first, *p, row_ptr, col_idx, col_capacity, nnz_out, stream);
     }
     if (n < 0) { bad = true; return; }
     launched += n;
@@ -488,28 +506,34 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
         elems += (int64_t)Hq * n1 * n1; blocks += n1;
         ++b1;
       }
-      run_band(blk_off, blk_off + blocks, 0, Hq, score_off, Hq * blk_off, Hq * (blk_off + blocks));
+      run_band({(int32_t)blk_off, (int32_t)(blk_off + blocks), 0, Hq, score_off, 0, 0}, Hq * blk_off, Hq * (blk_off + blocks));
       blk_off += blocks; score_off += elems;
       b = b1;
       continue;
     }
-    const int64_t ntile = (nb + kScoreTile - 1) / kScoreTile;
-    if (nb * nb <= cap) {
-      // whole heads of this sequence
-      const int hb = (int)(cap / (nb * nb));
+    // query blocks of the sequence that have scores: all of them, or those of its chunk
+    int64_t i_lo = 0;
+    if (shape->cu_seqlens_q_host) {
+      const int64_t sq = (int64_t)shape->cu_seqlens_q_host[b + 1] - shape->cu_seqlens_q_host[b], sk = (int64_t)cu[b + 1] - cu[b];
+      i_lo = sq > 0 ? (sk - sq) / shape->block : nb;
+    }
+    const int64_t per_head = (nb - i_lo) * nb;
+    if (per_head <= cap) {
+      // whole heads of this sequence, packed without the rows before the chunk
+      const int hb = per_head > 0 ? (int)(cap / per_head < Hq ? cap / per_head : Hq) : Hq;
       for (int h0 = 0; h0 < Hq; h0 += hb) {
         const int h1 = h0 + hb < Hq ? h0 + hb : Hq;
-        run_band(blk_off, blk_off + nb, h0, h1 - h0, score_off + (int64_t)h0 * nb * nb, Hq * blk_off + (int64_t)h0 * nb,
-                 Hq * blk_off + (int64_t)h1 * nb);
+        run_band({(int32_t)(blk_off + i_lo), (int32_t)(blk_off + nb), h0, h1 - h0, 0, per_head > 0 ? per_head : 1, (int32_t)i_lo},
+                 Hq * blk_off + (int64_t)h0 * nb, Hq * blk_off + (int64_t)h1 * nb);
       }
     } else {
       // runs of 64-row tiles of one head
-      const int64_t tb = cap / ((int64_t)kScoreTile * nb);   // >= 1: the workspace check above
+      const int64_t ntile = (nb + kScoreTile - 1) / kScoreTile, tb = cap / ((int64_t)kScoreTile * nb);   // tb >= 1: the workspace check above
       for (int h = 0; h < Hq; ++h)
         for (int64_t t0 = 0; t0 < ntile; t0 += tb) {
           const int64_t t1 = t0 + tb < ntile ? t0 + tb : ntile;
           const int64_t i0 = t0 * kScoreTile, i1 = t1 * kScoreTile < nb ? t1 * kScoreTile : nb;
-          run_band(blk_off + i0, blk_off + i1, h, 1, score_off + ((int64_t)h * nb + i0) * nb,
+          run_band({(int32_t)(blk_off + i0), (int32_t)(blk_off + i1), h, 1, score_off + ((int64_t)h * nb + i0) * nb, 0, 0},
                    Hq * blk_off + (int64_t)h * nb + i0, Hq * blk_off + (int64_t)h * nb + i1);
         }
     }

@@ -15,8 +15,7 @@ constexpr int kHeadDim = 128;
 constexpr int kGateDim = 128;
 constexpr int kMaxBatch = 4096;
 constexpr int kMetaSlots = 8;
-constexpr int kPoolChunk = 16;  // blocks pooled and projected by one CTA of the gate's first kernel
-constexpr int kScoreTile = 64;  // score rows (blocks of the packed batch) handled by one CTA of the gate's second kernel
+constexpr int kScoreTile = 64;  // column tile of the gate's score kernel, and granularity of the bands of the one-call gate + mask
 
 // Per-batch metadata the kernels read from device memory.
 struct SeqMeta {
@@ -29,7 +28,6 @@ struct SeqMeta {
   int32_t group;               // Hq / Hkv
   int32_t total_tokens;
   int32_t total_blocks;
-  int32_t total_chunks;
   int32_t max_nb;
   int64_t rows;                // Hq * total_blocks
   int64_t score_elems;
@@ -42,17 +40,44 @@ struct SeqMeta {
   int32_t chunked;             // 1 if the shape carries cu_seqlens_q
   // bounded waits of the tcgen05 attention kernel, and the test hook that makes one of them run out
   uint32_t wait_limit_us;      // a barrier wait that lasts this long is declared lost
+  int64_t score_tiles;         // host: 128 x 64 tiles of the score matrix, all heads, about
+  int32_t first_q_block;       // host: first block of the batch that can have queries (one chunked sequence: where its chunk starts)
   int32_t lose_v_copy;         // >= 0: stream 0 of CTA 0 never issues the V copy of its tile with this ordinal
 };
 
+// Projected pooled vectors: per (head, block) three bf16 planes (hi, mid, lo of the fp32 value) of 128 elements.  A head's
+// blocks are stored as tiles of 64 (aligned in the packed batch; the last one may be shorter) in the layout the score
+// kernel's MMAs read: plane -> k half (64 elements = 128 bytes) -> block of the tile -> 16-byte chunk XOR (block % 8), so that
+// a whole tile is one contiguous 48 KB copy.
+constexpr int kGatePairBytes = 3 * kGateDim * 2;
+struct GateTile {
+  size_t base;                 // byte offset from the head's first tile
+  int rows;
+  __host__ __device__ GateTile(int tile, int total_blocks) : base((size_t)tile * 64 * kGatePairBytes), rows(total_blocks - tile * 64 < 64 ? total_blocks - tile * 64 : 64) {}
+};
+
+// Softmax statistics of the gate are formed per segment of this many column tiles (of the packed batch) and combined in order.
+__host__ __device__ inline int gate_seg_tiles(int max_nb) { return max_nb <= 2048 ? 4 : 16; }
+// segments a sequence of max_nb blocks can touch, wherever it starts
+__host__ __device__ inline int gate_stat_segs(int max_nb) { const int c = gate_seg_tiles(max_nb) * kScoreTile; return (max_nb + c - 1) / c + 1; }
+
 // A rectangle of (block row of the packed batch, query head) pairs whose scores are produced and consumed together.
-// score_base is the offset, in the full score matrix, of the band's first element: the band's scores live at
-// (full offset - score_base) in whatever buffer the kernels are given.
+// head_stride == 0: the band's scores lie at (offset in the full score matrix - score_base) in whatever buffer the kernels are
+// given.  Otherwise the band is query blocks >= row0 of one sequence, packed: row i of head h lies at
+// (h - head_lo) * head_stride + (i - row0) * nb.
 struct ScoreBand {
   int32_t blk_lo, blk_hi;      // block rows [blk_lo, blk_hi), numbered over the batch (blk_off)
   int32_t head_lo, heads;
   int64_t score_base;
+  int64_t head_stride;
+  int32_t row0;
 };
+
+// Offset of entry (h, i, 0) of sequence b, which has nb blocks.
+__device__ __forceinline__ int64_t score_row_offset(const SeqMeta& m, const ScoreBand& sb, int b, int nb, int h, int i) {
+  if (sb.head_stride != 0) return (int64_t)(h - sb.head_lo) * sb.head_stride + (int64_t)(i - sb.row0) * nb;
+  return m.score_off[b] + ((int64_t)h * nb + i) * nb - sb.score_base;
+}
 
 struct MetaSlot {
   std::vector<int32_t> key;    // cu_seqlens + Hq: what the slot currently describes
@@ -92,22 +117,29 @@ void finish_call(seer_ctx* ctx, int slot, cudaStream_t stream);
 
 // Host-only shape arithmetic (no CUDA calls): returns SEER_OK and fills totals.
 struct ShapeTotals {
-  int64_t total_tokens, total_q_tokens, total_blocks, total_chunks, rows, score_elems, causal_blocks;
+  int64_t total_tokens, total_q_tokens, total_blocks, rows, score_elems, causal_blocks;
   int32_t max_nb;
 };
 seer_status shape_totals(const seer_shape* shape, ShapeTotals* t);
 
-size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* shape);
+size_t gate_planes_bytes(const ShapeTotals& t, const seer_shape* shape);      // the projected vectors
+size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* shape);   // ... and the softmax statistics behind them
 
 // Kernel launchers (each returns the number of kernels it launched, or a negative cudaError).
 int launch_gate(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const float* Wq, const float* Wk,
                 float* scores, void* ws, cudaStream_t stream);
 int launch_gate_ex(seer_ctx* ctx, const SeqMeta& m, const seer_gate_options& opt, const void* q, const void* k,
                    const float* Wq, const float* Wk, float* scores, void* ws, cudaStream_t stream);
-int launch_gate_scores_band(const SeqMeta& m, const ScoreBand& band, const void* ws, float* scores, cudaStream_t stream);
+// The one-call gate + mask: statistics of all rows once, then the scores of one band at a time, from the vectors a launch with
+// scores == nullptr left in `ws`.
+int launch_gate_stats_all(seer_ctx* ctx, const SeqMeta& m, void* ws, cudaStream_t stream);
+int launch_gate_scores_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& band, void* ws, float* scores, bool with_stats,
+                            cudaStream_t stream);
+const float2* gate_stats(const SeqMeta& m, void* ws);
+bool gate_split(const SeqMeta& m, int num_sms);   // scores of the whole problem: statistics apart from the scores?
 // Mask rows [row_lo, row_hi) from a band of scores; `first` starts row_ptr at 0, later bands continue from the
-// previous band's last entry.
-int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, int64_t score_base, int64_t row_lo,
+// previous band's last entry; `stats` (or nullptr) are the statistics the scores were made from.
+int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const float2* stats, const ScoreBand& sb, int64_t row_lo,
                      int64_t row_hi, bool first, const seer_mask_params& p, int32_t* row_ptr, int32_t* col_idx,
                      int64_t col_capacity, int64_t* nnz_out, cudaStream_t stream);
 // 128-token block lists -> the 64-token lists the attention kernels take (m128 and m64 describe the same batch).
