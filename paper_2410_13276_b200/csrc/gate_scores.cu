@@ -72,6 +72,12 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+// Parts of a row tile's causal columns when the batch is one sequence.
+__host__ __device__ __forceinline__ int part_count(const ScoreBand& band, int tile, int part_tiles) {
+  const int r0 = band.blk_lo + tile * kRows, last = (band.blk_hi - r0 < kRows ? band.blk_hi - r0 : kRows) + r0 - 1;
+  return last / (part_tiles * kCols) + 1;
+}
+
 // (m, l) of two disjoint sets of a row's columns, in units of log2: l counts 2^(x - m); m = -inf: empty
 __device__ __forceinline__ void combine(float& m, float& l, float m2, float l2) {
   const float nm = fmaxf(m, m2);
@@ -82,7 +88,8 @@ __device__ __forceinline__ void combine(float& m, float& l, float m2, float l2) 
 }  // namespace gs
 
 // grid.x = row tiles * band.heads (head fastest; row tiles are visited from the last rows to the first), grid.y = parts of
-// part_tiles column tiles (1 for kBoth; for kStats a part is a segment).  Row r of a tile is query block i_r of sequence b_r; its causal columns are the blocks seq_start_r .. r of
+// part_tiles column tiles (1 for kBoth; for kStats a part is a segment); with one sequence in the batch the parts are in grid.x
+// (a CTA that has nothing to do still takes an SM to itself for 2 us).  Row r of a tile is query block i_r of sequence b_r; its causal columns are the blocks seq_start_r .. r of
 // the batch.  The whole problem is the band (0, total_blocks, 0, Hq, 0).  Scores are written at their offset in the full
 // matrix minus band.score_base.  stats: [head][block of the batch][stat_segs] (m, l).
 template <int kMode>
@@ -102,7 +109,16 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
   const int row_tiles = (band.blk_hi - band.blk_lo + kRows - 1) / kRows;
-  const int tile = row_tiles - 1 - (int)(blockIdx.x / band.heads);
+  int tile = row_tiles - 1 - (int)(blockIdx.x / band.heads), part_of_tile = (int)blockIdx.y;
+  if (kMode != kBoth && m.batch == 1) {                                   // only the parts that exist: row tile t has part_count of them
+    int rest = (int)(blockIdx.x / band.heads);
+    for (tile = row_tiles - 1; tile > 0; --tile) {
+      const int parts = part_count(band, tile, part_tiles);
+      if (rest < parts) break;
+      rest -= parts;
+    }
+    part_of_tile = rest;
+  }
   const int h = band.head_lo + (int)(blockIdx.x % band.heads);
   const int g = h / m.group;
   const int r0 = band.blk_lo + tile * kRows;                              // first block row of the tile
@@ -114,7 +130,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   const int last_col = r0 + rows_valid - 1;
   int col_lo = first_col, col_hi = last_col;                              // columns of this CTA
   if (kMode != kBoth) {
-    const int part_cols = part_tiles * kCols, part = first_col / part_cols + (int)blockIdx.y;
+    const int part_cols = part_tiles * kCols, part = first_col / part_cols + part_of_tile;
     col_lo = max(col_lo, part * part_cols);
     col_hi = min(col_hi, (part + 1) * part_cols - 1);
     if (col_lo > col_hi) return;
@@ -344,6 +360,11 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
 // part_tiles == 0: one CTA per row tile and head
 static dim3 score_grid(const SeqMeta& m, const ScoreBand& band, int part_tiles) {
   const unsigned x = (unsigned)((band.blk_hi - band.blk_lo + gs::kRows - 1) / gs::kRows) * (unsigned)band.heads;
+  if (part_tiles && m.batch == 1) {
+    unsigned n = 0;
+    for (int t = 0; t < (int)(x / band.heads); ++t) n += (unsigned)gs::part_count(band, t, part_tiles);
+    return dim3(n * (unsigned)band.heads, 1);
+  }
   // a row tile that starts in one sequence and ends in another may touch a tile's worth of columns more than the longest one
   const int cols = part_tiles * gs::kCols;
   return dim3(x, part_tiles ? (unsigned)((m.max_nb + gs::kRows + cols - 1) / cols + 1) : 1u);

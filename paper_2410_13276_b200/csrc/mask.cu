@@ -132,52 +132,53 @@ count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mas
   if (lane == 0) row_ptr[r + 1] = c;
 }
 
+// TopK counts of scores whose softmax statistics are at hand, a thread per row.  A row whose maximum and sum are finite has no
+// NaN among its scores, so its length follows from n and the parameters and no score is read (4096 rows of 4096 blocks: 15 us
+// with count_kernel); a row that has not is counted by its thread.
+__global__ void __launch_bounds__(128)
+topk_count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, const float2* __restrict__ stats, seer_mask_params p,
+                  int32_t* __restrict__ row_ptr) {
+  const int64_t r = band.row_lo + (int64_t)blockIdx.x * 128 + threadIdx.x;
+  const RowInfo ri = decode_row(m, band, scores, r);
+  if (!ri.valid) return;
+  const int n = ri.i + 1;
+  int c = 0;
+  if (ri.skip) {
+    // nothing listed
+  } else if (ri.i >= ri.nb - p.dense_tail_blocks) {
+    c = n;
+  } else {
+    const int nf = num_forced(ri.i, p.flags), take = max(keep_count(n, p) - nf, 0);
+    const int seg_cols = gate_seg_tiles(m.max_nb) * kScoreTile, segs = ri.gb / seg_cols - (ri.gb - ri.i) / seg_cols + 1;
+    const float2* st = stats + ((size_t)ri.h * m.total_blocks + ri.gb) * gate_stat_segs(m.max_nb);
+    bool finite = true;
+    for (int s = 0; s < segs; ++s) { const float2 v = st[s]; finite = finite && fabsf(v.x) < 3.0e38f && v.y > 0.f && v.y < 3.0e38f; }
+    int ncand = n - nf;
+    if (!finite) {
+      ncand = 0;
+      for (int j = 0; j < n; ++j) ncand += (!is_forced(j, ri.i, p.flags) && score_key(ri.s[j]) != 0u) ? 1 : 0;
+    }
+    c = nf + min(take, ncand);
+  }
+  row_ptr[r + 1] = c;
+}
+
 // Single CTA: in-place inclusive scan of row_ptr[1..rows].  `first`: row_ptr[0] = 0; otherwise the scan continues from
 // row_ptr[0], the last entry of the rows scanned before.  Tiles of 8192 counts go through shared memory (coalesced loads and
 // stores, the next tile's loads in flight meanwhile), eight consecutive counts per thread, warp shuffles inside a warp; every
 // warp adds up the warp totals for itself.  It is bound by the latency of a tile's three barriers (65 536 rows: 33 us with
 // tiles of 4096 and their loads exposed).  All sums fit 32 bits (the host refuses shapes with 2^31 causal blocks).
-//
-// kCounts (TopK of scores whose softmax statistics are at hand): the counts come from here as well.  A row whose maximum and sum
-// are finite has no NaN among its scores, so its length follows from n and the parameters and no score is read (4096 rows of
-// 4096: 20 us for the two kernels, 6 us); a row that has not is counted by its thread.
-struct CountArgs {
-  SeqMeta m;
-  RowBand band;
-  const float* scores;
-  const float2* stats;
-  seer_mask_params p;
-};
-__device__ __forceinline__ int topk_count(const CountArgs& a, int64_t r) {
-  const RowInfo ri = decode_row(a.m, a.band, a.scores, r);
-  if (ri.skip) return 0;
-  const int n = ri.i + 1;
-  if (ri.i >= ri.nb - a.p.dense_tail_blocks) return n;
-  const int nf = num_forced(ri.i, a.p.flags), take = max(keep_count(n, a.p) - nf, 0);
-  const int seg_cols = gate_seg_tiles(a.m.max_nb) * kScoreTile, segs = (ri.gb / seg_cols) - (ri.gb - ri.i) / seg_cols + 1;
-  const float2* st = a.stats + ((size_t)ri.h * a.m.total_blocks + ri.gb) * gate_stat_segs(a.m.max_nb);
-  bool finite = true;
-  for (int s = 0; s < segs; ++s) { const float2 v = st[s]; finite = finite && fabsf(v.x) < 3.0e38f && v.y > 0.f && v.y < 3.0e38f; }
-  int ncand = n - nf;
-  if (!finite) {
-    ncand = 0;
-    for (int j = 0; j < n; ++j) ncand += (!is_forced(j, ri.i, a.p.flags) && score_key(ri.s[j]) != 0u) ? 1 : 0;
-  }
-  return nf + min(take, ncand);
-}
-
 constexpr int kScanPer = 8, kScanTile = 1024 * kScanPer;
-template <bool kCounts>
 __global__ void __launch_bounds__(1024)
 scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_capacity, int64_t* __restrict__ nnz_out,
-            int* __restrict__ status, CountArgs args) {
+            int* __restrict__ status) {
   __shared__ int32_t tile[kScanTile + kScanTile / 32];     // (one word of padding per 32: eight consecutive words per thread)
   __shared__ int32_t warp_tot[2][32];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   int carry = first ? 0 : row_ptr[0];
   int32_t next[kScanPer];
 #pragma unroll
-  for (int k = 0; k < kScanPer; ++k) next[k] = t + k * 1024 < rows ? (kCounts ? topk_count(args, args.band.row_lo + t + k * 1024) : row_ptr[t + k * 1024 + 1]) : 0;
+  for (int k = 0; k < kScanPer; ++k) next[k] = t + k * 1024 < rows ? row_ptr[t + k * 1024 + 1] : 0;
   int par = 0;
   for (int64_t base = 0; base < rows; base += kScanTile, par ^= 1) {
 #pragma unroll
@@ -186,7 +187,7 @@ scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) {
       const int64_t idx = base + kScanTile + t + k * 1024;
-      next[k] = idx < rows ? (kCounts ? topk_count(args, args.band.row_lo + idx) : row_ptr[idx + 1]) : 0;
+      next[k] = idx < rows ? row_ptr[idx + 1] : 0;
     }
     int v[kScanPer];
 #pragma unroll
@@ -644,9 +645,6 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   }
 }
 
-// Beyond this many rows one CTA's counting takes longer than a launch of its own.
-constexpr int64_t kCountRowsMax = 16384;
-
 template <int W>
 static void launch_topk_w(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
                           int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
@@ -669,18 +667,15 @@ int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const
   if (row_hi <= row_lo) return 0;
   const RowBand band = {row_lo, row_hi, sb};
   const unsigned grid = (unsigned)((row_hi - row_lo + kMaskWarps - 1) / kMaskWarps);
-  int launches = 2;
-  if (stats != nullptr && p.mode != SEER_THRESHOLD && row_hi - row_lo <= kCountRowsMax) {
-    scan_kernel<true><<<1, 1024, 0, stream>>>(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status, CountArgs{m, band, scores, stats, p});
-  } else {
+  if (stats != nullptr && p.mode != SEER_THRESHOLD)
+    topk_count_kernel<<<(unsigned)((row_hi - row_lo + 127) / 128), 128, 0, stream>>>(m, band, scores, stats, p, row_ptr);
+  else
     count_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr);
-    scan_kernel<false><<<1, 1024, 0, stream>>>(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status, CountArgs{});
-    ++launches;
-  }
+  scan_kernel<<<1, 1024, 0, stream>>>(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status);
   if (p.mode != SEER_THRESHOLD && m.max_nb <= kTopkRowMax) launch_topk(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
   else fill_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr, col_idx, col_capacity);
   cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? launches : -(int)e;
+  return e == cudaSuccess ? 3 : -(int)e;
 }
 
 int launch_mask(seer_ctx* ctx, const SeqMeta& m, const float* scores, const seer_mask_params& p, int32_t* row_ptr,
@@ -752,7 +747,7 @@ int launch_expand_lists(seer_ctx* ctx, const SeqMeta& m128, const SeqMeta& m64, 
   }
   const unsigned grid = (unsigned)((m64.rows + kMaskWarps - 1) / kMaskWarps);
   expand_kernel<false><<<grid, kMaskWarps * 32, 0, stream>>>(m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
-  scan_kernel<false><<<1, 1024, 0, stream>>>(m64.rows, row_ptr64, 1, col_capacity64, nnz_out, ctx->d_status, CountArgs{});
+  scan_kernel<<<1, 1024, 0, stream>>>(m64.rows, row_ptr64, 1, col_capacity64, nnz_out, ctx->d_status);
   expand_kernel<true><<<grid, kMaskWarps * 32, 0, stream>>>(m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? 3 : -(int)e;
