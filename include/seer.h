@@ -104,7 +104,10 @@ typedef struct {
  * Not supported with a chunk (SEER_ERR_UNSUPPORTED): seer_prefill_host, seer_gate_scores_static. */
 
 /* Sizing helpers (pure host arithmetic; return 0 / -1 on an invalid shape). */
-size_t seer_workspace_bytes(const seer_shape* shape); /* enough for any of the three calls */
+/* Enough for any of the three calls.  A gate call whose ws goes on behind these bytes with room for the rows' softmax statistics
+ * (at most 8 * seer_mask_rows * (max nb / 256 + 2) bytes) scores long sequences of few heads in two launches that fill the
+ * GPU; without that room it takes one.  The results are the same bit for bit. */
+size_t seer_workspace_bytes(const seer_shape* shape);
 size_t seer_scores_elems(const seer_shape* shape);    /* num_q_heads * sum_b nb_b^2 */
 int64_t seer_mask_rows(const seer_shape* shape);      /* num_q_heads * sum_b nb_b   */
 int64_t seer_causal_blocks(const seer_shape* shape);  /* num_q_heads * sum_b nb_b (nb_b + 1) / 2: capacity that always suffices */

@@ -344,21 +344,22 @@ int launch_gate_scores(const SeqMeta& m, const ScoreBand& band, const uint16_t* 
 bool init_gate_scores();
 
 namespace {
-// The workspace: planes of gq, of gk, statistics.
+// The workspace: planes of gq, of gk and, where it has room, the statistics.
 struct GateWs {
   char *gq, *gk;
   float2* stats;
-  GateWs(const SeqMeta& m, void* ws) {
+  GateWs(const SeqMeta& m, void* ws, size_t ws_bytes) {
     auto up = [](size_t x) { return (x + 255) / 256 * 256; };
     gq = (char*)ws;
     gk = gq + up((size_t)m.num_q_heads * m.total_blocks * kGatePairBytes);
     stats = (float2*)(gk + up((size_t)m.num_kv_heads * m.total_blocks * kGatePairBytes));
+    if ((size_t)((char*)stats - gq) + (size_t)m.num_q_heads * m.total_blocks * gate_stat_segs(m.max_nb) * sizeof(float2) > ws_bytes) stats = nullptr;
   }
 };
 
 int launch_scores_whole(seer_ctx* ctx, const SeqMeta& m, const GateWs& w, float* scores, cudaStream_t stream) {
-  // (the fixed scratch of the allocation-free variant, which has no context, has no room for the statistics)
   int* status = ctx ? ctx->d_status : nullptr;
+  // (the allocation-free variant has no context)
   float2* stats = ctx && gate_split(m, ctx->num_sms) ? w.stats : nullptr;
   const int n1 = stats ? launch_gate_stats(m, (const uint16_t*)w.gq, (const uint16_t*)w.gk, stats, status, stream) : 0;
   if (n1 < 0) return n1;
@@ -369,8 +370,8 @@ int launch_scores_whole(seer_ctx* ctx, const SeqMeta& m, const GateWs& w, float*
 }  // namespace
 
 int launch_gate(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const float* Wq, const float* Wk,
-                float* scores, void* ws, cudaStream_t stream) {
-  const GateWs w(m, ws);
+                float* scores, void* ws, size_t ws_bytes, cudaStream_t stream) {
+  const GateWs w(m, ws, ws_bytes);
   const unsigned heads = (unsigned)(m.num_q_heads + m.num_kv_heads);
   const unsigned big = (unsigned)((m.total_blocks + 15) / 16) * heads;
   if (big > kBigChunkFrom)
@@ -385,10 +386,10 @@ int launch_gate(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, c
 }
 
 int launch_gate_ex(seer_ctx* ctx, const SeqMeta& m, const seer_gate_options& opt, const void* q, const void* k,
-                   const float* Wq, const float* Wk, float* scores, void* ws, cudaStream_t stream) {
+                   const float* Wq, const float* Wk, float* scores, void* ws, size_t ws_bytes, cudaStream_t stream) {
   // averages alone and no rotation: the plain gate
-  if (opt.pool_q == SEER_POOL_AVG && opt.pool_k == SEER_POOL_AVG && opt.rope_theta == 0.f) return launch_gate(ctx, m, q, k, Wq, Wk, scores, ws, stream);
-  const GateWs w(m, ws);
+  if (opt.pool_q == SEER_POOL_AVG && opt.pool_k == SEER_POOL_AVG && opt.rope_theta == 0.f) return launch_gate(ctx, m, q, k, Wq, Wk, scores, ws, ws_bytes, stream);
+  const GateWs w(m, ws, ws_bytes);
   const unsigned grid1 = (unsigned)((m.total_blocks + kPoolChunkEx - 1) / kPoolChunkEx) * (unsigned)(m.num_q_heads + m.num_kv_heads);
   pool_project_ex_kernel<<<grid1, kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk,
                                                               opt.pool_q, opt.pool_k, opt.rope_theta);
@@ -400,18 +401,18 @@ int launch_gate_ex(seer_ctx* ctx, const SeqMeta& m, const seer_gate_options& opt
 }
 
 int launch_gate_stats_all(seer_ctx* ctx, const SeqMeta& m, void* ws, cudaStream_t stream) {
-  const GateWs w(m, ws);
+  const GateWs w(m, ws, SIZE_MAX);
   return launch_gate_stats(m, (const uint16_t*)w.gq, (const uint16_t*)w.gk, w.stats, ctx->d_status, stream);
 }
 
 int launch_gate_scores_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& band, void* ws, float* scores, bool with_stats,
                             cudaStream_t stream) {
-  const GateWs w(m, ws);
+  const GateWs w(m, ws, SIZE_MAX);
   return launch_gate_scores(m, band, (const uint16_t*)w.gq, (const uint16_t*)w.gk, scores, with_stats ? w.stats : nullptr, ctx->d_status,
                             ctx->num_sms, stream);
 }
 
-const float2* gate_stats(const SeqMeta& m, void* ws) { return GateWs(m, ws).stats; }
+const float2* gate_stats(const SeqMeta& m, void* ws) { return GateWs(m, ws, SIZE_MAX).stats; }
 
 // ----------------------------------------------------------------------------------------------- allocation-free variant
 // Scratch for seer_gate_scores_static lives in the library image: every GPU that loads the library carries these
@@ -451,7 +452,7 @@ seer_status gate_scores_static(const seer_shape* shape, const void* q, const voi
   if (t.total_blocks == 0) return SEER_OK;
   if (!q || !k || !Wq || !Wk || !scores) return SEER_ERR_INVALID_ARG;
   // sizes beyond the built-in scratch are refused, never truncated
-  if (shape->batch > kStaticMaxBatch || gate_planes_bytes(t, shape) > kStaticScratchBytes) return SEER_ERR_WORKSPACE;
+  if (shape->batch > kStaticMaxBatch || gate_workspace_bytes(t, shape) > kStaticScratchBytes) return SEER_ERR_WORKSPACE;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kStaticMaxDevices) return SEER_ERR_CUDA;
   unsigned char* base = nullptr;
@@ -501,7 +502,7 @@ seer_status gate_scores_static(const seer_shape* shape, const void* q, const voi
   m.score_tiles = 0; m.first_q_block = 0;
   // The two kernels below are the ones seer_gate_scores launches; only the scratch pointer differs.  Nothing in the
   // scratch has to start at zero: the first kernel writes every projected vector the second one reads.
-  const int n = launch_gate(nullptr, m, q, k, Wq, Wk, scores, base + kStaticMetaBytes, stream);
+  const int n = launch_gate(nullptr, m, q, k, Wq, Wk, scores, base + kStaticMetaBytes, kStaticScratchBytes, stream);
   return n < 0 ? SEER_ERR_CUDA : SEER_OK;
 }
 

@@ -57,15 +57,15 @@ seer_status shape_totals(const seer_shape* s, ShapeTotals* t) {
   return SEER_OK;
 }
 
-size_t gate_planes_bytes(const ShapeTotals& t, const seer_shape* s) {
+size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* s) {
   // projected pooled Q [Hq, blocks] and K [Hkv, blocks], three bf16 planes (hi, mid, lo of the fp32 value) each
   size_t gq = align_up((size_t)s->num_q_heads * t.total_blocks * kGatePairBytes, 256);
   size_t gk = align_up((size_t)s->num_kv_heads * t.total_blocks * kGatePairBytes, 256);
   return gq + gk;
 }
 
-size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* s) {
-  return gate_planes_bytes(t, s) + align_up((size_t)s->num_q_heads * t.total_blocks * gate_stat_segs(t.max_nb) * sizeof(float2), 256);
+size_t gate_stats_bytes(const ShapeTotals& t, const seer_shape* s) {
+  return align_up((size_t)s->num_q_heads * t.total_blocks * gate_stat_segs(t.max_nb) * sizeof(float2), 256);
 }
 
 seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream, SeqMeta* m, int* slot_out) {
@@ -290,7 +290,7 @@ seer_status seer_gate_scores(seer_ctx* ctx, const seer_shape* shape, const void*
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
-  int n = launch_gate(ctx, m, q, k, Wq, Wk, scores, ws, stream);
+  int n = launch_gate(ctx, m, q, k, Wq, Wk, scores, ws, ws_bytes, stream);
   finish_call(ctx, slot, stream);
   if (n < 0) return SEER_ERR_CUDA;
   ctx->launches += n;
@@ -310,7 +310,7 @@ seer_status seer_gate_project(seer_ctx* ctx, const seer_shape* shape, const void
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
-  int n = launch_gate(ctx, m, q, k, Wq, Wk, nullptr, ws, stream);   // no score buffer: pooling and projection only
+  int n = launch_gate(ctx, m, q, k, Wq, Wk, nullptr, ws, ws_bytes, stream);   // no score buffer: pooling and projection only
   finish_call(ctx, slot, stream);
   if (n < 0) return SEER_ERR_CUDA;
   ctx->launches += n;
@@ -334,7 +334,7 @@ seer_status seer_gate_scores_ex(seer_ctx* ctx, const seer_shape* shape, const se
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
-  int n = launch_gate_ex(ctx, m, *opt, q, k, Wq, Wk, scores, ws, stream);
+  int n = launch_gate_ex(ctx, m, *opt, q, k, Wq, Wk, scores, ws, ws_bytes, stream);
   finish_call(ctx, slot, stream);
   if (n < 0) return SEER_ERR_CUDA;
   ctx->launches += n;
@@ -452,8 +452,8 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
   if (p->flags & ~(uint32_t)(SEER_FORCE_DIAG | SEER_FORCE_SINK)) return SEER_ERR_INVALID_ARG;
   if (p->dense_tail_blocks < 0) return SEER_ERR_INVALID_ARG;
   if (t.total_blocks > 0 && ((!q && t.total_q_tokens > 0) || !k || !Wq || !Wk)) return SEER_ERR_INVALID_ARG;
-  const size_t gate_bytes = gate_workspace_bytes(t, shape);
-  if (t.total_blocks > 0 && !ws_ok(ws, ws_bytes, gate_bytes + min_band_bytes(t))) return SEER_ERR_WORKSPACE;
+  const size_t planes_bytes = gate_workspace_bytes(t, shape), stats_bytes = gate_stats_bytes(t, shape);
+  if (t.total_blocks > 0 && !ws_ok(ws, ws_bytes, planes_bytes + min_band_bytes(t))) return SEER_ERR_WORKSPACE;
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
@@ -462,15 +462,19 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
     finish_call(ctx, slot, stream);
     return n0 < 0 ? SEER_ERR_CUDA : SEER_OK;
   }
+  // Several bands, or a problem of few long rows: the statistics of all rows by one launch that fills the GPU, if what follows the
+  // projected vectors has room for them (1 / 28 of the scores of a 2048-block sequence, 1 / 51 at 4096) and for the smallest band
+  const auto band_elems = [&](size_t at) { return (int64_t)((ws_bytes - at) / sizeof(float)) - (int64_t)kBandSlackElems; };
+  const bool with_stats = ws_bytes >= planes_bytes + stats_bytes + min_band_bytes(t) &&
+                          (t.score_elems > band_elems(planes_bytes) || gate_split(m, ctx->num_sms));
+  const size_t gate_bytes = planes_bytes + (with_stats ? stats_bytes : 0);
   float* band_buf = (float*)((char*)ws + gate_bytes);
-  const int64_t cap = (int64_t)((ws_bytes - gate_bytes) / sizeof(float)) - (int64_t)kBandSlackElems;   // elements per band
+  const int64_t cap = band_elems(gate_bytes);          // elements per band
   int64_t launched = 0;
   bool bad = false, first = true;
-  // several bands: the statistics of all rows by one launch that fills the GPU
-  const bool with_stats = t.score_elems > cap || gate_split(m, ctx->num_sms);
   {
-    int n = opt ? launch_gate_ex(ctx, m, *opt, q, k, Wq, Wk, nullptr, ws, stream)
-                : launch_gate(ctx, m, q, k, Wq, Wk, nullptr, ws, stream);
+    int n = opt ? launch_gate_ex(ctx, m, *opt, q, k, Wq, Wk, nullptr, ws, ws_bytes, stream)
+                : launch_gate(ctx, m, q, k, Wq, Wk, nullptr, ws, ws_bytes, stream);
     if (n < 0) bad = true; else launched += n;
     if (!bad && with_stats) {
       n = launch_gate_stats_all(ctx, m, ws, stream);
@@ -613,7 +617,7 @@ namespace {
 // with num_q_heads = G, num_kv_heads = 1.  The arena holds two sets of slice inputs and outputs (copy of slice s + 1 and
 // read-back of slice s - 1 overlap the kernels of slice s) and one set of intermediates.
 struct ArenaLayout {
-  size_t q[2], k[2], v[2], o[2], lse[2], wq[2], wk[2], scores, row_ptr, col_idx, nnz, ws, total;
+  size_t q[2], k[2], v[2], o[2], lse[2], wq[2], wk[2], scores, row_ptr, col_idx, nnz, ws, ws_bytes, total;
 };
 ArenaLayout arena_layout(const seer_shape* slice, const ShapeTotals& t) {   // shape and totals of ONE slice
   ArenaLayout a;
@@ -633,7 +637,8 @@ ArenaLayout arena_layout(const seer_shape* slice, const ShapeTotals& t) {   // s
   a.row_ptr = take(((size_t)t.rows + 1) * 4);
   a.col_idx = take((size_t)t.causal_blocks * 4);
   a.nnz = take(8);
-  a.ws = take(gate_workspace_bytes(t, slice));
+  a.ws_bytes = gate_workspace_bytes(t, slice) + gate_stats_bytes(t, slice);
+  a.ws = take(a.ws_bytes);
   a.total = p;
   return a;
 }

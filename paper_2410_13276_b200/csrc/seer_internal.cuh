@@ -122,14 +122,14 @@ struct ShapeTotals {
 };
 seer_status shape_totals(const seer_shape* shape, ShapeTotals* t);
 
-size_t gate_planes_bytes(const ShapeTotals& t, const seer_shape* shape);      // the projected vectors
-size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* shape);   // ... and the softmax statistics behind them
+size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* shape);   // the projected vectors
+size_t gate_stats_bytes(const ShapeTotals& t, const seer_shape* shape);       // the softmax statistics that may follow them
 
 // Kernel launchers (each returns the number of kernels it launched, or a negative cudaError).
 int launch_gate(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const float* Wq, const float* Wk,
-                float* scores, void* ws, cudaStream_t stream);
+                float* scores, void* ws, size_t ws_bytes, cudaStream_t stream);
 int launch_gate_ex(seer_ctx* ctx, const SeqMeta& m, const seer_gate_options& opt, const void* q, const void* k,
-                   const float* Wq, const float* Wk, float* scores, void* ws, cudaStream_t stream);
+                   const float* Wq, const float* Wk, float* scores, void* ws, size_t ws_bytes, cudaStream_t stream);
 // The one-call gate + mask: statistics of all rows once, then the scores of one band at a time, from the vectors a launch with
 // scores == nullptr left in `ws`.
 int launch_gate_stats_all(seer_ctx* ctx, const SeqMeta& m, void* ws, cudaStream_t stream);

@@ -45,7 +45,10 @@ class Prefill:
         if self.rows < 0:
             raise B.SeerError(2, "shape")
         d = self.device
-        self.ws = torch.empty(max(B.seer_workspace_bytes(self.shape), 256), dtype=torch.uint8, device=d)
+        # the projected vectors and, behind them, room for the gate's row statistics (8 bytes per row and 256 blocks)
+        longest = (int(np.diff(self.cu).max(initial=0)) + block - 1) // block
+        room = 8 * self.rows * (longest // 256 + 2)
+        self.ws = torch.empty(max(B.seer_gate_mask_workspace_bytes(self.shape, room), 256), dtype=torch.uint8, device=d)
         self.scores = torch.empty(max(B.seer_scores_elems(self.shape), 1), dtype=torch.float32, device=d)
         self.row_ptr = torch.zeros(self.rows + 1, dtype=torch.int32, device=d)
         cap = self.causal_blocks if col_capacity is None else col_capacity
