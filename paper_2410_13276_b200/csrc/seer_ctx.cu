@@ -521,9 +521,9 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
       const int64_t sq = (int64_t)shape->cu_seqlens_q_host[b + 1] - shape->cu_seqlens_q_host[b], sk = (int64_t)cu[b + 1] - cu[b];
       i_lo = sq > 0 ? (sk - sq) / shape->block : nb;
     }
-    const int64_t per_head = (nb - i_lo) * nb;
+    const int64_t per_head = packed_rows((int)nb) - packed_rows((int)i_lo);
     if (per_head <= cap) {
-      // whole heads of this sequence, packed without the rows before the chunk
+      // whole heads of this sequence, packed: causal columns alone, no rows before the chunk
       const int hb = per_head > 0 ? (int)(cap / per_head < Hq ? cap / per_head : Hq) : Hq;
       for (int h0 = 0; h0 < Hq; h0 += hb) {
         const int h1 = h0 + hb < Hq ? h0 + hb : Hq;

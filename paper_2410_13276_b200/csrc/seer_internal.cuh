@@ -64,7 +64,9 @@ __host__ __device__ inline int gate_stat_segs(int max_nb) { const int c = gate_s
 // A rectangle of (block row of the packed batch, query head) pairs whose scores are produced and consumed together.
 // head_stride == 0: the band's scores lie at (offset in the full score matrix - score_base) in whatever buffer the kernels are
 // given.  Otherwise the band is query blocks >= row0 of one sequence, packed: row i of head h lies at
-// (h - head_lo) * head_stride + (i - row0) * nb.
+// (h - head_lo) * head_stride + packed_rows(i) - packed_rows(row0), its causal columns alone, rounded up to 64.  A band buffer
+// takes twice the heads of whole rows then, and a band's launches are as many times fewer (32 heads of 4096 blocks in 128 MB:
+// 32 bands -> 11, gate + mask 2.99 -> 2.60 ms).
 struct ScoreBand {
   int32_t blk_lo, blk_hi;      // block rows [blk_lo, blk_hi), numbered over the batch (blk_off)
   int32_t head_lo, heads;
@@ -73,9 +75,15 @@ struct ScoreBand {
   int32_t row0;
 };
 
+// Elements of the packed rows before row i: rows 64 t .. 64 t + 63 take 64 (t + 1) each.
+__host__ __device__ inline int64_t packed_rows(int i) {
+  const int64_t t = i / kScoreTile, w = kScoreTile;
+  return w * w * (t * (t + 1) / 2) + (i - t * w) * w * (t + 1);
+}
+
 // Offset of entry (h, i, 0) of sequence b, which has nb blocks.
 __device__ __forceinline__ int64_t score_row_offset(const SeqMeta& m, const ScoreBand& sb, int b, int nb, int h, int i) {
-  if (sb.head_stride != 0) return (int64_t)(h - sb.head_lo) * sb.head_stride + (int64_t)(i - sb.row0) * nb;
+  if (sb.head_stride != 0) return (int64_t)(h - sb.head_lo) * sb.head_stride + packed_rows(i) - packed_rows(sb.row0);
   return m.score_off[b] + ((int64_t)h * nb + i) * nb - sb.score_base;
 }
 

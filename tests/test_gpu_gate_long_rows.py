@@ -112,7 +112,8 @@ def test_packed_chunk_bands(rt, heads_per_band, mode):
     p.gate()
     p.mask(params)
     want = [x.copy() for x in p.lists_host()]
-    rows_bytes = (141 - starts[0] // 64) * 141 * 4
+    packed = lambda i: 4096 * ((i // 64) * (i // 64 + 1) // 2) + (i % 64) * 64 * (i // 64 + 1)   # columns rounded up to 64
+    rows_bytes = (packed(141) - packed(starts[0] // 64)) * 4
     # with room for the statistics behind the projected vectors (4 heads x 210 blocks x 2 segments x 8 bytes) and without
     for room in (0, 13568):
         p.row_ptr.fill_(-1)
