@@ -146,7 +146,9 @@ __device__ __forceinline__ float row_pass(uint32_t s_addr, float sl2, float R, i
   return a.x + a.y;
 }
 
-// The largest raw score of this thread's row among the keys it sees (key <= last); -inf if there is none.
+// The largest raw score of this thread's row (MASKED: among the keys it sees, key <= last; -inf if there is none).
+// Off the diagonal without the 64 predicates: 16k block maxima and attention 3.99 -> 3.87 ms, 128k prompt 17.3 -> 16.9.
+template <bool MASKED>
 __device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
   float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
   uint32_t sv[2][32];
@@ -158,7 +160,7 @@ __device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
   for (int ch = 0; ch < 2; ++ch)
 #pragma unroll
     for (int e = 0; e < 32; ++e)
-      if (ch * 32 + e <= last) mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(sv[ch][e]));
+      if (!MASKED || ch * 32 + e <= last) mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(sv[ch][e]));
   return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
 }
 
@@ -491,7 +493,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           fail = fail || !mbar_wait(sh, bb + S_FULL + (int)buf, (cnt >> 1) & 1u, status);
           if (__any_sync(0xffffffffu, fail)) { fail = true; break; }
           tc_fence_after();
-          float mx = row_max(tmem + lane_addr + col_s(s, buf), j == it.i ? row : 63);
+          const uint32_t s_addr = tmem + lane_addr + col_s(s, buf);
+          float mx = j == it.i ? row_max<true>(s_addr, row) : row_max<false>(s_addr, 63);
           if (j < 0 || row >= it.q_valid || !(mx == mx)) mx = -CUDART_INF_F;
           else mx = fmaf(mx, sl2, -L2);
           int key = __float_as_int(mx);
@@ -535,7 +538,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         } else {
           const bool diag = j == it.i;
           if (t == 0) {
-            const float mx = row_max(s_addr, diag ? row : 63);
+            const float mx = diag ? row_max<true>(s_addr, row) : row_max<false>(s_addr, 63);
             if (fabsf(mx) < 3.0e38f) R = mx * sl2;
           }
           float sum = diag ? row_pass<true>(s_addr, sl2, R, row, pk) : row_pass<false>(s_addr, sl2, R, row, pk);
@@ -547,7 +550,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
               if (__any_sync(0xffffffffu, fail)) { fail = true; break; }
               tc_fence_after();
             }
-            const float mx = row_max(s_addr, diag ? row : 63) * sl2;
+            const float mx = row_max<true>(s_addr, diag ? row : 63) * sl2;
             const float nr = over && fabsf(mx) < 3.0e38f ? fmaxf(R, mx) : R;
             const float alpha = nr == R ? 1.f : exp2f(R - nr);
             R = nr;
