@@ -61,15 +61,17 @@ constexpr uint32_t kStreamBytes = kStV + kVUnits * kUnit;         // 112 KB
 constexpr uint32_t kOffMl = 2 * kStreamBytes;                     // per stream: (reference, sum) of 128 rows; block maxima
 constexpr uint32_t kMlBytes = 1024;
 constexpr uint32_t kOffBar = kOffMl + 2 * kMlBytes;               // mbarriers
-constexpr int kBarsPerStream = 32;
+constexpr int kBarsPerStream = 40;
 constexpr uint32_t kOffRing = kOffBar + 2 * kBarsPerStream * 8;   // per stream: four item slots of 32 bytes
 constexpr uint32_t kOffMisc = kOffRing + 2 * 4 * 32;              // tmem base, abort flag
 constexpr uint32_t kSmemBytes = kOffMisc + 64;                    // (no slack: the kernel checks the base's alignment)
 static_assert(kSmemBytes <= 232448, "shared memory budget of one CTA");
 
 enum Bar { Q_FULL = 0 /* + buf */, Q_EMPTY = 2, K_FULL = 4 /* + unit */, K_EMPTY = 7, V_FULL = 10, V_EMPTY = 13,
-           S_FULL = 16 /* + buf */, P_FULL = 18, PV_DONE = 20, ITEM_FULL = 22 /* + slot */, ITEM_EMPTY = 26, kBars = 30 };
-static_assert(kBars <= kBarsPerStream && kKUnits <= 3 && kVUnits <= 3, "barrier map");
+           S_FULL = 16 /* + buf */, P_FULL = 18, PV_DONE = 20, ITEM_FULL = 22 /* + slot */, ITEM_EMPTY = 26, kBars = 30,
+           // the block maxima have no V, no P and no O: five K units, four S buffers (M_TAKEN: the group has its maxima)
+           M_KEMPTY = 30, M_TAKEN = 10, kBarsMax = 35 };
+static_assert(kBarsMax <= kBarsPerStream && kKUnits <= 3 && kVUnits <= 3, "barrier map");
 
 constexpr uint32_t kTmemCols = 512;
 // TMEM columns of a stream: two S buffers (P in their first 32 columns), O
@@ -187,6 +189,9 @@ __device__ __forceinline__ int slot_check(const Slot& it, int p, int raw) {
 // kBlockMax: the same pipeline without V: instead of softmax(S) V the kernel writes, for every list entry, the largest
 // probability exp(scale * s - lse) of its 64 x 64 tile (Sec. 3.2, Eq. 2 on the listed blocks), `lse` being an input: a
 // thread takes the maximum of its row, a block's maximum is one redux per warp and a word from its neighbour.
+// Without V and O a stream has five K units and four S buffers: with two of each it waited for copies and MMAs in turn (16k
+// tokens, 32 heads, all causal blocks: 1277 -> 1060 us, 520 clocks a tile; 440 are its 32 KB from L2, 384 its MMAs).  Tiles of four
+// blocks on N = 256 MMAs, 320 clocks per two blocks, gave nothing more.
 template <bool kTrace, bool kChunk, bool kBlockMax = false>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -211,10 +216,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
       const int b = s * kBarsPerStream;
-      for (int i = 0; i < kBars; ++i) {
+      for (int i = 0; i < (kBlockMax ? kBarsMax : kBars); ++i) {
         // Q_EMPTY, P_FULL: one arrival per warp of the softmax group; ITEM_EMPTY: those, the V producer and the issuer
-        const bool group = (i >= Q_EMPTY && i < Q_EMPTY + 2) || (i >= P_FULL && i < P_FULL + 2);
-        mbar_init(sh.bar(b + i), i >= ITEM_EMPTY ? (kBlockMax ? 5 : 6) : group ? 4 : 1);
+        const bool group = (i >= Q_EMPTY && i < Q_EMPTY + 2) || (kBlockMax ? i >= M_TAKEN && i < M_TAKEN + 4 : i >= P_FULL && i < P_FULL + 2);
+        mbar_init(sh.bar(b + i), i >= ITEM_EMPTY && i < ITEM_EMPTY + 4 ? (kBlockMax ? 5 : 6) : group ? 4 : 1);
       }
     }
     st_shared_u32(sh.abort_flag(), 0u);
@@ -236,6 +241,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   // the item and passes it to the other roles through a ring of four slots, each with a full and an empty mbarrier: a slot
   // is rewritten only when every other role has read it.  nlist < 0 ends the stream.  Results do not depend on which
   // stream runs an item.
+  constexpr uint32_t ring_k = kBlockMax ? kKUnits + kVUnits : kKUnits;   // without V its units are K's, without O its columns S buffers
+  constexpr int empty_k = kBlockMax ? M_KEMPTY : K_EMPTY;
   const bool dyn = work_counter != nullptr;
   auto ring_addr = [&](int s, uint32_t n) -> uint32_t { return sh.base + kOffRing + (uint32_t)s * 128u + (n & 3u) * 32u; };
   auto read_slot = [&](int s, uint32_t n) -> Slot {
@@ -296,12 +303,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             tr.sample(cnt); tr.ev(1);
 #pragma unroll
             for (int dh = 0; dh < 2; ++dh) {
-              if (!mbar_wait<kProducerSleepNs>(sh, bb + K_EMPTY + (int)ku, kph ^ 1u, status)) { ok = false; break; }
+              if (!mbar_wait<kProducerSleepNs>(sh, bb + empty_k + (int)ku, kph ^ 1u, status)) { ok = false; break; }
               const uint32_t fb = sh.bar(bb + K_FULL + (int)ku), dst = sbase + kStK + ku * kUnit;
               mbar_expect_tx(fb, has_b ? kUnit : kUnit / 2);   // (an odd list's last tile: the scores of the missing block are not looked at)
               tma_load_3d(dst, &map_k, fb, 64 * dh, it.g, ta);
               if (has_b) tma_load_3d(dst + kHalfQ, &map_k, fb, 64 * dh, it.g, tb);
-              if (++ku == kKUnits) { ku = 0; kph ^= 1u; }
+              if (++ku == ring_k) { ku = 0; kph ^= 1u; }
             }
             tr.ev(2);
             ja = na; jb = nb2;
@@ -392,9 +399,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             tr.sample(cs); tr.ev(10);
             if constexpr (kBlockMax) {
               // the group has taken the maxima of this S buffer's previous tile
-              if (cs >= 2 && !mbar_wait(sh, bb + P_FULL + (int)(cs & 1u), ((cs - 2) >> 1) & 1u, status)) { ok = false; break; }
+              if (cs >= 4 && !mbar_wait(sh, bb + M_TAKEN + (int)(cs & 3u), ((cs - 4) >> 2) & 1u, status)) { ok = false; break; }
             }
-            const uint32_t d = tmem + col_s(s, cs & 1u);     // (P V of tile cs - 2, which read P from it, is ahead on the pipe)
+            const uint32_t sbuf = cs & (kBlockMax ? 3u : 1u), d = tmem + col_s(s, sbuf);     // (P V of tile cs - 2, which read P from it, is ahead on the pipe)
 #pragma unroll
             for (int dh = 0; dh < 2 && ok; ++dh) {
               if (!mbar_wait(sh, bb + K_FULL + (int)ku, kph, status)) { ok = false; break; }
@@ -403,11 +410,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
 #pragma unroll
               for (int kk = 0; kk < 4; ++kk)
                 tc_mma_ws(d, desc_hi_k | (uint64_t)(qlo + (uint32_t)kk * 2u), desc_hi_k | (uint64_t)(klo + (uint32_t)kk * 2u), kIdescS, (dh | kk) != 0 ? 1u : 0u);
-              tc_commit(sh.bar(bb + K_EMPTY + (int)ku));
-              if (++ku == kKUnits) { ku = 0; kph ^= 1u; }
+              tc_commit(sh.bar(bb + empty_k + (int)ku));
+              if (++ku == ring_k) { ku = 0; kph ^= 1u; }
             }
             if (!ok) break;
-            tc_commit(sh.bar(bb + S_FULL + (int)(cs & 1u)));
+            tc_commit(sh.bar(bb + S_FULL + (int)sbuf));
             tr.ev(12);
             ++cs; --left;
             if constexpr (kBlockMax) ++cp;
@@ -487,13 +494,13 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         if (!(fabsf(L) < 3.0e38f)) L = 0.f;                 // a query without a key has no probabilities to report
         const float L2 = L * 1.4426950408889634f;
         for (int t = 0; t < ntiles; ++t, ++cnt) {
-          const uint32_t buf = cnt & 1u;
+          const uint32_t buf = cnt & 1u, sbuf = cnt & 3u;
           const int p = 2 * t + half, j = slot_check(it, p, raw);
           raw = slot_block(it, col_idx, p + 2);
-          fail = fail || !mbar_wait(sh, bb + S_FULL + (int)buf, (cnt >> 1) & 1u, status);
+          fail = fail || !mbar_wait(sh, bb + S_FULL + (int)sbuf, (cnt >> 2) & 1u, status);
           if (__any_sync(0xffffffffu, fail)) { fail = true; break; }
           tc_fence_after();
-          const uint32_t s_addr = tmem + lane_addr + col_s(s, buf);
+          const uint32_t s_addr = tmem + lane_addr + col_s(s, sbuf);
           float mx = j == it.i ? row_max<true>(s_addr, row) : row_max<false>(s_addr, 63);
           if (j < 0 || row >= it.q_valid || !(mx == mx)) mx = -CUDART_INF_F;
           else mx = fmaf(mx, sl2, -L2);
@@ -505,7 +512,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           // their maxima, the group as a whole does not
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(sh.bar(bb + P_FULL + (int)buf));
+          if (lane == 0) mbar_arrive(sh.bar(bb + M_TAKEN + (int)sbuf));
           if (named_bar_or(5 + 2 * s + half, 64, false)) break;
           if ((quad & 1) == 0 && lane == 0 && p < it.nlist) {
             int kx = max(wmax[buf * 4 + quad], wmax[buf * 4 + quad + 1]);

@@ -1,6 +1,7 @@
 """Attention over lists of every small length: tiles of two blocks, so lists of one block (no second half), of odd and of even
 length, across the two score buffers and the four item slots, with the diagonal first, last or absent, an entry that is
-rejected in either half, and rows of different lengths next to one another; against the fp64 oracle."""
+rejected in either half, and rows of different lengths next to one another; against the fp64 oracle.  The block maxima of the
+same lists, whose pipeline has four score buffers and five key units."""
 import math
 
 import numpy as np
@@ -48,3 +49,9 @@ def test_list_lengths(lengths, bad):
     lse = p.lse_host().astype(np.float64)
     fin = np.isfinite(lse_ref)
     assert np.array_equal(fin, np.isfinite(lse)) and np.all(np.abs(lse[fin] - lse_ref[fin]) <= 4e-4 + 2.0 ** -20 * np.abs(lse_ref[fin]))
+    if bad is None:
+        got = p.block_max().cpu().numpy()[:len(col)].astype(np.float64)
+        assert p.status() == 0
+        ref = O.maxpool_listed_blocks(w.q, w.k, w.cu_seqlens, rp, col, hq, 2, 64, 1 / math.sqrt(128))
+        # bf16 operands, fp32 sums of magnitude 10, the lse within its own bound
+        assert np.all(np.abs(got - ref) <= 1e-2 * np.abs(ref) + 1e-7)
