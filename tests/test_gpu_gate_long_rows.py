@@ -121,3 +121,33 @@ def test_packed_chunk_bands(rt, heads_per_band, mode):
         assert p.status() == 0
         for x, y in zip(p.lists_host(), want):
             assert np.array_equal(x, y)
+
+
+# 641 blocks and 16 KV heads: chunks of sixteen blocks; two heads: of two.  The question starts around the edges of both.
+@pytest.mark.parametrize("heads", [16, 2])
+@pytest.mark.parametrize("lens,starts", [([641 * 64 - 9], [b]) for b in (0, 1, 2, 15, 16, 17, 31, 623, 624, 639, 640)] +
+                         [([300 * 64, 65, 341 * 64 - 9], s) for s in ([299, 0, 340], [17, 1, 340], [300, 1, 0], [0, 2, 16])])
+def test_pooling_of_chunks(rt, heads, lens, starts):
+    import torch
+    B, Prefill, ctx = rt
+    cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    q, k = (torch.randn(int(cu[-1]), heads, 128, generator=gen, device="cuda").bfloat16() for _ in range(2))
+    wq, wk = (torch.randn(heads, 128, 128, generator=gen, device="cuda") / 11.3 for _ in range(2))
+    part = [q[min(int(cu[b]) + 64 * s, int(cu[b + 1])):int(cu[b + 1])] for b, s in enumerate(starts)]
+    cu_q = np.concatenate([[0], np.cumsum([len(x) for x in part])]).astype(np.int32)
+    scores = []
+    for qq, cuq in ((q, None), (torch.cat(part), cu_q)):
+        p = Prefill(cu, heads, heads, ctx=ctx, want_lse=False, cu_seqlens_q=cuq)
+        p.q, p.k, p.wq, p.wk = qq, k, wq, wk
+        p.scores.fill_(float("nan"))
+        p.gate()
+        assert p.status() == 0
+        scores.append(p.scores)
+    at = 0
+    for n, s in zip(lens, starts):
+        nb = (n + 63) // 64
+        a, b = (x[at:at + heads * nb * nb].view(heads, nb, nb)[:, s:] for x in scores)
+        tri = torch.ones(nb, nb, dtype=torch.bool, device="cuda").tril()[s:]
+        assert torch.equal(a[:, tri], b[:, tri]) and not torch.isnan(a[:, tri]).any()
+        at += heads * nb * nb
