@@ -275,7 +275,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         bool ok = true;
         int64_t w = draw();
         for (uint32_t n = 0; ok; ++n) {
-          const bool more = w < m.rows;
+          const bool more = w < m.q_rows;
           Item it{};
           if (more) it = decode_item<kChunk>(m, row_ptr, w);
           // the slot's previous content (item n - 4) has been read by everyone
@@ -721,7 +721,7 @@ seer_status init_attn_tc(seer_ctx* ctx) {
 int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const void* v,
                     const int32_t* row_ptr, const int32_t* col_idx, void* o, float* lse, int* work_counter,
                     cudaStream_t stream) {
-  if (m.rows == 0) return 0;
+  if (m.q_rows == 0) return 0;
   // the counter the streams draw their work items from (in the caller's workspace; without one the deal is static)
   if (work_counter != nullptr && cudaMemsetAsync(work_counter, 0, sizeof(int), stream) != cudaSuccess) return -(int)cudaErrorInvalidValue;
   // the input pointers must be 16-byte aligned for TMA
@@ -730,7 +730,7 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
   if (!tc::make_map(ctx, &mq, q, m.total_q_tokens, m.num_q_heads, 64) || !tc::make_map(ctx, &mk, k, m.total_tokens, m.num_kv_heads, 64) ||
       !tc::make_map(ctx, &mv, v, m.total_tokens, m.num_kv_heads, 32))
     return -(int)cudaErrorInvalidValue;
-  const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, (m.rows + 1) / 2);
+  const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, (m.q_rows + 1) / 2);
   unsigned long long* tb = (unsigned long long*)ctx->trace;
   if (m.chunked)               // chunked prefill (never instrumented)
     tc::attn_tc_kernel<false, true><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
@@ -745,12 +745,12 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
 // Max-pooled attention map on the listed blocks (Sec. 3.2, Eq. 2): the attention pipeline without V.
 int launch_block_max_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const int32_t* row_ptr,
                         const int32_t* col_idx, const float* lse, float* out, cudaStream_t stream) {
-  if (m.rows == 0) return 0;
+  if (m.q_rows == 0) return 0;
   if ((((uintptr_t)q | (uintptr_t)k) & 15) != 0) return -(int)cudaErrorMisalignedAddress;
   CUtensorMap mq, mk;
   if (!tc::make_map(ctx, &mq, q, m.total_q_tokens, m.num_q_heads, 64) || !tc::make_map(ctx, &mk, k, m.total_tokens, m.num_kv_heads, 64))
     return -(int)cudaErrorInvalidValue;
-  const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, (m.rows + 1) / 2);
+  const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, (m.q_rows + 1) / 2);
   float* lse_in = const_cast<float*>(lse);   // read only in this mode
   if (m.chunked)
     tc::attn_tc_kernel<false, true, true><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out);

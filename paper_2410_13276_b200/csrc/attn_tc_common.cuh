@@ -214,15 +214,19 @@ struct Item {
 };
 
 // kChunk: chunked prefill.  q / o / lse hold the last positions of each sequence only: their token index is the k / v
-// token index plus dq, and query blocks before the chunk have nothing to do whatever their lists say.
+// token index plus dq.  Query blocks before the chunk have nothing to do whatever their lists say, and no work item is counted for
+// them: a stream took about a microsecond to draw one, look it up and drop it (917 queries against 60k tokens: 29 888 items
+// for 512 of work, 163 -> 67 us; 8k against 128k, 65 536 for 4096: 90 us less).
 template <bool kChunk>
 __device__ __forceinline__ Item decode_item(const SeqMeta& m, const int32_t* __restrict__ row_ptr, int64_t w) {
   Item it;
-  it.b = find_sequence(m.blk_off, m.batch, (int)(w / m.num_q_heads));
+  const int32_t* off = kChunk ? m.qblk_off : m.blk_off;    // blocks with queries: the last ones of each sequence
+  it.b = find_sequence(off, m.batch, (int)(w / m.num_q_heads));
   it.nb = m.blk_off[it.b + 1] - m.blk_off[it.b];
-  const int local = (int)(w - (int64_t)m.num_q_heads * m.blk_off[it.b]);
-  it.g = local / (it.nb * m.group);
-  const int rem = local - it.g * it.nb * m.group;
+  const int nq = kChunk ? off[it.b + 1] - off[it.b] : it.nb;
+  const int local = (int)(w - (int64_t)m.num_q_heads * off[it.b]);
+  it.g = local / (nq * m.group);
+  const int rem = local - it.g * nq * m.group;
   it.i = it.nb - 1 - rem / m.group;
   it.h = it.g * m.group + rem % m.group;
   it.row = (int64_t)m.num_q_heads * m.blk_off[it.b] + (int64_t)it.h * it.nb + it.i;
@@ -231,11 +235,7 @@ __device__ __forceinline__ Item decode_item(const SeqMeta& m, const int32_t* __r
   it.q_valid = min(kBlock, it.slen - it.i * kBlock);
   it.l0 = row_ptr[it.row];
   it.nlist = row_ptr[it.row + 1] - it.l0;
-  it.dq = 0;
-  if (kChunk) {
-    it.dq = m.qdelta[it.b];
-    if (it.i < m.qoff[it.b]) { it.nlist = 0; it.q_valid = 0; }   // no tiles, and no row of o / lse is written
-  }
+  it.dq = kChunk ? m.qdelta[it.b] : 0;
   it.ntiles = (it.nlist + 1) >> 1;
   return it;
 }

@@ -13,7 +13,8 @@ constexpr size_t kOffBlk = kOffCu + sizeof(int32_t) * (kMaxBatch + 1 + 3);
 constexpr size_t kOffScore = kOffBlk + sizeof(int32_t) * (kMaxBatch + 1 + 3);
 constexpr size_t kOffQoff = kOffScore + sizeof(int64_t) * (kMaxBatch + 1);
 constexpr size_t kOffQdelta = kOffQoff + sizeof(int32_t) * (kMaxBatch + 4);
-constexpr size_t kSlotBytes = kOffQdelta + sizeof(int32_t) * (kMaxBatch + 4);
+constexpr size_t kOffQblk = kOffQdelta + sizeof(int32_t) * (kMaxBatch + 4);
+constexpr size_t kSlotBytes = kOffQblk + sizeof(int32_t) * (kMaxBatch + 4);
 
 seer_status shape_totals(const seer_shape* s, ShapeTotals* t) {
   if (!s || !s->cu_seqlens_host || s->batch < 1) return SEER_ERR_INVALID_ARG;
@@ -108,7 +109,8 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
     int64_t* sc = (int64_t*)(h + kOffScore);
     int32_t* qo = (int32_t*)(h + kOffQoff);
     int32_t* qd = (int32_t*)(h + kOffQdelta);
-    blk[0] = 0; sc[0] = 0;
+    int32_t* qb = (int32_t*)(h + kOffQblk);
+    blk[0] = 0; sc[0] = 0; qb[0] = 0;
     for (int b = 0; b < shape->batch; ++b) {
       cu[b] = shape->cu_seqlens_host[b];
       int32_t nb = (shape->cu_seqlens_host[b + 1] - shape->cu_seqlens_host[b] + shape->block - 1) / shape->block;
@@ -120,6 +122,7 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
         qo[b] = sq > 0 ? (sk - sq) / shape->block : nb;          // no queries: past the last block
         qd[b] = cq[b] - (shape->cu_seqlens_host[b] + (sk - sq));  // first query token <-> key token cu[b] + sk - sq
       }
+      qb[b + 1] = qb[b] + nb - qo[b];
     }
     cu[shape->batch] = shape->cu_seqlens_host[shape->batch];
     if (cudaMemcpyAsync(s.dev, s.pinned, kSlotBytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SEER_ERR_CUDA;
@@ -148,18 +151,23 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
   m->block = shape->block;
   m->qoff = (const int32_t*)(d + kOffQoff);
   m->qdelta = (const int32_t*)(d + kOffQdelta);
+  m->qblk_off = (const int32_t*)(d + kOffQblk);
   m->total_q_tokens = (int32_t)t.total_q_tokens;
   m->chunked = shape->cu_seqlens_q_host ? 1 : 0;
   double tiles = 0;
+  int64_t q_blocks = 0;
   for (int b = 0; b < shape->batch; ++b) {
     const double nb = (shape->cu_seqlens_host[b + 1] - shape->cu_seqlens_host[b] + shape->block - 1) / shape->block;
     double before = 0;                                 // blocks before the chunk
     if (const int32_t* cq = shape->cu_seqlens_q_host)
       before = ((shape->cu_seqlens_host[b + 1] - shape->cu_seqlens_host[b]) - (cq[b + 1] - cq[b])) / shape->block;
     tiles += (nb * nb - before * before) / 2 / (128.0 * kScoreTile);
+    const int32_t* cq = shape->cu_seqlens_q_host;
+    if (!cq || cq[b + 1] > cq[b]) q_blocks += (int64_t)(nb - before);   // (a chunk starts on a block)
     if (shape->batch == 1) m->first_q_block = (int32_t)before;
   }
   if (shape->batch != 1) m->first_q_block = 0;
+  m->q_rows = q_blocks * shape->num_q_heads;
   m->score_tiles = (int64_t)(tiles * shape->num_q_heads);
   m->wait_limit_us = ctx->wait_limit_us;
   m->lose_v_copy = ctx->lose_v_copy;

@@ -36,11 +36,13 @@ struct SeqMeta {
   // chunked prefill (all zero without a chunk): the queries of sequence b are its last positions
   const int32_t* qoff;         // [batch] block position of the chunk's first query block
   const int32_t* qdelta;       // [batch] token index in q / o / lse = token index in k / v + qdelta
+  const int32_t* qblk_off;     // [batch + 1] query blocks of the chunks before sequence b
   int32_t total_q_tokens;      // tokens in q / o / lse
   int32_t chunked;             // 1 if the shape carries cu_seqlens_q
   // bounded waits of the tcgen05 attention kernel, and the test hook that makes one of them run out
   uint32_t wait_limit_us;      // a barrier wait that lasts this long is declared lost
   int64_t score_tiles;         // host: 128 x 64 tiles of the score matrix, all heads, about
+  int64_t q_rows;              // host: rows that have queries (all of them without a chunk)
   int32_t first_q_block;       // host: first block of the batch that can have queries (one chunked sequence: where its chunk starts)
   int32_t lose_v_copy;         // >= 0: stream 0 of CTA 0 never issues the V copy of its tile with this ordinal
 };
