@@ -163,30 +163,39 @@ topk_count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, con
   row_ptr[r + 1] = c;
 }
 
-// Single CTA: in-place inclusive scan of row_ptr[1..rows].  `first`: row_ptr[0] = 0; otherwise the scan continues from
-// row_ptr[0], the last entry of the rows scanned before.  Tiles of 8192 counts go through shared memory (coalesced loads and
-// stores, the next tile's loads in flight meanwhile), eight consecutive counts per thread, warp shuffles inside a warp; every
-// warp adds up the warp totals for itself.  It is bound by the latency of a tile's three barriers (65 536 rows: 33 us with
-// tiles of 4096 and their loads exposed).  All sums fit 32 bits (the host refuses shapes with 2^31 causal blocks).
-constexpr int kScanPer = 8, kScanTile = 1024 * kScanPer;
+// In-place inclusive scan of row_ptr[1..rows] by one CTA or a cluster of eight.  `first`: row_ptr[0] = 0; otherwise the scan
+// continues from row_ptr[0], the last entry of the rows scanned before.  Tiles of 8192 counts go through shared memory (coalesced
+// loads and stores, the next tile's loads in flight meanwhile), eight consecutive counts per thread, warp shuffles inside a
+// warp; every warp adds up the warp totals for itself, every CTA the tile totals that the others have put into its shared memory.
+// A CTA alone is bound by the latency of a tile's three barriers, about 2 us (counts, scan and lists of 65 536 rows 248 -> 238 us with
+// the cluster, of 76 800 123 -> 111); beyond one tile the cluster takes eight at a time.  All sums fit 32 bits (the host refuses shapes with 2^31 causal blocks).
+constexpr int kScanPer = 8, kScanTile = 1024 * kScanPer, kScanRanks = 8;
+template <int kRanks>
 __global__ void __launch_bounds__(1024)
 scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_capacity, int64_t* __restrict__ nnz_out,
             int* __restrict__ status) {
   __shared__ int32_t tile[kScanTile + kScanTile / 32];     // (one word of padding per 32: eight consecutive words per thread)
-  __shared__ int32_t warp_tot[2][32];
+  __shared__ int32_t warp_tot[2][32], rank_tot[2][kRanks];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int rank = kRanks > 1 ? (int)blockIdx.x : 0;       // (the grid is one cluster)
   int carry = first ? 0 : row_ptr[0];
   int32_t next[kScanPer];
 #pragma unroll
-  for (int k = 0; k < kScanPer; ++k) next[k] = t + k * 1024 < rows ? row_ptr[t + k * 1024 + 1] : 0;
+  for (int k = 0; k < kScanPer; ++k) {
+    const int64_t idx = (int64_t)rank * kScanTile + t + k * 1024;
+    next[k] = idx < rows ? row_ptr[idx + 1] : 0;
+  }
+  // (a CTA's shared memory may be written to once it runs)
+  if (kRanks > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   int par = 0;
-  for (int64_t base = 0; base < rows; base += kScanTile, par ^= 1) {
+  for (int64_t base0 = 0; base0 < rows; base0 += kRanks * kScanTile, par ^= 1) {
+    const int64_t base = base0 + rank * kScanTile;
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) { const int idx = t + k * 1024; tile[idx + (idx >> 5)] = next[k]; }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) {
-      const int64_t idx = base + kScanTile + t + k * 1024;
+      const int64_t idx = base + kRanks * kScanTile + t + k * 1024;
       next[k] = idx < rows ? row_ptr[idx + 1] : 0;
     }
     int v[kScanPer];
@@ -206,7 +215,23 @@ scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_
       const int o = __shfl_up_sync(0xffffffffu, w, off);
       if (lane >= off) w += o;
     }
-    const int before_warp = __shfl_sync(0xffffffffu, w, (warp + 31) & 31), total = __shfl_sync(0xffffffffu, w, 31);
+    const int before_warp = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+    int total = __shfl_sync(0xffffffffu, w, 31);
+    if (kRanks > 1) {
+      if (t < kRanks) {                                    // this CTA's total to CTA t
+        const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&rank_tot[par][rank]);
+        uint32_t theirs;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(theirs) : "r"(mine), "r"(t));
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(theirs), "r"(total) : "memory");
+      }
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+      total = 0;
+#pragma unroll
+      for (int q = 0; q < kRanks; ++q) {
+        const int x = rank_tot[par][q];
+        if (q < rank) carry += x; else total += x;         // (carry: counts before this CTA's tile)
+      }
+    }
     const int before = carry + (warp > 0 ? before_warp : 0) + (incl - v[kScanPer - 1]);
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) { const int idx = kScanPer * t + k; tile[idx + (idx >> 5)] = before + v[k]; }
@@ -219,11 +244,29 @@ scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_
     }
     // (a thread's stores of the next tile go to the words it has just read)
   }
-  if (t == 0) {
+  if (t == 0 && rank == 0) {
     if (first) row_ptr[0] = 0;
     if (nnz_out) *nnz_out = carry;
     if (carry > col_capacity) atomicCAS(status, 0, (int)SEER_ERR_CAPACITY);
   }
+}
+
+static cudaError_t launch_scan(int64_t rows, int32_t* row_ptr, int first, int64_t col_capacity, int64_t* nnz_out, int* status,
+                               cudaStream_t stream) {
+  if (rows <= kScanTile) {
+    scan_kernel<1><<<1, 1024, 0, stream>>>(rows, row_ptr, first, col_capacity, nnz_out, status);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kScanRanks);
+  cfg.blockDim = dim3(1024);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kScanRanks; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, scan_kernel<kScanRanks>, rows, row_ptr, first, col_capacity, nnz_out, status);
 }
 
 // The key a TopK row is ranked by, in fewer instructions than score_key (the loops are bound by instruction issue).
@@ -671,7 +714,8 @@ int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const
     topk_count_kernel<<<(unsigned)((row_hi - row_lo + 127) / 128), 128, 0, stream>>>(m, band, scores, stats, p, row_ptr);
   else
     count_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr);
-  scan_kernel<<<1, 1024, 0, stream>>>(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status);
+  const cudaError_t es = launch_scan(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status, stream);
+  if (es != cudaSuccess) return -(int)es;
   if (p.mode != SEER_THRESHOLD && m.max_nb <= kTopkRowMax) launch_topk(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
   else fill_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr, col_idx, col_capacity);
   cudaError_t e = cudaGetLastError();
@@ -747,7 +791,8 @@ int launch_expand_lists(seer_ctx* ctx, const SeqMeta& m128, const SeqMeta& m64, 
   }
   const unsigned grid = (unsigned)((m64.rows + kMaskWarps - 1) / kMaskWarps);
   expand_kernel<false><<<grid, kMaskWarps * 32, 0, stream>>>(m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
-  scan_kernel<<<1, 1024, 0, stream>>>(m64.rows, row_ptr64, 1, col_capacity64, nnz_out, ctx->d_status);
+  const cudaError_t es = launch_scan(m64.rows, row_ptr64, 1, col_capacity64, nnz_out, ctx->d_status, stream);
+  if (es != cudaSuccess) return -(int)es;
   expand_kernel<true><<<grid, kMaskWarps * 32, 0, stream>>>(m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? 3 : -(int)e;

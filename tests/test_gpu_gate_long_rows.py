@@ -151,3 +151,16 @@ def test_pooling_of_chunks(rt, heads, lens, starts):
         tri = torch.ones(nb, nb, dtype=torch.bool, device="cuda").tril()[s:]
         assert torch.equal(a[:, tri], b[:, tri]) and not torch.isnan(a[:, tri]).any()
         at += heads * nb * nb
+
+
+# rows of the mask: one tile of the scan (8192), a tile and a row, a cluster's eight tiles, and beyond
+@pytest.mark.parametrize("hq,seqs", [(1, 1), (2, 4095), (2, 4096), (3, 2731), (17, 3855), (16, 4096), (18, 3641), (40, 3500)])
+def test_scan_sizes(rt, hq, seqs):
+    B, Prefill, ctx = rt
+    p = Prefill(np.arange(seqs + 1, dtype=np.int32), hq, 1, ctx=ctx, want_lse=False)   # a block each: lists of no or one entry
+    p.scores.uniform_()
+    p.mask(B.make_mask_params(B.SEER_THRESHOLD, threshold=0.7, flags=0))
+    assert p.status() == 0
+    rp, col = p.lists_host()
+    kept = p.scores_host().reshape(-1)[:hq * seqs] > np.float32(0.7)
+    assert np.array_equal(rp, np.concatenate([[0], np.cumsum(kept)])) and int(p.nnz.item()) == kept.sum() and not col[:kept.sum()].any()
