@@ -207,6 +207,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   sh.abort_addr = sh.base + kOffMisc + 8;
   sh.limit_us = m.wait_limit_us;
   if ((sh.base & 1023u) != 0u) {                           // the swizzled tiles need the alignment
+    grid_wait();
     if (threadIdx.x == 0) atomicCAS(status, 0, (int)SEER_ERR_CUDA);
     return;
   }
@@ -232,6 +233,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_wait();
   const uint32_t tmem = *tmem_slot;
   const unsigned long long cta_t0 = kTrace ? global_ns() : 0ull;
   const long long cta_c0 = kTrace ? clock64() : 0ll;
@@ -680,6 +682,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   }
 }
 
+__global__ void zero_kernel(int* __restrict__ word) {
+  grid_wait();
+  if (threadIdx.x == 0) *word = 0;
+}
+
 // ------------------------------------------------------------------------------------------------ host side
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -722,8 +729,6 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
                     const int32_t* row_ptr, const int32_t* col_idx, void* o, float* lse, int* work_counter,
                     cudaStream_t stream) {
   if (m.q_rows == 0) return 0;
-  // the counter the streams draw their work items from (in the caller's workspace; without one the deal is static)
-  if (work_counter != nullptr && cudaMemsetAsync(work_counter, 0, sizeof(int), stream) != cudaSuccess) return -(int)cudaErrorInvalidValue;
   // the input pointers must be 16-byte aligned for TMA
   if ((((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)o) & 15) != 0) return -(int)cudaErrorMisalignedAddress;
   CUtensorMap mq, mk, mv;
@@ -731,15 +736,24 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
       !tc::make_map(ctx, &mv, v, m.total_tokens, m.num_kv_heads, 32))
     return -(int)cudaErrorInvalidValue;
   const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, (m.q_rows + 1) / 2);
+  // The counter the streams draw their work items from lies in the caller's workspace; without one, or with an item a stream at
+  // most, the deal is static.  (Its zero by a kernel: a memset would make this launch wait for all that precedes it.)
+  cudaError_t e = cudaSuccess;
+  int launched = 0;
+  if (m.q_rows <= 2 * (int64_t)grid) work_counter = nullptr;
+  if (work_counter != nullptr) {
+    e = launch_next(tc::zero_kernel, 1, 32, 0, stream, work_counter);
+    if (e != cudaSuccess) return -(int)e;
+    launched = 1;
+  }
   unsigned long long* tb = (unsigned long long*)ctx->trace;
   if (m.chunked)               // chunked prefill (never instrumented)
-    tc::attn_tc_kernel<false, true><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
+    e = launch_next(tc::attn_tc_kernel<false, true>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
   else if (tb != nullptr)      // the instrumented instantiation
-    tc::attn_tc_kernel<true, false><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
+    e = launch_next(tc::attn_tc_kernel<true, false>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
   else
-    tc::attn_tc_kernel<false, false><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? 1 : -(int)e;
+    e = launch_next(tc::attn_tc_kernel<false, false>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
+  return e == cudaSuccess ? launched + 1 : -(int)e;
 }
 
 // Max-pooled attention map on the listed blocks (Sec. 3.2, Eq. 2): the attention pipeline without V.
@@ -752,11 +766,9 @@ int launch_block_max_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const vo
     return -(int)cudaErrorInvalidValue;
   const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, (m.q_rows + 1) / 2);
   float* lse_in = const_cast<float*>(lse);   // read only in this mode
-  if (m.chunked)
-    tc::attn_tc_kernel<false, true, true><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out);
-  else
-    tc::attn_tc_kernel<false, false, true><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = m.chunked
+      ? launch_next(tc::attn_tc_kernel<false, true, true>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr)
+      : launch_next(tc::attn_tc_kernel<false, false, true>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr);
   return e == cudaSuccess ? 1 : -(int)e;
 }
 

@@ -112,6 +112,7 @@ pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* _
   __shared__ __align__(16) float part[kSplit > 1 ? kChunk * kMaxSteps * 2 * kHeadDim : kChunk * kHeadDim];
 
   const PoolWork work(m, kChunk);
+  grid_wait();
   if (work.idle) return;
   const int chunk = work.chunk, H = work.H, h = work.h;
   const bool is_q = work.is_q;
@@ -252,6 +253,7 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
   __shared__ int block_pos[kChunk];                        // position of each block in its sequence (block RoPE)
 
   const PoolWork work(m, kChunk);
+  grid_wait();
   if (work.idle) return;
   const int chunk = work.chunk, H = work.H, h = work.h;
   const bool is_q = work.is_q;
@@ -409,11 +411,9 @@ int launch_gate(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, c
                 float* scores, void* ws, size_t ws_bytes, cudaStream_t stream) {
   const GateWs w(m, ws, ws_bytes);
   const unsigned big = PoolWork::grid(m, 16);
-  if (big > kBigChunkFrom)
-    pool_project_kernel<16><<<big, kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk);
-  else
-    pool_project_kernel<2><<<PoolWork::grid(m, 2), kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk);
-  cudaError_t e0 = cudaGetLastError();
+  const cudaError_t e0 = big > kBigChunkFrom
+      ? launch_next(pool_project_kernel<16>, big, kPoolThreads, 0, stream, m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk)
+      : launch_next(pool_project_kernel<2>, PoolWork::grid(m, 2), kPoolThreads, 0, stream, m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk);
   if (e0 != cudaSuccess) return -(int)e0;
   if (scores == nullptr) return 1;                     // projection only: the scores follow band by band
   const int n2 = launch_scores_whole(ctx, m, w, scores, stream);
@@ -426,9 +426,8 @@ int launch_gate_ex(seer_ctx* ctx, const SeqMeta& m, const seer_gate_options& opt
   if (opt.pool_q == SEER_POOL_AVG && opt.pool_k == SEER_POOL_AVG && opt.rope_theta == 0.f) return launch_gate(ctx, m, q, k, Wq, Wk, scores, ws, ws_bytes, stream);
   const GateWs w(m, ws, ws_bytes);
   const unsigned grid1 = PoolWork::grid(m, kPoolChunkEx);
-  pool_project_ex_kernel<<<grid1, kPoolThreads, 0, stream>>>(m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk,
-                                                              opt.pool_q, opt.pool_k, opt.rope_theta);
-  cudaError_t e0 = cudaGetLastError();
+  const cudaError_t e0 = launch_next(pool_project_ex_kernel, grid1, kPoolThreads, 0, stream, m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk,
+                                     w.gq, w.gk, opt.pool_q, opt.pool_k, opt.rope_theta);
   if (e0 != cudaSuccess) return -(int)e0;
   if (scores == nullptr) return 1;
   const int n2 = launch_scores_whole(ctx, m, w, scores, stream);

@@ -101,6 +101,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(gs_raw);
   unsigned char* smem = gs_raw;
   if ((base & 1023u) != 0u) {
+    grid_wait();
     if (threadIdx.x == 0 && status != nullptr) atomicCAS(status, 0, (int)SEER_ERR_CUDA);
     return;
   }
@@ -133,7 +134,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
     const int part_cols = part_tiles * kCols, part = first_col / part_cols + part_of_tile;
     col_lo = max(col_lo, part * part_cols);
     col_hi = min(col_hi, (part + 1) * part_cols - 1);
-    if (col_lo > col_hi) return;
+    if (col_lo > col_hi) { grid_wait(); return; }
   }
 
   // this thread's row (threads t, t + 128, .. share row t; the helpers only need the tile's column range)
@@ -154,7 +155,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   } else if (threadIdx.x < kRows) {
     *reinterpret_cast<int2*>(smem + kOffMeta + row * 16 + 8) = make_int2(0, -1);
   }
-  if (!__syncthreads_or(my_last >= 0 ? 1 : 0)) return;                    // a tile of query blocks before their chunks
+  if (!__syncthreads_or(my_last >= 0 ? 1 : 0)) { grid_wait(); return; }                    // a tile of query blocks before their chunks
   const int tile_lo = col_lo / kCols;
   const int ntiles = col_hi / kCols - tile_lo + 1;                        // column tiles of one sweep
   const int total = kMode == kBoth ? 2 * ntiles : ntiles;
@@ -172,6 +173,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_wait();
   const uint32_t tmem = *tmem_slot;
   const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
   const int half = (warp >> 2) & 1;                                       // which 32 columns of a tile this row warp takes
@@ -388,8 +390,7 @@ int launch_gate_stats(const SeqMeta& m, const uint16_t* gq, const uint16_t* gk, 
   const int part = gate_seg_tiles(m.max_nb);
   const dim3 grid = score_grid(m, all, part);
   if (grid.x == 0) return 0;
-  gate_scores_kernel<gs::kStats><<<grid, gs::kThreads, gs::kSmemBytes, stream>>>(m, all, gq, gk, nullptr, stats, status, part);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = launch_next(gate_scores_kernel<gs::kStats>, grid, gs::kThreads, gs::kSmemBytes, stream, m, all, gq, gk, nullptr, stats, status, part);
   return e == cudaSuccess ? 1 : -(int)e;
 }
 
@@ -402,9 +403,9 @@ int launch_gate_scores(const SeqMeta& m, const ScoreBand& band, const uint16_t* 
   while (part < 16 && tiles / part > num_sms) part *= 2;
   const dim3 grid = score_grid(m, band, stats != nullptr ? part : 0);
   if (grid.x == 0) return 0;
-  if (stats != nullptr) gate_scores_kernel<gs::kWrite><<<grid, gs::kThreads, gs::kSmemBytes, stream>>>(m, band, gq, gk, scores, stats, status, part);
-  else gate_scores_kernel<gs::kBoth><<<grid, gs::kThreads, gs::kSmemBytes, stream>>>(m, band, gq, gk, scores, nullptr, status, 0);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = stats != nullptr
+      ? launch_next(gate_scores_kernel<gs::kWrite>, grid, gs::kThreads, gs::kSmemBytes, stream, m, band, gq, gk, scores, stats, status, part)
+      : launch_next(gate_scores_kernel<gs::kBoth>, grid, gs::kThreads, gs::kSmemBytes, stream, m, band, gq, gk, scores, nullptr, status, 0);
   return e == cudaSuccess ? 1 : -(int)e;
 }
 

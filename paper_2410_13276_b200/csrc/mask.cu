@@ -90,6 +90,7 @@ count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mas
   const int lane = threadIdx.x & 31;
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * kMaskWarps + (threadIdx.x >> 5);
   const RowInfo ri = decode_row(m, band, scores, r);
+  grid_wait();
   if (!ri.valid) return;
   const int n = ri.i + 1;
   int c = 0;
@@ -140,6 +141,7 @@ topk_count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, con
                   int32_t* __restrict__ row_ptr) {
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * 128 + threadIdx.x;
   const RowInfo ri = decode_row(m, band, scores, r);
+  grid_wait();
   if (!ri.valid) return;
   const int n = ri.i + 1;
   int c = 0;
@@ -178,12 +180,13 @@ scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_
   __shared__ int32_t warp_tot[2][32], rank_tot[2][kRanks];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int rank = kRanks > 1 ? (int)blockIdx.x : 0;       // (the grid is one cluster)
-  int carry = first ? 0 : row_ptr[0];
+  grid_wait();
+  int carry = first ? 0 : __ldcg(row_ptr);                 // (read past L1: the kernel rewrites it)
   int32_t next[kScanPer];
 #pragma unroll
   for (int k = 0; k < kScanPer; ++k) {
     const int64_t idx = (int64_t)rank * kScanTile + t + k * 1024;
-    next[k] = idx < rows ? row_ptr[idx + 1] : 0;
+    next[k] = idx < rows ? __ldcg(row_ptr + idx + 1) : 0;
   }
   // (a CTA's shared memory may be written to once it runs)
   if (kRanks > 1) asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -196,7 +199,7 @@ scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_
 #pragma unroll
     for (int k = 0; k < kScanPer; ++k) {
       const int64_t idx = base + kRanks * kScanTile + t + k * 1024;
-      next[k] = idx < rows ? row_ptr[idx + 1] : 0;
+      next[k] = idx < rows ? __ldcg(row_ptr + idx + 1) : 0;
     }
     int v[kScanPer];
 #pragma unroll
@@ -253,19 +256,19 @@ scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_
 
 static cudaError_t launch_scan(int64_t rows, int32_t* row_ptr, int first, int64_t col_capacity, int64_t* nnz_out, int* status,
                                cudaStream_t stream) {
-  if (rows <= kScanTile) {
-    scan_kernel<1><<<1, 1024, 0, stream>>>(rows, row_ptr, first, col_capacity, nnz_out, status);
-    return cudaGetLastError();
-  }
+  if (rows <= kScanTile)
+    return launch_next(scan_kernel<1>, 1, 1024, 0, stream, rows, row_ptr, first, col_capacity, nnz_out, status);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kScanRanks);
   cfg.blockDim = dim3(1024);
   cfg.stream = stream;
-  cudaLaunchAttribute attr = {};
-  attr.id = cudaLaunchAttributeClusterDimension;
-  attr.val.clusterDim.x = kScanRanks; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2] = {};
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kScanRanks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, scan_kernel<kScanRanks>, rows, row_ptr, first, col_capacity, nnz_out, status);
 }
 
@@ -305,6 +308,7 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   };
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * kRows + rr;
   const RowInfo ri = decode_row(m, band, scores, r);
+  grid_wait();
   if (!ri.valid || ri.skip) return;                              // (uniform in a row's group)
   const int n = ri.i + 1;
   const int32_t out0 = row_ptr[r], out1 = row_ptr[r + 1];
@@ -546,6 +550,7 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * kMaskWarps + warp;
   const RowInfo ri = decode_row(m, band, scores, r);
+  grid_wait();
   if (!ri.valid || ri.skip) return;
   const int n = ri.i + 1;
   const int32_t out0 = row_ptr[r], out1 = row_ptr[r + 1];
@@ -689,19 +694,19 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
 }
 
 template <int W>
-static void launch_topk_w(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
+static cudaError_t launch_topk_w(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
                           int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
   constexpr int kRows = W < 4 ? 4 / W : 1, kThreads = W < 4 ? 128 : W * 32;
   const int cap = (m.max_nb + 128 * W - 1) / (128 * W) * (128 * W);
-  topk_kernel<W><<<(unsigned)((band.row_hi - band.row_lo + kRows - 1) / kRows), kThreads, (size_t)kRows * cap * 4, stream>>>(
-      m, band, scores, p, row_ptr, col_idx, col_capacity, cap);
+  return launch_next(topk_kernel<W>, (unsigned)((band.row_hi - band.row_lo + kRows - 1) / kRows), kThreads, (size_t)kRows * cap * 4, stream, m, band,
+                     scores, p, row_ptr, col_idx, col_capacity, cap);
 }
 // At most 2048 keys per warp (4096-block rows: two warps 4 % slower than four); kTopkRowMax = 8 warps' worth.
-static void launch_topk(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
+static cudaError_t launch_topk(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
                         int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
-  if (m.max_nb <= 2048) launch_topk_w<1>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
-  else if (m.max_nb <= 8192) launch_topk_w<4>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
-  else launch_topk_w<8>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
+  if (m.max_nb <= 2048) return launch_topk_w<1>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
+  if (m.max_nb <= 8192) return launch_topk_w<4>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
+  return launch_topk_w<8>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
 }
 
 int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const float2* stats, const ScoreBand& sb, int64_t row_lo,
@@ -710,15 +715,14 @@ int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const
   if (row_hi <= row_lo) return 0;
   const RowBand band = {row_lo, row_hi, sb};
   const unsigned grid = (unsigned)((row_hi - row_lo + kMaskWarps - 1) / kMaskWarps);
-  if (stats != nullptr && p.mode != SEER_THRESHOLD)
-    topk_count_kernel<<<(unsigned)((row_hi - row_lo + 127) / 128), 128, 0, stream>>>(m, band, scores, stats, p, row_ptr);
-  else
-    count_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr);
-  const cudaError_t es = launch_scan(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status, stream);
-  if (es != cudaSuccess) return -(int)es;
-  if (p.mode != SEER_THRESHOLD && m.max_nb <= kTopkRowMax) launch_topk(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
-  else fill_kernel<<<grid, kMaskWarps * 32, 0, stream>>>(m, band, scores, p, row_ptr, col_idx, col_capacity);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = stats != nullptr && p.mode != SEER_THRESHOLD
+      ? launch_next(topk_count_kernel, (unsigned)((row_hi - row_lo + 127) / 128), 128, 0, stream, m, band, scores, stats, p, row_ptr)
+      : launch_next(count_kernel, grid, kMaskWarps * 32, 0, stream, m, band, scores, p, row_ptr);
+  if (e == cudaSuccess) e = launch_scan(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status, stream);
+  if (e == cudaSuccess)
+    e = p.mode != SEER_THRESHOLD && m.max_nb <= kTopkRowMax
+        ? launch_topk(m, band, scores, p, row_ptr, col_idx, col_capacity, stream)
+        : launch_next(fill_kernel, grid, kMaskWarps * 32, 0, stream, m, band, scores, p, row_ptr, col_idx, col_capacity);
   return e == cudaSuccess ? 3 : -(int)e;
 }
 
@@ -743,6 +747,7 @@ template <bool kFill>
 __global__ void __launch_bounds__(kMaskWarps * 32)
 expand_kernel(SeqMeta m128, SeqMeta m64, const int32_t* __restrict__ row_ptr128, const int32_t* __restrict__ col_idx128,
               int32_t* __restrict__ row_ptr64, int32_t* __restrict__ col_idx64, int64_t col_capacity64) {
+  grid_wait();
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * kMaskWarps + (threadIdx.x >> 5);
   if (r >= m64.rows) return;
@@ -790,11 +795,10 @@ int launch_expand_lists(seer_ctx* ctx, const SeqMeta& m128, const SeqMeta& m64, 
     return 0;
   }
   const unsigned grid = (unsigned)((m64.rows + kMaskWarps - 1) / kMaskWarps);
-  expand_kernel<false><<<grid, kMaskWarps * 32, 0, stream>>>(m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
-  const cudaError_t es = launch_scan(m64.rows, row_ptr64, 1, col_capacity64, nnz_out, ctx->d_status, stream);
-  if (es != cudaSuccess) return -(int)es;
-  expand_kernel<true><<<grid, kMaskWarps * 32, 0, stream>>>(m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_next(expand_kernel<false>, grid, kMaskWarps * 32, 0, stream, m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
+  if (e == cudaSuccess) e = launch_scan(m64.rows, row_ptr64, 1, col_capacity64, nnz_out, ctx->d_status, stream);
+  if (e == cudaSuccess)
+    e = launch_next(expand_kernel<true>, grid, kMaskWarps * 32, 0, stream, m128, m64, row_ptr128, col_idx128, row_ptr64, col_idx64, col_capacity64);
   return e == cudaSuccess ? 3 : -(int)e;
 }
 
