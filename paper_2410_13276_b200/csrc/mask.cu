@@ -280,35 +280,44 @@ __device__ __forceinline__ uint32_t lean_key(float sc) {
   return z != z ? 0u : kk;                                       // NaN: never a candidate
 }
 
-// TopK lists, W warps per row, the row's keys in shared memory (`cap` of them, a multiple of 128 W; step k of a row is the
-// columns 128 W k + 4 t + u of thread t, u < 4).
+// TopK lists, W warps per row, the row's keys in shared memory (`cap` of them, a multiple of 128 W).  A warp works on a contiguous
+// run of the row's columns, 128 at a time, a lane four of them.
 //
-// It is bound by instruction issue, so the loops are short and rolled: with the keys in registers and the loops unrolled the
-// kernel waited for instructions (a row of 2048 keys took 2300 instructions and 20 000 clocks, and more warps did not help).
+// It is bound by instruction issue (3.5 of 4 per clock), so the loops are short and rolled (with the keys in registers and the
+// loops unrolled it waited for instructions), what a row needs once is done by one of its warps and passed on, and the
+// counts that order the warps' parts of the list are taken in the pass that gathers the threshold's class.
 // A row gets one warp up to 2048 blocks, and as many as keep it at 2048 keys per warp beyond.  Measured: 65 536 rows of up to
-// 2048 blocks 251 -> 183 us, 4096 rows of up to 4096 blocks (which re-read their scores in every pass) 158 -> 34 us.
+// 2048 blocks 251 -> 176 us, 4096 rows of up to 4096 blocks (which re-read their scores in every pass) 158 -> 31 us; what a row
+// needs once done by every warp of it, and a pass of its own for the counts: 183 and 34.
 template <int W>
-__global__ void __launch_bounds__(W < 4 ? 128 : W * 32)
+__global__ void __launch_bounds__(W < 4 ? 128 : W * 32, W < 8 ? 12 : 6)
 topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask_params p, const int32_t* __restrict__ row_ptr,
             int32_t* __restrict__ col_idx, int64_t col_capacity, int cap) {
-  constexpr int kWarps = W < 4 ? 4 : W, kRows = kWarps / W, kStep = 128 * W;
-  constexpr int kMaxSteps = 16, kEntries = kMaxSteps * W;        // (the launcher keeps cap <= 16 steps)
+  constexpr int kWarps = W < 4 ? 4 : W, kRows = kWarps / W;
   extern __shared__ __align__(16) uint32_t key_smem[];
   __shared__ __align__(16) uint32_t s_hist[kRows][256];
   __shared__ uint32_t s_red[kRows][3][W];
   __shared__ uint32_t s_list[kRows][32];
+  __shared__ uint32_t s_own[kRows][32];
   __shared__ uint32_t s_found[kRows];
-  __shared__ int s_cnt[kRows][2][W > 1 ? kEntries : 1];
+  __shared__ int s_cnt[kRows][2][W];
+  __shared__ uint32_t s_pick[kRows][4];
+  __shared__ RowInfo s_row[kRows];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rr = warp / W, w = warp % W, t = w * 32 + lane;      // row of the CTA, warp and thread within the row's group
+  const int rr = warp / W, w = warp % W;                         // row of the CTA, warp within the row's group
   auto meet = [&]() {                                            // the warps of a row
     if (W == 1) __syncwarp();
     else if (W < 4) asm volatile("bar.sync %0, %1;" ::"r"(1 + rr), "n"(W * 32) : "memory");
     else __syncthreads();
   };
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * kRows + rr;
-  const RowInfo ri = decode_row(m, band, scores, r);
+  RowInfo ri;
+  if (W == 1 || w == 0) {
+    ri = decode_row(m, band, scores, r);
+    if (W > 1 && lane == 0) s_row[rr] = ri;
+  }
   grid_wait();
+  if (W > 1) { meet(); ri = s_row[rr]; }
   if (!ri.valid || ri.skip) return;                              // (uniform in a row's group)
   const int n = ri.i + 1;
   const int32_t out0 = row_ptr[r], out1 = row_ptr[r + 1];
@@ -316,7 +325,7 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   int32_t* __restrict__ out = col_idx + out0;
   const uint32_t lt_mask = (1u << lane) - 1u;
   if (ri.i >= ri.nb - p.dense_tail_blocks) {           // a dense row at the end of the sequence: every causal block
-    for (int j = t; j < n; j += W * 32) out[j] = j;
+    for (int j = w * 32 + lane; j < n; j += W * 32) out[j] = j;
     return;
   }
   uint32_t* keys = key_smem + (size_t)rr * cap;
@@ -324,30 +333,32 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   const bool sink_f = (p.flags & SEER_FORCE_SINK) != 0u;
   const bool diag_f = (p.flags & SEER_FORCE_DIAG) != 0u && !(sink_f && ri.i == 0);
   const int take = max(keep_count(n, p) - num_forced(ri.i, p.flags), 0);
+  const int run_cols = (n + 128 * W - 1) / (128 * W) * 128;      // columns of a warp
+  const int j_lo = w * run_cols, j_hi = min(j_lo + run_cols, n), j_mine = j_lo + 4 * lane;
 
   // ---- keys (0: not a candidate: past the row, NaN, or forced, which the writer puts in its place by itself)
   uint32_t c = 0, k_min = 0xffffffffu, k_max = 0u;               // over the candidates
   const uint32_t nan_bits = 0x7fffffffu;
   const uint32_t* __restrict__ src = reinterpret_cast<const uint32_t*>(ri.s);
   const bool vec = (reinterpret_cast<uintptr_t>(ri.s) & 15) == 0;
-  for (int j0 = 4 * t; j0 - 4 * t < n; j0 += 4 * kStep) {
+  for (int j0 = j_mine; j0 - 4 * lane < j_hi; j0 += 512) {
     uint4 v[4];                                                  // four loads in flight per lane
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int j = j0 + q * kStep;
+      const int j = j0 + q * 128;
       v[q] = make_uint4(nan_bits, nan_bits, nan_bits, nan_bits);
-      if (vec && j + 3 < n) v[q] = __ldg(reinterpret_cast<const uint4*>(src + j));
-      else if (j < n) {
+      if (vec && j + 3 < j_hi) v[q] = __ldg(reinterpret_cast<const uint4*>(src + j));
+      else if (j < j_hi) {
         v[q].x = __ldg(src + j);
-        if (j + 1 < n) v[q].y = __ldg(src + j + 1);
-        if (j + 2 < n) v[q].z = __ldg(src + j + 2);
-        if (j + 3 < n) v[q].w = __ldg(src + j + 3);
+        if (j + 1 < j_hi) v[q].y = __ldg(src + j + 1);
+        if (j + 2 < j_hi) v[q].z = __ldg(src + j + 2);
+        if (j + 3 < j_hi) v[q].w = __ldg(src + j + 3);
       }
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int j = j0 + q * kStep;
-      if (j - 4 * t >= n) break;                                 // (uniform)
+      const int j = j0 + q * 128;
+      if (j - 4 * lane >= j_hi) break;                           // (uniform)
       uint4 kq = make_uint4(lean_key(__uint_as_float(v[q].x)), lean_key(__uint_as_float(v[q].y)), lean_key(__uint_as_float(v[q].z)), lean_key(__uint_as_float(v[q].w)));
       if (sink_f && j == 0) kq.x = 0u;
       if (diag_f && (uint32_t)(ri.i - j) < 4u) {
@@ -362,9 +373,14 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
       k_min = min(min(k_min, min(kq.x - 1u, kq.y - 1u)), min(kq.z - 1u, kq.w - 1u));   // (0, not a candidate, wraps to the largest)
     }
   }
-  *reinterpret_cast<uint4*>(hist + (t & 31) * 8) = make_uint4(0u, 0u, 0u, 0u);
-  *reinterpret_cast<uint4*>(hist + (t & 31) * 8 + 4) = make_uint4(0u, 0u, 0u, 0u);
-  if (t == 0) s_found[rr] = 0u;
+  auto clear_hist = [&]() {
+    *reinterpret_cast<uint4*>(hist + lane * 8) = make_uint4(0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4*>(hist + lane * 8 + 4) = make_uint4(0u, 0u, 0u, 0u);
+  };
+  if (w == 0) {
+    clear_hist();
+    if (lane == 0) s_found[rr] = 0u;
+  }
   uint32_t ncand = __reduce_add_sync(0xffffffffu, c);
   k_min = __reduce_min_sync(0xffffffffu, k_min);
   k_max = __reduce_max_sync(0xffffffffu, k_max);
@@ -379,6 +395,7 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   // ---- T: kept are the candidates with key >= T, of those with key == T only the first need_eq of n_eq
   uint32_t T = 1u;
   int need_eq = 0, n_eq = 0;
+  bool counted = W == 1;                                         // s_cnt[.][0] holds the warps' kept columns
   if (take >= (int)ncand) {
     // every candidate is kept
   } else if (take == 0) {
@@ -386,13 +403,12 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   } else {
     // The scores of a row are close together (probabilities of one softmax), often on both sides of a power of two.  So the
     // first pass bins the distance from the smallest key, scaled to 128..256 bins: binning the keys' own leading bits put a
-    // flat row into a dozen bins, 32 lanes adding to a few shared-memory words, and took another pass.  Every warp of the row
-    // walks the bins for itself.
+    // flat row into a dozen bins, 32 lanes adding to a few shared-memory words, and took another pass.
     uint32_t lo = k_min + 1u, span = k_max - lo;                          // the class: keys lo .. lo + span
     int shift = max(24 - __clz(span | 1u), 0);
     int remaining = take;           // rank (1-based, from the top) still to locate inside the current class
     for (;;) {
-      for (int j = 4 * t; j - 4 * t < n; j += kStep) {
+      for (int j = j_mine; j - 4 * lane < j_hi; j += 128) {
         const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
         if (kq.x - lo <= span) atomicAdd(&hist[(kq.x - lo) >> shift], 1u);
         if (kq.y - lo <= span) atomicAdd(&hist[(kq.y - lo) >> shift], 1u);
@@ -400,143 +416,154 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
         if (kq.w - lo <= span) atomicAdd(&hist[(kq.w - lo) >> shift], 1u);
       }
       meet();
-      // lane l owns digits 8l .. 8l+7; suffix sums over lanes give the number of keys with a larger digit
-      uint32_t b[8], lane_total = 0u;
-      {
-        const uint4 h0 = *reinterpret_cast<const uint4*>(hist + lane * 8), h1 = *reinterpret_cast<const uint4*>(hist + lane * 8 + 4);
-        b[0] = h0.x; b[1] = h0.y; b[2] = h0.z; b[3] = h0.w; b[4] = h1.x; b[5] = h1.y; b[6] = h1.z; b[7] = h1.w;
-      }
+      uint32_t found = 0u;                               // digit that holds the rank sought, its keys and the rank within them
+      int cls = 0;
+      if (W == 1 || w == 0) {
+        // lane l owns digits 8l .. 8l+7; suffix sums over lanes give the number of keys with a larger digit
+        uint32_t b[8], lane_total = 0u;
+        {
+          const uint4 h0 = *reinterpret_cast<const uint4*>(hist + lane * 8), h1 = *reinterpret_cast<const uint4*>(hist + lane * 8 + 4);
+          b[0] = h0.x; b[1] = h0.y; b[2] = h0.z; b[3] = h0.w; b[4] = h1.x; b[5] = h1.y; b[6] = h1.z; b[7] = h1.w;
+        }
 #pragma unroll
-      for (int e = 0; e < 8; ++e) lane_total += b[e];
-      uint32_t above = lane_total;                       // inclusive suffix sum over lanes >= this lane
+        for (int e = 0; e < 8; ++e) lane_total += b[e];
+        uint32_t above = lane_total;                     // inclusive suffix sum over lanes >= this lane
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t x = __shfl_down_sync(0xffffffffu, above, o);
-        if (lane + o < 32) above += x;
-      }
-      above -= lane_total;                               // keys in lanes with larger digits
-      // the digit holding rank `remaining` lies in the lane where above < remaining <= above + lane_total
-      const bool mine = (int)above < remaining && remaining <= (int)(above + lane_total);
-      uint32_t found = 0u;                               // digit, its keys and the rank within them
-      int cls = 0, rank = 0;
-      if (mine) {
-        uint32_t acc = above;
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t x = __shfl_down_sync(0xffffffffu, above, o);
+          if (lane + o < 32) above += x;
+        }
+        above -= lane_total;                             // keys in lanes with larger digits
+        // the digit holding rank `remaining` lies in the lane where above < remaining <= above + lane_total
+        const bool mine = (int)above < remaining && remaining <= (int)(above + lane_total);
+        int rank = 0;
+        if (mine) {
+          uint32_t acc = above;
 #pragma unroll
-        for (int e = 7; e >= 0; --e) {
-          if ((int)acc < remaining && remaining <= (int)(acc + b[e])) { found = (uint32_t)(lane * 8 + e); rank = remaining - (int)acc; cls = (int)b[e]; }
-          acc += b[e];
+          for (int e = 7; e >= 0; --e) {
+            if ((int)acc < remaining && remaining <= (int)(acc + b[e])) { found = (uint32_t)(lane * 8 + e); rank = remaining - (int)acc; cls = (int)b[e]; }
+            acc += b[e];
+          }
+        }
+        if (W > 1) {
+          clear_hist();
+          if (mine) { s_pick[rr][0] = found; s_pick[rr][1] = (uint32_t)rank; s_pick[rr][2] = (uint32_t)cls; }
+        } else {
+          const int at = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
+          found = __shfl_sync(0xffffffffu, found, at);
+          remaining = __shfl_sync(0xffffffffu, rank, at);
+          cls = __shfl_sync(0xffffffffu, cls, at);
         }
       }
-      const int at = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
-      found = __shfl_sync(0xffffffffu, found, at);
-      remaining = __shfl_sync(0xffffffffu, rank, at);
-      cls = __shfl_sync(0xffffffffu, cls, at);
+      meet();
+      if (W > 1) { found = s_pick[rr][0]; remaining = (int)s_pick[rr][1]; cls = (int)s_pick[rr][2]; }
       lo += found << shift;
       span = (1u << shift) - 1u;
       if (shift == 0) { T = lo; need_eq = remaining; n_eq = cls; break; }
-      // A class of at most 32 keys (the usual case after one pass) is finished by rank: its keys are gathered, every lane of
-      // every warp ranks one of them against the others.
+      // A class of at most 32 keys (the usual case after one pass) is finished by rank: its keys are gathered, each lane of one
+      // warp ranks one of them against the others.  The columns above the class are kept: their number is taken on the way.
       if (cls <= 32) {
-        for (int j = 4 * t; j - 4 * t < n; j += kStep) {
+        int kept = 0;
+        for (int j = j_mine; j - 4 * lane < j_hi; j += 128) {
           const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
           const bool a0 = kq.x - lo <= span, a1 = kq.y - lo <= span, a2 = kq.z - lo <= span, a3 = kq.w - lo <= span;
+          if (W > 1) kept += (kq.x > lo + span) + (kq.y > lo + span) + (kq.z > lo + span) + (kq.w > lo + span);
           if (a0 | a1 | a2 | a3) {
-            int to = (int)atomicAdd(&s_found[rr], (uint32_t)a0 + (uint32_t)a1 + (uint32_t)a2 + (uint32_t)a3);
+            const int first = (int)atomicAdd(&s_found[rr], (uint32_t)a0 + (uint32_t)a1 + (uint32_t)a2 + (uint32_t)a3);
+            int to = first;
             if (a0) s_list[rr][to++] = kq.x;
             if (a1) s_list[rr][to++] = kq.y;
             if (a2) s_list[rr][to++] = kq.z;
-            if (a3) s_list[rr][to] = kq.w;
+            if (a3) s_list[rr][to++] = kq.w;
+            if (W > 1) for (int q = first; q < to; ++q) s_own[rr][q] = (uint32_t)w;
           }
         }
-        meet();
-        const uint32_t x = lane < cls ? s_list[rr][lane] : 0u;
-        int G = 0, E = 0;                                // keys of the class larger than / equal to this lane's
-#pragma unroll 4
-        for (int l = 0; l < cls; ++l) {
-          const uint32_t y = __shfl_sync(0xffffffffu, x, l);
-          G += y > x; E += y == x;
+        if (W > 1) {
+          kept = (int)__reduce_add_sync(0xffffffffu, (uint32_t)kept);
+          if (lane == 0) s_cnt[rr][0][w] = kept;
         }
-        const int ts = __ffs(__ballot_sync(0xffffffffu, x != 0u && G < remaining && remaining <= G + E)) - 1;
-        T = __shfl_sync(0xffffffffu, x, ts);
-        need_eq = remaining - __shfl_sync(0xffffffffu, G, ts);
-        n_eq = __shfl_sync(0xffffffffu, E, ts);
+        meet();
+        if (W == 1 || w == 0) {
+          const uint32_t x = lane < cls ? s_list[rr][lane] : 0u;
+          int G = 0, E = 0;                              // keys of the class larger than / equal to this lane's
+#pragma unroll 4
+          for (int l = 0; l < cls; ++l) {
+            const uint32_t y = __shfl_sync(0xffffffffu, x, l);
+            G += y > x; E += y == x;
+          }
+          const int ts = __ffs(__ballot_sync(0xffffffffu, x != 0u && G < remaining && remaining <= G + E)) - 1;
+          T = __shfl_sync(0xffffffffu, x, ts);
+          need_eq = remaining - __shfl_sync(0xffffffffu, G, ts);
+          n_eq = __shfl_sync(0xffffffffu, E, ts);
+          if (W > 1) {
+            const uint32_t own = lane < cls ? s_own[rr][lane] : 0xffffffffu;
+            int add = 0;
+#pragma unroll
+            for (int q = 0; q < W; ++q) { const int more = __popc(__ballot_sync(0xffffffffu, own == (uint32_t)q && x >= T)); if (lane == q) add = more; }
+            if (lane < W) s_cnt[rr][0][lane] += add;
+            if (lane == 0) { s_pick[rr][0] = T; s_pick[rr][1] = (uint32_t)need_eq; s_pick[rr][2] = (uint32_t)n_eq; }
+          }
+        }
+        if (W > 1) {
+          meet();
+          T = s_pick[rr][0]; need_eq = (int)s_pick[rr][1]; n_eq = (int)s_pick[rr][2];
+          counted = true;
+        }
         break;
       }
       shift = max(shift - 8, 0);
-      meet();                                            // every warp has walked the bins
-      *reinterpret_cast<uint4*>(hist + (t & 31) * 8) = make_uint4(0u, 0u, 0u, 0u);
-      *reinterpret_cast<uint4*>(hist + (t & 31) * 8 + 4) = make_uint4(0u, 0u, 0u, 0u);
-      meet();
+      if (W == 1) { clear_hist(); meet(); }
     }
   }
-  // ---- the list: kept columns in ascending order.  With several warps the counts of all (step, warp) meet first: `excl` and
-  // `ent` are the exclusive sums a lane holds of them, before(k) the columns that precede this warp's in step k.
-  constexpr int kPer = (kEntries + 31) / 32;             // (step, warp) entries per lane, in order
-  int run = 0, ent[kPer], excl = 0;
-  auto publish = [&](int which, uint32_t limit, bool equal) {   // columns with key >= limit, or == limit
-    run = 0;
-    if (W == 1) return;
-    for (int k = 0; k < kMaxSteps; ++k) {
-      int cnt = 0;
-      if (k * kStep < n) {
-        const uint4 kq = *reinterpret_cast<const uint4*>(keys + k * kStep + 4 * t);
-        cnt = (equal ? kq.x == limit : kq.x >= limit) + (equal ? kq.y == limit : kq.y >= limit) + (equal ? kq.z == limit : kq.z >= limit) +
-              (equal ? kq.w == limit : kq.w >= limit);
-        cnt = (int)__reduce_add_sync(0xffffffffu, (uint32_t)cnt);
-      }
-      if (lane == 0) s_cnt[rr][which][k * W + w] = cnt;
+  // ---- the list: kept columns in ascending order.  A warp's columns follow those of the warps before it.
+  auto publish = [&](int which, uint32_t limit, bool equal) {   // a warp's columns with key >= limit, or == limit
+    int cnt = 0;
+    for (int j = j_mine; j - 4 * lane < j_hi; j += 128) {
+      const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
+      cnt += (equal ? kq.x == limit : kq.x >= limit) + (equal ? kq.y == limit : kq.y >= limit) + (equal ? kq.z == limit : kq.z >= limit) +
+             (equal ? kq.w == limit : kq.w >= limit);
     }
+    cnt = (int)__reduce_add_sync(0xffffffffu, (uint32_t)cnt);
+    if (lane == 0) s_cnt[rr][which][w] = cnt;
     meet();
-    int tot = 0;
-#pragma unroll
-    for (int q = 0; q < kPer; ++q) { const int idx = lane * kPer + q; ent[q] = idx < kEntries ? s_cnt[rr][which][idx] : 0; tot += ent[q]; }
-    int incl = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += x;
-    }
-    excl = incl - tot;
   };
-  auto before = [&](int k, int cnt) -> int {
-    if (W == 1) { const int x = run; run += cnt; return x; }
-    const int idx = k * W + w;
-    int x = excl;
-#pragma unroll
-    for (int q = 0; q + 1 < kPer; ++q) if (q < idx % kPer) x += ent[q];
-    return __shfl_sync(0xffffffffu, x, idx / kPer);
+  auto before = [&](int which) -> int {                  // columns of the warps before this one
+    int x = 0;
+    if (W > 1) for (int q = 0; q < w; ++q) x += s_cnt[rr][which][q];
+    return x;
   };
   if (need_eq < n_eq) {              // ties at T that are not all kept: the later ones are struck out (rare)
-    publish(1, T, true);
-    for (int k = 0; k * kStep < n; ++k) {
-      uint32_t* at = keys + k * kStep + 4 * t;
-      int cnt = 0, rank = 0;
+    if (W > 1) publish(1, T, true);
+    int rank0 = before(1);
+    for (int j = j_mine; j - 4 * lane < j_hi; j += 128) {
+      uint32_t* at = keys + j;
+      int cnt = 0, rank = rank0;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const uint32_t bal = __ballot_sync(0xffffffffu, at[u] == T);
         cnt += __popc(bal); rank += __popc(bal & lt_mask);
       }
-      rank += before(k, cnt);
+      rank0 += cnt;
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (at[u] == T) { if (rank >= need_eq) at[u] = 0u; ++rank; }
     }
+    counted = W == 1;
   }
-  publish(0, T, false);
-  const int base = sink_f ? 1 : 0;
-  for (int k = 0; k * kStep < n; ++k) {
-    const int j = k * kStep + 4 * t;
+  if (!counted) publish(0, T, false);
+  int run = (sink_f ? 1 : 0) + before(0);
+  for (int j = j_mine; j - 4 * lane < j_hi; j += 128) {
     const uint4 kq = *reinterpret_cast<const uint4*>(keys + j);
     const uint32_t b0 = __ballot_sync(0xffffffffu, kq.x >= T), b1 = __ballot_sync(0xffffffffu, kq.y >= T);
     const uint32_t b2 = __ballot_sync(0xffffffffu, kq.z >= T), b3 = __ballot_sync(0xffffffffu, kq.w >= T);
-    int at = base + before(k, __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3)) +
-             __popc(b0 & lt_mask) + __popc(b1 & lt_mask) + __popc(b2 & lt_mask) + __popc(b3 & lt_mask);
+    int at = run + __popc(b0 & lt_mask) + __popc(b1 & lt_mask) + __popc(b2 & lt_mask) + __popc(b3 & lt_mask);
+    run += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
     if (kq.x >= T) out[at++] = j;
     if (kq.y >= T) out[at++] = j + 1;
     if (kq.z >= T) out[at++] = j + 2;
     if (kq.w >= T) out[at] = j + 3;
   }
-  if (t == 0) {
+  if (w == 0 && lane == 0) {
     if (sink_f) out[0] = 0;
     if (diag_f) out[out1 - out0 - 1] = ri.i;
   }
