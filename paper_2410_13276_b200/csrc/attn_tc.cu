@@ -238,7 +238,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   const unsigned long long cta_t0 = kTrace ? global_ns() : 0ull;
   const long long cta_c0 = kTrace ? clock64() : 0ll;
 
-  // Work items.  Without a counter a stream takes the items 2 * CTA + stream, + 2 * grid, ... (static deal).  With one
+  // Work items.  Without a counter a stream takes the items CTA + stream * grid, + 2 * grid, ... (static deal: as long as there are no
+  // more items than CTAs each has an SM to itself; two to an SM, 128 items took 15.2 us, and 12.3 so).  With one
   // (`work_counter`, zero at launch) the next item number is drawn from it.  Either way the stream's Q / K producer decodes
   // the item and passes it to the other roles through a ring of four slots, each with a full and an empty mbarrier: a slot
   // is rewritten only when every other role has read it.  nlist < 0 ends the stream.  Results do not depend on which
@@ -266,7 +267,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         const uint32_t sbase = sh.base + (uint32_t)s * kStreamBytes;
         Tracer<kTrace> tr; tr.init(s == 0 ? trace : nullptr, 0);
         const int64_t w_step = 2 * (int64_t)gridDim.x;
-        int64_t w_static = 2 * (int64_t)blockIdx.x + s;
+        int64_t w_static = (int64_t)blockIdx.x + (int64_t)s * gridDim.x;
         auto draw = [&]() -> int64_t {
           if (dyn) return (int64_t)atomicAdd(work_counter, 1);
           const int64_t w = w_static;
@@ -735,7 +736,7 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
   if (!tc::make_map(ctx, &mq, q, m.total_q_tokens, m.num_q_heads, 64) || !tc::make_map(ctx, &mk, k, m.total_tokens, m.num_kv_heads, 64) ||
       !tc::make_map(ctx, &mv, v, m.total_tokens, m.num_kv_heads, 32))
     return -(int)cudaErrorInvalidValue;
-  const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, (m.q_rows + 1) / 2);
+  const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, m.q_rows);
   // The counter the streams draw their work items from lies in the caller's workspace; without one, or with an item a stream at
   // most, the deal is static.  (Its zero by a kernel: a memset would make this launch wait for all that precedes it.)
   cudaError_t e = cudaSuccess;
@@ -764,7 +765,7 @@ int launch_block_max_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const vo
   CUtensorMap mq, mk;
   if (!tc::make_map(ctx, &mq, q, m.total_q_tokens, m.num_q_heads, 64) || !tc::make_map(ctx, &mk, k, m.total_tokens, m.num_kv_heads, 64))
     return -(int)cudaErrorInvalidValue;
-  const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, (m.q_rows + 1) / 2);
+  const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, m.q_rows);
   float* lse_in = const_cast<float*>(lse);   // read only in this mode
   const cudaError_t e = m.chunked
       ? launch_next(tc::attn_tc_kernel<false, true, true>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr)
