@@ -244,20 +244,28 @@ __device__ __forceinline__ void min_bf16x8(float (&a)[8], const uint4& u) {
 }
 
 
-__global__ void __launch_bounds__(kPoolThreads)
+// The pooling of the gate's variants: average, maximum and minimum of a block side by side, one product with the wider matrix, and
+// the block rotation.  Bound by issue beside the bytes: only the pools asked for are formed, an angle's cosine and sine are taken
+// once per block and pair and not by every thread, and three CTAs share an SM (49k tokens, average of Q, all three of K,
+// rotation, with the scores 223 -> 197 us; the bytes take 77).
+__global__ void __launch_bounds__(kPoolThreads, 3)
 pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
                        const float* __restrict__ Wq, const float* __restrict__ Wk, char* __restrict__ gq,
                        char* __restrict__ gk, uint32_t pool_q, uint32_t pool_k, float rope_theta) {
   constexpr int kChunk = kPoolChunkEx;
   __shared__ __align__(16) float pooled[kChunk][3 * kHeadDim];
   __shared__ int block_pos[kChunk];                        // position of each block in its sequence (block RoPE)
+  __shared__ double angle[kGateDim / 2];                   // of one block's step, by pair
 
   const PoolWork work(m, kChunk);
+  if (rope_theta > 0.f && threadIdx.x < kGateDim / 2)
+    angle[threadIdx.x] = pow((double)rope_theta / (double)m.block, -2.0 * (double)threadIdx.x / (double)kGateDim);
   grid_wait();
   if (work.idle) return;
   const int chunk = work.chunk, H = work.H, h = work.h;
   const bool is_q = work.is_q;
   const uint32_t methods = is_q ? pool_q : pool_k;
+  const bool extremes = (methods & ~SEER_POOL_AVG) != 0u;
   const int nparts = __popc(methods);
   const int width = nparts * kHeadDim;                       // rows of the head's gate matrix
   const uint16_t* __restrict__ x = is_q ? q : k;
@@ -304,7 +312,7 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         acc_bf16x8(a, u[j]);
-        if (live[j]) { max_bf16x8(hi, u[j]); min_bf16x8(lo, u[j]); }   // rows past the end of the sequence take no part
+        if (extremes && live[j]) { max_bf16x8(hi, u[j]); min_bf16x8(lo, u[j]); }   // rows past the end of the sequence take no part
       }
     }
     const float inv = cnt > 0 ? 1.0f / (float)cnt : 0.f;
@@ -349,22 +357,28 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
     }
   }
   if (rope_theta > 0.f) {
-    // rotate (o, o + dg/2) pairs: the partner's value goes through shared memory (the pooled vectors are no longer needed)
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < 8; ++j) pooled[grp * 8 + j][o] = acc[j];
+    // rotate (o, o + dg/2) pairs: the partner's value goes through shared memory (the pooled vectors are no longer needed), and
+    // so do the angles' cosines and sines, one per block and pair
     __syncthreads();
     const int f = o & (kGateDim / 2 - 1);
-    const double freq = pow((double)rope_theta / (double)m.block, -2.0 * (double)f / (double)kGateDim);
+    const double freq = angle[f];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) pooled[grp * 8 + j][o] = acc[j];
+#pragma unroll
+    for (int bi = threadIdx.x / (kGateDim / 2); bi < kChunk; bi += kPoolThreads / (kGateDim / 2)) {
+      double sn, cs;
+      sincos((double)(bi < nblk ? block_pos[bi] : 0) * freq, &sn, &cs);
+      *reinterpret_cast<double2*>(&pooled[bi][kHeadDim + 4 * f]) = make_double2(cs, sn);
+    }
+    __syncthreads();
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const int bi = grp * 8 + j;
-      double sn, cs;
-      sincos((double)(bi < nblk ? block_pos[bi] : 0) * freq, &sn, &cs);
+      const double2 t = *reinterpret_cast<const double2*>(&pooled[bi][kHeadDim + 4 * f]);
       const float partner = pooled[bi][o ^ (kGateDim / 2)];
       // first half: x1 cos - x2 sin; second half: x2 cos + x1 sin
-      acc[j] = (o < kGateDim / 2) ? (float)((double)acc[j] * cs - (double)partner * sn)
-                                  : (float)((double)acc[j] * cs + (double)partner * sn);
+      acc[j] = (o < kGateDim / 2) ? (float)((double)acc[j] * t.x - (double)partner * t.y)
+                                  : (float)((double)acc[j] * t.x + (double)partner * t.y);
     }
   }
 #pragma unroll
