@@ -37,6 +37,29 @@ __device__ __forceinline__ void store_split3(char* __restrict__ head, int total_
   *reinterpret_cast<uint16_t*>(dst + 2 * plane) = __bfloat16_as_ushort(lo);
 }
 
+// Four consecutive elements, the first a multiple of four.
+__device__ __forceinline__ void store_split3x4(char* __restrict__ head, int total_blocks, int gb, int o, const float4& x) {
+  const float v[4] = {x.x, x.y, x.z, x.w};
+  uint32_t pl[3][2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const __nv_bfloat162 hi = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    const float2 h = __bfloat1622float2(hi);
+    const float a1 = v[2 * i] - h.x, b1 = v[2 * i + 1] - h.y;
+    const __nv_bfloat162 mid = __floats2bfloat162_rn(a1, b1);
+    const float2 g = __bfloat1622float2(mid);
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(a1 - g.x, b1 - g.y);
+    pl[0][i] = *reinterpret_cast<const uint32_t*>(&hi);
+    pl[1][i] = *reinterpret_cast<const uint32_t*>(&mid);
+    pl[2][i] = *reinterpret_cast<const uint32_t*>(&lo);
+  }
+  const GateTile t(gb >> 6, total_blocks);
+  const int plane = t.rows * 256;
+  char* dst = head + t.base + (size_t)((o >> 6) * t.rows * 128 + (gb & 63) * 128 + ((((o >> 3) & 7) ^ (gb & 7)) << 4) + (o & 7) * 2);
+#pragma unroll
+  for (int q = 0; q < 3; ++q) *reinterpret_cast<uint2*>(dst + q * plane) = make_uint2(pl[q][0], pl[q][1]);
+}
+
 __device__ __forceinline__ uint4 ld_stream_16(const void* p) {
   uint4 r;
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -108,7 +131,8 @@ pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* _
   constexpr int kWarps = kPoolThreads / 32;
   constexpr int kSplit = kChunk < kWarps ? kWarps / kChunk : 1;      // warps per block
   constexpr int kMaxSteps = 8;                                       // groups of 16 rows in a block of 128 tokens
-  __shared__ __align__(16) float pooled[kChunk][kHeadDim];
+  __shared__ __align__(16) float pooled[kChunk == 16 ? 1 : kChunk][kHeadDim];
+  __shared__ __align__(16) float by_col[kChunk == 16 ? kHeadDim * 16 + kHeadDim / 2 : 4];   // [column][block], 16 bytes more per eight columns
   __shared__ __align__(16) float part[kSplit > 1 ? kChunk * kMaxSteps * 2 * kHeadDim : kChunk * kHeadDim];
 
   const PoolWork work(m, kChunk);
@@ -165,11 +189,8 @@ pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* _
       const float inv = cnt > 0 ? 1.0f / (float)cnt : 0.f;
 #pragma unroll
       for (int j = 0; j < 8; ++j) a[j] = __fmul_rn(__fadd_rn(a[j], __shfl_xor_sync(0xffffffffu, a[j], 16)), inv);
-      if (half == 0) {
-        float4* dst = reinterpret_cast<float4*>(&pooled[bi][cchunk * 8]);
-        dst[0] = make_float4(a[0], a[1], a[2], a[3]);
-        dst[1] = make_float4(a[4], a[5], a[6], a[7]);
-      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) by_col[(cchunk * 8 + half * 4 + e) * 16 + cchunk * 4 + bi] = half ? a[4 + e] : a[e];
     } else if (lane == 0 && warp % kSplit == 0) pooled[bi][0] = cnt > 0 ? 1.0f / (float)cnt : 0.f;   // (until the sums are combined)
   }
   if (!__syncthreads_or(any ? 1 : 0)) return;                   // every block of the chunk lies before its queries
@@ -191,6 +212,48 @@ pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* _
 #pragma unroll
     for (int idx = threadIdx.x; idx < kChunk * kHeadDim; idx += kPoolThreads, ++e) pooled[idx / kHeadDim][idx % kHeadDim] = v[e];
     __syncthreads();
+  }
+
+  if constexpr (kChunk == 16) {
+    // projection: a thread takes four output columns, four blocks and one half of the matrix's rows, two columns to an instruction.
+    // What bounds it is the 128 bytes a clock that loads return to the registers: a step is 16 bytes of W, 16 of four blocks'
+    // column and 16 products (a column and sixteen blocks to a thread: 68 bytes for as many; 128k tokens, 32 / 8 heads 296 -> 266 us,
+    // 205 of them the bytes; 32k 76 -> 67; blocks of 128 tokens, 64k 123 -> 113; two columns of blocks to an instruction alone 275).
+    const int bg = warp & 3, ch = warp >> 2, o = 4 * lane;
+    float2 acc[4][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+    const float4* __restrict__ Wh = reinterpret_cast<const float4*>(W + (size_t)ch * 64 * kGateDim + o);
+#pragma unroll 2
+    for (int c = 0; c < 64; c += 8) {
+      float4 w[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) w[e] = __ldg(Wh + (size_t)(c + e) * (kGateDim / 4));
+      const float4* col = reinterpret_cast<const float4*>(by_col + (ch * 64 + c) * 16 + (ch * 64 + c) / 2) + bg;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const float4 pv = col[e * 4];
+        const float2 w0 = make_float2(w[e].x, w[e].y), w1 = make_float2(w[e].z, w[e].w);
+        acc[0][0] = __ffma2_rn(make_float2(pv.x, pv.x), w0, acc[0][0]); acc[0][1] = __ffma2_rn(make_float2(pv.x, pv.x), w1, acc[0][1]);
+        acc[1][0] = __ffma2_rn(make_float2(pv.y, pv.y), w0, acc[1][0]); acc[1][1] = __ffma2_rn(make_float2(pv.y, pv.y), w1, acc[1][1]);
+        acc[2][0] = __ffma2_rn(make_float2(pv.z, pv.z), w0, acc[2][0]); acc[2][1] = __ffma2_rn(make_float2(pv.z, pv.z), w1, acc[2][1]);
+        acc[3][0] = __ffma2_rn(make_float2(pv.w, pv.w), w0, acc[3][0]); acc[3][1] = __ffma2_rn(make_float2(pv.w, pv.w), w1, acc[3][1]);
+      }
+    }
+    // the halves are added by the thread that stores: the first half's threads two blocks, the second half's the other two
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if ((j >= 2) != (ch == 1))
+        *reinterpret_cast<float4*>(&part[(bg * 4 + j) * kGateDim + o]) = make_float4(acc[j][0].x, acc[j][0].y, acc[j][1].x, acc[j][1].y);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if ((j >= 2) == (ch == 1) && bg * 4 + j < nblk) {
+        const float4 t = *reinterpret_cast<const float4*>(&part[(bg * 4 + j) * kGateDim + o]);
+        store_split3x4(out, m.total_blocks, g0 + bg * 4 + j, o, make_float4(__fadd_rn(acc[j][0].x, t.x), __fadd_rn(acc[j][0].y, t.y),
+                                                                            __fadd_rn(acc[j][1].x, t.z), __fadd_rn(acc[j][1].y, t.w)));
+      }
+    return;
   }
 
   // projection: a thread takes output column o, one half of the matrix's rows and all blocks of the chunk
