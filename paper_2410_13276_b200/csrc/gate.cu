@@ -308,15 +308,16 @@ __device__ __forceinline__ void min_bf16x8(float (&a)[8], const uint4& u) {
 
 
 // The pooling of the gate's variants: average, maximum and minimum of a block side by side, one product with the wider matrix, and
-// the block rotation.  Bound by issue beside the bytes: only the pools asked for are formed, an angle's cosine and sine are taken
-// once per block and pair and not by every thread, and three CTAs share an SM (49k tokens, average of Q, all three of K,
-// rotation, with the scores 223 -> 197 us; the bytes take 77).
+// the block rotation.  Bound by issue and shared memory beside the bytes: only the pools asked for are formed, an angle's cosine and
+// sine are taken once per block and pair, by the warps that do not project, and three CTAs share an SM (49k tokens, average of Q, all
+// three of K, rotation, with the scores: 223 us, 197 so, 178 with four columns and four blocks to a thread; the bytes take 77).
 __global__ void __launch_bounds__(kPoolThreads, 3)
 pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
                        const float* __restrict__ Wq, const float* __restrict__ Wk, char* __restrict__ gq,
                        char* __restrict__ gk, uint32_t pool_q, uint32_t pool_k, float rope_theta) {
   constexpr int kChunk = kPoolChunkEx;
-  __shared__ __align__(16) float pooled[kChunk][3 * kHeadDim];
+  __shared__ __align__(16) float by_col[3 * kHeadDim * kChunk + 3 * kHeadDim / 2];   // [column][block], 16 bytes more per eight columns
+  __shared__ __align__(16) double2 turn[kChunk][kGateDim / 2];   // cosine and sine of each block's angle, by pair
   __shared__ int block_pos[kChunk];                        // position of each block in its sequence (block RoPE)
   __shared__ double angle[kGateDim / 2];                   // of one block's step, by pair
 
@@ -386,68 +387,66 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
       lo[j] = fminf(lo[j], __shfl_xor_sync(0xffffffffu, lo[j], 16));
       if (cnt == 0) { hi[j] = 0.f; lo[j] = 0.f; }      // a skipped block: zeros, not the identities of max and min
     }
-    if (half == 0) {
-      if (methods & SEER_POOL_AVG) {
-        float4* dst = reinterpret_cast<float4*>(&pooled[bi][off_avg + cchunk * 8]);
-        dst[0] = make_float4(a[0], a[1], a[2], a[3]); dst[1] = make_float4(a[4], a[5], a[6], a[7]);
-      }
-      if (methods & SEER_POOL_MAX) {
-        float4* dst = reinterpret_cast<float4*>(&pooled[bi][off_max + cchunk * 8]);
-        dst[0] = make_float4(hi[0], hi[1], hi[2], hi[3]); dst[1] = make_float4(hi[4], hi[5], hi[6], hi[7]);
-      }
-      if (methods & SEER_POOL_MIN) {
-        float4* dst = reinterpret_cast<float4*>(&pooled[bi][off_min + cchunk * 8]);
-        dst[0] = make_float4(lo[0], lo[1], lo[2], lo[3]); dst[1] = make_float4(lo[4], lo[5], lo[6], lo[7]);
-      }
-    }
+    auto put = [&](int off, const float (&v)[8]) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) by_col[(off + cchunk * 8 + half * 4 + e) * kChunk + (off / 8 + cchunk) * 4 + bi] = half ? v[4 + e] : v[e];
+    };
+    if (methods & SEER_POOL_AVG) put(off_avg, a);
+    if (methods & SEER_POOL_MAX) put(off_max, hi);
+    if (methods & SEER_POOL_MIN) put(off_min, lo);
   }
   if (!__syncthreads_or(any ? 1 : 0)) return;                   // every block of the chunk lies before its queries
 
-  // projection: thread -> output column o, 8 of the 16 blocks
-  const int o = threadIdx.x & (kGateDim - 1);
-  const int grp = threadIdx.x >> 7;  // 0 or 1
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  // projection, by four warps: a thread takes four output columns and four blocks, as in pool_project_kernel; the other four warps take
+  // the cosines and sines meanwhile
+  const int o = 4 * lane, bg = warp & 3;
+  float2 acc[4][2];
+  if (warp < 4) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
+    const float4* __restrict__ Wh = reinterpret_cast<const float4*>(W + o);
 #pragma unroll 2
-  for (int c = 0; c < width; c += 8) {
-    float w[8];
+    for (int c = 0; c < width; c += 8) {
+      float4 w[8];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) w[e] = __ldg(W + (size_t)(c + e) * kGateDim + o);
+      for (int e = 0; e < 8; ++e) w[e] = __ldg(Wh + (size_t)(c + e) * (kGateDim / 4));
+      const float4* col = reinterpret_cast<const float4*>(by_col + c * kChunk + c / 2) + bg;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const float4 p0 = *reinterpret_cast<const float4*>(&pooled[grp * 8 + j][c]), p1 = *reinterpret_cast<const float4*>(&pooled[grp * 8 + j][c + 4]);
-      acc[j] = fmaf(p0.x, w[0], acc[j]); acc[j] = fmaf(p0.y, w[1], acc[j]); acc[j] = fmaf(p0.z, w[2], acc[j]); acc[j] = fmaf(p0.w, w[3], acc[j]);
-      acc[j] = fmaf(p1.x, w[4], acc[j]); acc[j] = fmaf(p1.y, w[5], acc[j]); acc[j] = fmaf(p1.z, w[6], acc[j]); acc[j] = fmaf(p1.w, w[7], acc[j]);
+      for (int e = 0; e < 8; ++e) {
+        const float4 pv = col[e * (kChunk / 4)];
+        const float2 w0 = make_float2(w[e].x, w[e].y), w1 = make_float2(w[e].z, w[e].w);
+        acc[0][0] = __ffma2_rn(make_float2(pv.x, pv.x), w0, acc[0][0]); acc[0][1] = __ffma2_rn(make_float2(pv.x, pv.x), w1, acc[0][1]);
+        acc[1][0] = __ffma2_rn(make_float2(pv.y, pv.y), w0, acc[1][0]); acc[1][1] = __ffma2_rn(make_float2(pv.y, pv.y), w1, acc[1][1]);
+        acc[2][0] = __ffma2_rn(make_float2(pv.z, pv.z), w0, acc[2][0]); acc[2][1] = __ffma2_rn(make_float2(pv.z, pv.z), w1, acc[2][1]);
+        acc[3][0] = __ffma2_rn(make_float2(pv.w, pv.w), w0, acc[3][0]); acc[3][1] = __ffma2_rn(make_float2(pv.w, pv.w), w1, acc[3][1]);
+      }
     }
-  }
-  if (rope_theta > 0.f) {
-    // rotate (o, o + dg/2) pairs: the partner's value goes through shared memory (the pooled vectors are no longer needed), and
-    // so do the angles' cosines and sines, one per block and pair
-    __syncthreads();
-    const int f = o & (kGateDim / 2 - 1);
+  } else if (rope_theta > 0.f) {
+    const int f = threadIdx.x & (kGateDim / 2 - 1);
     const double freq = angle[f];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) pooled[grp * 8 + j][o] = acc[j];
-#pragma unroll
-    for (int bi = threadIdx.x / (kGateDim / 2); bi < kChunk; bi += kPoolThreads / (kGateDim / 2)) {
+    for (int bi = (threadIdx.x - 128) / (kGateDim / 2); bi < nblk; bi += 128 / (kGateDim / 2)) {
       double sn, cs;
-      sincos((double)(bi < nblk ? block_pos[bi] : 0) * freq, &sn, &cs);
-      *reinterpret_cast<double2*>(&pooled[bi][kHeadDim + 4 * f]) = make_double2(cs, sn);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int bi = grp * 8 + j;
-      const double2 t = *reinterpret_cast<const double2*>(&pooled[bi][kHeadDim + 4 * f]);
-      const float partner = pooled[bi][o ^ (kGateDim / 2)];
-      // first half: x1 cos - x2 sin; second half: x2 cos + x1 sin
-      acc[j] = (o < kGateDim / 2) ? (float)((double)acc[j] * t.x - (double)partner * t.y)
-                                  : (float)((double)acc[j] * t.x + (double)partner * t.y);
+      sincos((double)block_pos[bi] * freq, &sn, &cs);
+      turn[bi][f] = make_double2(cs, sn);
     }
   }
+  if (rope_theta > 0.f) __syncthreads();
+  if (warp >= 4) return;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int bi = grp * 8 + j;
-    if (bi < nblk) store_split3(out, m.total_blocks, g0 + bi, o, acc[j]);
+  for (int j = 0; j < 4; ++j) {
+    const int bi = bg * 4 + j;
+    float v[4] = {acc[j][0].x, acc[j][0].y, acc[j][1].x, acc[j][1].y};
+    if (rope_theta > 0.f) {
+      // rotate (o, o + dg/2) pairs: the partner's value is that of lane ^ 16
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float partner = __shfl_xor_sync(0xffffffffu, v[u], 16);
+        const double2 t = turn[bi][(o + u) & (kGateDim / 2 - 1)];
+        // first half: x1 cos - x2 sin; second half: x2 cos + x1 sin
+        v[u] = lane < 16 ? (float)((double)v[u] * t.x - (double)partner * t.y) : (float)((double)v[u] * t.x + (double)partner * t.y);
+      }
+    }
+    if (bi < nblk) store_split3x4(out, m.total_blocks, g0 + bi, o, make_float4(v[0], v[1], v[2], v[3]));
   }
 }
 
