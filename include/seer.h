@@ -15,8 +15,10 @@
  *    work has finished, and only if all 8 are still in flight does it wait on the host for the oldest one.
  *    The library allocates device memory only in seer_create; per-call scratch comes from the caller's
  *    workspace `ws` (>= seer_workspace_bytes(shape), 256-byte aligned).
+ *  - A call's kernels may become resident while the kernel before them in the stream ends; they wait for its completion
+ *    before they touch memory.  Work that the caller enqueues before or behind a call keeps its order.
  *  - The tcgen05 attention kernel takes all 512 tensor-memory columns and 227 KB of shared memory of an SM, the
- *    gate's score kernel 256 columns and 226 KB: one CTA of either is resident per SM (the two cannot share an SM
+ *    gate's score kernel 512 columns and 210 KB: one CTA of either is resident per SM (the two cannot share an SM
  *    either), so a tensor-memory allocation never waits on another CTA of this library.  A kernel of ANOTHER
  *    library that holds tensor memory on the same device at the same time (another stream or process) can make
  *    that allocation wait; it is the one wait in these kernels the library cannot bound.
@@ -160,8 +162,8 @@ seer_status seer_block_mask(seer_ctx* ctx, const seer_shape* shape, const float*
  *    A row with an empty list yields o = 0 and lse = -inf.
  *    ws (optional): with a workspace of at least 256 bytes (256-byte aligned, as for the other calls) the first word
  *    becomes the counter from which the tcgen05 kernel's persistent CTAs draw their (head, query block) work items,
- *    so that a CTA that finishes early takes more of them; without one (NULL) the items are dealt statically.  The
- *    results are identical bit for bit.  Calls that may run at the same time must not share the workspace. */
+ *    so that a CTA that finishes early takes more of them; without one (NULL), and where there are no more than two items
+ *    a CTA, the items are dealt statically.  The results are identical bit for bit.  Calls that may run at the same time must not share the workspace. */
 seer_status seer_sparse_attn(seer_ctx* ctx, const seer_shape* shape, const void* q, const void* k, const void* v,
                              const int32_t* row_ptr, const int32_t* col_idx, void* o, float* lse, void* ws,
                              size_t ws_bytes, void* stream);
