@@ -397,10 +397,20 @@ int launch_gate_stats(const SeqMeta& m, const uint16_t* gq, const uint16_t* gk, 
 // Scores of a band; with `stats` launch_gate_stats has run, without the rows' statistics are formed by the same launch.
 int launch_gate_scores(const SeqMeta& m, const ScoreBand& band, const uint16_t* gq, const uint16_t* gk, float* scores,
                        float2* stats, int* status, int num_sms, cudaStream_t stream) {
-  // parts of 4 to 16 tiles, so that the band's tiles make about one wave of CTAs (a 4096-block head: 16 tiles a CTA 30 us, 8: 17)
-  const int64_t tiles = (int64_t)((band.blk_hi - band.blk_lo + gs::kRows - 1) / gs::kRows) * band.heads * (m.max_nb / gs::kCols / 2 + 1);
+  // Parts of 4, 8 or 16 tiles: what lasts shortest, in units of a tile.  A CTA's start is about three of them; a launch lasts as long as
+  // a full part or its share of all tiles and starts.  (128 rows of 32 heads against 2048 blocks: 8 tiles to a part instead of
+  // 4: gate and mask of the chunk 170 -> 162 us; three 4096-block heads: 16, where 8 take 7 % longer.)
   int part = 4;
-  while (part < 16 && tiles / part > num_sms) part *= 2;
+  if (stats != nullptr) {
+    const dim3 all = score_grid(m, band, 1);
+    const int64_t tiles = (int64_t)all.x * all.y;
+    int64_t best = INT64_MAX;
+    for (int p = 4; p <= 16; p *= 2) {
+      const dim3 g = score_grid(m, band, p);
+      const int64_t share = (tiles + 3 * (int64_t)g.x * g.y) / num_sms, cost = share > p + 3 ? share : p + 3;
+      if (cost < best) { best = cost; part = p; }
+    }
+  }
   const dim3 grid = score_grid(m, band, stats != nullptr ? part : 0);
   if (grid.x == 0) return 0;
   const cudaError_t e = stats != nullptr
