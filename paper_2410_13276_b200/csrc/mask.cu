@@ -457,8 +457,10 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
       }
       meet();
       if (W > 1) { found = s_pick[rr][0]; remaining = (int)s_pick[rr][1]; cls = (int)s_pick[rr][2]; }
+      // (The class ends at the largest key.  Without that limit lo + span would wrap where scores of both signs meet scores from 2^127
+      // on, or infinities: key 0 would lie inside the class, and the test for keys above it would take nearly all of them.)
+      span = min((1u << shift) - 1u, span - (found << shift));
       lo += found << shift;
-      span = (1u << shift) - 1u;
       if (shift == 0) { T = lo; need_eq = remaining; n_eq = cls; break; }
       // A class of at most 32 keys (the usual case after one pass) is finished by rank: its keys are gathered, each lane of one
       // warp ranks one of them against the others.  The columns above the class are kept: their number is taken on the way.
