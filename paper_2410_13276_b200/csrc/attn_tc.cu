@@ -166,7 +166,13 @@ __device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
   return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
 }
 
-__device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8]) {   // 32 bytes
+// 32 bytes, at once where the address allows it (the host asks for 16)
+__device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bool aligned) {
+  if (!aligned) {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    return;
+  }
   asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]),
                "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
 }
@@ -192,7 +198,8 @@ __device__ __forceinline__ int slot_check(const Slot& it, int p, int raw) {
 // Without V and O a stream has five K units and four S buffers: with two of each it waited for copies and MMAs in turn (16k
 // tokens, 32 heads, all causal blocks: 1277 -> 1060 us, 520 clocks a tile; 440 are its 32 KB from L2, 384 its MMAs).  Tiles of four
 // blocks on N = 256 MMAs, 320 clocks per two blocks, gave nothing more.
-template <bool kTrace, bool kChunk, bool kBlockMax = false>
+// kO32: o begins on 32 bytes.  (A test of the address in the kernel instead: 32k tokens 1392 -> 1404 us.)
+template <bool kTrace, bool kChunk, bool kBlockMax = false, bool kO32 = true>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, SeqMeta m,
@@ -464,6 +471,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     const uint32_t ml = sh.base + kOffMl + (uint32_t)s * kMlBytes;
     const uint32_t o_addr = tmem + lane_addr + col_o(s);
     const int64_t lse_stride = kChunk ? m.total_q_tokens : m.total_tokens;
+    const bool o32 = kTrace ? (reinterpret_cast<uintptr_t>(o) & 31) == 0 : kO32;
     Tracer<kTrace> tr; tr.init(r == 0 ? trace : nullptr, 4 + s);
     uint32_t cnt = 0, nitem = 0;                            // tiles and items with tiles this stream has processed
     for (uint32_t n = 0;; ++n) {
@@ -636,8 +644,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             if (store) {
               const uint32_t o0[8] = {out[0], out[1], out[2], out[3], out[4], out[5], out[6], out[7]};
               const uint32_t o1[8] = {out[8], out[9], out[10], out[11], out[12], out[13], out[14], out[15]};
-              st_global_32(orow + half * 64 + i * 32, o0);
-              st_global_32(orow + half * 64 + i * 32 + 16, o1);
+              st_global_32(orow + half * 64 + i * 32, o0, o32);
+              st_global_32(orow + half * 64 + i * 32 + 16, o1, o32);
             }
           }
           fence_async_smem();                               // before the next Q copy into this buffer
@@ -656,8 +664,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             if (store) {
               const uint32_t o0[8] = {out[0], out[1], out[2], out[3], out[4], out[5], out[6], out[7]};
               const uint32_t o1[8] = {out[8], out[9], out[10], out[11], out[12], out[13], out[14], out[15]};
-              st_global_32(orow + ch * 32, o0);
-              st_global_32(orow + ch * 32 + 16, o1);
+              st_global_32(orow + ch * 32, o0, o32);
+              st_global_32(orow + ch * 32 + 16, o1, o32);
             }
           }
         }
@@ -682,6 +690,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
   }
 }
+
+using Kernel = void(CUtensorMap, CUtensorMap, CUtensorMap, SeqMeta, const int32_t*, const int32_t*, uint16_t*, float*, int*, unsigned long long*, float*, int*);
 
 __global__ void zero_kernel(int* __restrict__ word) {
   grid_wait();
@@ -714,16 +724,11 @@ seer_status init_attn_tc(seer_ctx* ctx) {
       qres != cudaDriverEntryPointSuccess)
     return SEER_ERR_CUDA;
   ctx->tmap_encode = fn;
-  cudaError_t e = cudaFuncSetAttribute(tc::attn_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc::attn_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc::attn_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc::attn_tc_kernel<false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(tc::attn_tc_kernel<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes);
-  return e == cudaSuccess ? SEER_OK : SEER_ERR_CUDA;
+  for (tc::Kernel* k : {tc::attn_tc_kernel<false, false>, tc::attn_tc_kernel<false, true>, tc::attn_tc_kernel<true, false>,
+                        tc::attn_tc_kernel<false, false, false, false>, tc::attn_tc_kernel<false, true, false, false>,
+                        tc::attn_tc_kernel<false, false, true>, tc::attn_tc_kernel<false, true, true>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes) != cudaSuccess) return SEER_ERR_CUDA;
+  return SEER_OK;
 }
 
 int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const void* v,
@@ -748,12 +753,11 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
     launched = 1;
   }
   unsigned long long* tb = (unsigned long long*)ctx->trace;
-  if (m.chunked)               // chunked prefill (never instrumented)
-    e = launch_next(tc::attn_tc_kernel<false, true>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
-  else if (tb != nullptr)      // the instrumented instantiation
-    e = launch_next(tc::attn_tc_kernel<true, false>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
-  else
-    e = launch_next(tc::attn_tc_kernel<false, false>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
+  const bool o32 = ((uintptr_t)o & 31) == 0;
+  tc::Kernel* kernel = m.chunked ? (o32 ? tc::attn_tc_kernel<false, true> : tc::attn_tc_kernel<false, true, false, false>)   // (never instrumented)
+                     : tb != nullptr ? tc::attn_tc_kernel<true, false>
+                     : o32 ? tc::attn_tc_kernel<false, false> : tc::attn_tc_kernel<false, false, false, false>;
+  e = launch_next(kernel, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter);
   return e == cudaSuccess ? launched + 1 : -(int)e;
 }
 

@@ -1,0 +1,50 @@
+"""Tensors that begin where their type allows but not on the width of the kernels' widest accesses, as slices of larger buffers
+do: bit for bit what the calls return for tensors on their own."""
+import numpy as np
+import pytest
+
+from oracle import seer_oracle as O
+from paper_2410_13276_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def shifted(t, elements):
+    """A copy of t that begins `elements` elements behind a 256-byte boundary."""
+    import torch
+    room = torch.empty(t.numel() + elements + 256, dtype=t.dtype, device=t.device)
+    assert room.data_ptr() % 256 == 0
+    out = room[elements:elements + t.numel()].view(t.shape)
+    out.copy_(t)
+    return out
+
+
+@pytest.mark.parametrize("chunk", [False, True])
+def test_attention_output_on_16_bytes(chunk):
+    import torch
+    from paper_2410_13276_b200 import binding as B
+    from paper_2410_13276_b200.prefill import Prefill
+    lens, starts = [64 * 9 - 5, 70, 64 * 5], [128, 64, 0]
+    w = W.make_small(seed=210, seqlens=lens, hq=4, hkv=2)
+    q, cu_q = w.q, None
+    if chunk:
+        part = [w.q[w.cu_seqlens[b] + s:w.cu_seqlens[b + 1]] for b, s in enumerate(starts)]
+        q, cu_q = np.concatenate(part), np.concatenate([[0], np.cumsum([len(x) for x in part])]).astype(np.int32)
+    p = Prefill(w.cu_seqlens, 4, 2, cu_seqlens_q=cu_q)
+    p.set_inputs(q, w.k, w.v, w.wq, w.wk)
+    r = np.random.default_rng(3)
+    rows = [sorted(r.choice(i + 1, min(n, i + 1), replace=False).tolist()) for x in lens for h in range(4) for i, n in
+            enumerate(r.integers(0, 6, (x + 63) // 64))]          # no, one, odd and even numbers of blocks
+    p.set_lists(np.concatenate([[0], np.cumsum([len(x) for x in rows])]), np.array([j for x in rows for j in x]))
+    p.o.fill_(-1.0)
+    p.attn()
+    want = p.o
+    p.o = shifted(torch.full_like(want, -1.0), 8)                  # 16 bytes on
+    assert p.o.data_ptr() % 32 == 16
+    p.attn()
+    assert p.status() == 0 and torch.equal(p.o, want)
+    trace = torch.zeros(7 * 8192, dtype=torch.int64, device="cuda")   # the instrumented kernel
+    B.seer_set_trace_buffer(p.ctx, trace)
+    p.o.fill_(-1.0)
+    p.attn()
+    assert p.status() == 0 and torch.equal(p.o, want)
