@@ -60,6 +60,14 @@ __device__ __forceinline__ void store_split3x4(char* __restrict__ head, int tota
   for (int q = 0; q < 3; ++q) *reinterpret_cast<uint2*>(dst + q * plane) = make_uint2(pl[q][0], pl[q][1]);
 }
 
+// Four consecutive columns of a gate matrix: one load where the matrices begin on 16 bytes, otherwise four.
+template <bool kVecW>
+__device__ __forceinline__ float4 ld_w4(const float* __restrict__ p) {
+  if (kVecW) return __ldg(reinterpret_cast<const float4*>(p));
+  return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+static bool vec_w(const float* Wq, const float* Wk) { return (((uintptr_t)Wq | (uintptr_t)Wk) & 15) == 0; }   // (a head's matrix is 64 KB)
+
 __device__ __forceinline__ uint4 ld_stream_16(const void* p) {
   uint4 r;
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -123,7 +131,7 @@ struct PoolWork {
 // matrix, read once per CTA from L2, is then a fifth of its traffic) and 2 blocks otherwise, with four warps per block.
 // The sums are formed in the same order for every chunk size (16 rows at a time; the two halves of the matrix's rows apart),
 // so the result does not depend on it.
-template <int kChunk>
+template <int kChunk, bool kVecW = true>
 __global__ void __launch_bounds__(kPoolThreads, kChunk == 16 ? 3 : 1)
 pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
                     const float* __restrict__ Wq, const float* __restrict__ Wk, char* __restrict__ gq,
@@ -223,12 +231,12 @@ pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* _
     float2 acc[4][2];
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
-    const float4* __restrict__ Wh = reinterpret_cast<const float4*>(W + (size_t)ch * 64 * kGateDim + o);
+    const float* __restrict__ Wh = W + (size_t)ch * 64 * kGateDim + o;
 #pragma unroll 2
     for (int c = 0; c < 64; c += 8) {
       float4 w[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) w[e] = __ldg(Wh + (size_t)(c + e) * (kGateDim / 4));
+      for (int e = 0; e < 8; ++e) w[e] = ld_w4<kVecW>(Wh + (size_t)(c + e) * kGateDim);
       const float4* col = reinterpret_cast<const float4*>(by_col + (ch * 64 + c) * 16 + (ch * 64 + c) / 2) + bg;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
@@ -311,6 +319,7 @@ __device__ __forceinline__ void min_bf16x8(float (&a)[8], const uint4& u) {
 // the block rotation.  Bound by issue and shared memory beside the bytes: only the pools asked for are formed, an angle's cosine and
 // sine are taken once per block and pair, by the warps that do not project, and three CTAs share an SM (49k tokens, average of Q, all
 // three of K, rotation, with the scores: 223 us, 197 so, 178 with four columns and four blocks to a thread; the bytes take 77).
+template <bool kVecW>
 __global__ void __launch_bounds__(kPoolThreads, 3)
 pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
                        const float* __restrict__ Wq, const float* __restrict__ Wk, char* __restrict__ gq,
@@ -404,12 +413,12 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
   if (warp < 4) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = make_float2(0.f, 0.f);
-    const float4* __restrict__ Wh = reinterpret_cast<const float4*>(W + o);
+    const float* __restrict__ Wh = W + o;
 #pragma unroll 2
     for (int c = 0; c < width; c += 8) {
       float4 w[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) w[e] = __ldg(Wh + (size_t)(c + e) * (kGateDim / 4));
+      for (int e = 0; e < 8; ++e) w[e] = ld_w4<kVecW>(Wh + (size_t)(c + e) * kGateDim);
       const float4* col = reinterpret_cast<const float4*>(by_col + c * kChunk + c / 2) + bg;
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
@@ -488,7 +497,7 @@ int launch_gate(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, c
   const GateWs w(m, ws, ws_bytes);
   const unsigned big = PoolWork::grid(m, 16);
   const cudaError_t e0 = big > kBigChunkFrom
-      ? launch_next(pool_project_kernel<16>, big, kPoolThreads, 0, stream, m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk)
+      ? launch_next(vec_w(Wq, Wk) ? pool_project_kernel<16> : pool_project_kernel<16, false>, big, kPoolThreads, 0, stream, m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk)
       : launch_next(pool_project_kernel<2>, PoolWork::grid(m, 2), kPoolThreads, 0, stream, m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk, w.gq, w.gk);
   if (e0 != cudaSuccess) return -(int)e0;
   if (scores == nullptr) return 1;                     // projection only: the scores follow band by band
@@ -502,7 +511,7 @@ int launch_gate_ex(seer_ctx* ctx, const SeqMeta& m, const seer_gate_options& opt
   if (opt.pool_q == SEER_POOL_AVG && opt.pool_k == SEER_POOL_AVG && opt.rope_theta == 0.f) return launch_gate(ctx, m, q, k, Wq, Wk, scores, ws, ws_bytes, stream);
   const GateWs w(m, ws, ws_bytes);
   const unsigned grid1 = PoolWork::grid(m, kPoolChunkEx);
-  const cudaError_t e0 = launch_next(pool_project_ex_kernel, grid1, kPoolThreads, 0, stream, m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk,
+  const cudaError_t e0 = launch_next(vec_w(Wq, Wk) ? pool_project_ex_kernel<true> : pool_project_ex_kernel<false>, grid1, kPoolThreads, 0, stream, m, (const uint16_t*)q, (const uint16_t*)k, Wq, Wk,
                                      w.gq, w.gk, opt.pool_q, opt.pool_k, opt.rope_theta);
   if (e0 != cudaSuccess) return -(int)e0;
   if (scores == nullptr) return 1;

@@ -48,3 +48,31 @@ def test_attention_output_on_16_bytes(chunk):
     p.o.fill_(-1.0)
     p.attn()
     assert p.status() == 0 and torch.equal(p.o, want)
+
+
+# 12 + 4 heads: pooled two blocks a CTA, and sixteen
+@pytest.mark.parametrize("lens", [[300, 65], [300 * 64 - 5, 310 * 64 + 1]])
+@pytest.mark.parametrize("elements", [1, 2])
+def test_gate_matrices_on_4_and_8_bytes(lens, elements):
+    import torch
+    from paper_2410_13276_b200 import binding as B
+    from paper_2410_13276_b200.prefill import Prefill
+    w = W.make_small(seed=211, seqlens=lens, hq=12, hkv=4)
+    p = Prefill(w.cu_seqlens, 12, 4, want_lse=False)
+    p.set_inputs(w.q, w.k, w.v, w.wq, w.wk)
+    wq3, wk3 = (torch.cat([x, 0.1 * x, -0.1 * x], 1).contiguous() for x in (p.wq, p.wk))
+    options = B.seer_gate_options(B.SEER_POOL_AVG | B.SEER_POOL_MAX | B.SEER_POOL_MIN, B.SEER_POOL_AVG | B.SEER_POOL_MAX | B.SEER_POOL_MIN, 10000.0)
+    got = {}
+    for name, move in (("aligned", lambda t, k: t), ("both", lambda t, k: shifted(t, elements)), ("Wk", lambda t, k: shifted(t, elements * k))):
+        p.scores.fill_(-1.0)                                       # (above the diagonal nothing is written)
+        B.seer_gate_scores(p.ctx, p.shape, p.q, p.k, move(p.wq, 0), move(p.wk, 1), p.scores, p.ws)
+        plain = p.scores.clone()
+        p.gate_ex(options, move(wq3, 0), move(wk3, 1))
+        got[name] = (plain, p.scores.clone())
+        if lens[0] == 300:
+            p.scores.fill_(-1.0)
+            B.seer_gate_scores_static(p.shape, p.q, p.k, move(p.wq, 0), move(p.wk, 1), p.scores)
+            got[name] += (p.scores.clone(),)
+    assert p.status() == 0
+    for name in ("both", "Wk"):
+        assert all(torch.equal(a, b) for a, b in zip(got[name], got["aligned"]))
