@@ -344,9 +344,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           for (int t = 0; t < it.ntiles() && ok; ++t, ++cnt) {
             const int ra = slot_block(it, col_idx, 2 * t + 2), rb = slot_block(it, col_idx, 2 * t + 3);   // next pair
             const int ta = it.s0 + (ja < 0 ? 0 : ja) * kBlock;
-            // the last tile of an odd list: the second half multiplies zeros, by the values of the first block (whatever
-            // else lies in the buffer might not be finite); a list of one block has no second half to spoil
-            const int tb = jb == -1 ? ta : it.s0 + (jb < 0 ? 0 : jb) * kBlock;
+            // the last tile of an odd list: the second half multiplies zeros by zeros, which a copy from past the last token brings
+            // (values of another block, or what else lies in the buffer, might not be finite); a list of one block has no second
+            // half to spoil
+            const int tb = jb == -1 ? m.total_tokens : it.s0 + (jb < 0 ? 0 : jb) * kBlock;
             const bool two = it.nlist > 1;
             tr.sample(cnt); tr.ev(1);
             // test hook: one V copy that is never issued, so that the issuer's wait for it runs out

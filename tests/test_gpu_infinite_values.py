@@ -1,0 +1,47 @@
+"""Values and gate logits past the range of their type stay where they belong: an infinite value reaches the columns of the rows
+that attend to it and no others, and a logit of -inf is a probability of zero."""
+import math
+
+import numpy as np
+import pytest
+
+from oracle import seer_oracle as O
+from paper_2410_13276_b200 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("chunk", [False, True])
+@pytest.mark.parametrize("lengths", [(1, 2, 3), (3, 4, 5), (5, 6, 7, 9)])
+def test_infinite_values(lengths, chunk):
+    from paper_2410_13276_b200 import binding as B
+    from paper_2410_13276_b200.prefill import Prefill
+    nb, hq, first = 20, 4, 10
+    w = W.make_small(seed=220, seqlens=[nb * 64 - 7], hq=hq, hkv=2)
+    v = w.v.copy()
+    inf = np.uint16(0x7f80)
+    v[3 * 64 + 5, 0, 7] = inf                            # blocks 3 and 8 of either KV head
+    v[3 * 64 + 63, 1, 100] = inf | np.uint16(0x8000)
+    v[8 * 64, 0, 64] = inf
+    r = np.random.default_rng(sum(lengths))
+    rows = []
+    for h in range(hq):
+        for i in range(nb):
+            n = min(lengths[(h + i) % len(lengths)], i) if i >= first else 0
+            row = sorted(r.choice(i, n, replace=False).tolist()) if n else []      # (no diagonal: every row sees every listed key)
+            if n and i % 2:                                  # an infinite value in the last block of the list
+                row = sorted(r.choice(8, n - 1, replace=False).tolist() + [8]) if n <= 9 else row
+            rows.append(row)
+    rp, col = np.concatenate([[0], np.cumsum([len(x) for x in rows])]).astype(np.int32), np.array([j for x in rows for j in x], np.int32)
+    p = Prefill(w.cu_seqlens, hq, 2, cu_seqlens_q=np.array([0, (nb - first) * 64 - 7], np.int32) if chunk else None)
+    p.set_inputs(w.q[first * 64:] if chunk else w.q, w.k, v, w.wq, w.wk)
+    p.set_lists(rp, col)
+    p.attn()
+    assert p.status() == 0
+    want, _ = O.sparse_attention(w.q, w.k, v, w.cu_seqlens, rp, col, hq, 2, 64, 1 / math.sqrt(128))
+    got = p.o_host().astype(np.float64)
+    got, want = got if chunk else got[first * 64:], want[first * 64:]
+    assert np.isinf(want).any() and not np.isnan(want).any() and np.isfinite(want).mean() > 0.9
+    off = ~np.isfinite(want)
+    assert np.array_equal(got[off], want[off]) and np.isfinite(got[~off]).all()
+    assert np.all(np.abs(got[~off] - want[~off]) <= 2e-2 + 1e-2 * np.abs(want[~off]))   # the attention's tolerance
