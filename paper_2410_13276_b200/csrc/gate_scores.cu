@@ -297,12 +297,13 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
           float mx[4] = {x[0], x[1], x[2], x[3]};
 #pragma unroll
           for (int c = 4; c < 32; ++c) mx[c & 3] = fmaxf(mx[c & 3], x[c]);
-          const float nm = fmaxf(seg_m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])));   // finite: there is a causal column
+          const float nm = fmaxf(seg_m, fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])));
+          const float ref = fmaxf(nm, -CUDART_MAX_NORMAL_F);   // (nm = -inf: nothing but logits below the range of fp32 so far)
           float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-          for (int c = 0; c < 32; ++c) sum[c & 3] = __fadd_rn(sum[c & 3], ex2f(__fsub_rn(x[c], nm)));   // 2^(-inf) = 0 for the masked columns
+          for (int c = 0; c < 32; ++c) sum[c & 3] = __fadd_rn(sum[c & 3], ex2f(__fsub_rn(x[c], ref)));   // 2^(-inf) = 0 for the masked columns
           const float s4 = __fadd_rn(__fadd_rn(sum[0], sum[1]), __fadd_rn(sum[2], sum[3]));
-          seg_l = __fadd_rn(__fmul_rn(seg_l, ex2f(__fsub_rn(seg_m, nm))), s4);              // 2^(-inf) = 0 on the first contribution
+          seg_l = __fadd_rn(__fmul_rn(seg_l, ex2f(__fsub_rn(seg_m, ref))), s4);              // 2^(-inf) = 0 on the first contribution
           seg_m = nm;
         }
       } else {

@@ -45,3 +45,38 @@ def test_infinite_values(lengths, chunk):
     off = ~np.isfinite(want)
     assert np.array_equal(got[off], want[off]) and np.isfinite(got[~off]).all()
     assert np.all(np.abs(got[~off] - want[~off]) <= 2e-2 + 1e-2 * np.abs(want[~off]))   # the attention's tolerance
+
+
+# blocks whose logits lie below the range of fp32, alone among a row's columns of a 32-column group, at the edges of groups, tiles
+# and 256-column segments; by one launch and by two
+@pytest.mark.parametrize("nb,two", [(300, False), (640, True)])
+def test_logits_below_the_range(nb, two):
+    from paper_2410_13276_b200 import binding as B
+    from paper_2410_13276_b200.prefill import Prefill
+    low = [31, 32, 64, 95, 96, 128, 255, 256, 257, 288, nb - 1]
+    q, k = np.zeros((nb * 64, 1, 128), np.float32), np.zeros((nb * 64, 1, 128), np.float32)
+    q[:, 0, 0] = 2.0 ** 64                                   # (powers of two: pooling, projection and products are exact)
+    q[:, 0, 1] = 1.0
+    k[:, 0, 1] = np.repeat(np.arange(nb) % 7, 64)
+    for j in low:
+        k[j * 64:(j + 1) * 64, 0, 0] = -2.0 ** 100           # a logit of -2^164 / sqrt(128)
+    eye = np.eye(128, dtype=np.float32)[None]
+    bits = [W.f32_to_bf16_bits(x) for x in (q, k)]
+    p = Prefill(np.array([0, nb * 64], np.int32), 1, 1, want_lse=False)
+    p.set_inputs(bits[0], bits[1], bits[1], eye, eye)
+    p.scores.zero_()
+    n0 = B.seer_launch_count(p.ctx)
+    p.gate()
+    assert p.status() == 0 and B.seer_launch_count(p.ctx) - n0 == (3 if two else 2)
+    got = O.unflatten_scores(p.scores_host(), p.cu, 64, 1)[0][0].astype(np.float64)
+    want = O.gate_scores(bits[0], bits[1], eye, eye, p.cu, 64)[0][0]
+    tri = np.tril(np.ones((nb, nb), bool))
+    assert all((want[j:, j] == 0).all() for j in low)
+    assert np.all(np.abs(got - want)[tri] <= 1e-3 * want[tri])      # the gate's tolerance
+    # lists from those scores by one call
+    params = B.make_mask_params(B.SEER_TOPK_RATIO, keep_num=1, keep_den=3, flags=3)
+    p.mask(params)
+    lists = [x.copy() for x in p.lists_host()]
+    p.row_ptr.fill_(-1)
+    p.gate_mask(params, band_bytes=1 << 20)
+    assert p.status() == 0 and all(np.array_equal(a, b) for a, b in zip(lists, p.lists_host()))
