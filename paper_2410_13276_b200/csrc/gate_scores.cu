@@ -256,6 +256,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
     float2* ml = reinterpret_cast<float2*>(smem + kOffStage);   // [segment parity][group][half][row]
     int nseg = 0;
     uint32_t uses = 0;                                    // tiles this group has worked on
+    const uint32_t base4 = (uint32_t)(reinterpret_cast<uintptr_t>(scores) >> 2);   // scores may begin on any four bytes
     if (kMode == kWrite && my_last >= 0) {
       const int s_lo = my_start / seg_cols, s_hi = my_last / seg_cols;
       const float2* st = stats + ((size_t)h * m.total_blocks + r0 + row) * stat_segs;
@@ -323,7 +324,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, c
           const int j = j0 + 4 * (lane & 7);
           const float4 v = *reinterpret_cast<const float4*>(stage + lr * 32 + (((lane & 7) ^ (lr & 7)) << 2));
           float* dst = scores + (off + j);
-          if (j >= se.x && j + 3 <= se.y && ((off + j) & 3) == 0) *reinterpret_cast<float4*>(dst) = v;
+          if (j >= se.x && j + 3 <= se.y && (((uint32_t)off + base4) & 3u) == 0u) *reinterpret_cast<float4*>(dst) = v;   // (j is a multiple of four)
           else {
             if (j >= se.x && j <= se.y) dst[0] = v.x;
             if (j + 1 >= se.x && j + 1 <= se.y) dst[1] = v.y;

@@ -76,3 +76,23 @@ def test_gate_matrices_on_4_and_8_bytes(lens, elements):
     assert p.status() == 0
     for name in ("both", "Wk"):
         assert all(torch.equal(a, b) for a, b in zip(got[name], got["aligned"]))
+
+
+@pytest.mark.parametrize("lens", [[64 * 5], [300, 65, 64 * 7 - 1], [640 * 64]])
+def test_scores_on_4_bytes(lens):
+    import torch
+    from paper_2410_13276_b200 import binding as B
+    from paper_2410_13276_b200.prefill import Prefill
+    w = W.make_small(seed=212, seqlens=lens, hq=2, hkv=1)
+    p = Prefill(w.cu_seqlens, 2, 1, want_lse=False)
+    p.set_inputs(w.q, w.k, w.v, w.wq, w.wk)
+    params = B.make_mask_params(B.SEER_TOPK_RATIO, keep_num=1, keep_den=3, flags=3)
+    got = []
+    for elements in (0, 1, 2, 3):
+        p.scores = shifted(torch.full_like(p.scores, -1.0), elements)
+        p.row_ptr.fill_(-1)
+        p.gate()
+        p.mask(params)
+        got.append((p.scores, p.row_ptr.clone(), p.col_idx[:int(p.nnz.item())].clone()))
+    assert p.status() == 0
+    assert all(torch.equal(a, b) for x in got[1:] for a, b in zip(x, got[0]))
