@@ -26,7 +26,8 @@
  *    Errors only the device can see (list capacity exceeded, a list entry out of range, a bounded wait
  *    that ran out) are recorded in a status word owned by the context; the offending work is skipped and
  *    the kernel exits normally.  seer_poll_device_status reads that word.
- *  - bf16 tensors are passed as const void* / void*; element type is the 16-bit bfloat16 bit pattern.
+ *  - bf16 tensors are passed as const void* / void*; element type is the 16-bit bfloat16 bit pattern.  On the device they
+ *    begin on 16 bytes (SEER_ERR_CUDA otherwise); the fp32 and int32 tensors may begin on any element.
  *
  * Shapes and layouts ("THD", packed variable-length batch)
  *    T            total tokens of all sequences = cu_seqlens[batch]

@@ -736,8 +736,6 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
                     const int32_t* row_ptr, const int32_t* col_idx, void* o, float* lse, int* work_counter,
                     cudaStream_t stream) {
   if (m.q_rows == 0) return 0;
-  // the input pointers must be 16-byte aligned for TMA
-  if ((((uintptr_t)q | (uintptr_t)k | (uintptr_t)v | (uintptr_t)o) & 15) != 0) return -(int)cudaErrorMisalignedAddress;
   CUtensorMap mq, mk, mv;
   if (!tc::make_map(ctx, &mq, q, m.total_q_tokens, m.num_q_heads, 64) || !tc::make_map(ctx, &mk, k, m.total_tokens, m.num_kv_heads, 64) ||
       !tc::make_map(ctx, &mv, v, m.total_tokens, m.num_kv_heads, 32))
@@ -766,7 +764,6 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
 int launch_block_max_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const int32_t* row_ptr,
                         const int32_t* col_idx, const float* lse, float* out, cudaStream_t stream) {
   if (m.q_rows == 0) return 0;
-  if ((((uintptr_t)q | (uintptr_t)k) & 15) != 0) return -(int)cudaErrorMisalignedAddress;
   CUtensorMap mq, mk;
   if (!tc::make_map(ctx, &mq, q, m.total_q_tokens, m.num_q_heads, 64) || !tc::make_map(ctx, &mk, k, m.total_tokens, m.num_kv_heads, 64))
     return -(int)cudaErrorInvalidValue;

@@ -572,6 +572,7 @@ seer_status gate_scores_static(const seer_shape* shape, const void* q, const voi
   if (!q || !k || !Wq || !Wk || !scores) return SEER_ERR_INVALID_ARG;
   // sizes beyond the built-in scratch are refused, never truncated
   if (shape->batch > kStaticMaxBatch || gate_workspace_bytes(t, shape) > kStaticScratchBytes) return SEER_ERR_WORKSPACE;
+  if (!on_16(q, k)) return SEER_ERR_CUDA;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kStaticMaxDevices) return SEER_ERR_CUDA;
   unsigned char* base = nullptr;

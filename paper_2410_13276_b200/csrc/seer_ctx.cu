@@ -184,6 +184,10 @@ static bool ws_ok(const void* ws, size_t have, size_t need) {
   return ws && ((uintptr_t)ws & 255) == 0 && have >= need;
 }
 
+bool on_16(const void* a, const void* b, const void* c, const void* d) {
+  return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 15) == 0;
+}
+
 }  // namespace seer
 
 using namespace seer;
@@ -295,6 +299,7 @@ seer_status seer_gate_scores(seer_ctx* ctx, const seer_shape* shape, const void*
   if (t.total_blocks == 0 || t.total_q_tokens == 0) return SEER_OK;   // no score row to write
   if (!q || !k || !Wq || !Wk || !scores) return SEER_ERR_INVALID_ARG;
   if (!ws_ok(ws, ws_bytes, gate_workspace_bytes(t, shape))) return SEER_ERR_WORKSPACE;
+  if (!on_16(q, k)) return SEER_ERR_CUDA;
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
@@ -315,6 +320,7 @@ seer_status seer_gate_project(seer_ctx* ctx, const seer_shape* shape, const void
   if (t.total_blocks == 0 || t.total_q_tokens == 0) return SEER_OK;
   if (!q || !k || !Wq || !Wk) return SEER_ERR_INVALID_ARG;
   if (!ws_ok(ws, ws_bytes, gate_workspace_bytes(t, shape))) return SEER_ERR_WORKSPACE;
+  if (!on_16(q, k)) return SEER_ERR_CUDA;
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
@@ -339,6 +345,7 @@ seer_status seer_gate_scores_ex(seer_ctx* ctx, const seer_shape* shape, const se
   if (t.total_blocks == 0 || t.total_q_tokens == 0) return SEER_OK;   // no score row to write
   if (!q || !k || !Wq || !Wk || !scores) return SEER_ERR_INVALID_ARG;
   if (!ws_ok(ws, ws_bytes, gate_workspace_bytes(t, shape))) return SEER_ERR_WORKSPACE;
+  if (!on_16(q, k)) return SEER_ERR_CUDA;
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
@@ -388,6 +395,7 @@ seer_status seer_sparse_attn(seer_ctx* ctx, const seer_shape* shape, const void*
   int* work_counter = ws_ok(ws, ws_bytes, 256) ? (int*)ws : nullptr;
   if (t.total_blocks == 0 || t.total_q_tokens == 0) return SEER_OK;   // no output row
   if (!q || !k || !v || !row_ptr || !col_idx || !o) return SEER_ERR_INVALID_ARG;
+  if (!on_16(q, k, v, o)) return SEER_ERR_CUDA;
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
@@ -413,6 +421,7 @@ seer_status seer_attn_block_max(seer_ctx* ctx, const seer_shape* shape, const vo
   if (shape->block != kBlock) return SEER_ERR_UNSUPPORTED;
   if (t.total_blocks == 0 || t.total_q_tokens == 0) return SEER_OK;
   if (!q || !k || !row_ptr || !col_idx || !lse || !block_max) return SEER_ERR_INVALID_ARG;
+  if (!on_16(q, k)) return SEER_ERR_CUDA;
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
@@ -462,6 +471,7 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
   if (t.total_blocks > 0 && ((!q && t.total_q_tokens > 0) || !k || !Wq || !Wk)) return SEER_ERR_INVALID_ARG;
   const size_t planes_bytes = gate_workspace_bytes(t, shape), stats_bytes = gate_stats_bytes(t, shape);
   if (t.total_blocks > 0 && !ws_ok(ws, ws_bytes, planes_bytes + min_band_bytes(t))) return SEER_ERR_WORKSPACE;
+  if (t.total_blocks > 0 && !on_16(t.total_q_tokens > 0 ? q : nullptr, k)) return SEER_ERR_CUDA;
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;

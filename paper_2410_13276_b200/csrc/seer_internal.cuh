@@ -124,6 +124,8 @@ namespace seer {
 // and fills `m`.  `slot_out` identifies the slot to pass to finish_call.
 seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream, SeqMeta* m, int* slot_out);
 void finish_call(seer_ctx* ctx, int slot, cudaStream_t stream);
+// Whether tensors that the kernels copy 16 bytes at a time begin on 16 bytes (a misaligned access would end the context).
+bool on_16(const void* a, const void* b, const void* c = nullptr, const void* d = nullptr);
 
 // Host-only shape arithmetic (no CUDA calls): returns SEER_OK and fills totals.
 struct ShapeTotals {

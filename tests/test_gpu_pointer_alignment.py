@@ -96,3 +96,39 @@ def test_scores_on_4_bytes(lens):
         got.append((p.scores, p.row_ptr.clone(), p.col_idx[:int(p.nnz.item())].clone()))
     assert p.status() == 0
     assert all(torch.equal(a, b) for x in got[1:] for a, b in zip(x, got[0]))
+
+
+@pytest.mark.parametrize("elements", [1, 4])
+def test_bf16_tensors_off_16_bytes_are_refused(elements):
+    import torch
+    from paper_2410_13276_b200 import binding as B
+    from paper_2410_13276_b200.prefill import Prefill
+    w = W.make_small(seed=213, seqlens=[300, 65], hq=2, hkv=1)
+    p = Prefill(w.cu_seqlens, 2, 1)
+    p.set_inputs(w.q, w.k, w.v, w.wq, w.wk)
+    params = B.make_mask_params(B.SEER_TOPK_RATIO, keep_num=1, keep_den=3, flags=3)
+    options = B.seer_gate_options(B.SEER_POOL_AVG, B.SEER_POOL_AVG, 10000.0)
+    p.run(params)
+    want, good = p.o.clone(), {x: getattr(p, x) for x in "qkvo"}
+    calls = [("qk", p.gate), ("qk", p.gate_project), ("qk", lambda: p.gate_ex(options, p.wq, p.wk)), ("qk", lambda: p.gate_mask(params)),
+             ("qk", lambda: B.seer_gate_scores_static(p.shape, p.q, p.k, p.wq, p.wk, p.scores)), ("qkvo", p.attn), ("qk", p.block_max)]
+    for impl in (1, 0):
+        B.seer_set_attn_impl(p.ctx, impl)
+        for names, call in calls:
+            for x in names:
+                launched = B.seer_launch_count(p.ctx)
+                setattr(p, x, shifted(good[x], elements))
+                with pytest.raises(B.SeerError) as e:
+                    call()
+                setattr(p, x, good[x])
+                assert e.value.status == 7 and B.seer_launch_count(p.ctx) == launched
+    p.o.fill_(-1.0)
+    p.run(params)
+    assert p.status() == 0 and torch.equal(p.o, want)
+    # a pointer that nothing reads may be anything: queries of a chunk without any, inputs of an empty batch
+    for lens, cu_q in (([300], np.array([0, 0], np.int32)), ([0], None)):
+        e = Prefill(np.array([0, lens[0]], np.int32), 2, 1, ctx=p.ctx, cu_seqlens_q=cu_q)
+        e.q, e.k, e.wq, e.wk = shifted(good["q"], elements), good["k"] if lens[0] else shifted(good["k"], elements), p.wq, p.wk
+        e.row_ptr.fill_(-1)
+        e.gate_mask(params)
+        assert e.status() == 0 and not e.row_ptr.any()
