@@ -210,7 +210,8 @@ seer_status seer_poll_device_status(seer_ctx* ctx, void* stream);
  * Host buffers should be page-locked for the copies to be asynchronous; they must stay valid, and o_host must not be read,
  * until `stream` has been synchronised.  `arena` is a caller-owned DEVICE buffer of at least
  * seer_prefill_host_arena_bytes(shape) bytes, 256-byte aligned, that holds two sets of slice inputs / outputs and one set of
- * slice intermediates; the call allocates nothing.  col_idx inside the arena is sized for the full causal mask of a slice,
+ * slice intermediates, the rows' softmax statistics (see seer_workspace_bytes) last: an arena without room for these is taken too,
+ * with the same result.  The call allocates nothing.  col_idx inside the arena is sized for the full causal mask of a slice,
  * so SEER_ERR_CAPACITY cannot occur.  One call at a time per context. */
 size_t seer_prefill_host_arena_bytes(const seer_shape* shape);
 seer_status seer_prefill_host(seer_ctx* ctx, const seer_shape* shape, const void* q_host, const void* k_host,

@@ -635,7 +635,7 @@ namespace {
 // with num_q_heads = G, num_kv_heads = 1.  The arena holds two sets of slice inputs and outputs (copy of slice s + 1 and
 // read-back of slice s - 1 overlap the kernels of slice s) and one set of intermediates.
 struct ArenaLayout {
-  size_t q[2], k[2], v[2], o[2], lse[2], wq[2], wk[2], scores, row_ptr, col_idx, nnz, ws, ws_bytes, total;
+  size_t q[2], k[2], v[2], o[2], lse[2], wq[2], wk[2], scores, row_ptr, col_idx, nnz, ws, need, total;
 };
 ArenaLayout arena_layout(const seer_shape* slice, const ShapeTotals& t) {   // shape and totals of ONE slice
   ArenaLayout a;
@@ -655,8 +655,9 @@ ArenaLayout arena_layout(const seer_shape* slice, const ShapeTotals& t) {   // s
   a.row_ptr = take(((size_t)t.rows + 1) * 4);
   a.col_idx = take((size_t)t.causal_blocks * 4);
   a.nnz = take(8);
-  a.ws_bytes = gate_workspace_bytes(t, slice) + gate_stats_bytes(t, slice);
-  a.ws = take(a.ws_bytes);
+  a.ws = take(gate_workspace_bytes(t, slice));
+  a.need = p;
+  take(gate_stats_bytes(t, slice));                        // behind the projected vectors: used where there is room
   a.total = p;
   return a;
 }
@@ -692,7 +693,8 @@ seer_status seer_prefill_host(seer_ctx* ctx, const seer_shape* shape, const void
   seer_shape slice;
   if (!slice_of(shape, &slice, &t)) return SEER_ERR_INVALID_ARG;
   const ArenaLayout a = arena_layout(&slice, t);
-  if (!ws_ok(arena, arena_bytes, a.total)) return SEER_ERR_WORKSPACE;
+  if (!ws_ok(arena, arena_bytes, a.need)) return SEER_ERR_WORKSPACE;
+  const size_t ws_bytes = (arena_bytes < a.total ? arena_bytes : a.total) - a.ws;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return SEER_ERR_CUDA;
   char* d = (char*)arena;
   const size_t T = (size_t)t.total_tokens;
@@ -736,13 +738,13 @@ seer_status seer_prefill_host(seer_ctx* ctx, const seer_shape* shape, const void
       // ---- the three calls, on the caller's stream
       SEER_TRY(cudaStreamWaitEvent(stream, ctx->ev_h2d[b], 0));
       st = seer_gate_scores(ctx, &part, dq, d + a.k[b], (const float*)(d + a.wq[b]) + h0 * kHeadDim * kGateDim, (const float*)(d + a.wk[b]),
-                            (float*)(d + a.scores), d + a.ws, a.total - a.ws, stream);
+                            (float*)(d + a.scores), d + a.ws, ws_bytes, stream);
       if (st != SEER_OK) return st;
       st = seer_block_mask(ctx, &part, (const float*)(d + a.scores), params, (int32_t*)(d + a.row_ptr),
                            (int32_t*)(d + a.col_idx), t.causal_blocks, (int64_t*)(d + a.nnz), nullptr, 0, stream);
       if (st != SEER_OK) return st;
       st = seer_sparse_attn(ctx, &part, dq, d + a.k[b], d + a.v[b], (const int32_t*)(d + a.row_ptr), (const int32_t*)(d + a.col_idx),
-                            dout, dlse, d + a.ws, a.total - a.ws, stream);   // (the gate's workspace is free again: the attention's work counter)
+                            dout, dlse, d + a.ws, ws_bytes, stream);   // (the gate's workspace is free again: the attention's work counter)
       if (st != SEER_OK) return st;
       SEER_TRY(cudaEventRecord(ctx->ev_comp[b], stream));
       // ---- device -> host
