@@ -182,8 +182,8 @@ struct Slot {
   int h, i, l0, nlist, q_valid, s0, tok0;   // tok0: first row of the item in q / o / lse
   __device__ __forceinline__ int ntiles() const { return (nlist + 1) >> 1; }
 };
-__device__ __forceinline__ int slot_block(const Slot& it, const int32_t* __restrict__ col_idx, int p) {
-  return p < it.nlist ? __ldg(col_idx + it.l0 + p) : -1;
+__device__ __forceinline__ int slot_block(const Slot& it, const int32_t* col_idx, int p) {
+  return p < it.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + it.l0 + p) : -1;
 }
 // Block index of a list entry: -1 past the end of the list, -2 outside [0, i].
 __device__ __forceinline__ int slot_check(const Slot& it, int p, int raw) {
@@ -203,9 +203,9 @@ template <bool kTrace, bool kChunk, bool kBlockMax = false, bool kO32 = true>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, SeqMeta m,
-                const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
-                uint16_t* __restrict__ o, float* __restrict__ lse, int* __restrict__ status,
-                unsigned long long* __restrict__ trace, float* __restrict__ block_max = nullptr,
+                const int32_t* row_ptr, const int32_t* col_idx,
+                uint16_t* __restrict__ o, float* lse, int* __restrict__ status,
+                unsigned long long* __restrict__ trace, float* block_max = nullptr,
                 int* __restrict__ work_counter = nullptr) {
   extern __shared__ __align__(1024) unsigned char smem[];
   Shared sh;

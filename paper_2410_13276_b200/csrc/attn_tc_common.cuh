@@ -218,7 +218,7 @@ struct Item {
 // them: a stream took about a microsecond to draw one, look it up and drop it (917 queries against 60k tokens: 29 888 items
 // for 512 of work, 163 -> 67 us; 8k against 128k, 65 536 for 4096: 90 us less).
 template <bool kChunk>
-__device__ __forceinline__ Item decode_item(const SeqMeta& m, const int32_t* __restrict__ row_ptr, int64_t w) {
+__device__ __forceinline__ Item decode_item(const SeqMeta& m, const int32_t* row_ptr, int64_t w) {
   Item it;
   const int32_t* off = kChunk ? m.qblk_off : m.blk_off;    // blocks with queries: the last ones of each sequence
   it.b = find_sequence(off, m.batch, (int)(w / m.num_q_heads));
@@ -241,7 +241,7 @@ __device__ __forceinline__ Item decode_item(const SeqMeta& m, const int32_t* __r
 }
 
 // Block index of list position p of an item: -1 past the end of the list, -2 for an entry outside [0, i].
-__device__ __forceinline__ int list_block(const Item& it, const int32_t* __restrict__ col_idx, int p) {
+__device__ __forceinline__ int list_block(const Item& it, const int32_t* col_idx, int p) {
   if (p >= it.nlist) return -1;
   const int j = col_idx[it.l0 + p];
   return (j < 0 || j > it.i) ? -2 : j;

@@ -94,8 +94,8 @@ __device__ __forceinline__ void combine(float& m, float& l, float m2, float l2) 
 // matrix minus band.score_base.  stats: [head][block of the batch][stat_segs] (m, l).
 template <int kMode>
 __global__ void __launch_bounds__(gs::kThreads, 1)
-gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* __restrict__ gq, const uint16_t* __restrict__ gk,
-                   float* __restrict__ scores, float2* __restrict__ stats, int* __restrict__ status, int part_tiles) {
+gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t* gk,
+                   float* scores, float2* stats, int* __restrict__ status, int part_tiles) {
   using namespace gs;
   extern __shared__ __align__(1024) unsigned char gs_raw[];   // (the swizzled tiles need 1024-byte alignment)
   const uint32_t base = (uint32_t)__cvta_generic_to_shared(gs_raw);

@@ -30,7 +30,7 @@ struct RowBand {
   ScoreBand sb;
 };
 
-__device__ __forceinline__ RowInfo decode_row(const SeqMeta& m, const RowBand& band, const float* __restrict__ scores, int64_t r) {
+__device__ __forceinline__ RowInfo decode_row(const SeqMeta& m, const RowBand& band, const float* scores, int64_t r) {
   RowInfo ri;
   ri.valid = r < band.row_hi;
   ri.skip = false;
@@ -86,7 +86,7 @@ __device__ __forceinline__ int warp_sum(int v) {
 }
 
 __global__ void __launch_bounds__(kMaskWarps * 32)
-count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask_params p, int32_t* __restrict__ row_ptr) {
+count_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, int32_t* row_ptr) {
   const int lane = threadIdx.x & 31;
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * kMaskWarps + (threadIdx.x >> 5);
   const RowInfo ri = decode_row(m, band, scores, r);
@@ -137,8 +137,8 @@ count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mas
 // NaN among its scores, so its length follows from n and the parameters and no score is read (4096 rows of 4096 blocks: 15 us
 // with count_kernel); a row that has not is counted by its thread.
 __global__ void __launch_bounds__(128)
-topk_count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, const float2* __restrict__ stats, seer_mask_params p,
-                  int32_t* __restrict__ row_ptr) {
+topk_count_kernel(SeqMeta m, RowBand band, const float* scores, const float2* stats, seer_mask_params p,
+                  int32_t* row_ptr) {
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * 128 + threadIdx.x;
   const RowInfo ri = decode_row(m, band, scores, r);
   grid_wait();
@@ -174,7 +174,7 @@ topk_count_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, con
 constexpr int kScanPer = 8, kScanTile = 1024 * kScanPer, kScanRanks = 8;
 template <int kRanks>
 __global__ void __launch_bounds__(1024)
-scan_kernel(int64_t rows, int32_t* __restrict__ row_ptr, int first, int64_t col_capacity, int64_t* __restrict__ nnz_out,
+scan_kernel(int64_t rows, int32_t* row_ptr, int first, int64_t col_capacity, int64_t* __restrict__ nnz_out,
             int* __restrict__ status) {
   __shared__ int32_t tile[kScanTile + kScanTile / 32];     // (one word of padding per 32: eight consecutive words per thread)
   __shared__ int32_t warp_tot[2][32], rank_tot[2][kRanks];
@@ -291,8 +291,8 @@ __device__ __forceinline__ uint32_t lean_key(float sc) {
 // needs once done by every warp of it, and a pass of its own for the counts: 183 and 34.
 template <int W>
 __global__ void __launch_bounds__(W < 4 ? 128 : W * 32, W < 8 ? 12 : 6)
-topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask_params p, const int32_t* __restrict__ row_ptr,
-            int32_t* __restrict__ col_idx, int64_t col_capacity, int cap) {
+topk_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, const int32_t* row_ptr,
+            int32_t* col_idx, int64_t col_capacity, int cap) {
   constexpr int kWarps = W < 4 ? 4 : W, kRows = kWarps / W;
   extern __shared__ __align__(16) uint32_t key_smem[];
   __shared__ __align__(16) uint32_t s_hist[kRows][256];
@@ -322,7 +322,7 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   const int n = ri.i + 1;
   const int32_t out0 = row_ptr[r], out1 = row_ptr[r + 1];
   if ((int64_t)out1 > col_capacity) return;   // this row (and all later ones) do not fit; status already raised
-  int32_t* __restrict__ out = col_idx + out0;
+  int32_t* out = col_idx + out0;
   const uint32_t lt_mask = (1u << lane) - 1u;
   if (ri.i >= ri.nb - p.dense_tail_blocks) {           // a dense row at the end of the sequence: every causal block
     for (int j = w * 32 + lane; j < n; j += W * 32) out[j] = j;
@@ -339,7 +339,7 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   // ---- keys (0: not a candidate: past the row, NaN, or forced, which the writer puts in its place by itself)
   uint32_t c = 0, k_min = 0xffffffffu, k_max = 0u;               // over the candidates
   const uint32_t nan_bits = 0x7fffffffu;
-  const uint32_t* __restrict__ src = reinterpret_cast<const uint32_t*>(ri.s);
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(ri.s);
   const bool vec = (reinterpret_cast<uintptr_t>(ri.s) & 15) == 0;
   for (int j0 = j_mine; j0 - 4 * lane < j_hi; j0 += 512) {
     uint4 v[4];                                                  // four loads in flight per lane
@@ -347,12 +347,12 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
     for (int q = 0; q < 4; ++q) {
       const int j = j0 + q * 128;
       v[q] = make_uint4(nan_bits, nan_bits, nan_bits, nan_bits);
-      if (vec && j + 3 < j_hi) v[q] = __ldg(reinterpret_cast<const uint4*>(src + j));
+      if (vec && j + 3 < j_hi) v[q] = ld_global_v4(src + j);
       else if (j < j_hi) {
-        v[q].x = __ldg(src + j);
-        if (j + 1 < j_hi) v[q].y = __ldg(src + j + 1);
-        if (j + 2 < j_hi) v[q].z = __ldg(src + j + 2);
-        if (j + 3 < j_hi) v[q].w = __ldg(src + j + 3);
+        v[q].x = ld_global(src + j);
+        if (j + 1 < j_hi) v[q].y = ld_global(src + j + 1);
+        if (j + 2 < j_hi) v[q].z = ld_global(src + j + 2);
+        if (j + 3 < j_hi) v[q].w = ld_global(src + j + 3);
       }
     }
 #pragma unroll
@@ -573,8 +573,8 @@ topk_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
 
 // Threshold lists, and TopK lists of rows beyond kTopkRowMax: a warp per row.
 __global__ void __launch_bounds__(kMaskWarps * 32)
-fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask_params p, const int32_t* __restrict__ row_ptr,
-            int32_t* __restrict__ col_idx, int64_t col_capacity) {
+fill_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, const int32_t* row_ptr,
+            int32_t* col_idx, int64_t col_capacity) {
   __shared__ __align__(16) uint32_t hist_smem[kMaskWarps * 256];      // 256 bins per warp
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * kMaskWarps + warp;
@@ -584,7 +584,7 @@ fill_kernel(SeqMeta m, RowBand band, const float* __restrict__ scores, seer_mask
   const int n = ri.i + 1;
   const int32_t out0 = row_ptr[r], out1 = row_ptr[r + 1];
   if ((int64_t)out1 > col_capacity) return;   // this row (and all later ones) do not fit; status already raised
-  int32_t* __restrict__ out = col_idx + out0;
+  int32_t* out = col_idx + out0;
   const uint32_t lt_mask = (1u << lane) - 1u;
 
   if (ri.i >= ri.nb - p.dense_tail_blocks) {           // a dense row at the end of the sequence: every causal block
@@ -774,8 +774,8 @@ int launch_mask(seer_ctx* ctx, const SeqMeta& m, const float* scores, const seer
 // reports it.  One warp per 64-token row; `fill` = false counts, true writes.
 template <bool kFill>
 __global__ void __launch_bounds__(kMaskWarps * 32)
-expand_kernel(SeqMeta m128, SeqMeta m64, const int32_t* __restrict__ row_ptr128, const int32_t* __restrict__ col_idx128,
-              int32_t* __restrict__ row_ptr64, int32_t* __restrict__ col_idx64, int64_t col_capacity64) {
+expand_kernel(SeqMeta m128, SeqMeta m64, const int32_t* row_ptr128, const int32_t* col_idx128,
+              int32_t* row_ptr64, int32_t* col_idx64, int64_t col_capacity64) {
   grid_wait();
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * kMaskWarps + (threadIdx.x >> 5);

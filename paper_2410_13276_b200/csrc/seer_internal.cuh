@@ -163,6 +163,19 @@ __device__ __forceinline__ void grid_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// What the kernel before writes (scores, statistics, projected vectors, row_ptr, col_idx, lse) changes while this kernel is resident,
+// so nothing may promise the compiler that it does not: no __restrict__ and no __ldg on it, which allow a load to move above the
+// wait.  These loads name the address space of a pointer that the compiler has lost sight of.
+__device__ __forceinline__ uint32_t ld_global(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint4 ld_global_v4(const uint32_t* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+  return v;
+}
 
 // Kernel launchers (each returns the number of kernels it launched, or a negative cudaError).
 int launch_gate(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k, const float* Wq, const float* Wk,
