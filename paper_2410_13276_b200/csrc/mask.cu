@@ -3,8 +3,8 @@
 //   scan_kernel  : exclusive prefix sum of the counts -> row_ptr, nnz, capacity check
 //   topk_kernel / fill_kernel : repeat the selection and write the ascending lists
 // Selection order in the TopK modes is (score descending, block index ascending): scores become order-preserving
-// 32-bit keys, the key of the last kept candidate is found by a radix select (at most four 8-bit passes), and ties at that
-// key are resolved by rank in index order.
+// 32-bit keys, the key of the last kept candidate is found (by bins of the keys' distance from the smallest in topk_kernel, by a radix
+// select of at most four 8-bit passes in fill_kernel), and ties at that key are resolved by rank in index order.
 #include <math_constants.h>
 
 #include "seer_internal.cuh"
@@ -280,7 +280,7 @@ __device__ __forceinline__ uint32_t lean_key(float sc) {
   return z != z ? 0u : kk;                                       // NaN: never a candidate
 }
 
-// TopK lists, W warps per row, the row's keys in shared memory (`cap` of them, a multiple of 128 W).  A warp works on a contiguous
+// TopK lists, W = 1, 4 or 8 warps per row, the row's keys in shared memory (`cap` of them, a multiple of 128 W).  A warp works on a contiguous
 // run of the row's columns, 128 at a time, a lane four of them.
 //
 // It is bound by instruction issue (3.5 of 4 per clock), so the loops are short and rolled (with the keys in registers and the
@@ -290,10 +290,11 @@ __device__ __forceinline__ uint32_t lean_key(float sc) {
 // 2048 blocks 251 -> 176 us, 4096 rows of up to 4096 blocks (which re-read their scores in every pass) 158 -> 31 us; what a row
 // needs once done by every warp of it, and a pass of its own for the counts: 183 and 34.
 template <int W>
-__global__ void __launch_bounds__(W < 4 ? 128 : W * 32, W < 8 ? 12 : 6)
+__global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W < 8 ? 12 : 6)
 topk_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, const int32_t* row_ptr,
             int32_t* col_idx, int64_t col_capacity, int cap) {
-  constexpr int kWarps = W < 4 ? 4 : W, kRows = kWarps / W;
+  static_assert(W == 1 || W == 4 || W == 8, "a row has a warp or a CTA to itself");
+  constexpr int kRows = W == 1 ? 4 : 1;
   extern __shared__ __align__(16) uint32_t key_smem[];
   __shared__ __align__(16) uint32_t s_hist[kRows][256];
   __shared__ uint32_t s_red[kRows][3][W];
@@ -307,7 +308,6 @@ topk_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, co
   const int rr = warp / W, w = warp % W;                         // row of the CTA, warp within the row's group
   auto meet = [&]() {                                            // the warps of a row
     if (W == 1) __syncwarp();
-    else if (W < 4) asm volatile("bar.sync %0, %1;" ::"r"(1 + rr), "n"(W * 32) : "memory");
     else __syncthreads();
   };
   const int64_t r = band.row_lo + (int64_t)blockIdx.x * kRows + rr;
@@ -653,7 +653,8 @@ fill_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, co
   } else if (take == 0) {
     T = 0xffffffffu; need_eq = 0;   // nothing beyond the forced blocks
   } else {
-    // radix select as in topk_kernel, the scores re-read in every pass
+    // radix select, up to 8 bits a pass from the top, the scores re-read in every pass: a histogram of the current digit of the keys
+    // that match the prefix found so far, walked from the largest digit down.  The leading bits that all keys share need no pass.
     uint32_t* hist = hist_smem + warp * 256;
     const uint32_t differ = k_and ^ k_or;                                 // bit set: not all keys agree there
     int hi_bit = differ == 0u ? 0 : 31 - __clz(differ);                   // highest differing bit
@@ -725,7 +726,7 @@ fill_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, co
 template <int W>
 static cudaError_t launch_topk_w(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
                           int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
-  constexpr int kRows = W < 4 ? 4 / W : 1, kThreads = W < 4 ? 128 : W * 32;
+  constexpr int kRows = W == 1 ? 4 : 1, kThreads = W == 1 ? 128 : W * 32;
   const int cap = (m.max_nb + 128 * W - 1) / (128 * W) * (128 * W);
   return launch_next(topk_kernel<W>, (unsigned)((band.row_hi - band.row_lo + kRows - 1) / kRows), kThreads, (size_t)kRows * cap * 4, stream, m, band,
                      scores, p, row_ptr, col_idx, col_capacity, cap);
