@@ -160,7 +160,8 @@ seer_status seer_block_mask(seer_ctx* ctx, const seer_shape* shape, const float*
  *    blocks listed for its (sequence, head, query block) row that are not later than the query.  bf16 operands, fp32
  *    accumulation and softmax, probabilities rounded to bf16 before the P V product, o written as bf16.
  *    lse (optional, may be NULL): [num_q_heads, T] fp32, natural log of the softmax denominator of the scaled logits.
- *    A row with an empty list yields o = 0 and lse = -inf.
+ *    A row with an empty list yields o = 0 and lse = -inf.  Values up to 2^50 are safe whatever the scores; larger ones may
+ *    overflow where a row's scores rise far (by up to 2^60 in probability) above those of the first block of its list.
  *    ws (optional): with a workspace of at least 256 bytes (256-byte aligned, as for the other calls) the first word
  *    becomes the counter from which the tcgen05 kernel's persistent CTAs draw their (head, query block) work items,
  *    so that a CTA that finishes early takes more of them; without one (NULL), and where there are no more than two items
@@ -182,11 +183,10 @@ seer_status seer_attn_block_max(seer_ctx* ctx, const seer_shape* shape, const vo
                                 void* stream);
 
 /* Selects the attention kernel used by seer_sparse_attn (and, by the same rule, the kernel of seer_attn_block_max: the
- * tcgen05 pipeline without V, or the mma.sync kernel): 0 = tcgen05 / TMEM / TMA kernel (default),
- * 1 = mma.sync kernel (on-device cross-check; also the faster one for very short lists), 2 = chosen per call from
- * the shape: the persistent tcgen05 kernel pays a few microseconds per (head, query block) row whatever its list
- * length, so batches whose rows have at most 8 causal blocks on average (many short sequences) go to the mma.sync
- * kernel and everything else to the tcgen05 kernel.  Returns SEER_ERR_INVALID_ARG for other values. */
+ * tcgen05 pipeline without V, or the mma.sync kernel): 0 = tcgen05 / TMEM / TMA kernel (default, and the faster one or
+ * equal at every shape measured), 1 = mma.sync kernel (on-device cross-check), 2 = chosen per call from the shape: batches whose
+ * rows have at most 8 causal blocks on average (many short sequences) go to the mma.sync kernel and everything else to the
+ * tcgen05 kernel.  Returns SEER_ERR_INVALID_ARG for other values. */
 seer_status seer_set_attn_impl(seer_ctx* ctx, int impl);
 
 /* Test hook for the bounded waits of the tcgen05 attention kernel (no counterpart in the paper).  Every barrier
@@ -226,8 +226,8 @@ seer_status seer_prefill_host(seer_ctx* ctx, const seer_shape* shape, const void
  * call cudaMalloc behind its back, a latency-critical loop where cudaMalloc's implicit device synchronisation is not
  * acceptable.  Such a caller cannot create a seer_ctx (seer_create allocates) nor provide a workspace.
  *
- * What it does: the same two kernels as seer_gate_scores, same arguments and results (q, k, Wq, Wk in, scores out, all
- * DEVICE pointers owned by the caller), on the CURRENT device, without a context and without a workspace.  The
+ * What it does: the two kernels of seer_gate_scores without room for statistics, same arguments and results (q, k, Wq, Wk in,
+ * scores out, all DEVICE pointers owned by the caller), on the CURRENT device, without a context and without a workspace.  The
  * intermediate projected vectors and the per-batch offsets live in a fixed array inside the library image: every GPU
  * that loads the library holds SEER_STATIC_SCRATCH_BYTES + 16 KiB for it until the process exits.
  *
@@ -235,7 +235,7 @@ seer_status seer_prefill_host(seer_ctx* ctx, const seer_shape* shape, const void
  * 256 per tensor) <= SEER_STATIC_SCRATCH_BYTES, i.e. 10922 (head, block) pairs: e.g. 40 heads x 17000 tokens.  Larger shapes
  * return SEER_ERR_WORKSPACE and enqueue nothing.
  *
- * First call on a device: looks up the array's device address and raises one kernel's shared-memory limit (no allocation).
+ * First call on a device: looks up the array's device address and raises the score kernels' shared-memory limit (no allocation).
  * Make that first call outside of any stream capture.  The call itself performs no cudaMalloc / cudaFree and uses no
  * allocating library routine; it copies about 5 KiB of offsets from the host stack with cudaMemcpyAsync and launches.
  *

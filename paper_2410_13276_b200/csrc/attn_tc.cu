@@ -1,8 +1,9 @@
 // Block-sparse causal GQA attention (Sec. 3.3) on the Blackwell tensor path, two work items in flight per CTA.
 //
-// What bounds it: the copies of K and V into shared memory (64 KB per pair of listed 64 x 64 blocks, an SM takes about 70
-// bytes per clock from L2) before the MMA pipe (8 x 48 + 4 x 76 clocks per pair), and in launches of more than a few
-// milliseconds the board's power limit; short lists are bound by the latencies of an item's start and end.
+// What bounds it.  Long lists: the copies of K and V into shared memory (64 KB per pair of listed 64 x 64 blocks, about 885 clocks
+// at the 74 bytes a clock that an SM takes from L2, of 917 to 1060 that a pair takes), close before the MMA pipe (8 x 48 + 4 x 76 =
+// 688 clocks: 75 % active on dense lists of 16k tokens), and in launches of more than a few milliseconds the board's power limit.
+// Short lists: an item's start and end, about 6000 clocks beside 2000 for a stream's tile (13 tiles an item: the pipe 61 % active).
 //
 // Tiles.  A query block is 64 rows and every (head, query block) has its own list, so no two items share their keys.
 // The MMAs are the weight-stationary form (tcgen05.mma.ws) with M = 64: the 128 lanes of tensor memory hold two 64-row
@@ -14,12 +15,13 @@
 // so all 128 lanes work for arbitrary lists at 82 % of the full MMA rate (K = 16 in 48 clocks for N = 128, 76 for 256; the
 // ordinary M = 64 form takes 64 and 128).  A thread owns a query row and all 64 keys of one block: the softmax needs no
 // other thread.  The two halves are two partial results with their own references and sums (as in split-KV decoding), merged
-// once per item.  Against the transposed product it replaced (S^T = K Q^T with a thread per key, references per column
-// subtracted by a ninth MMA step, a vote of the group per tile, P^T through shared memory; 17 MMAs of 48 clocks per
-// tile): 128k tokens at one block in ten 20.5 -> 15.3 ms, 24 short prompts 331 -> 187 us, dense 16k 2.80 -> 2.22 ms.
+// once per item.  The transposed product (S^T = K Q^T, a thread per key, a vote of the group per tile, P^T through shared memory)
+// takes 17 MMAs of 48 clocks per tile and 20.5 ms where this takes 15.3 (128k tokens, one block in ten).
 //
 // References.  p = 2^(s * scale * log2(e) - R), R the row's maximum over the half's first live block.  P is bf16 and the sums are
-// fp32, so p may grow to 2^60 before R has to move: the sum of a tile's 64 probabilities says so, without a maximum.
+// fp32, so p may grow to 2^60 before R has to move: the sum of a tile's 64 probabilities says so, without a maximum.  O
+// holds the values at that scale, so values up to 2^50 stay finite however a row's scores rise.  (2^30 here, for values up to 2^80:
+// short prompts 253.6 us against 252.1, long ones alike; 2^20: 264; 2^10: 338 and long ones 10 to 30 % more.)
 // When it does, the warp waits for the previous P V, rescales its rows of O and its sums and takes the tile again.
 //
 // Arrangement.  A CTA runs two independent streams; a stream owns a whole work item (head, query block) from its first
@@ -149,7 +151,7 @@ __device__ __forceinline__ float row_pass(uint32_t s_addr, float sl2, float R, i
 }
 
 // The largest raw score of this thread's row (MASKED: among the keys it sees, key <= last; -inf if there is none).
-// Off the diagonal without the 64 predicates: 16k block maxima and attention 3.99 -> 3.87 ms, 128k prompt 17.3 -> 16.9.
+// Off the diagonal the 64 predicates are left out (with them a 128k prompt takes 2 % longer).
 template <bool MASKED>
 __device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
   float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
@@ -195,9 +197,8 @@ __device__ __forceinline__ int slot_check(const Slot& it, int p, int raw) {
 // kBlockMax: the same pipeline without V: instead of softmax(S) V the kernel writes, for every list entry, the largest
 // probability exp(scale * s - lse) of its 64 x 64 tile (Sec. 3.2, Eq. 2 on the listed blocks), `lse` being an input: a
 // thread takes the maximum of its row, a block's maximum is one redux per warp and a word from its neighbour.
-// Without V and O a stream has five K units and four S buffers: with two of each it waited for copies and MMAs in turn (16k
-// tokens, 32 heads, all causal blocks: 1277 -> 1060 us, 520 clocks a tile; 440 are its 32 KB from L2, 384 its MMAs).  Tiles of four
-// blocks on N = 256 MMAs, 320 clocks per two blocks, gave nothing more.
+// Without V and O a stream has five K units and four S buffers: with two of each it waits for copies and MMAs in turn (16k tokens, 32
+// heads, all causal blocks: 1277 us and 1060 so, 520 clocks a tile; 440 are its 32 KB from L2, 384 its MMAs).
 // kO32: o begins on 32 bytes.  (A test of the address in the kernel instead: 32k tokens 1392 -> 1404 us.)
 template <bool kTrace, bool kChunk, bool kBlockMax = false, bool kO32 = true>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -246,7 +247,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   const long long cta_c0 = kTrace ? clock64() : 0ll;
 
   // Work items.  Without a counter a stream takes the items CTA + stream * grid, + 2 * grid, ... (static deal: as long as there are no
-  // more items than CTAs each has an SM to itself; two to an SM, 128 items took 15.2 us, and 12.3 so).  With one
+  // more items than CTAs each has an SM to itself: 128 items 12.3 us, two to an SM 15.2).  With one
   // (`work_counter`, zero at launch) the next item number is drawn from it.  Either way the stream's Q / K producer decodes
   // the item and passes it to the other roles through a ring of four slots, each with a full and an empty mbarrier: a slot
   // is rewritten only when every other role has read it.  nlist < 0 ends the stream.  Results do not depend on which

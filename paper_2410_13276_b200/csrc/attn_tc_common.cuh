@@ -1,5 +1,5 @@
-// Pieces shared by the tcgen05 attention kernels: PTX wrappers (mbarrier, TMA, tcgen05, named barriers), shared-memory
-// matrix descriptors, the work-item decoder, warp-level column reductions and the optional cycle accounting.
+// Pieces shared by the tcgen05 kernels of the attention and of the gate's scores: PTX wrappers (mbarrier, TMA, tcgen05, named barriers),
+// shared-memory matrix descriptors, the work-item decoder and the optional cycle accounting.
 #pragma once
 
 #include <cuda.h>
@@ -215,8 +215,8 @@ struct Item {
 
 // kChunk: chunked prefill.  q / o / lse hold the last positions of each sequence only: their token index is the k / v
 // token index plus dq.  Query blocks before the chunk have nothing to do whatever their lists say, and no work item is counted for
-// them: a stream took about a microsecond to draw one, look it up and drop it (917 queries against 60k tokens: 29 888 items
-// for 512 of work, 163 -> 67 us; 8k against 128k, 65 536 for 4096: 90 us less).
+// them: a stream takes about a microsecond to draw one, look it up and drop it (917 queries against 60k tokens: 29 888 items
+// for 512 of work, 163 us and 67 so).
 template <bool kChunk>
 __device__ __forceinline__ Item decode_item(const SeqMeta& m, const int32_t* row_ptr, int64_t w) {
   Item it;

@@ -84,9 +84,8 @@ __device__ __forceinline__ void acc_bf16x8(float (&a)[8], const uint4& u) {
 
 // What a CTA pools: a chunk of blocks of one head, the head varying fastest so that CTAs running together read neighbouring
 // 256-byte segments of the same token rows.  Chunked prefill: most chunks of Q lie before its queries, and CTAs with nothing to
-// do between those of K kept the memory system idle.  So K comes first there, and of Q the chunks of a single sequence that
-// lie before its queries have no CTA, other such CTAs leave at once (8k tokens against 128k: 135 -> 78 us, the bytes take 51;
-// four sequences of 60k tokens with 917 queries: 70 -> 47 us).
+// do between those of K keep the memory system idle.  So K comes first there, and of Q the chunks of a single sequence that
+// lie before its queries have no CTA, other such CTAs leave at once (8k tokens against 128k: 135 us, 78 so).
 struct PoolWork {
   int chunk, h, H;
   bool is_q, idle;
@@ -225,8 +224,8 @@ pool_project_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* _
   if constexpr (kChunk == 16) {
     // projection: a thread takes four output columns, four blocks and one half of the matrix's rows, two columns to an instruction.
     // What bounds it is the 128 bytes a clock that loads return to the registers: a step is 16 bytes of W, 16 of four blocks'
-    // column and 16 products (a column and sixteen blocks to a thread: 68 bytes for as many; 128k tokens, 32 / 8 heads 296 -> 266 us,
-    // 205 of them the bytes; 32k 76 -> 67; blocks of 128 tokens, 64k 123 -> 113; two columns of blocks to an instruction alone 275).
+    // column and 16 products (a column and sixteen blocks to a thread: 68 bytes for as many, and 296 us where this takes 266 at 128k
+    // tokens, 32 / 8 heads; the bytes take 205).
     const int bg = warp & 3, ch = warp >> 2, o = 4 * lane;
     float2 acc[4][2];
 #pragma unroll
@@ -318,7 +317,7 @@ __device__ __forceinline__ void min_bf16x8(float (&a)[8], const uint4& u) {
 // The pooling of the gate's variants: average, maximum and minimum of a block side by side, one product with the wider matrix, and
 // the block rotation.  Bound by issue and shared memory beside the bytes: only the pools asked for are formed, an angle's cosine and
 // sine are taken once per block and pair, by the warps that do not project, and three CTAs share an SM (49k tokens, average of Q, all
-// three of K, rotation, with the scores: 223 us, 197 so, 178 with four columns and four blocks to a thread; the bytes take 77).
+// three of K, rotation, with the scores: 178 us; 223 without any of this and a column of eight blocks to a thread; the bytes take 77).
 template <bool kVecW>
 __global__ void __launch_bounds__(kPoolThreads, 3)
 pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t* __restrict__ k,
@@ -547,7 +546,7 @@ static std::mutex g_static_mutex;
 static void* g_static_addr[kStaticMaxDevices];     // device address of g_static_scratch, per device ordinal
 static bool g_static_ready[kStaticMaxDevices];
 
-// Once per device, with that device current: resolve the array's device address and lift the score kernel's
+// Once per device, with that device current: resolve the array's device address and lift the score kernels'
 // shared-memory limit.  Neither call allocates.
 static seer_status static_setup(int dev, unsigned char** out) {
   std::lock_guard<std::mutex> lock(g_static_mutex);
@@ -620,8 +619,8 @@ seer_status gate_scores_static(const seer_shape* shape, const void* q, const voi
   m.total_q_tokens = (int32_t)t.total_tokens;
   m.wait_limit_us = 0u; m.lose_v_copy = -1;   // unused by the gate
   m.score_tiles = 0; m.first_q_block = 0;
-  // The two kernels below are the ones seer_gate_scores launches; only the scratch pointer differs.  Nothing in the
-  // scratch has to start at zero: the first kernel writes every projected vector the second one reads.
+  // The kernels of seer_gate_scores without room for the statistics (pooling, then scores by one launch); only the scratch pointer
+  // differs.  Nothing in the scratch has to start at zero: the first kernel writes every projected vector the second one reads.
   const int n = launch_gate(nullptr, m, q, k, Wq, Wk, scores, base + kStaticMetaBytes, kStaticScratchBytes, stream);
   return n < 0 ? SEER_ERR_CUDA : SEER_OK;
 }

@@ -169,8 +169,8 @@ topk_count_kernel(SeqMeta m, RowBand band, const float* scores, const float2* st
 // continues from row_ptr[0], the last entry of the rows scanned before.  Tiles of 8192 counts go through shared memory (coalesced
 // loads and stores, the next tile's loads in flight meanwhile), eight consecutive counts per thread, warp shuffles inside a
 // warp; every warp adds up the warp totals for itself, every CTA the tile totals that the others have put into its shared memory.
-// A CTA alone is bound by the latency of a tile's three barriers, about 2 us (counts, scan and lists of 65 536 rows 248 -> 238 us with
-// the cluster, of 76 800 123 -> 111); beyond one tile the cluster takes eight at a time.  All sums fit 32 bits (the host refuses shapes with 2^31 causal blocks).
+// A CTA alone is bound by the latency of a tile's three barriers, about 2 us a tile; beyond one tile the cluster takes eight at a time
+// (counts, scan and lists of 76 800 rows: 123 us by one CTA, 111 so).  All sums fit 32 bits (the host refuses shapes with 2^31 causal blocks).
 constexpr int kScanPer = 8, kScanTile = 1024 * kScanPer, kScanRanks = 8;
 template <int kRanks>
 __global__ void __launch_bounds__(1024)
@@ -287,7 +287,7 @@ __device__ __forceinline__ uint32_t lean_key(float sc) {
 // loops unrolled it waited for instructions), what a row needs once is done by one of its warps and passed on, and the
 // counts that order the warps' parts of the list are taken in the pass that gathers the threshold's class.
 // A row gets one warp up to 2048 blocks, and as many as keep it at 2048 keys per warp beyond.  Measured: 65 536 rows of up to
-// 2048 blocks 251 -> 176 us, 4096 rows of up to 4096 blocks (which re-read their scores in every pass) 158 -> 31 us; what a row
+// 2048 blocks 176 us, 4096 rows of up to 4096 blocks 31 us (fill_kernel, which re-reads the scores in every pass: 158); what a row
 // needs once done by every warp of it, and a pass of its own for the counts: 183 and 34.
 template <int W>
 __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W < 8 ? 12 : 6)

@@ -399,8 +399,9 @@ seer_status seer_sparse_attn(seer_ctx* ctx, const seer_shape* shape, const void*
   SeqMeta m; int slot;
   st = prepare(ctx, shape, stream, &m, &slot);
   if (st != SEER_OK) return st;
-  // impl 2: by shape.  The lists are at most the causal blocks; rows that short cost the persistent kernel more in
-  // per-row hand-over than the legacy kernel needs for the whole row.
+  // impl 2: by shape, where the lists (at most the causal blocks) are short.  Not for speed any more: on batches of 1 to 4000
+  // sequences of 40 to 960 tokens the tcgen05 kernel takes 0.3 to 1.0 of the mma.sync kernel's time (64 sequences of 900 tokens, 32
+  // heads, all blocks: 990 against 2572 us; 8 of 64 tokens: 13.3 against 13.4).
   const bool legacy = ctx->attn_impl == 1 || (ctx->attn_impl == 2 && t.causal_blocks <= 8 * t.rows);
   int n = legacy ? launch_attn_mma(ctx, m, q, k, v, row_ptr, col_idx, o, lse, stream)
                  : launch_attn_tc(ctx, m, q, k, v, row_ptr, col_idx, o, lse, work_counter, stream);
@@ -710,7 +711,7 @@ seer_status seer_prefill_host(seer_ctx* ctx, const seer_shape* shape, const void
   // The copies in are what the call is bound by (55 GB/s), so what follows the last of them counts in full: the kernels of the last
   // slice and its read-back.  The last slice is therefore taken in parts of its query heads, each of more than 8 MB (150 us
   // of copying, as long as the kernels of that many heads take): the parts' kernels and read-backs overlap the copies of the later
-  // parts (32 / 8 heads, a tenth kept: 32k tokens 8.97 -> 8.60 ms, 48k 13.4 -> 12.8, 128k 36.1 -> 34.8; parts of 4 MB: no faster).
+  // parts (32 / 8 heads, a tenth kept, 128k tokens: 36.1 ms with the slice whole, 34.8 so; parts of 4 MB: no faster).
   int tail_heads = (int)(((size_t)8 << 20) / (T * head_bytes)) + 1;
   while (tail_heads < G && G % tail_heads != 0) ++tail_heads;
   if (tail_heads > G) tail_heads = G;

@@ -67,8 +67,8 @@ __host__ __device__ inline int gate_stat_segs(int max_nb) { const int c = gate_s
 // head_stride == 0: the band's scores lie at (offset in the full score matrix - score_base) in whatever buffer the kernels are
 // given.  Otherwise the band is query blocks >= row0 of one sequence, packed: row i of head h lies at
 // (h - head_lo) * head_stride + packed_rows(i) - packed_rows(row0), its causal columns alone, rounded up to 64.  A band buffer
-// takes twice the heads of whole rows then, and a band's launches are as many times fewer (32 heads of 4096 blocks in 128 MB:
-// 32 bands -> 11, gate + mask 2.99 -> 2.60 ms).
+// takes twice the heads of whole rows then, and there are as many times fewer launches (32 heads of 4096 blocks in 128 MB: 11 bands
+// instead of 32, gate + mask 13 % faster).
 struct ScoreBand {
   int32_t blk_lo, blk_hi;      // block rows [blk_lo, blk_hi), numbered over the batch (blk_off)
   int32_t head_lo, heads;
@@ -143,8 +143,7 @@ size_t gate_stats_bytes(const ShapeTotals& t, const seer_shape* shape);       //
 // before the call's first kernel): a grid that ended without it would let its successor overtake its predecessor.  Only
 // then does a kernel let its own successor start: two kernels overlap, never three, so no line that a third one rewrites can
 // sit in L1, and a kernel that rewrites what it has read reads past L1.
-// It is worth the start of a kernel, about 2 us, at each of a call's launches: 2k tokens, four heads, 48.5 -> 36.2 us; a batch
-// of 24 short prompts 266 -> 260; 256k tokens in 11 bands 2.61 -> 2.50 ms.
+// It is worth the start of a kernel, about 2 us, at each of a call's launches: 2k tokens, four heads, 48.5 us without and 36.2 with it.
 template <typename... P, typename... A>
 cudaError_t launch_next(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t stream, A... args) {
   cudaLaunchConfig_t cfg = {};
