@@ -93,9 +93,15 @@ __device__ __forceinline__ bool mbar_test(uint32_t addr, uint32_t parity) {
 // 2^x for two values at once on the FMA pipe (the special-function unit does 16 exponentials per clock and SM): x = n + f
 // with n = round(x), 2^f by a cubic (relative error 7.5e-5, far below the bf16 rounding of P), 2^n by adding n to the
 // exponent field.  x is clamped to [-125, 128] so that the exponent field stays in 1..255: below gives ~2^-125, above
-// something no smaller than 2^127 or a NaN, which the caller's test of the sum sees.
+// something no smaller than 2^127, which the caller's test of the sum sees; so does a NaN, which the clamp lets through.
+__device__ __forceinline__ float clamp_nan(float x) {
+  float y;
+  asm("max.NaN.f32 %0, %1, 0fC2FA0000;" : "=f"(y) : "f"(x));   // -125
+  asm("min.NaN.f32 %0, %1, 0f43000000;" : "=f"(x) : "f"(y));   // 128
+  return x;
+}
 __device__ __forceinline__ float2 exp2_poly2(float2 x) {
-  x.x = fminf(fmaxf(x.x, -125.f), 128.f); x.y = fminf(fmaxf(x.y, -125.f), 128.f);
+  x.x = clamp_nan(x.x); x.y = clamp_nan(x.y);
   const float2 magic = make_float2(12582912.f, 12582912.f);        // 1.5 * 2^23: the sum's low mantissa bits are round(x)
   const float2 t = __fadd2_rn(x, magic);
   const float2 n = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
@@ -587,6 +593,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
               }
             }
             sum = diag ? row_pass<true>(s_addr, sl2, R, row, pk) : row_pass<false>(s_addr, sl2, R, row, pk);
+            if (!(sum < kRise)) sum = CUDART_NAN_F;         // an infinite score or a NaN: so is the row
             tr.ev(40);
           }
           l = __fadd_rn(l, sum);

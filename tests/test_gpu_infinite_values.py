@@ -1,5 +1,6 @@
 """Values and gate logits past the range of their type stay where they belong: an infinite value reaches the columns of the rows
-that attend to it and no others, and a logit of -inf is a probability of zero."""
+that attend to it and no others, a key that is not finite makes NaN of the rows that attend to it, and a gate logit of -inf is a
+probability of zero."""
 import math
 
 import numpy as np
@@ -45,6 +46,47 @@ def test_infinite_values(lengths, chunk):
     off = ~np.isfinite(want)
     assert np.array_equal(got[off], want[off]) and np.isfinite(got[~off]).all()
     assert np.all(np.abs(got[~off] - want[~off]) <= 2e-2 + 1e-2 * np.abs(want[~off]))   # the attention's tolerance
+
+
+# keys of a block by their place: exponentials run on either of two pipes
+@pytest.mark.parametrize("what", [float("nan"), float("inf")])
+def test_keys_that_are_not_finite(what):
+    from paper_2410_13276_b200 import binding as B
+    from paper_2410_13276_b200.prefill import Prefill
+    nb, hq = 70, 2
+    w = W.make_small(seed=221, seqlens=[nb * 64], hq=hq, hkv=1)
+    q, k = w.q.copy(), w.k.copy()
+    q[:, :, 3] = np.where(np.arange(nb * 64) % 5 == 0, 0xbf80, 0x3f80)[:, None]   # -1 or 1: an infinite key scores +inf or -inf
+    for j in range(64):
+        k[j * 64 + j, 0, 3] = 0x7fc0 if np.isnan(what) else 0x7f80              # block j: its key j
+    rows = [[] for _ in range(hq * nb)]
+    r = np.random.default_rng(4)
+    for h in range(hq):
+        for i in range(64, nb):
+            n = (i - 64 + h) % 5 + 1
+            rows[h * nb + i] = sorted(r.choice(64, n, replace=False).tolist()) if i % 2 else [64] * (i > 64) + [65] * (i > 65)
+    rows[64], rows[66] = list(range(64)), [0, 17, 64]
+    rp, col = np.concatenate([[0], np.cumsum([len(x) for x in rows])]).astype(np.int32), np.array([j for x in rows for j in x], np.int32)
+    p = Prefill(w.cu_seqlens, hq, 1)
+    p.set_inputs(q, k, w.v, w.wq, w.wk)
+    p.set_lists(rp, col)
+    p.attn()
+    assert p.status() == 0
+    got = p.o_host().astype(np.float64)
+    clean = np.where((k & 0x7f80) == 0x7f80, 0, k).astype(np.uint16)             # (the key of -inf scores is replaced below)
+    for h in range(hq):
+        for i in range(64, nb):
+            row = rows[h * nb + i]
+            bad = any(j < 64 for j in row)
+            for t in range(i * 64, i * 64 + 64, 7):
+                if bad and (np.isnan(what) or t % 5):
+                    assert np.isnan(got[t, h]).all(), (h, i, t)
+                elif row:
+                    keys = [x for j in row for x in range(j * 64, j * 64 + 64) if not (j < 64 and x == j * 65)]   # 2^(-inf) = 0
+                    s = O.bf16_bits_to_f64(clean[keys, 0]) @ O.bf16_bits_to_f64(q[t, h]) / math.sqrt(128)
+                    e = np.exp(s - s.max())
+                    want = e @ O.bf16_bits_to_f64(w.v[keys, 0]) / e.sum()
+                    assert np.all(np.abs(got[t, h] - want) <= 2e-2 + 1e-2 * np.abs(want)), (h, i, t)   # the attention's tolerance
 
 
 # blocks whose logits lie below the range of fp32, alone among a row's columns of a 32-column group, at the edges of groups, tiles
