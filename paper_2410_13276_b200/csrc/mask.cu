@@ -170,18 +170,19 @@ topk_count_kernel(SeqMeta m, RowBand band, const float* scores, const float2* st
 // loads and stores, the next tile's loads in flight meanwhile), eight consecutive counts per thread, warp shuffles inside a
 // warp; every warp adds up the warp totals for itself, every CTA the tile totals that the others have put into its shared memory.
 // A CTA alone is bound by the latency of a tile's three barriers, about 2 us a tile; beyond one tile the cluster takes eight at a time
-// (counts, scan and lists of 76 800 rows: 123 us by one CTA, 111 so).  All sums fit 32 bits (the host refuses shapes with 2^31 causal blocks).
+// (counts, scan and lists of 76 800 rows: 123 us by one CTA, 111 so).  All sums fit 32 bits, unsigned: the host
+// refuses shapes with 2^31 causal blocks, and lists to be expanded may hold entries past the diagonal, twice as many at most.
 constexpr int kScanPer = 8, kScanTile = 1024 * kScanPer, kScanRanks = 8;
 template <int kRanks>
 __global__ void __launch_bounds__(1024)
 scan_kernel(int64_t rows, int32_t* row_ptr, int first, int64_t col_capacity, int64_t* __restrict__ nnz_out,
             int* __restrict__ status) {
   __shared__ int32_t tile[kScanTile + kScanTile / 32];     // (one word of padding per 32: eight consecutive words per thread)
-  __shared__ int32_t warp_tot[2][32], rank_tot[2][kRanks];
+  __shared__ uint32_t warp_tot[2][32], rank_tot[2][kRanks];
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int rank = kRanks > 1 ? (int)blockIdx.x : 0;       // (the grid is one cluster)
   grid_wait();
-  int carry = first ? 0 : __ldcg(row_ptr);                 // (read past L1: the kernel rewrites it)
+  uint32_t carry = first ? 0u : (uint32_t)__ldcg(row_ptr); // (read past L1: the kernel rewrites it)
   int32_t next[kScanPer];
 #pragma unroll
   for (int k = 0; k < kScanPer; ++k) {
@@ -201,25 +202,25 @@ scan_kernel(int64_t rows, int32_t* row_ptr, int first, int64_t col_capacity, int
       const int64_t idx = base + kRanks * kScanTile + t + k * 1024;
       next[k] = idx < rows ? __ldcg(row_ptr + idx + 1) : 0;
     }
-    int v[kScanPer];
+    uint32_t v[kScanPer];
 #pragma unroll
-    for (int k = 0; k < kScanPer; ++k) { const int idx = kScanPer * t + k; v[k] = tile[idx + (idx >> 5)] + (k > 0 ? v[k - 1] : 0); }
-    int incl = v[kScanPer - 1];
+    for (int k = 0; k < kScanPer; ++k) { const int idx = kScanPer * t + k; v[k] = (uint32_t)tile[idx + (idx >> 5)] + (k > 0 ? v[k - 1] : 0u); }
+    uint32_t incl = v[kScanPer - 1];
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-      const int o = __shfl_up_sync(0xffffffffu, incl, off);
+      const uint32_t o = __shfl_up_sync(0xffffffffu, incl, off);
       if (lane >= off) incl += o;
     }
     if (lane == 31) warp_tot[par][warp] = incl;
     __syncthreads();
-    int w = warp_tot[par][lane];
+    uint32_t w = warp_tot[par][lane];
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-      const int o = __shfl_up_sync(0xffffffffu, w, off);
+      const uint32_t o = __shfl_up_sync(0xffffffffu, w, off);
       if (lane >= off) w += o;
     }
-    const int before_warp = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
-    int total = __shfl_sync(0xffffffffu, w, 31);
+    const uint32_t before_warp = __shfl_sync(0xffffffffu, w, (warp + 31) & 31);
+    uint32_t total = __shfl_sync(0xffffffffu, w, 31);
     if (kRanks > 1) {
       if (t < kRanks) {                                    // this CTA's total to CTA t
         const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&rank_tot[par][rank]);
@@ -231,13 +232,13 @@ scan_kernel(int64_t rows, int32_t* row_ptr, int first, int64_t col_capacity, int
       total = 0;
 #pragma unroll
       for (int q = 0; q < kRanks; ++q) {
-        const int x = rank_tot[par][q];
+        const uint32_t x = rank_tot[par][q];
         if (q < rank) carry += x; else total += x;         // (carry: counts before this CTA's tile)
       }
     }
-    const int before = carry + (warp > 0 ? before_warp : 0) + (incl - v[kScanPer - 1]);
+    const uint32_t before = carry + (warp > 0 ? before_warp : 0u) + (incl - v[kScanPer - 1]);
 #pragma unroll
-    for (int k = 0; k < kScanPer; ++k) { const int idx = kScanPer * t + k; tile[idx + (idx >> 5)] = before + v[k]; }
+    for (int k = 0; k < kScanPer; ++k) { const int idx = kScanPer * t + k; tile[idx + (idx >> 5)] = (int32_t)(before + v[k]); }
     carry += total;
     __syncthreads();
 #pragma unroll
@@ -249,8 +250,8 @@ scan_kernel(int64_t rows, int32_t* row_ptr, int first, int64_t col_capacity, int
   }
   if (t == 0 && rank == 0) {
     if (first) row_ptr[0] = 0;
-    if (nnz_out) *nnz_out = carry;
-    if (carry > col_capacity) atomicCAS(status, 0, (int)SEER_ERR_CAPACITY);
+    if (nnz_out) *nnz_out = (int64_t)carry;
+    if ((int64_t)carry > col_capacity) atomicCAS(status, 0, (int)SEER_ERR_CAPACITY);
   }
 }
 
@@ -790,10 +791,10 @@ expand_kernel(SeqMeta m128, SeqMeta m64, const int32_t* row_ptr128, const int32_
   const bool odd = (i64 & 1) != 0;
   const int64_t src = (int64_t)m128.num_q_heads * m128.blk_off[b] + (int64_t)h * nb128 + i128;
   const int32_t s0 = row_ptr128[src], s1 = row_ptr128[src + 1];
-  int32_t out0 = 0;
+  uint32_t out0 = 0;
   if (kFill) {
-    out0 = row_ptr64[r];
-    if ((int64_t)row_ptr64[r + 1] > col_capacity64) return;    // does not fit; status already raised by the scan
+    out0 = (uint32_t)row_ptr64[r];
+    if ((int64_t)(uint32_t)row_ptr64[r + 1] > col_capacity64) return;    // does not fit; status already raised by the scan
   }
   int written = 0;
   for (int base = s0; base < s1; base += 32) {
@@ -807,7 +808,7 @@ expand_kernel(SeqMeta m128, SeqMeta m64, const int32_t* row_ptr128, const int32_
       if (lane >= o) incl += v;
     }
     if (kFill && c > 0) {
-      int32_t* dst = col_idx64 + out0 + written + incl - c;
+      int32_t* dst = col_idx64 + (size_t)out0 + written + incl - c;
       dst[0] = 2 * j;
       if (c == 2) dst[1] = 2 * j + 1;
     }

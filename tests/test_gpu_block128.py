@@ -121,3 +121,30 @@ def test_block128_unsupported_calls_and_capacity(rt):
     B.seer_expand_block_lists(ctx, p.shape, p.row_ptr, p.col_idx, p.row_ptr64, small, 100, p.nnz64)
     assert p.status() == 4                                 # SEER_ERR_CAPACITY
     assert int(p.nnz64.item()) == 2 * 136
+
+
+def test_expanded_lists_of_more_than_2_31_entries(rt):
+    """Full lists with the entries past the diagonal: the count stays right and what does not fit is not written."""
+    import torch
+    B, _, ctx = rt
+    nb, hq, cap = 4100, 32, 100_000
+    shape = B.make_shape(np.array([0, nb * 128], np.int32), hq, 1, block=128)
+    col = torch.arange(nb, dtype=torch.int32, device="cuda").repeat(hq * nb)
+    rp = torch.arange(hq * nb + 1, dtype=torch.int32, device="cuda") * nb
+    rp64 = torch.zeros(2 * hq * nb + 1, dtype=torch.int32, device="cuda")
+    col64 = torch.full((cap + 4096,), -9, dtype=torch.int32, device="cuda")
+    nnz = torch.zeros(1, dtype=torch.int64, device="cuda")
+    B.seer_expand_block_lists(ctx, shape, rp, col, rp64, col64, cap, nnz)
+    assert B.seer_poll_device_status(ctx) == 4
+    lengths = np.full(2 * hq * nb, 2 * nb, np.int64)
+    lengths[::2] -= 1                                       # the first half of a block does not see the second
+    ends = np.cumsum(lengths)
+    assert int(nnz.item()) == ends[-1] and ends[-1] > 1 << 31
+    assert np.array_equal(rp64.cpu().numpy()[1:].view(np.uint32), ends.astype(np.uint32))
+    fit = int(np.searchsorted(ends, cap, side="right"))
+    got, at = col64.cpu().numpy(), 0
+    for r in range(fit):
+        want = [j for j in range(2 * nb) if r % 2 or j != r + 1]
+        assert got[at:at + len(want)].tolist() == want
+        at += len(want)
+    assert (got[at:] == -9).all()
