@@ -3,7 +3,10 @@
 // What bounds it.  Long lists: the copies of K and V into shared memory (64 KB per pair of listed 64 x 64 blocks, about 885 clocks
 // at the 74 bytes a clock that an SM takes from L2, of 917 to 1060 that a pair takes), close before the MMA pipe (8 x 48 + 4 x 76 =
 // 688 clocks: 75 % active on dense lists of 16k tokens), and in launches of more than a few milliseconds the board's power limit.
-// Short lists: an item's start and end, about 6000 clocks beside 2000 for a stream's tile (13 tiles an item: the pipe 61 % active).
+// Short lists: an item's start and end, about 4800 clocks beside 2000 for a stream's tile.  Of them the wait for the last P V 1300, merge and
+// stores 2700; everything that needs no O is done during the wait, and an item's row pointers and first list entries are fetched
+// while the item before it is copied.  With those after the wait, the entries fetched at the item's start, and producers that slept between
+// their polls: 6000 clocks; 24 prompts of 16 900 tokens 173 us where this takes 163, 32k tokens 1384 and 1335, 128k 16.7 and 16.1 ms.
 //
 // Tiles.  A query block is 64 rows and every (head, query block) has its own list, so no two items share their keys.
 // The MMAs are the weight-stationary form (tcgen05.mma.ws) with M = 64: the 128 lanes of tensor memory hold two 64-row
@@ -48,9 +51,11 @@ constexpr float kNoRef = -1e30f;   // reference of a row that has not seen a liv
 // A tile whose row sum reaches this moves the row's reference: 2^60 above the first block's maximum, far from the 2^127 at
 // which P or the sums would overflow, and far above what a prompt's sink or stripes rise (a move costs about two tiles).
 constexpr float kRise = 1.152921504606847e18f;   // 2^60
-constexpr int kHelperRegs = 56, kSoftmaxRegs = 200;   // (2 * 56 + 2 * 200) * 128 = 65536
+// Registers of the helpers' and the softmax warpgroups, two each: 2 * (helper + softmax) * 128 = 65536.  (The softmax pass wants 200; the
+// block maxima want less, and their producer spills with 56.)
+template <bool kBlockMax> constexpr int kHelperRegs = kBlockMax ? 64 : 56;
+template <bool kBlockMax> constexpr int kSoftmaxRegs = 256 - kHelperRegs<kBlockMax>;
 constexpr int kGroupThreads = 128;
-constexpr int kProducerSleepNs = 32;   // a producer that polls a barrier shares its scheduler with two softmax warps
 // of every eight pairs of a pass this many take their exponentials on the FMA pipe (0, 1 and 3 measured within 2 % of it)
 constexpr int kPolyPairsOf8 = 2;
 constexpr uint32_t kHalfQ = 64 * 128;            // bytes of one d half of a 64-row tile (8 KB)
@@ -188,12 +193,14 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bo
 // What the roles need to know of a work item (decoded once, by the stream's Q / K producer).
 struct Slot {
   int h, i, l0, nlist, q_valid, s0, tok0;   // tok0: first row of the item in q / o / lse
+  int first[2];                             // the list's first two entries
   __device__ __forceinline__ int ntiles() const { return (nlist + 1) >> 1; }
 };
 __device__ __forceinline__ int slot_block(const Slot& it, const int32_t* col_idx, int p) {
   return p < it.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + it.l0 + p) : -1;
 }
 // Block index of a list entry: -1 past the end of the list, -2 outside [0, i].
+__device__ __forceinline__ int list_entry(const Item& it, int p, int raw) { return p >= it.nlist ? -1 : (raw < 0 || raw > it.i) ? -2 : raw; }
 __device__ __forceinline__ int slot_check(const Slot& it, int p, int raw) {
   if (p >= it.nlist) return -1;
   return (raw < 0 || raw > it.i) ? -2 : raw;
@@ -265,15 +272,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   auto read_slot = [&](int s, uint32_t n) -> Slot {
     const uint4 a = ld_shared_v4(ring_addr(s, n)), b = ld_shared_v4(ring_addr(s, n) + 16u);
     Slot it;
-    it.h = (int)a.x; it.i = (int)a.y; it.l0 = (int)a.z; it.nlist = (int)a.w;
-    it.q_valid = (int)b.x; it.s0 = (int)b.y; it.tok0 = (int)b.z;
+    it.h = (int)a.x; it.i = (int)(a.y >> 7); it.q_valid = (int)(a.y & 127u);   // (a batch has at most 2^25 blocks)
+    it.l0 = (int)a.z; it.nlist = (int)a.w;
+    it.s0 = (int)b.x; it.tok0 = (int)b.y; it.first[0] = (int)b.z; it.first[1] = (int)b.w;
     return it;
   };
   auto item_full = [&](int s, uint32_t n) -> int { return s * kBarsPerStream + ITEM_FULL + (int)(n & 3u); };
   auto release_item = [&](int s, uint32_t n) { mbar_arrive(sh.bar(s * kBarsPerStream + ITEM_EMPTY + (int)(n & 3u))); };
 
   if (warp < 4 || warp >= 12) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kHelperRegs));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kHelperRegs<kBlockMax>));
     // ========================================================================================== producer of Q and K (TMA)
     if (warp == 0 || warp == 2) {
       if (elect_one()) {
@@ -290,28 +298,42 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         };
         uint32_t nitem = 0, cnt = 0, ku = 0, kph = 0;
         bool ok = true;
-        int64_t w = draw();
-        for (uint32_t n = 0; ok; ++n) {
-          const bool more = w < m.q_rows;
-          Item it{};
-          if (more) it = decode_item<kChunk>(m, row_ptr, w);
+        // An item is decoded and announced while the one before it is copied: its row pointers and its first list entries are two
+        // trips to L2, one after the other, that every role of the stream would wait for at the item's start.
+        Item it{}, nx{};
+        int na0 = -1, nb0 = -1;                            // first entries of the next list
+        bool more = false;
+        auto locate = [&](int64_t w) {                     // which item comes next
+          more = w < m.q_rows;
+          nx = Item{};
+          if (more) nx = decode_item<kChunk>(m, row_ptr, w);
+        };
+        auto announce = [&](uint32_t n) -> bool {
+          na0 = 0 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0) : -1;
+          nb0 = 1 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0 + 1) : -1;
           // the slot's previous content (item n - 4) has been read by everyone
-          if (!mbar_wait<kProducerSleepNs>(sh, bb + ITEM_EMPTY + (int)(n & 3u), ((n >> 2) & 1u) ^ 1u, status)) break;
-          const int tok0 = it.s0 + it.i * kBlock + (kChunk ? it.dq : 0);
-          st_shared_v4(ring_addr(s, n), (uint32_t)it.h, (uint32_t)it.i, (uint32_t)it.l0, more ? (uint32_t)it.nlist : 0xffffffffu);
-          st_shared_v4(ring_addr(s, n) + 16u, (uint32_t)it.q_valid, (uint32_t)it.s0, (uint32_t)tok0, 0u);
+          if (!mbar_wait(sh, bb + ITEM_EMPTY + (int)(n & 3u), ((n >> 2) & 1u) ^ 1u, status)) return false;
+          const int tok0 = nx.s0 + nx.i * kBlock + (kChunk ? nx.dq : 0);
+          st_shared_v4(ring_addr(s, n), (uint32_t)nx.h, (uint32_t)nx.i << 7 | (uint32_t)nx.q_valid, (uint32_t)nx.l0, more ? (uint32_t)nx.nlist : 0xffffffffu);
+          st_shared_v4(ring_addr(s, n) + 16u, (uint32_t)nx.s0, (uint32_t)tok0, (uint32_t)na0, (uint32_t)nb0);
           mbar_arrive(sh.bar(item_full(s, n)));
-          if (!more) break;
-          w = draw();                                      // the next one is on its way while this one is copied
-          if (it.ntiles == 0) continue;
-          int ja = list_block(it, col_idx, 0), jb = list_block(it, col_idx, 1);
+          return true;
+        };
+        locate(draw());
+        ok = announce(0);
+        for (uint32_t n = 0; ok && more; ++n) {
+          it = nx;
+          int ja = list_entry(it, 0, na0), jb = list_entry(it, 1, nb0);
+          const int64_t w = draw();                        // the next one is on its way while this one is copied
+          if (it.ntiles == 0) { locate(w); ok = announce(n + 1); continue; }
+          const int tok0 = it.s0 + it.i * kBlock + (kChunk ? it.dq : 0);
           const uint32_t qb = nitem & 1u;
-          if (!mbar_wait<kProducerSleepNs>(sh, bb + Q_EMPTY + (int)qb, ((nitem >> 1) & 1u) ^ 1u, status)) break;
+          if (!mbar_wait(sh, bb + Q_EMPTY + (int)qb, ((nitem >> 1) & 1u) ^ 1u, status)) break;
           mbar_expect_tx(sh.bar(bb + Q_FULL + (int)qb), kQBytes);
           tma_load_3d(sbase + kStQ + qb * kQBytes, &map_q, sh.bar(bb + Q_FULL + (int)qb), 0, it.h, tok0);
           tma_load_3d(sbase + kStQ + qb * kQBytes + kHalfQ, &map_q, sh.bar(bb + Q_FULL + (int)qb), 64, it.h, tok0);
           ++nitem;
-          for (int t = 0; t < it.ntiles && ok; ++t, ++cnt) {
+          for (int t = 0; t < it.ntiles; ++t, ++cnt) {
             const int na = list_block(it, col_idx, 2 * t + 2), nb2 = list_block(it, col_idx, 2 * t + 3);   // next pair
             if (ja == -2 || jb == -2) atomicCAS(status, 0, (int)SEER_ERR_INVALID_INDEX);
             const bool has_b = jb != -1;
@@ -320,7 +342,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             tr.sample(cnt); tr.ev(1);
 #pragma unroll
             for (int dh = 0; dh < 2; ++dh) {
-              if (!mbar_wait<kProducerSleepNs>(sh, bb + empty_k + (int)ku, kph ^ 1u, status)) { ok = false; break; }
+              if (!mbar_wait(sh, bb + empty_k + (int)ku, kph ^ 1u, status)) { ok = false; break; }
               const uint32_t fb = sh.bar(bb + K_FULL + (int)ku), dst = sbase + kStK + ku * kUnit;
               mbar_expect_tx(fb, has_b ? kUnit : kUnit / 2);   // (an odd list's last tile: the scores of the missing block are not looked at)
               tma_load_3d(dst, &map_k, fb, 64 * dh, it.g, ta);
@@ -328,7 +350,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
               if (++ku == ring_k) { ku = 0; kph ^= 1u; }
             }
             tr.ev(2);
+            if (!ok) break;
             ja = na; jb = nb2;
+            if (t == 0) locate(w);
+            if (t == min(1, it.ntiles - 1) && !announce(n + 1)) { ok = false; break; }
           }
         }
       }
@@ -342,12 +367,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         uint32_t cnt = 0, vu = 0, vph = 0;
         bool ok = true;
         for (uint32_t n = 0; ok; ++n) {
-          if (!mbar_wait<kProducerSleepNs>(sh, item_full(s, n), (n >> 2) & 1u, status)) break;
+          if (!mbar_wait(sh, item_full(s, n), (n >> 2) & 1u, status)) break;
           const Slot it = read_slot(s, n);
           release_item(s, n);
           if (it.nlist < 0) break;
           const int g = it.h / m.group;
-          int ja = slot_check(it, 0, slot_block(it, col_idx, 0)), jb = slot_check(it, 1, slot_block(it, col_idx, 1));
+          int ja = slot_check(it, 0, it.first[0]), jb = slot_check(it, 1, it.first[1]);
           for (int t = 0; t < it.ntiles() && ok; ++t, ++cnt) {
             const int ra = slot_block(it, col_idx, 2 * t + 2), rb = slot_block(it, col_idx, 2 * t + 3);   // next pair
             const int ta = it.s0 + (ja < 0 ? 0 : ja) * kBlock;
@@ -361,7 +386,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             const bool lost = s == 0 && blockIdx.x == 0 && m.lose_v_copy >= 0 && cnt == (uint32_t)m.lose_v_copy;
 #pragma unroll
             for (int kh = 0; kh < 2; ++kh) {
-              if (!mbar_wait<kProducerSleepNs>(sh, bb + V_EMPTY + (int)vu, vph ^ 1u, status)) { ok = false; break; }
+              if (!mbar_wait(sh, bb + V_EMPTY + (int)vu, vph ^ 1u, status)) { ok = false; break; }
               const uint32_t fb = sh.bar(bb + V_FULL + (int)vu), dst = sbase + kStV + vu * kUnit;
               if (!lost) {
                 mbar_expect_tx(fb, two ? kUnit : kUnit / 2);
@@ -467,7 +492,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   }   // helper warpgroups
   // ============================================================================================ softmax groups
   else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs));
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSoftmaxRegs<kBlockMax>));
     const int s = (warp - 4) >> 2, bb = s * kBarsPerStream;
     const int quad = warp & 3;                              // TMEM lane quadrant this warp may access
     const int half = quad >> 1;                             // which of a tile's two blocks this warp works on
@@ -505,7 +530,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         }
         continue;
       }
-      int raw = slot_block(it, col_idx, half);
+      int raw = half ? it.first[1] : it.first[0];
       tr.ev(36);
       if constexpr (kBlockMax) {
         int* wmax = reinterpret_cast<int*>(smem + kOffMl + s * kMlBytes);   // [2 tile parities][4 warps]: maxima as order-preserving integers
@@ -609,45 +634,60 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
       if constexpr (!kBlockMax) {
         // ---------------------------------------------------------------------------------------- epilogue: merge, store
         tr.sample(0); tr.ev(36);
-        if (!fail) fail = !mbar_wait(sh, bb + PV_DONE + (int)((cnt - 1) & 1u), ((cnt - 1) >> 1) & 1u, status);   // the last P V of the item
-        tc_fence_after();
-        tr.ev(37);
         const bool two = it.nlist > 1;                      // the second half has something to contribute
         if (two) st_shared_v2(ml + (uint32_t)r * 8u, __float_as_uint(R), __float_as_uint(l));
         if (named_bar_or(bar_vote, kGroupThreads, fail)) break;
         uint16_t* orow = o + (((int64_t)it.tok0 + row) * m.num_q_heads + it.h) * kHeadDim;
-        const bool store = row < it.q_valid;
         const uint32_t qbuf = nitem & 1u;
+        float sc, lse_row;
         if (two) {
-          // out = (2^(R_a - R) O_a + 2^(R_b - R) O_b) / l, R = max(R_a, R_b).  The thread of lane r ends with d columns
-          // 64 * half ..: it hands the other 64 of its partial row to lane r ^ 64 through the item's Q buffer (Q has been
-          // read: the last S is done), 32 columns at a time, 16-byte chunks XOR (row % 8)
+          // out = (2^(R_a - R) O_a + 2^(R_b - R) O_b) / l, R = max(R_a, R_b)
           const float Ro = ld_shared_f32(ml + (uint32_t)(r ^ 64) * 8u), lo = ld_shared_f32(ml + (uint32_t)(r ^ 64) * 8u + 4u);
           const float Rm = fmaxf(R, Ro);
           const float f = l == 0.f ? 0.f : ex2f(R - Rm), fo = lo == 0.f ? 0.f : ex2f(Ro - Rm);
           const float la = __fmul_rn(l, f), lb = __fmul_rn(lo, fo), total = __fadd_rn(la, lb);   // (the same in both threads)
-          const float sc = total > 0.f ? f / total : 0.f;
-          if (half == 0 && lse != nullptr && store)
-            lse[(int64_t)it.h * lse_stride + it.tok0 + row] = total > 0.f ? (Rm + log2f(total)) * 0.6931471805599453f : -CUDART_INF_F;
+          sc = total > 0.f ? f / total : 0.f;
+          lse_row = total > 0.f ? (Rm + log2f(total)) * 0.6931471805599453f : -CUDART_INF_F;
+        } else {
+          sc = l > 0.f ? 1.f / l : 0.f;
+          lse_row = l > 0.f ? (R + log2f(l)) * 0.6931471805599453f : -CUDART_INF_F;
+        }
+        // The last P V of the item.  A warp whose wait for it is lost keeps the group's barriers, stores nothing and leaves afterwards.
+        fail = !mbar_wait(sh, bb + PV_DONE + (int)((cnt - 1) & 1u), ((cnt - 1) >> 1) & 1u, status);
+        fail = __any_sync(0xffffffffu, fail);
+        const bool store = row < it.q_valid && !fail;
+        tc_fence_after();
+        tr.ev(37);
+        if (half == 0 && lse != nullptr && store) lse[(int64_t)it.h * lse_stride + it.tok0 + row] = lse_row;
+        if (two) {
+          // The thread of lane r ends with d columns 64 * half ..: it hands the other 64 of its partial row to lane r ^ 64 through the
+          // item's Q buffer (Q has been read: the last S is done), 32 columns at a time, 16-byte chunks XOR (row % 8)
           uint32_t mine[2][32], other[2][32];
-          tc_ld32(o_addr + half * 64, mine[0]); tc_ld32(o_addr + half * 64 + 32, mine[1]);
-          tc_ld32(o_addr + (half ^ 1) * 64, other[0]); tc_ld32(o_addr + (half ^ 1) * 64 + 32, other[1]);
-          tc_wait_ld32(mine[0]); tc_wait_ld32(mine[1]); tc_wait_ld32(other[0]); tc_wait_ld32(other[1]);
+          tc_ld32(o_addr + (half ^ 1) * 64, other[0]);
+          tc_wait_ld32(other[0]);
+          tc_ld32(o_addr + half * 64, mine[0]);
+          tc_ld32(o_addr + (half ^ 1) * 64 + 32, other[1]); tc_ld32(o_addr + half * 64 + 32, mine[1]);
           const uint32_t buf = sh.base + (uint32_t)s * kStreamBytes + kStQ + qbuf * kQBytes;
           const uint32_t wr = buf + (uint32_t)r * 128u, rd = buf + (uint32_t)(r ^ 64) * 128u;
+          const float2 sc2 = make_float2(sc, sc);
 #pragma unroll
           for (int i = 0; i < 2; ++i) {
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-              st_shared_v4(wr + (uint32_t)((c ^ (r & 7)) << 4), __float_as_uint(__uint_as_float(other[i][4 * c]) * sc), __float_as_uint(__uint_as_float(other[i][4 * c + 1]) * sc),
-                           __float_as_uint(__uint_as_float(other[i][4 * c + 2]) * sc), __float_as_uint(__uint_as_float(other[i][4 * c + 3]) * sc));
+            for (int c = 0; c < 8; ++c) {
+              const float2 x = __fmul2_rn(make_float2(__uint_as_float(other[i][4 * c]), __uint_as_float(other[i][4 * c + 1])), sc2);
+              const float2 y = __fmul2_rn(make_float2(__uint_as_float(other[i][4 * c + 2]), __uint_as_float(other[i][4 * c + 3])), sc2);
+              st_shared_v4(wr + (uint32_t)((c ^ (r & 7)) << 4), __float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(y.x), __float_as_uint(y.y));
+            }
+            if (i == 0) { tc_wait_ld32(mine[0]); tc_wait_ld32(other[1]); tc_wait_ld32(mine[1]); }
             named_bar_sync(bar_merge, kGroupThreads);
             uint32_t out[16];
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
               const float4 v = ld_shared_f4(rd + (uint32_t)((c ^ (r & 7)) << 4));
-              out[2 * c] = pack_bf16(fmaf(__uint_as_float(mine[i][4 * c]), sc, v.x), fmaf(__uint_as_float(mine[i][4 * c + 1]), sc, v.y));
-              out[2 * c + 1] = pack_bf16(fmaf(__uint_as_float(mine[i][4 * c + 2]), sc, v.z), fmaf(__uint_as_float(mine[i][4 * c + 3]), sc, v.w));
+              const float2 x = __ffma2_rn(make_float2(__uint_as_float(mine[i][4 * c]), __uint_as_float(mine[i][4 * c + 1])), sc2, make_float2(v.x, v.y));
+              const float2 y = __ffma2_rn(make_float2(__uint_as_float(mine[i][4 * c + 2]), __uint_as_float(mine[i][4 * c + 3])), sc2, make_float2(v.z, v.w));
+              out[2 * c] = pack_bf16(x.x, x.y);
+              out[2 * c + 1] = pack_bf16(y.x, y.y);
             }
             if (i == 0) named_bar_sync(bar_merge, kGroupThreads);
             if (store) {
@@ -659,9 +699,6 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           }
           fence_async_smem();                               // before the next Q copy into this buffer
         } else if (half == 0) {
-          const float sc = l > 0.f ? 1.f / l : 0.f;
-          if (lse != nullptr && store)
-            lse[(int64_t)it.h * lse_stride + it.tok0 + row] = l > 0.f ? (R + log2f(l)) * 0.6931471805599453f : -CUDART_INF_F;
 #pragma unroll
           for (int ch = 0; ch < 4; ++ch) {
             uint32_t ov[32];
@@ -683,6 +720,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         if (lane == 0) mbar_arrive(sh.bar(bb + Q_EMPTY + (int)qbuf));
         ++nitem;
         tr.ev(38);
+        if (fail) { named_bar_or(bar_vote, kGroupThreads, true); break; }
       }
     }
   }

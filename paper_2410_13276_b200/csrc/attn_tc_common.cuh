@@ -73,7 +73,6 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 // Bounded wait.  Returns false after the limit (or when another role has already given up); the caller drains.
-template <int kSleepNs = 0>
 __device__ __forceinline__ bool mbar_wait(const Shared& sh, int bar, uint32_t parity, int* status) {
   const uint32_t addr = sh.bar(bar);
   {
@@ -86,7 +85,6 @@ __device__ __forceinline__ bool mbar_wait(const Shared& sh, int bar, uint32_t pa
   const unsigned long long t0 = global_ns();
   for (uint32_t it = 1;; ++it) {
     if (mbar_try(addr, parity)) return true;
-    if (kSleepNs > 0) __nanosleep(kSleepNs);   // a waiting helper must not take issue slots from the softmax warps of its scheduler
     if ((it & 255u) == 0u) {
       if (ld_shared_u32(sh.abort_flag()) != 0u) return false;
       if (global_ns() - t0 > (unsigned long long)sh.limit_us * 1000ull) break;
