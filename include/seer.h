@@ -287,8 +287,9 @@ seer_status seer_gate_scores_ex(seer_ctx* ctx, const seer_shape* shape, const se
  * the L2 cache, so the scores never reach DRAM.
  *
  * Results (row_ptr, col_idx, *nnz_out) are identical, bit for bit, to seer_gate_scores (options == NULL) or
- * seer_gate_scores_ex (options != NULL) followed by seer_block_mask with the same params: the same kernels compute
- * the same scores in the same order.  Arguments, layouts, ownership and errors are those of these calls.
+ * seer_gate_scores_ex (options != NULL) followed by seer_block_mask with the same params: the same scores are formed
+ * in the same order (in the TopK modes, where the scratch has room for the rows' statistics and rows have at most 16384 blocks, by the
+ * selection itself, from a band of logits).  Arguments, layouts, ownership and errors are those of these calls.
  *
  * Workspace: DEVICE memory, 256-byte aligned, seer_gate_mask_workspace_bytes(shape, band_bytes) bytes: the projected
  * vectors (seer_workspace_bytes) followed by the band scratch.  The call uses whatever follows the projected vectors

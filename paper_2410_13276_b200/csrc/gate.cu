@@ -463,6 +463,8 @@ pool_project_ex_kernel(SeqMeta m, const uint16_t* __restrict__ q, const uint16_t
 int launch_gate_stats(const SeqMeta& m, const uint16_t* gq, const uint16_t* gk, float2* stats, int* status, cudaStream_t stream);
 int launch_gate_scores(const SeqMeta& m, const ScoreBand& band, const uint16_t* gq, const uint16_t* gk, float* scores,
                        float2* stats, int* status, int num_sms, cudaStream_t stream);
+int launch_gate_logits(const SeqMeta& m, const ScoreBand& band, const uint16_t* gq, const uint16_t* gk, float* logits, float2* stats,
+                       int* status, int num_sms, cudaStream_t stream);
 bool init_gate_scores();
 
 namespace {
@@ -528,6 +530,11 @@ int launch_gate_scores_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& ba
   const GateWs w(m, ws, SIZE_MAX);
   return launch_gate_scores(m, band, (const uint16_t*)w.gq, (const uint16_t*)w.gk, scores, with_stats ? w.stats : nullptr, ctx->d_status,
                             ctx->num_sms, stream);
+}
+
+int launch_gate_logits_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& band, void* ws, float* logits, cudaStream_t stream) {
+  const GateWs w(m, ws, SIZE_MAX);
+  return launch_gate_logits(m, band, (const uint16_t*)w.gq, (const uint16_t*)w.gk, logits, w.stats, ctx->d_status, ctx->num_sms, stream);
 }
 
 const float2* gate_stats(const SeqMeta& m, void* ws) { return GateWs(m, ws, SIZE_MAX).stats; }

@@ -14,6 +14,10 @@
 //   kBoth   one CTA walks all causal tiles of its rows twice (short sequences: one launch)
 //   kStats  a CTA walks one segment of up to SegTiles tiles and leaves the rows' (maximum, sum) of that segment
 //   kWrite  a CTA walks part_tiles tiles, after combining its rows' statistics, and writes exp(x - m) / l
+// Where the scores are only read again by this library's selection, which can form them itself, one sweep is enough:
+//   kLogits a CTA walks part_tiles tiles, whole segments, and leaves the logits and the segments' statistics
+// (lists of 262 144 tokens, 32 heads: 2.40 ms by statistics of all rows, then scores band by band; 2.11 so; 8k tokens against 128k:
+// 163 and 142 us; 917 against 60k in a batch of four: 90 and 74).
 // With long sequences the first form has few CTAs of very unequal length (one head of a 262 144-token prompt: 32 CTAs, 245 us
 // a launch).  Statistics are always formed per segment of the batch's column grid and combined in segment order, so the
 // scores are the same bit for bit whichever form computes them and however the rows are grouped into calls.
@@ -27,6 +31,8 @@
 // three times slower).
 #include <cuda_bf16.h>
 #include <math_constants.h>
+
+#include <algorithm>
 
 #include "attn_tc_common.cuh"
 #include "seer_internal.cuh"
@@ -43,8 +49,9 @@ constexpr int kThreads = kRowThreads + 96;
 constexpr uint32_t kBPlane = kCols * kGateDim * 2;   // 16 KB: one plane of a column tile, [2 k halves][64 rows][128 B]
 constexpr uint32_t kBBuf = 3 * kBPlane;
 constexpr uint32_t kBBufs = 3;
-constexpr uint32_t kOffStage = kBBufs * kBBuf;       // 16 warps x [32 rows][32 columns] fp32; in the first sweep: (m, l) of the parts
-constexpr uint32_t kOffMeta = kOffStage + 16 * 4096;   // per row: element offset of column 0 (int64), first and last causal block
+constexpr uint32_t kOffStage = kBBufs * kBBuf;       // 16 warps x [32 rows][32 columns] fp32
+constexpr uint32_t kOffSeg = kOffStage + 16 * 4096;    // (m, l) of a segment: [segment parity][group][half][row]
+constexpr uint32_t kOffMeta = kOffSeg + 8 * kRows * 8;   // per row: element offset of column 0 (int64), first and last causal block
 constexpr uint32_t kOffBar = kOffMeta + kRows * 16;
 constexpr uint32_t kOffMisc = kOffBar + 128;         // tmem base, abort flag
 constexpr uint32_t kSmemBytes = kOffMisc + 64;
@@ -54,7 +61,7 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColA = 256;                      // columns 0..255: two accumulator pairs; 256..447: the A planes
 constexpr uint32_t kIdesc = make_idesc(false, false, kCols);
 constexpr uint32_t kWaitSpins = 1u << 24;            // a wait that lasts this many polls (seconds) is declared lost
-enum Mode { kBoth = 0, kStats = 1, kWrite = 2 };
+enum Mode { kBoth = 0, kStats = 1, kWrite = 2, kLogits = 3 };
 
 // Bounded wait that never changes the control flow: after the limit the error is recorded and the wait counts as
 // satisfied, so every role still reaches its barriers and the CTA ends normally (with a wrong result and a status).
@@ -78,17 +85,10 @@ __host__ __device__ __forceinline__ int part_count(const ScoreBand& band, int ti
   return last / (part_tiles * kCols) + 1;
 }
 
-// (m, l) of two disjoint sets of a row's columns, in units of log2: l counts 2^(x - m); m = -inf: empty
-__device__ __forceinline__ void combine(float& m, float& l, float m2, float l2) {
-  const float nm = fmaxf(m, m2);
-  const float f = m == -CUDART_INF_F ? 0.f : ex2f(m - nm), f2 = m2 == -CUDART_INF_F ? 0.f : ex2f(m2 - nm);
-  l = __fadd_rn(__fmul_rn(l, f), __fmul_rn(l2, f2));
-  m = nm;
-}
 }  // namespace gs
 
 // grid.x = row tiles * band.heads (head fastest; row tiles are visited from the last rows to the first), grid.y = parts of
-// part_tiles column tiles (1 for kBoth; for kStats a part is a segment); with one sequence in the batch the parts are in grid.x
+// part_tiles column tiles (part_tiles = 0, always so for kBoth: one part; for kStats a part is a segment); with one sequence in the batch the parts are in grid.x
 // (a CTA that has nothing to do still takes an SM to itself for 2 us).  Row r of a tile is query block i_r of sequence b_r; its causal columns are the blocks seq_start_r .. r of
 // the batch.  The whole problem is the band (0, total_blocks, 0, Hq, 0).  Scores are written at their offset in the full
 // matrix minus band.score_base.  stats: [head][block of the batch][stat_segs] (m, l).
@@ -111,7 +111,8 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
 
   const int row_tiles = (band.blk_hi - band.blk_lo + kRows - 1) / kRows;
   int tile = row_tiles - 1 - (int)(blockIdx.x / band.heads), part_of_tile = (int)blockIdx.y;
-  if (kMode != kBoth && m.batch == 1) {                                   // only the parts that exist: row tile t has part_count of them
+  const bool parted = kMode != kBoth && part_tiles != 0;
+  if (parted && m.batch == 1) {                                   // only the parts that exist: row tile t has part_count of them
     int rest = (int)(blockIdx.x / band.heads);
     for (tile = row_tiles - 1; tile > 0; --tile) {
       const int parts = part_count(band, tile, part_tiles);
@@ -130,7 +131,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
   const int first_col = m.blk_off[find_sequence(m.blk_off, m.batch, r0)]; // rows ascend, so do their sequence starts
   const int last_col = r0 + rows_valid - 1;
   int col_lo = first_col, col_hi = last_col;                              // columns of this CTA
-  if (kMode != kBoth) {
+  if (parted) {
     const int part_cols = part_tiles * kCols, part = first_col / part_cols + part_of_tile;
     col_lo = max(col_lo, part * part_cols);
     col_hi = min(col_hi, (part + 1) * part_cols - 1);
@@ -253,24 +254,19 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
     const float scale2 = rsqrtf((float)kGateDim) * 1.4426950408889634f;
     float seg_m = -CUDART_INF_F, seg_l = 0.f;             // this thread's columns of the current segment
     float row_m = -CUDART_INF_F, row_l = 0.f, inv_l = 0.f;   // the whole row
-    float2* ml = reinterpret_cast<float2*>(smem + kOffStage);   // [segment parity][group][half][row]
+    float2* ml = reinterpret_cast<float2*>(smem + kOffSeg);
     int nseg = 0;
     uint32_t uses = 0;                                    // tiles this group has worked on
     const uint32_t base4 = (uint32_t)(reinterpret_cast<uintptr_t>(scores) >> 2);   // scores may begin on any four bytes
     if (kMode == kWrite && my_last >= 0) {
-      const int s_lo = my_start / seg_cols, s_hi = my_last / seg_cols;
-      const float2* st = stats + ((size_t)h * m.total_blocks + r0 + row) * stat_segs;
-      for (int s = 0; s <= s_hi - s_lo; ++s) { const float2 v = st[s]; combine(row_m, row_l, v.x, v.y); }
+      gate_row_stats(m, stats, h, my_last, my_start, row_m, row_l);
       inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
     }
     for (int n = 0; n < total; ++n) {
       const bool write = kMode == kWrite || (kMode == kBoth && n >= ntiles);
       const int ct = tile_lo + (kMode == kBoth && n >= ntiles ? n - ntiles : n);
       const int j0 = ct * kCols + half * 32;              // first column of this thread
-      if (kMode == kBoth && n == ntiles) {
-        inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
-        named_bar_sync(1, kRowThreads);                   // (the staging area held the segments' statistics)
-      }
+      if (kMode == kBoth && n == ntiles) inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
       if ((ct & 1) == grp) {
       wait_bar(bar0 + 8 * (ACC_FULL + grp), uses & 1u, abort_addr, status);
       ++uses;
@@ -289,7 +285,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
       for (int c = 0; c < 32; ++c) x[c] = __fmul_rn(__fadd_rn(__uint_as_float(vs[c]), __uint_as_float(vl[c])), scale2);
       // columns that are causal for this row: j in [my_start, my_last]
       const int lo = my_start - j0, hi = my_last - j0;
-      if (!write) {
+      if (!write) {                                        // statistics
         if (hi >= 0 && lo <= 31) {
           if (lo > 0 || hi < 31) {
 #pragma unroll
@@ -307,9 +303,12 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
           seg_l = __fadd_rn(__fmul_rn(seg_l, ex2f(__fsub_rn(seg_m, ref))), s4);              // 2^(-inf) = 0 on the first contribution
           seg_m = nm;
         }
-      } else {
+      }
+      if (write || kMode == kLogits) {
+        if (write) {
 #pragma unroll
-        for (int c = 0; c < 32; ++c) x[c] = __fmul_rn(ex2f(__fsub_rn(x[c], row_m)), inv_l);
+          for (int c = 0; c < 32; ++c) x[c] = gate_score(x[c], row_m, inv_l);
+        }
         float* stage = reinterpret_cast<float*>(smem + kOffStage) + warp * 1024;
 #pragma unroll
         for (int c = 0; c < 32; c += 4)
@@ -342,12 +341,12 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
         named_bar_sync(1, kRowThreads);
         float sm = -CUDART_INF_F, sl = 0.f;
 #pragma unroll
-        for (int p = 0; p < 4; ++p) { const float2 v = buf[p * kRows + row]; combine(sm, sl, v.x, v.y); }
+        for (int p = 0; p < 4; ++p) { const float2 v = buf[p * kRows + row]; gate_combine(sm, sl, v.x, v.y); }
         const int seg = ct * kCols / seg_cols, s_lo = my_start / seg_cols;
         const bool mine = my_last >= 0 && seg >= s_lo && seg <= my_last / seg_cols;
-        if (kMode == kStats) {
+        if (kMode == kStats || kMode == kLogits) {
           if (mine && half == 0 && grp == 0) stats[((size_t)h * m.total_blocks + r0 + row) * stat_segs + (seg - s_lo)] = make_float2(sm, sl);
-        } else if (mine) combine(row_m, row_l, sm, sl);
+        } else if (mine) gate_combine(row_m, row_l, sm, sl);
         seg_m = -CUDART_INF_F; seg_l = 0.f;
         ++nseg;
       }
@@ -421,11 +420,30 @@ int launch_gate_scores(const SeqMeta& m, const ScoreBand& band, const uint16_t* 
   return e == cudaSuccess ? 1 : -(int)e;
 }
 
+// Logits of a band and the statistics of its rows by one launch, for selection kernels that form the scores themselves.  Parts of 1, 2, 4 ..
+// segments, or whole rows: what lasts shortest, by the same estimate.
+int launch_gate_logits(const SeqMeta& m, const ScoreBand& band, const uint16_t* gq, const uint16_t* gk, float* logits, float2* stats,
+                       int* status, int num_sms, cudaStream_t stream) {
+  const dim3 all = score_grid(m, band, 1), rows = score_grid(m, band, 0);
+  if (rows.x == 0) return 0;
+  const int64_t tiles = (int64_t)all.x * all.y, longest = (m.max_nb + gs::kCols - 1) / gs::kCols;
+  int part = 0;
+  int64_t best = std::max((tiles + 3 * (int64_t)rows.x) / num_sms, longest + 3);
+  for (int p = gate_seg_tiles(m.max_nb); p < longest; p *= 2) {
+    const dim3 g = score_grid(m, band, p);
+    const int64_t cost = std::max((tiles + 3 * (int64_t)g.x * g.y) / num_sms, (int64_t)p + 3);
+    if (cost < best) { best = cost; part = p; }
+  }
+  const cudaError_t e = launch_next(gate_scores_kernel<gs::kLogits>, score_grid(m, band, part), gs::kThreads, gs::kSmemBytes, stream, m, band, gq, gk, logits, stats, status, part);
+  return e == cudaSuccess ? 1 : -(int)e;
+}
+
 // Lifts the kernels' shared-memory limit on the current device (no allocation).
 bool init_gate_scores() {
   return cudaFuncSetAttribute(gate_scores_kernel<gs::kBoth>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess &&
          cudaFuncSetAttribute(gate_scores_kernel<gs::kStats>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess &&
-         cudaFuncSetAttribute(gate_scores_kernel<gs::kWrite>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess;
+         cudaFuncSetAttribute(gate_scores_kernel<gs::kWrite>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess &&
+         cudaFuncSetAttribute(gate_scores_kernel<gs::kLogits>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gs::kSmemBytes) == cudaSuccess;
 }
 
 }  // namespace seer

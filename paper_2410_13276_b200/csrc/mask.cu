@@ -135,7 +135,8 @@ count_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, i
 
 // TopK counts of scores whose softmax statistics are at hand, a thread per row.  A row whose maximum and sum are finite has no
 // NaN among its scores, so its length follows from n and the parameters and no score is read (4096 rows of 4096 blocks: 15 us
-// with count_kernel); a row that has not is counted by its thread.
+// with count_kernel); a row that has not is counted by its thread (kLogits: from the scores that the selection will form).
+template <bool kLogits>
 __global__ void __launch_bounds__(128)
 topk_count_kernel(SeqMeta m, RowBand band, const float* scores, const float2* stats, seer_mask_params p,
                   int32_t* row_ptr) {
@@ -158,7 +159,13 @@ topk_count_kernel(SeqMeta m, RowBand band, const float* scores, const float2* st
     int ncand = n - nf;
     if (!finite) {
       ncand = 0;
-      for (int j = 0; j < n; ++j) ncand += (!is_forced(j, ri.i, p.flags) && score_key(ri.s[j]) != 0u) ? 1 : 0;
+      float row_m = 0.f, row_l = 0.f;
+      if (kLogits) gate_row_stats(m, stats, ri.h, ri.gb, ri.gb - ri.i, row_m, row_l);
+      const float inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
+      for (int j = 0; j < n; ++j) {
+        const float x = kLogits ? gate_score(ri.s[j], row_m, inv_l) : ri.s[j];
+        ncand += (!is_forced(j, ri.i, p.flags) && score_key(x) != 0u) ? 1 : 0;
+      }
     }
     c = nf + min(take, ncand);
   }
@@ -290,9 +297,12 @@ __device__ __forceinline__ uint32_t lean_key(float sc) {
 // A row gets one warp up to 2048 blocks, and as many as keep it at 2048 keys per warp beyond.  Measured: 65 536 rows of up to
 // 2048 blocks 176 us, 4096 rows of up to 4096 blocks 31 us (fill_kernel, which re-reads the scores in every pass: 158); what a row
 // needs once done by every warp of it, and a pass of its own for the counts: 183 and 34.
-template <int W>
+//
+// kLogits: the rows hold logits in units of log2, not scores; `stats` are the softmax statistics of the row's segments.  A score
+// is formed here as the score kernel forms it, bit for bit.
+template <int W, bool kLogits>
 __global__ void __launch_bounds__(W == 1 ? 128 : W * 32, W < 8 ? 12 : 6)
-topk_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, const int32_t* row_ptr,
+topk_kernel(SeqMeta m, RowBand band, const float* scores, const float2* stats, seer_mask_params p, const int32_t* row_ptr,
             int32_t* col_idx, int64_t col_capacity, int cap) {
   static_assert(W == 1 || W == 4 || W == 8, "a row has a warp or a CTA to itself");
   constexpr int kRows = W == 1 ? 4 : 1;
@@ -340,6 +350,13 @@ topk_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, co
   // ---- keys (0: not a candidate: past the row, NaN, or forced, which the writer puts in its place by itself)
   uint32_t c = 0, k_min = 0xffffffffu, k_max = 0u;               // over the candidates
   const uint32_t nan_bits = 0x7fffffffu;
+  float row_m = 0.f, inv_l = 0.f;
+  if (kLogits) {
+    float row_l = 0.f;
+    gate_row_stats(m, stats, ri.h, ri.gb, ri.gb - ri.i, row_m, row_l);
+    inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
+  }
+  auto key_of = [&](uint32_t raw) -> uint32_t { return lean_key(kLogits ? gate_score(__uint_as_float(raw), row_m, inv_l) : __uint_as_float(raw)); };
   const uint32_t* src = reinterpret_cast<const uint32_t*>(ri.s);
   const bool vec = (reinterpret_cast<uintptr_t>(ri.s) & 15) == 0;
   for (int j0 = j_mine; j0 - 4 * lane < j_hi; j0 += 512) {
@@ -360,7 +377,7 @@ topk_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, co
     for (int q = 0; q < 4; ++q) {
       const int j = j0 + q * 128;
       if (j - 4 * lane >= j_hi) break;                           // (uniform)
-      uint4 kq = make_uint4(lean_key(__uint_as_float(v[q].x)), lean_key(__uint_as_float(v[q].y)), lean_key(__uint_as_float(v[q].z)), lean_key(__uint_as_float(v[q].w)));
+      uint4 kq = make_uint4(key_of(v[q].x), key_of(v[q].y), key_of(v[q].z), key_of(v[q].w));
       if (sink_f && j == 0) kq.x = 0u;
       if (diag_f && (uint32_t)(ri.i - j) < 4u) {
         if (j == ri.i) kq.x = 0u;
@@ -725,34 +742,37 @@ fill_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, co
 }
 
 template <int W>
-static cudaError_t launch_topk_w(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
-                          int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
+static cudaError_t launch_topk_w(const SeqMeta& m, const RowBand& band, const float* scores, const float2* stats, bool logits, const seer_mask_params& p,
+                                 const int32_t* row_ptr, int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
   constexpr int kRows = W == 1 ? 4 : 1, kThreads = W == 1 ? 128 : W * 32;
   const int cap = (m.max_nb + 128 * W - 1) / (128 * W) * (128 * W);
-  return launch_next(topk_kernel<W>, (unsigned)((band.row_hi - band.row_lo + kRows - 1) / kRows), kThreads, (size_t)kRows * cap * 4, stream, m, band,
-                     scores, p, row_ptr, col_idx, col_capacity, cap);
+  return launch_next(logits ? topk_kernel<W, true> : topk_kernel<W, false>, (unsigned)((band.row_hi - band.row_lo + kRows - 1) / kRows), kThreads, (size_t)kRows * cap * 4,
+                     stream, m, band, scores, stats, p, row_ptr, col_idx, col_capacity, cap);
 }
-// At most 2048 keys per warp (4096-block rows: two warps 4 % slower than four); kTopkRowMax = 8 warps' worth.
-static cudaError_t launch_topk(const SeqMeta& m, const RowBand& band, const float* scores, const seer_mask_params& p, const int32_t* row_ptr,
-                        int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
-  if (m.max_nb <= 2048) return launch_topk_w<1>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
-  if (m.max_nb <= 8192) return launch_topk_w<4>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
-  return launch_topk_w<8>(m, band, scores, p, row_ptr, col_idx, col_capacity, stream);
+// At most 2048 keys per warp (4096-block rows: two warps 4 % slower than four); kTopkRowMax = 8 warps' worth.  `logits`: the scores'
+// place holds logits (launch_gate_logits_band), `stats` their statistics.
+static cudaError_t launch_topk(const SeqMeta& m, const RowBand& band, const float* scores, const float2* stats, bool logits, const seer_mask_params& p,
+                               const int32_t* row_ptr, int32_t* col_idx, int64_t col_capacity, cudaStream_t stream) {
+  if (m.max_nb <= 2048) return launch_topk_w<1>(m, band, scores, stats, logits, p, row_ptr, col_idx, col_capacity, stream);
+  if (m.max_nb <= 8192) return launch_topk_w<4>(m, band, scores, stats, logits, p, row_ptr, col_idx, col_capacity, stream);
+  return launch_topk_w<8>(m, band, scores, stats, logits, p, row_ptr, col_idx, col_capacity, stream);
 }
 
-int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const float2* stats, const ScoreBand& sb, int64_t row_lo,
+bool mask_takes_logits(const SeqMeta& m, const seer_mask_params& p) { return p.mode != SEER_THRESHOLD && m.max_nb <= kTopkRowMax; }
+
+int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const float2* stats, bool logits, const ScoreBand& sb, int64_t row_lo,
                      int64_t row_hi, bool first, const seer_mask_params& p, int32_t* row_ptr, int32_t* col_idx,
                      int64_t col_capacity, int64_t* nnz_out, cudaStream_t stream) {
   if (row_hi <= row_lo) return 0;
   const RowBand band = {row_lo, row_hi, sb};
   const unsigned grid = (unsigned)((row_hi - row_lo + kMaskWarps - 1) / kMaskWarps);
   cudaError_t e = stats != nullptr && p.mode != SEER_THRESHOLD
-      ? launch_next(topk_count_kernel, (unsigned)((row_hi - row_lo + 127) / 128), 128, 0, stream, m, band, scores, stats, p, row_ptr)
+      ? launch_next(logits ? topk_count_kernel<true> : topk_count_kernel<false>, (unsigned)((row_hi - row_lo + 127) / 128), 128, 0, stream, m, band, scores, stats, p, row_ptr)
       : launch_next(count_kernel, grid, kMaskWarps * 32, 0, stream, m, band, scores, p, row_ptr);
   if (e == cudaSuccess) e = launch_scan(row_hi - row_lo, row_ptr + row_lo, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status, stream);
   if (e == cudaSuccess)
     e = p.mode != SEER_THRESHOLD && m.max_nb <= kTopkRowMax
-        ? launch_topk(m, band, scores, p, row_ptr, col_idx, col_capacity, stream)
+        ? launch_topk(m, band, scores, stats, logits, p, row_ptr, col_idx, col_capacity, stream)
         : launch_next(fill_kernel, grid, kMaskWarps * 32, 0, stream, m, band, scores, p, row_ptr, col_idx, col_capacity);
   return e == cudaSuccess ? 3 : -(int)e;
 }
@@ -765,7 +785,7 @@ int launch_mask(seer_ctx* ctx, const SeqMeta& m, const float* scores, const seer
     return 0;
   }
   const ScoreBand all = {0, m.total_blocks, 0, m.num_q_heads, 0, 0, 0};
-  return launch_mask_band(ctx, m, scores, nullptr, all, 0, m.rows, true, p, row_ptr, col_idx, col_capacity, nnz_out, stream);
+  return launch_mask_band(ctx, m, scores, nullptr, false, all, 0, m.rows, true, p, row_ptr, col_idx, col_capacity, nnz_out, stream);
 }
 
 // ----------------------------------------------------------------------------------------------- 128-token lists -> 64-token lists
@@ -835,8 +855,9 @@ int launch_expand_lists(seer_ctx* ctx, const SeqMeta& m128, const SeqMeta& m64, 
 
 seer_status init_mask(seer_ctx* ctx) {
   (void)ctx;
-  const cudaError_t e = cudaFuncSetAttribute(topk_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkRowMax * 4);
-  return e == cudaSuccess ? SEER_OK : SEER_ERR_CUDA;
+  const bool ok = cudaFuncSetAttribute(topk_kernel<8, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkRowMax * 4) == cudaSuccess &&
+                  cudaFuncSetAttribute(topk_kernel<8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTopkRowMax * 4) == cudaSuccess;
+  return ok ? SEER_OK : SEER_ERR_CUDA;
 }
 
 }  // namespace seer

@@ -484,8 +484,10 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
   // Several bands, or a problem of few long rows: the statistics of all rows by one launch that fills the GPU, if what follows the
   // projected vectors has room for them (1 / 28 of the scores of a 2048-block sequence, 1 / 51 at 4096) and for the smallest band
   const auto band_elems = [&](size_t at) { return (int64_t)((ws_bytes - at) / sizeof(float)) - (int64_t)kBandSlackElems; };
-  const bool with_stats = ws_bytes >= planes_bytes + stats_bytes + min_band_bytes(t) &&
-                          (t.score_elems > band_elems(planes_bytes) || gate_split(m, ctx->num_sms));
+  const bool room = ws_bytes >= planes_bytes + stats_bytes + min_band_bytes(t);
+  // Where the selection can form the scores itself the bands hold logits: every logit is computed once, its row's statistics beside it.
+  const bool logits = room && mask_takes_logits(m, *p);
+  const bool with_stats = logits || (room && (t.score_elems > band_elems(planes_bytes) || gate_split(m, ctx->num_sms)));
   const size_t gate_bytes = planes_bytes + (with_stats ? stats_bytes : 0);
   float* band_buf = (float*)((char*)ws + gate_bytes);
   const int64_t cap = band_elems(gate_bytes);          // elements per band
@@ -495,7 +497,7 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
     int n = opt ? launch_gate_ex(ctx, m, *opt, q, k, Wq, Wk, nullptr, ws, ws_bytes, stream)
                 : launch_gate(ctx, m, q, k, Wq, Wk, nullptr, ws, ws_bytes, stream);
     if (n < 0) bad = true; else launched += n;
-    if (!bad && with_stats) {
+    if (!bad && with_stats && !logits) {
       n = launch_gate_stats_all(ctx, m, ws, stream);
       if (n < 0) bad = true; else launched += n;
     }
@@ -504,10 +506,11 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
   auto run_band = [&](ScoreBand band, int64_t row_lo, int64_t row_hi) {
     if (bad || row_hi <= row_lo) return;
     band.score_base &= ~(int64_t)3;
-    int n = band.blk_hi > band.blk_lo ? launch_gate_scores_band(ctx, m, band, ws, band_buf, with_stats, stream) : 0;
+    int n = band.blk_hi <= band.blk_lo ? 0
+            : logits ? launch_gate_logits_band(ctx, m, band, ws, band_buf, stream) : launch_gate_scores_band(ctx, m, band, ws, band_buf, with_stats, stream);
     if (n >= 0) {
       launched += n;
-      n = launch_mask_band(ctx, m, band_buf, with_stats ? gate_stats(m, ws) : nullptr, band, row_lo, row_hi, first, *p, row_ptr, col_idx, col_capacity, nnz_out, stream);
+      n = launch_mask_band(ctx, m, band_buf, with_stats ? gate_stats(m, ws) : nullptr, logits, band, row_lo, row_hi, first, *p, row_ptr, col_idx, col_capacity, nnz_out, stream);
     }
     if (n < 0) { bad = true; return; }
     launched += n;

@@ -137,6 +137,28 @@ seer_status shape_totals(const seer_shape* shape, ShapeTotals* t);
 size_t gate_workspace_bytes(const ShapeTotals& t, const seer_shape* shape);   // the projected vectors
 size_t gate_stats_bytes(const ShapeTotals& t, const seer_shape* shape);       // the softmax statistics that may follow them
 
+// The gate's row softmax, everything in units of log2: x = logit * log2(e), m the maximum of x, l the sum of 2^(x - m).
+__device__ __forceinline__ float gate_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float gate_score(float x, float row_m, float inv_l) { return __fmul_rn(gate_ex2(__fsub_rn(x, row_m)), inv_l); }
+// (m, l) of two disjoint sets of a row's columns; m = -inf: empty
+__device__ __forceinline__ void gate_combine(float& m, float& l, float m2, float l2) {
+  const float inf = __int_as_float(0x7f800000), nm = fmaxf(m, m2);
+  const float f = m == -inf ? 0.f : gate_ex2(m - nm), f2 = m2 == -inf ? 0.f : gate_ex2(m2 - nm);
+  l = __fadd_rn(__fmul_rn(l, f), __fmul_rn(l2, f2));
+  m = nm;
+}
+// Statistics of block row gb (numbered over the batch) of head h, whose sequence starts at block `start`.
+__device__ __forceinline__ void gate_row_stats(const SeqMeta& m, const float2* stats, int h, int gb, int start, float& row_m, float& row_l) {
+  const int seg_cols = gate_seg_tiles(m.max_nb) * kScoreTile, segs = gb / seg_cols - start / seg_cols + 1;
+  const float2* st = stats + ((size_t)h * m.total_blocks + gb) * gate_stat_segs(m.max_nb);
+  row_m = __int_as_float(0xff800000); row_l = 0.f;
+  for (int s = 0; s < segs; ++s) { const float2 v = st[s]; gate_combine(row_m, row_l, v.x, v.y); }
+}
+
 // Launch of a kernel that may start while its predecessor in the stream still runs (programmatic dependent launch): its CTAs get
 // ready as the predecessor's leave, and grid_wait() in the kernel holds them until the predecessor has completed and its writes are
 // visible.  Every CTA calls it, on every path, before it touches anything but its arguments and the shape's offsets (uploaded
@@ -186,11 +208,15 @@ int launch_gate_ex(seer_ctx* ctx, const SeqMeta& m, const seer_gate_options& opt
 int launch_gate_stats_all(seer_ctx* ctx, const SeqMeta& m, void* ws, cudaStream_t stream);
 int launch_gate_scores_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& band, void* ws, float* scores, bool with_stats,
                             cudaStream_t stream);
+// ... or its logits (units of log2) and its rows' statistics at once, for launch_mask_band with `logits`.
+int launch_gate_logits_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& band, void* ws, float* logits, cudaStream_t stream);
 const float2* gate_stats(const SeqMeta& m, void* ws);
 bool gate_split(const SeqMeta& m, int num_sms);   // scores of the whole problem: statistics apart from the scores?
 // Mask rows [row_lo, row_hi) from a band of scores; `first` starts row_ptr at 0, later bands continue from the
-// previous band's last entry; `stats` (or nullptr) are the statistics the scores were made from.
-int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const float2* stats, const ScoreBand& sb, int64_t row_lo,
+// previous band's last entry; `stats` (or nullptr) are the statistics the scores were made from; `logits`: `scores` holds logits
+// (mask_takes_logits).
+bool mask_takes_logits(const SeqMeta& m, const seer_mask_params& p);
+int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const float2* stats, bool logits, const ScoreBand& sb, int64_t row_lo,
                      int64_t row_hi, bool first, const seer_mask_params& p, int32_t* row_ptr, int32_t* col_idx,
                      int64_t col_capacity, int64_t* nnz_out, cudaStream_t stream);
 // 128-token block lists -> the 64-token lists the attention kernels take (m128 and m64 describe the same batch).
