@@ -10,7 +10,7 @@
 //
 // One CTA = 128 consecutive block rows of one head (rows of the packed batch, whatever sequences they belong to) times a
 // range of column tiles of 64 blocks (tiles of the packed batch, aligned to 64).  A score needs the softmax statistics of
-// its whole row first, so every tile is computed twice and every score is written once:
+// its whole row first, so every tile is computed twice (unless there are two at most) and every score is written once:
 //   kBoth   one CTA walks all causal tiles of its rows twice (short sequences: one launch)
 //   kStats  a CTA walks one segment of up to SegTiles tiles and leaves the rows' (maximum, sum) of that segment
 //   kWrite  a CTA walks part_tiles tiles, after combining its rows' statistics, and writes exp(x - m) / l
@@ -160,6 +160,9 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
   const int tile_lo = col_lo / kCols;
   const int ntiles = col_hi / kCols - tile_lo + 1;                        // column tiles of one sweep
   const int total = kMode == kBoth ? 2 * ntiles : ntiles;
+  // of two tiles each group of row warps has one: its logits stay in registers between the sweeps
+  const bool kept = kMode == kBoth && ntiles <= 2;
+  const int products = kept ? ntiles : total;                             // tiles that are multiplied
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < (int)kBars; ++i)                                  // one commit per issuing thread; one arrival per row warp
@@ -207,7 +210,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
     if (elect_one()) {
       const char* src = reinterpret_cast<const char*>(gk) + (size_t)g * m.total_blocks * kGatePairBytes;
       uint32_t buf = 0, ph = 1;
-      for (int n = 0; n < total; ++n) {
+      for (int n = 0; n < products; ++n) {
         wait_bar(bar0 + 8 * (B_EMPTY + buf), ph, abort_addr, status);
         const GateTile bt(tile_lo + (n >= ntiles ? n - ntiles : n), m.total_blocks);
         const uint32_t full = bar0 + 8 * (B_FULL + buf), dst = base + buf * kBBuf;
@@ -228,7 +231,7 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
       const uint32_t pa[3] = {0u, part ? 1u : 2u, part ? 0u : 1u}, pb[3] = {part ? 1u : 2u, 0u, part ? 0u : 1u};
       uint32_t buf = 0, ph = 0, uses[2] = {0u, 0u};
       wait_bar(bar0 + 8 * A_FULL, 0u, abort_addr, status);
-      for (int n = 0; n < total; ++n) {
+      for (int n = 0; n < products; ++n) {
         const int acc = (tile_lo + (n >= ntiles ? n - ntiles : n)) & 1;
         wait_bar(bar0 + 8 * (B_FULL + buf), ph, abort_addr, status);
         // the rows have taken the previous tile out of this accumulator pair
@@ -262,27 +265,29 @@ gate_scores_kernel(SeqMeta m, ScoreBand band, const uint16_t* gq, const uint16_t
       gate_row_stats(m, stats, h, my_last, my_start, row_m, row_l);
       inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
     }
+    float x[32];
     for (int n = 0; n < total; ++n) {
       const bool write = kMode == kWrite || (kMode == kBoth && n >= ntiles);
       const int ct = tile_lo + (kMode == kBoth && n >= ntiles ? n - ntiles : n);
       const int j0 = ct * kCols + half * 32;              // first column of this thread
       if (kMode == kBoth && n == ntiles) inv_l = row_l > 0.f ? 1.0f / row_l : 0.f;
       if ((ct & 1) == grp) {
-      wait_bar(bar0 + 8 * (ACC_FULL + grp), uses & 1u, abort_addr, status);
-      ++uses;
-      tc_fence_after();
-      const uint32_t a = tmem + lane_addr + (uint32_t)grp * 2u * kCols + (uint32_t)half * 32u;
-      uint32_t vs[32], vl[32];
-      tc_ld32(a, vs);
-      tc_ld32(a + kCols, vl);
-      tc_wait_ld32(vs);
-      tc_wait_ld32(vl);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar0 + 8 * (ACC_EMPTY + grp));
-      float x[32];
+      if (!kept || n < ntiles) {
+        wait_bar(bar0 + 8 * (ACC_FULL + grp), uses & 1u, abort_addr, status);
+        ++uses;
+        tc_fence_after();
+        const uint32_t a = tmem + lane_addr + (uint32_t)grp * 2u * kCols + (uint32_t)half * 32u;
+        uint32_t vs[32], vl[32];
+        tc_ld32(a, vs);
+        tc_ld32(a + kCols, vl);
+        tc_wait_ld32(vs);
+        tc_wait_ld32(vl);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar0 + 8 * (ACC_EMPTY + grp));
 #pragma unroll
-      for (int c = 0; c < 32; ++c) x[c] = __fmul_rn(__fadd_rn(__uint_as_float(vs[c]), __uint_as_float(vl[c])), scale2);
+        for (int c = 0; c < 32; ++c) x[c] = __fmul_rn(__fadd_rn(__uint_as_float(vs[c]), __uint_as_float(vl[c])), scale2);
+      }
       // columns that are causal for this row: j in [my_start, my_last]
       const int lo = my_start - j0, hi = my_last - j0;
       if (!write) {                                        // statistics
