@@ -654,13 +654,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           sc = l > 0.f ? 1.f / l : 0.f;
           lse_row = l > 0.f ? (R + log2f(l)) * 0.6931471805599453f : -CUDART_INF_F;
         }
-        // The last P V of the item.  A warp whose wait for it is lost keeps the group's barriers, stores nothing and leaves afterwards.
+        // The last P V of the item.  A warp whose wait for it is lost keeps the group's barriers and leaves afterwards.  Warps that hand each other
+        // partial rows agree on the outcome at their first exchange: one lost wait and none of them stores.  (A one-block list's rows are
+        // each a warp's own.)
         fail = !mbar_wait(sh, bb + PV_DONE + (int)((cnt - 1) & 1u), ((cnt - 1) >> 1) & 1u, status);
         fail = __any_sync(0xffffffffu, fail);
-        const bool store = row < it.q_valid && !fail;
+        bool store = row < it.q_valid && !fail;
         tc_fence_after();
         tr.ev(37);
-        if (half == 0 && lse != nullptr && store) lse[(int64_t)it.h * lse_stride + it.tok0 + row] = lse_row;
+        auto store_lse = [&] { if (half == 0 && lse != nullptr && store) lse[(int64_t)it.h * lse_stride + it.tok0 + row] = lse_row; };
         if (two) {
           // The thread of lane r ends with d columns 64 * half ..: it hands the other 64 of its partial row to lane r ^ 64 through the
           // item's Q buffer (Q has been read: the last S is done), 32 columns at a time, 16-byte chunks XOR (row % 8)
@@ -680,8 +682,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
               const float2 y = __fmul2_rn(make_float2(__uint_as_float(other[i][4 * c + 2]), __uint_as_float(other[i][4 * c + 3])), sc2);
               st_shared_v4(wr + (uint32_t)((c ^ (r & 7)) << 4), __float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(y.x), __float_as_uint(y.y));
             }
-            if (i == 0) { tc_wait_ld32(mine[0]); tc_wait_ld32(other[1]); tc_wait_ld32(mine[1]); }
-            named_bar_sync(bar_merge, kGroupThreads);
+            if (i == 0) {
+              tc_wait_ld32(mine[0]); tc_wait_ld32(other[1]); tc_wait_ld32(mine[1]);
+              fail = named_bar_or(bar_merge, kGroupThreads, fail);
+              store = store && !fail;
+              store_lse();
+            } else named_bar_sync(bar_merge, kGroupThreads);
             uint32_t out[16];
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
@@ -701,6 +707,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           }
           fence_async_smem();                               // before the next Q copy into this buffer
         } else if (half == 0) {
+          store_lse();
 #pragma unroll
           for (int ch = 0; ch < 4; ++ch) {
             uint32_t ov[32];

@@ -80,6 +80,50 @@ def test_a_lost_copy_raises_timeout_and_the_context_survives(rt, lost_tile):
     assert torch.equal(p.o, o_ref) and torch.equal(p.lse, lse_ref)
 
 
+@pytest.mark.parametrize("keep,lost_tile,lost_item", [(32, 15, 0), (2, 0, 0), (2, 1, 1), (3, 1, 0), (3, 3, 1), (1, 0, 0), (1, 1, 1)])
+def test_a_lost_last_copy_leaves_the_items_rows_unwritten(rt, keep, lost_tile, lost_item):
+    """The copy of an item's last tile: the group finds out at the item's merge, when everything but O is settled.  Neither o nor lse of any of the
+    item's rows is written (lists of two blocks or more are merged by pairs of warps, a list of one block by one), items that the stream
+    had finished are, and nothing of another stream changes."""
+    import torch
+    B, Prefill, ctx = rt
+    hq, hkv, S = 8, 2, 4096
+    w = W.make_small(seed=4243, seqlens=[S], hq=hq, hkv=hkv)
+    p = Prefill(w.cu_seqlens, hq, hkv, ctx=ctx, want_lse=True)
+    p.set_inputs(w.q, w.k, w.v, w.wq, w.wk)
+    p.gate(); p.mask(B.make_mask_params(B.SEER_TOPK_COUNT, k=keep, flags=B.SEER_FORCE_DIAG))
+    p.attn(dynamic=False); torch.cuda.synchronize()
+    assert p.status() == 0
+    o_ref, lse_ref = p.o.clone(), p.lse.clone()
+    nb, group = S // 64, hq // hkv
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = []                                                      # (head, query block) of the items of CTA 0's first stream, in order
+    for wi in range(0, hq * nb, 2 * min(sms, hq * nb // 2)):
+        g, rem = divmod(wi, nb * group)
+        rows.append((g * group + rem % group, nb - 1 - rem // group))
+    assert lost_item < len(rows) and all(i + 1 >= keep for _, i in rows[:lost_item + 1])   # every list so far has `keep` blocks
+    B.seer_debug_lost_wait(ctx, 2_000, lost_tile)
+    try:
+        p.o.fill_(float("nan")); p.lse.fill_(float("nan"))
+        p.attn(dynamic=False)
+        status = B.seer_poll_device_status(ctx)
+    finally:
+        B.seer_debug_lost_wait(ctx, 2_000_000, -1)
+    assert B.STATUS_NAMES[status] == "SEER_ERR_TIMEOUT"
+    for n, (h, i) in enumerate(rows):
+        o, lse = p.o[i * 64:(i + 1) * 64, h], p.lse[h, i * 64:(i + 1) * 64]
+        if n < lost_item:
+            assert torch.equal(o, o_ref[i * 64:(i + 1) * 64, h]) and torch.equal(lse, lse_ref[h, i * 64:(i + 1) * 64])
+        elif n == lost_item:
+            assert torch.isnan(o.float()).all() and torch.isnan(lse).all()
+        p.o[i * 64:(i + 1) * 64, h] = o_ref[i * 64:(i + 1) * 64, h]
+        p.lse[h, i * 64:(i + 1) * 64] = lse_ref[h, i * 64:(i + 1) * 64]
+    assert torch.equal(p.o, o_ref) and torch.equal(p.lse, lse_ref), "a row of another stream changed"
+    p.o.fill_(float("nan")); p.lse.fill_(float("nan"))
+    p.attn(); torch.cuda.synchronize()
+    assert p.status() == 0 and torch.equal(p.o, o_ref) and torch.equal(p.lse, lse_ref)
+
+
 def test_lost_wait_hook_rejects_a_zero_limit(rt):
     B, _, ctx = rt
     with pytest.raises(B.SeerError):
