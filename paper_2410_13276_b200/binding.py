@@ -129,17 +129,26 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
-_raw_stream = _current_device = None
+_stream_handle = None
+
+
+def _resolve_stream_handle():
+    """A function that gives the handle of torch's current stream on the current device, by the cheapest way this torch has."""
+    import torch
+    torch.cuda.current_stream()                         # (initialises CUDA)
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+    if raw is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
 
 
 def _current_stream() -> int:
     """Handle of torch's current stream on the current device."""
-    global _raw_stream, _current_device
-    if _raw_stream is None:
-        import torch
-        torch.cuda.current_stream()                     # (initialises CUDA)
-        _raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
-    return _raw_stream(_current_device())
+    global _stream_handle
+    handle = _stream_handle
+    if handle is None:                                  # (threads that get here at the same time find the same way)
+        handle = _stream_handle = _resolve_stream_handle()
+    return handle()
 
 
 def _stream(stream) -> Optional[int]:
