@@ -294,7 +294,10 @@ seer_status seer_gate_scores_ex(seer_ctx* ctx, const seer_shape* shape, const se
  * Workspace: DEVICE memory, 256-byte aligned, seer_gate_mask_workspace_bytes(shape, band_bytes) bytes: the projected
  * vectors (seer_workspace_bytes) followed by the band scratch.  The call uses whatever follows the projected vectors
  * as scratch, so `band_bytes` is the caller's choice; at least 64 rows of the longest sequence (64 * max nb * 4 + 16
- * bytes) are needed and the size query never returns less.  SEER_ERR_WORKSPACE if ws is smaller than that. */
+ * bytes) are needed and the size query never returns less.  SEER_ERR_WORKSPACE if ws is smaller than that.
+ * The softmax statistics of the rows (8 bytes per row and started 256 blocks of the longest sequence, and 8 more) are taken out of the
+ * band's bytes where that leaves one band one, or several at most twice as many: with `band_bytes` of the scores and those
+ * statistics a TopK mask takes one sweep over the logits, with less it takes two. */
 size_t seer_gate_mask_workspace_bytes(const seer_shape* shape, size_t band_bytes);
 seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const seer_gate_options* options, const void* q,
                                  const void* k, const float* Wq, const float* Wk, const seer_mask_params* params,

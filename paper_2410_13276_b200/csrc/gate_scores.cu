@@ -390,6 +390,19 @@ bool gate_split(const SeqMeta& m, int num_sms) {
   return two < one;
 }
 
+// Whether bands of logits, `bands` of them, take less time than the statistics of all rows and then bands of scores, in the same units.  A
+// part of the logits is a whole segment at least, so a band of few rows lasts as long as that (16 tiles beyond 2048 blocks), where
+// one of scores is split by four; and a band's selection takes about 1.5 longer to form the scores.  (Start of a CTA three; 200 000
+// tokens, 16 heads in bands of 8 MB: 5.0 ms by 112 bands of logits, 3.3 by scores; 262 144 tokens, 32 heads in 128 MB: 2.1 and 2.4.)
+bool gate_logits_pay(const SeqMeta& m, int64_t bands, int num_sms) {
+  const double tiles = (double)m.score_tiles, sms = num_sms, seg = gate_seg_tiles(m.max_nb), longest = (m.max_nb + gs::kCols - 1) / gs::kCols;
+  const auto launch = [&](double all, double part) { return std::max(all * (1.0 + 3.0 / part) / sms, std::min(part, longest) + 3.0); };
+  double of_logits = 1e30, of_scores = 1e30;
+  for (double p = seg; p < 2.0 * std::max(longest, seg); p *= 2.0) of_logits = std::min(of_logits, launch(tiles / (double)bands, p));
+  for (double p = 4.0; p <= 16.0; p *= 2.0) of_scores = std::min(of_scores, launch(tiles / (double)bands, p));
+  return (double)bands * (of_logits + 1.5 - of_scores) <= launch(tiles, seg) + 3.0;
+}
+
 // Statistics of all rows.
 int launch_gate_stats(const SeqMeta& m, const uint16_t* gq, const uint16_t* gk, float2* stats, int* status, cudaStream_t stream) {
   const ScoreBand all = {m.first_q_block, m.total_blocks, 0, m.num_q_heads, 0, 0, 0};

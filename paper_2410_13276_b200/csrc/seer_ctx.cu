@@ -196,6 +196,74 @@ bool on_16(const void* a, const void* b, const void* c, const void* d) {
   return (((uintptr_t)a | (uintptr_t)b | (uintptr_t)c | (uintptr_t)d) & 15) == 0;
 }
 
+// ---- bands of the one-call gate + mask
+namespace {
+constexpr size_t kBandSlackElems = 4;   // the band's base is rounded down to a multiple of four elements
+
+size_t min_band_bytes(const ShapeTotals& t) { return ((size_t)kScoreTile * (size_t)t.max_nb + kBandSlackElems) * sizeof(float); }
+
+// The bands of a scratch of `cap` elements, in CSR row order: fn(band, first row, last row + 1) until it returns false.
+template <class Fn>
+void walk_bands(const seer_shape* shape, int64_t cap, Fn&& fn) {
+  const int32_t* cu = shape->cu_seqlens_host;
+  const int Hq = shape->num_q_heads;
+  auto blocks_of = [&](int b) { return ((int64_t)cu[b + 1] - cu[b] + shape->block - 1) / shape->block; };
+  int64_t blk_off = 0, score_off = 0;                  // of sequence b
+  for (int b = 0; b < shape->batch;) {
+    const int64_t nb = blocks_of(b);
+    if ((int64_t)Hq * nb * nb <= cap) {
+      // whole sequences, as many as fit
+      int b1 = b;
+      int64_t blocks = 0, elems = 0;
+      while (b1 < shape->batch) {
+        const int64_t n1 = blocks_of(b1);
+        if (elems + (int64_t)Hq * n1 * n1 > cap) break;
+        elems += (int64_t)Hq * n1 * n1; blocks += n1;
+        ++b1;
+      }
+      if (!fn({(int32_t)blk_off, (int32_t)(blk_off + blocks), 0, Hq, score_off, 0, 0}, Hq * blk_off, Hq * (blk_off + blocks))) return;
+      blk_off += blocks; score_off += elems;
+      b = b1;
+      continue;
+    }
+    // query blocks of the sequence that have scores: all of them, or those of its chunk
+    int64_t i_lo = 0;
+    if (shape->cu_seqlens_q_host) {
+      const int64_t sq = (int64_t)shape->cu_seqlens_q_host[b + 1] - shape->cu_seqlens_q_host[b], sk = (int64_t)cu[b + 1] - cu[b];
+      i_lo = sq > 0 ? (sk - sq) / shape->block : nb;
+    }
+    const int64_t per_head = packed_rows((int)nb) - packed_rows((int)i_lo);
+    if (per_head <= cap) {
+      // whole heads of this sequence, packed: causal columns alone, no rows before the chunk
+      const int hb = per_head > 0 ? (int)(cap / per_head < Hq ? cap / per_head : Hq) : Hq;
+      for (int h0 = 0; h0 < Hq; h0 += hb) {
+        const int h1 = h0 + hb < Hq ? h0 + hb : Hq;
+        if (!fn({(int32_t)(blk_off + i_lo), (int32_t)(blk_off + nb), h0, h1 - h0, 0, per_head > 0 ? per_head : 1, (int32_t)i_lo},
+                Hq * blk_off + (int64_t)h0 * nb, Hq * blk_off + (int64_t)h1 * nb)) return;
+      }
+    } else {
+      // runs of 64-row tiles of one head
+      const int64_t ntile = (nb + kScoreTile - 1) / kScoreTile, tb = cap / ((int64_t)kScoreTile * nb);   // tb >= 1: the workspace check above
+      for (int h = 0; h < Hq; ++h)
+        for (int64_t t0 = 0; t0 < ntile; t0 += tb) {
+          const int64_t t1 = t0 + tb < ntile ? t0 + tb : ntile;
+          const int64_t i0 = t0 * kScoreTile, i1 = t1 * kScoreTile < nb ? t1 * kScoreTile : nb;
+          if (!fn({(int32_t)(blk_off + i0), (int32_t)(blk_off + i1), h, 1, score_off + ((int64_t)h * nb + i0) * nb, 0, 0},
+                  Hq * blk_off + (int64_t)h * nb + i0, Hq * blk_off + (int64_t)h * nb + i1)) return;
+        }
+    }
+    blk_off += nb; score_off += (int64_t)Hq * nb * nb;
+    ++b;
+  }
+}
+
+int64_t count_bands(const seer_shape* shape, int64_t cap, int64_t limit) {
+  int64_t n = 0;
+  walk_bands(shape, cap, [&](const ScoreBand&, int64_t row_lo, int64_t row_hi) { n += row_hi > row_lo ? 1 : 0; return n < limit; });
+  return n;
+}
+}  // namespace
+
 }  // namespace seer
 
 using namespace seer;
@@ -445,12 +513,6 @@ seer_status seer_attn_block_max(seer_ctx* ctx, const seer_shape* shape, const vo
 }
 
 // ---- gate and mask in one call, the scores held one band at a time
-namespace {
-constexpr size_t kBandSlackElems = 4;   // the band's base is rounded down to a multiple of four elements
-
-size_t min_band_bytes(const ShapeTotals& t) { return ((size_t)kScoreTile * (size_t)t.max_nb + kBandSlackElems) * sizeof(float); }
-}  // namespace
-
 size_t seer_gate_mask_workspace_bytes(const seer_shape* shape, size_t band_bytes) {
   ShapeTotals t;
   if (shape_totals(shape, &t) != SEER_OK) return 0;
@@ -490,12 +552,27 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
     return n0 < 0 ? SEER_ERR_CUDA : SEER_OK;
   }
   // Several bands, or a problem of few long rows: the statistics of all rows by one launch that fills the GPU, if what follows the
-  // projected vectors has room for them (1 / 28 of the scores of a 2048-block sequence, 1 / 51 at 4096) and for the smallest band
+  // projected vectors has room for them (1 / 28 of the scores of a 2048-block sequence, 1 / 51 at 4096) and for the smallest band.  For
+  // short sequences they are as large as the scores: statistics that would make several bands of one, or more than twice as many, are not
+  // worth their room.  (700 tokens, 32 heads, a scratch of exactly the scores: 18 us in one band, 133 in eleven.)
   const auto band_elems = [&](size_t at) { return (int64_t)((ws_bytes - at) / sizeof(float)) - (int64_t)kBandSlackElems; };
   const bool room = ws_bytes >= planes_bytes + stats_bytes + min_band_bytes(t);
-  // Where the selection can form the scores itself the bands hold logits: every logit is computed once, its row's statistics beside it.
-  const bool logits = room && mask_takes_logits(m, *p);
-  const bool with_stats = logits || (room && (t.score_elems > band_elems(planes_bytes) || gate_split(m, ctx->num_sms)));
+  bool with_stats = false, logits = false;
+  if (room) {
+    const int64_t plain = band_elems(planes_bytes), rest = band_elems(planes_bytes + stats_bytes);
+    const bool split = gate_split(m, ctx->num_sms);
+    int64_t bands = 1, limit = 1;
+    if (t.score_elems > rest) {
+      const int64_t without = count_bands(shape, plain, INT64_MAX);
+      limit = without > 1 ? 2 * without : 1;
+      bands = count_bands(shape, rest, limit + 1);
+      if (split && bands > limit) bands = count_bands(shape, rest, INT64_MAX);
+    }
+    with_stats = split || (t.score_elems > plain && bands <= limit);
+    // Where the selection can form the scores itself the bands hold logits: every logit is computed once, its row's statistics beside it.
+    logits = mask_takes_logits(m, *p) && (bands == 1 || (with_stats && gate_logits_pay(m, bands, ctx->num_sms)));
+    with_stats = with_stats || logits;
+  }
   const size_t gate_bytes = planes_bytes + (with_stats ? stats_bytes : 0);
   float* band_buf = (float*)((char*)ws + gate_bytes);
   const int64_t cap = band_elems(gate_bytes);          // elements per band
@@ -524,56 +601,7 @@ seer_status seer_gate_block_mask(seer_ctx* ctx, const seer_shape* shape, const s
     launched += n;
     first = false;
   };
-  const int32_t* cu = shape->cu_seqlens_host;
-  const int Hq = shape->num_q_heads;
-  auto blocks_of = [&](int b) { return ((int64_t)cu[b + 1] - cu[b] + shape->block - 1) / shape->block; };
-  int64_t blk_off = 0, score_off = 0;                  // of sequence b
-  for (int b = 0; b < shape->batch && !bad;) {
-    const int64_t nb = blocks_of(b);
-    if ((int64_t)Hq * nb * nb <= cap) {
-      // whole sequences, as many as fit
-      int b1 = b;
-      int64_t blocks = 0, elems = 0;
-      while (b1 < shape->batch) {
-        const int64_t n1 = blocks_of(b1);
-        if (elems + (int64_t)Hq * n1 * n1 > cap) break;
-        elems += (int64_t)Hq * n1 * n1; blocks += n1;
-        ++b1;
-      }
-      run_band({(int32_t)blk_off, (int32_t)(blk_off + blocks), 0, Hq, score_off, 0, 0}, Hq * blk_off, Hq * (blk_off + blocks));
-      blk_off += blocks; score_off += elems;
-      b = b1;
-      continue;
-    }
-    // query blocks of the sequence that have scores: all of them, or those of its chunk
-    int64_t i_lo = 0;
-    if (shape->cu_seqlens_q_host) {
-      const int64_t sq = (int64_t)shape->cu_seqlens_q_host[b + 1] - shape->cu_seqlens_q_host[b], sk = (int64_t)cu[b + 1] - cu[b];
-      i_lo = sq > 0 ? (sk - sq) / shape->block : nb;
-    }
-    const int64_t per_head = packed_rows((int)nb) - packed_rows((int)i_lo);
-    if (per_head <= cap) {
-      // whole heads of this sequence, packed: causal columns alone, no rows before the chunk
-      const int hb = per_head > 0 ? (int)(cap / per_head < Hq ? cap / per_head : Hq) : Hq;
-      for (int h0 = 0; h0 < Hq; h0 += hb) {
-        const int h1 = h0 + hb < Hq ? h0 + hb : Hq;
-        run_band({(int32_t)(blk_off + i_lo), (int32_t)(blk_off + nb), h0, h1 - h0, 0, per_head > 0 ? per_head : 1, (int32_t)i_lo},
-                 Hq * blk_off + (int64_t)h0 * nb, Hq * blk_off + (int64_t)h1 * nb);
-      }
-    } else {
-      // runs of 64-row tiles of one head
-      const int64_t ntile = (nb + kScoreTile - 1) / kScoreTile, tb = cap / ((int64_t)kScoreTile * nb);   // tb >= 1: the workspace check above
-      for (int h = 0; h < Hq; ++h)
-        for (int64_t t0 = 0; t0 < ntile; t0 += tb) {
-          const int64_t t1 = t0 + tb < ntile ? t0 + tb : ntile;
-          const int64_t i0 = t0 * kScoreTile, i1 = t1 * kScoreTile < nb ? t1 * kScoreTile : nb;
-          run_band({(int32_t)(blk_off + i0), (int32_t)(blk_off + i1), h, 1, score_off + ((int64_t)h * nb + i0) * nb, 0, 0},
-                   Hq * blk_off + (int64_t)h * nb + i0, Hq * blk_off + (int64_t)h * nb + i1);
-        }
-    }
-    blk_off += nb; score_off += (int64_t)Hq * nb * nb;
-    ++b;
-  }
+  walk_bands(shape, cap, [&](const ScoreBand& band, int64_t row_lo, int64_t row_hi) { run_band(band, row_lo, row_hi); return !bad; });
   finish_call(ctx, slot, stream);
   if (bad) return SEER_ERR_CUDA;
   ctx->launches += launched;

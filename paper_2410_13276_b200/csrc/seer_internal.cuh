@@ -213,6 +213,7 @@ int launch_gate_scores_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& ba
 // ... or its logits (units of log2) and its rows' statistics at once, for launch_mask_band with `logits`.
 int launch_gate_logits_band(seer_ctx* ctx, const SeqMeta& m, const ScoreBand& band, void* ws, float* logits, cudaStream_t stream);
 const float2* gate_stats(const SeqMeta& m, void* ws);
+bool gate_logits_pay(const SeqMeta& m, int64_t bands, int num_sms);   // bands of logits, or statistics and bands of scores?
 bool gate_split(const SeqMeta& m, int num_sms);   // scores of the whole problem: statistics apart from the scores?
 // Mask rows [row_lo, row_hi) from a band of scores; `first` starts row_ptr at 0, later bands continue from the
 // previous band's last entry; `stats` (or nullptr) are the statistics the scores were made from; `logits`: `scores` holds logits
