@@ -295,7 +295,7 @@ seer_status seer_gate_scores_ex(seer_ctx* ctx, const seer_shape* shape, const se
  * vectors (seer_workspace_bytes) followed by the band scratch.  The call uses whatever follows the projected vectors
  * as scratch, so `band_bytes` is the caller's choice; at least 64 rows of the longest sequence (64 * max nb * 4 + 16
  * bytes) are needed and the size query never returns less.  SEER_ERR_WORKSPACE if ws is smaller than that.
- * The softmax statistics of the rows (8 bytes per row and started 256 blocks of the longest sequence, and 8 more) are taken out of the
+ * The softmax statistics of the rows (per row 8 bytes, and 8 more for each 256 blocks of the longest sequence, 1024 where it has more than 2048) are taken out of the
  * band's bytes where that leaves one band one, or several at most twice as many: with `band_bytes` of the scores and those
  * statistics a TopK mask takes one sweep over the logits, with less it takes two. */
 size_t seer_gate_mask_workspace_bytes(const seer_shape* shape, size_t band_bytes);

@@ -263,9 +263,15 @@ scan_kernel(int64_t rows, int32_t* row_ptr, int first, int64_t col_capacity, int
 }
 
 // Counts and their scan by one CTA, for masks of few short rows: the two kernels are a launch and a few latencies each, and there is nothing
-// else to do meanwhile (2048 tokens, 4 heads: mask alone 16.5 us by two kernels, 11.6 so).  Eight lanes take a
-// row, 128 rows go at a time.
+// else to do meanwhile.  Eight lanes take a row, 128 rows go at a time, and each pass begins with the rows' addresses: past two to four of
+// them the one CTA is the slower way.  Mask alone, two kernels and this, one to sixteen sequences: 256 rows of 64 blocks, TopK 9.9 and
+// 8.1 to 8.5 us; 384 of 48 9.9 and 9.2 to 9.9; 384 of 64 10.0 and 10.0 to 10.6; 512 of 32 10.1 and 11.3 to 11.9.  Thresholds take fewer instructions
+// an entry: 384 of 64 9.8 and 8.6 to 9.1, 512 of 32 10.1 and 8.9 to 9.7, 512 of 64 9.7 and 10.3 to 11.4.
 constexpr int kSmallRows = 512, kSmallBlocks = 64;
+static bool small_mask(int64_t rows, int max_nb, int mode) {
+  if (max_nb > kSmallBlocks) return false;
+  return rows <= (mode == SEER_THRESHOLD ? (max_nb <= 32 ? kSmallRows : 384) : max_nb <= 48 ? 384 : 256);
+}
 __global__ void __launch_bounds__(1024)
 count_scan_kernel(SeqMeta m, RowBand band, const float* scores, seer_mask_params p, int32_t* row_ptr, int first, int64_t col_capacity,
                   int64_t* __restrict__ nnz_out, int* __restrict__ status) {
@@ -821,7 +827,7 @@ int launch_mask_band(seer_ctx* ctx, const SeqMeta& m, const float* scores, const
   if (row_hi <= row_lo) return 0;
   const RowBand band = {row_lo, row_hi, sb};
   const unsigned grid = (unsigned)((row_hi - row_lo + kMaskWarps - 1) / kMaskWarps);
-  const bool from_stats = stats != nullptr && p.mode != SEER_THRESHOLD, small = !from_stats && row_hi - row_lo <= kSmallRows && m.max_nb <= kSmallBlocks;
+  const bool from_stats = stats != nullptr && p.mode != SEER_THRESHOLD, small = !from_stats && small_mask(row_hi - row_lo, m.max_nb, p.mode);
   cudaError_t e = small
       ? launch_next(count_scan_kernel, 1, 1024, 0, stream, m, band, scores, p, row_ptr, first ? 1 : 0, col_capacity, nnz_out, ctx->d_status)
       : from_stats

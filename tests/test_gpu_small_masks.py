@@ -1,4 +1,5 @@
-"""Masks of few short rows, counted and scanned by one CTA: around its limits (512 rows, 64 blocks a row; beyond, two kernels), with ties,
+"""Masks of few short rows, counted and scanned by one CTA: around its limits (TopK 384 rows of up to 48 blocks or 256 of up to 64, thresholds
+512 rows of up to 32 or 384 of up to 64; beyond, two kernels), with ties,
 NaN, forced blocks, dense tails, chunks, a capacity that does not suffice, and scores that begin on any element."""
 import numpy as np
 import pytest
@@ -11,7 +12,8 @@ KW = [dict(mode=O.MODE_TOPK_RATIO, keep_num=1, keep_den=3, flags=3), dict(mode=O
 
 
 @pytest.mark.parametrize("lens,hq", [([5], 1), ([64 * 64], 8), ([64 * 64, 1], 8), ([64 * 64 + 1], 2), ([700, 0, 64, 4000, 65], 4), ([130] * 43, 4), ([64] * 511, 1), ([64] * 512, 1),
-                                     ([64] * 513, 1)])
+                                     ([64] * 513, 1), ([64 * 64], 4), ([64 * 49, 64 * 15, 1], 4), ([64 * 48], 8), ([64 * 48, 1], 8), ([64 * 64], 6), ([64 * 64, 1], 6),
+                                     ([64 * 49], 8), ([64 * 32], 16), ([64 * 33 - 5, 64 * 31], 6), ([64 * 33, 64 * 31], 8), ([64 * 32] * 2 + [64], 8)])
 @pytest.mark.parametrize("tail", [0, 2])
 def test_lists_of_few_short_rows(lens, hq, tail):
     import torch
@@ -20,7 +22,13 @@ def test_lists_of_few_short_rows(lens, hq, tail):
     rng = np.random.default_rng(len(lens) + hq)
     cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
     blocks = [(n + 63) // 64 for n in lens]
-    few = hq * sum(blocks) <= 512 and max(blocks) <= 64
+    rows = hq * sum(blocks)
+
+    def few(mode):
+        if mode == O.MODE_THRESHOLD:
+            return rows <= (512 if max(blocks) <= 32 else 384 if max(blocks) <= 64 else 0)
+        return rows <= (384 if max(blocks) <= 48 else 256 if max(blocks) <= 64 else 0)
+
     full = [np.round(rng.random((hq, nb, nb)), 1).astype(np.float32) for nb in blocks]
     for s in full:
         s[rng.random(s.shape) < 0.1] = np.nan
@@ -41,7 +49,7 @@ def test_lists_of_few_short_rows(lens, hq, tail):
                 p.nnz.fill_(-7)
                 before = B.seer_launch_count(p.ctx)
                 p.mask(params)
-                assert p.status() == 0 and B.seer_launch_count(p.ctx) - before == (2 if few else 3)
+                assert p.status() == 0 and B.seer_launch_count(p.ctx) - before == (2 if few(kw["mode"]) else 3)
                 got_rp, got = p.lists_host()
                 assert np.array_equal(got_rp, rp) and np.array_equal(got[:len(col)], col) and int(p.nnz.item()) == len(col)
                 if len(col) > 1:
