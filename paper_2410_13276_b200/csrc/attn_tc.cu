@@ -655,8 +655,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           lse_row = l > 0.f ? (R + log2f(l)) * 0.6931471805599453f : -CUDART_INF_F;
         }
         // The last P V of the item.  A warp whose wait for it is lost keeps the group's barriers and leaves afterwards.  Warps that hand each other
-        // partial rows agree on the outcome at their first exchange: one lost wait and none of them stores.  (A one-block list's rows are
-        // each a warp's own.)
+        // partial rows agree on the outcome between their first exchange and their first store: one lost wait and none of them stores.  (A
+        // one-block list's rows are each a warp's own.)
         fail = !mbar_wait(sh, bb + PV_DONE + (int)((cnt - 1) & 1u), ((cnt - 1) >> 1) & 1u, status);
         fail = __any_sync(0xffffffffu, fail);
         bool store = row < it.q_valid && !fail;
@@ -682,12 +682,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
               const float2 y = __fmul2_rn(make_float2(__uint_as_float(other[i][4 * c + 2]), __uint_as_float(other[i][4 * c + 3])), sc2);
               st_shared_v4(wr + (uint32_t)((c ^ (r & 7)) << 4), __float_as_uint(x.x), __float_as_uint(x.y), __float_as_uint(y.x), __float_as_uint(y.y));
             }
-            if (i == 0) {
-              tc_wait_ld32(mine[0]); tc_wait_ld32(other[1]); tc_wait_ld32(mine[1]);
-              fail = named_bar_or(bar_merge, kGroupThreads, fail);
-              store = store && !fail;
-              store_lse();
-            } else named_bar_sync(bar_merge, kGroupThreads);
+            if (i == 0) { tc_wait_ld32(mine[0]); tc_wait_ld32(other[1]); tc_wait_ld32(mine[1]); }
+            named_bar_sync(bar_merge, kGroupThreads);
             uint32_t out[16];
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
@@ -697,7 +693,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
               out[2 * c] = pack_bf16(x.x, x.y);
               out[2 * c + 1] = pack_bf16(y.x, y.y);
             }
-            if (i == 0) named_bar_sync(bar_merge, kGroupThreads);
+            if (i == 0) {                                   // (the vote on the first barrier: short lists 1 to 3 % slower)
+              fail = named_bar_or(bar_merge, kGroupThreads, fail);
+              store = store && !fail;
+              store_lse();
+            }
             if (store) {
               const uint32_t o0[8] = {out[0], out[1], out[2], out[3], out[4], out[5], out[6], out[7]};
               const uint32_t o1[8] = {out[8], out[9], out[10], out[11], out[12], out[13], out[14], out[15]};
