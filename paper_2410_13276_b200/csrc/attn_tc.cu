@@ -308,7 +308,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         auto locate = [&](int64_t w) {                     // which item comes next
           more = w < m.q_rows;
           nx = Item{};
-          if (more) nx = decode_item<kChunk>(m, row_ptr, w);
+          if (more) nx = decode_item<kChunk, kChunk || !kBlockMax>(m, row_ptr, w);
         };
         auto announce = [&](uint32_t n) -> bool {
           na0 = 0 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0) : -1;

@@ -622,7 +622,7 @@ seer_status gate_scores_static(const seer_shape* shape, const void* q, const voi
   m.score_elems = t.score_elems;
   m.softmax_scale = 0.f;   // unused by the gate
   m.block = shape->block;
-  m.qoff = nullptr; m.qdelta = nullptr; m.qblk_off = nullptr; m.order = nullptr; m.chunked = 0; m.q_rows = t.rows;
+  m.qoff = nullptr; m.qdelta = nullptr; m.qblk_off = nullptr; m.place = nullptr; m.chunked = 0; m.q_rows = t.rows;
   m.total_q_tokens = (int32_t)t.total_tokens;
   m.wait_limit_us = 0u; m.lose_v_copy = -1;   // unused by the gate
   m.score_tiles = 0; m.first_q_block = 0;

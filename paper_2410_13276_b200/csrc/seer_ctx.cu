@@ -8,15 +8,15 @@ namespace seer {
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Byte offsets of the arrays inside a metadata slot.
-constexpr size_t kOffCu = 0;
-constexpr size_t kOffBlk = kOffCu + sizeof(int32_t) * (kMaxBatch + 1 + 3);
-constexpr size_t kOffScore = kOffBlk + sizeof(int32_t) * (kMaxBatch + 1 + 3);
-constexpr size_t kOffQoff = kOffScore + sizeof(int64_t) * (kMaxBatch + 1);
-constexpr size_t kOffQdelta = kOffQoff + sizeof(int32_t) * (kMaxBatch + 4);
-constexpr size_t kOffQblk = kOffQdelta + sizeof(int32_t) * (kMaxBatch + 4);
-constexpr size_t kOffOrder = kOffQblk + sizeof(int32_t) * (kMaxBatch + 4);
-constexpr size_t kSlotBytes = kOffOrder + sizeof(int32_t) * (kMaxBatch + 4);
+// Byte offsets of the arrays inside a metadata slot: as long as the batch, so that a new shape's upload is.
+struct SlotLayout {
+  size_t place, score, cu, blk, qoff, qdelta, qblk, bytes;
+  explicit constexpr SlotLayout(int batch)
+      : place(0), score(place + sizeof(int4) * batch), cu(score + sizeof(int64_t) * (batch + 1)), blk(cu + sizeof(int32_t) * (batch + 1)),
+        qoff(blk + sizeof(int32_t) * (batch + 1)), qdelta(qoff + sizeof(int32_t) * batch), qblk(qdelta + sizeof(int32_t) * batch),
+        bytes(qblk + sizeof(int32_t) * (batch + 1)) {}
+};
+constexpr size_t kSlotBytes = (SlotLayout(kMaxBatch).bytes + 255) / 256 * 256;
 
 seer_status shape_totals(const seer_shape* s, ShapeTotals* t) {
   if (!s || !s->cu_seqlens_host || s->batch < 1) return SEER_ERR_INVALID_ARG;
@@ -78,6 +78,7 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
   if (st != SEER_OK) return st;
   if (cudaSetDevice(ctx->device) != cudaSuccess) return SEER_ERR_CUDA;
 
+  const SlotLayout at(shape->batch);
   const int n = shape->batch + 1;
   std::vector<int32_t> key(shape->cu_seqlens_host, shape->cu_seqlens_host + n);
   key.push_back(shape->num_q_heads);
@@ -106,13 +107,14 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
     }
     MetaSlot& s = ctx->slots[slot];
     char* h = (char*)s.pinned;
-    int32_t* cu = (int32_t*)(h + kOffCu);
-    int32_t* blk = (int32_t*)(h + kOffBlk);
-    int64_t* sc = (int64_t*)(h + kOffScore);
-    int32_t* qo = (int32_t*)(h + kOffQoff);
-    int32_t* qd = (int32_t*)(h + kOffQdelta);
-    int32_t* qb = (int32_t*)(h + kOffQblk);
-    int32_t* ord = (int32_t*)(h + kOffOrder);
+    int32_t* cu = (int32_t*)(h + at.cu);
+    int32_t* blk = (int32_t*)(h + at.blk);
+    int64_t* sc = (int64_t*)(h + at.score);
+    int32_t* qo = (int32_t*)(h + at.qoff);
+    int32_t* qd = (int32_t*)(h + at.qdelta);
+    int32_t* qb = (int32_t*)(h + at.qblk);
+    int4* place = (int4*)(h + at.place);
+    int32_t* order = qb + 1;                           // (its places are read before they become block counts)
     blk[0] = 0; sc[0] = 0; qb[0] = 0;
     for (int b = 0; b < shape->batch; ++b) {
       cu[b] = shape->cu_seqlens_host[b];
@@ -125,14 +127,22 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
         qo[b] = sq > 0 ? (sk - sq) / shape->block : nb;          // no queries: past the last block
         qd[b] = cq[b] - (shape->cu_seqlens_host[b] + (sk - sq));  // first query token <-> key token cu[b] + sk - sq
       }
-      ord[b] = b;
+      order[b] = b;
     }
-    // the attention works from the longest sequence to the shortest, so that the longest lists are not begun last (917 tokens
-    // against 60k in a batch of four, 512 items for 296 streams: 58 us in batch order, 49 so)
-    std::stable_sort(ord, ord + shape->batch, [blk](int32_t x, int32_t y) { return blk[x + 1] - blk[x] > blk[y + 1] - blk[y]; });
-    for (int p = 0; p < shape->batch; ++p) qb[p + 1] = qb[p] + blk[ord[p] + 1] - blk[ord[p]] - qo[ord[p]];
+    // The attention works from the longest sequence to the shortest, so that the longest lists are not begun last (917 tokens
+    // against 60k in a batch of four, 512 items for 296 streams: 58 us in batch order, 49 so).  Whole prompts of fewer than three items
+    // a stream stay in the batch's order: a sequence's lists are of every length then, and a stream's second item, which it draws when
+    // it begins its first, goes to the streams that begin first, those of the longest lists (prompts of 815 and 1965 tokens, 8
+    // heads, 352 items: 30 us, 34 longest first; 8 prompts of 90 to 6295, 16 heads, 2960 items: 165 and 157).
+    if (shape->cu_seqlens_q_host || (int64_t)blk[shape->batch] * shape->num_q_heads >= 6 * (int64_t)ctx->num_sms)
+      std::stable_sort(order, order + shape->batch, [blk](int32_t x, int32_t y) { return blk[x + 1] - blk[x] > blk[y + 1] - blk[y]; });
     cu[shape->batch] = shape->cu_seqlens_host[shape->batch];
-    if (cudaMemcpyAsync(s.dev, s.pinned, kSlotBytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SEER_ERR_CUDA;
+    for (int p = 0; p < shape->batch; ++p) {
+      const int b = order[p];
+      place[p] = make_int4(cu[b], cu[b + 1] - cu[b], blk[b], qd[b]);
+      qb[p + 1] = qb[p] + blk[b + 1] - blk[b] - qo[b];
+    }
+    if (cudaMemcpyAsync(s.dev, s.pinned, at.bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SEER_ERR_CUDA;
     if (cudaEventRecord(s.ready, stream) != cudaSuccess) return SEER_ERR_CUDA;
     s.key = key;
   } else {
@@ -142,9 +152,9 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
   MetaSlot& s = ctx->slots[slot];
   s.stamp = ++ctx->clock;
   const char* d = (const char*)s.dev;
-  m->cu_seqlens = (const int32_t*)(d + kOffCu);
-  m->blk_off = (const int32_t*)(d + kOffBlk);
-  m->score_off = (const int64_t*)(d + kOffScore);
+  m->cu_seqlens = (const int32_t*)(d + at.cu);
+  m->blk_off = (const int32_t*)(d + at.blk);
+  m->score_off = (const int64_t*)(d + at.score);
   m->batch = shape->batch;
   m->num_q_heads = shape->num_q_heads;
   m->num_kv_heads = shape->num_kv_heads;
@@ -156,10 +166,10 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
   m->score_elems = t.score_elems;
   m->softmax_scale = shape->softmax_scale > 0.f ? shape->softmax_scale : 0.08838834764831845f;  // 1/sqrt(128)
   m->block = shape->block;
-  m->qoff = (const int32_t*)(d + kOffQoff);
-  m->qdelta = (const int32_t*)(d + kOffQdelta);
-  m->qblk_off = (const int32_t*)(d + kOffQblk);
-  m->order = (const int32_t*)(d + kOffOrder);
+  m->qoff = (const int32_t*)(d + at.qoff);
+  m->qdelta = (const int32_t*)(d + at.qdelta);
+  m->qblk_off = (const int32_t*)(d + at.qblk);
+  m->place = (const int4*)(d + at.place);
   m->total_q_tokens = (int32_t)t.total_q_tokens;
   m->chunked = shape->cu_seqlens_q_host ? 1 : 0;
   double tiles = 0;

@@ -36,8 +36,8 @@ struct SeqMeta {
   // chunked prefill (all zero without a chunk): the queries of sequence b are its last positions
   const int32_t* qoff;         // [batch] block position of the chunk's first query block
   const int32_t* qdelta;       // [batch] token index in q / o / lse = token index in k / v + qdelta
-  // the attention's order of the sequences, the longest first
-  const int32_t* order;        // [batch] sequence at each place
+  // the attention's order of the sequences
+  const int4* place;           // [batch] (first token, tokens, first block, qdelta) of the sequence at each place
   const int32_t* qblk_off;     // [batch + 1] blocks with queries at the places before
   int32_t total_q_tokens;      // tokens in q / o / lse
   int32_t chunked;             // 1 if the shape carries cu_seqlens_q

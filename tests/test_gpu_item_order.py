@@ -1,5 +1,6 @@
-"""The attention visits the sequences of a batch from the longest to the shortest: results of batches in any order of lengths, with empty
-sequences and sequences without queries among them, equal those of each sequence by itself, bit for bit."""
+"""The attention visits the sequences of chunks, and of batches of three work items a stream and more, from the longest to the shortest, and others in
+the batch's order: results of batches in any order of lengths, with empty sequences and sequences without queries among them, equal those of
+each sequence by itself, bit for bit, on both sides of that line (888 items), and so do the block maxima."""
 import numpy as np
 import pytest
 
@@ -7,7 +8,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("lens,qlens", [([64, 1500, 1, 900, 0, 1500, 333], None), ([0, 0, 65, 700, 64, 700], None), ([700, 2000, 300, 2000, 128], [60, 80, 0, 16, 128]),
-                                        ([5000] + [70] * 40, [8] + [6] * 40)])
+                                        ([5000] + [70] * 40, [8] + [6] * 40), ([64 * 40, 0, 64 * 100 - 9, 64 * 7], None), ([64 * 41, 0, 64 * 100 - 9, 64 * 7], None)])
 def test_batch_equals_its_sequences(lens, qlens):
     import torch
     from paper_2410_13276_b200 import binding as B
@@ -27,12 +28,15 @@ def test_batch_equals_its_sequences(lens, qlens):
         p.mask(B.make_mask_params(B.SEER_TOPK_COUNT, k=1 << 20, flags=3))
         p.attn()
         assert p.status() == 0
-        return p.o, p.lse
+        return p.o, p.lse, (p.row_ptr.cpu(), p.block_max().clone(), p.status())
 
-    o, lse = attend(cu, cu_q, q, k, v)
+    o, lse, (rp, bmax, status) = attend(cu, cu_q, q, k, v)
     for b in range(len(lens)):
         if ql[b] == 0:
             continue
         s, e, qs, qe = cu[b], cu[b + 1], cu_q[b], cu_q[b + 1]
-        o1, lse1 = attend(np.array([0, e - s], np.int32), np.array([0, qe - qs], np.int32), q[qs:qe].contiguous(), k[s:e].contiguous(), v[s:e].contiguous())
+        o1, lse1, (rp1, bmax1, status1) = attend(np.array([0, e - s], np.int32), np.array([0, qe - qs], np.int32), q[qs:qe].contiguous(), k[s:e].contiguous(), v[s:e].contiguous())
         assert torch.equal(o1.view(torch.int16), o[qs:qe].view(torch.int16)) and torch.equal(lse1, lse[:, qs:qe])
+        at = hq * int(sum((n + 63) // 64 for n in lens[:b]))
+        assert status == status1 == 0
+        assert torch.equal(bmax[int(rp[at]):int(rp[at + len(rp1) - 1])], bmax1[:int(rp1[-1])])
