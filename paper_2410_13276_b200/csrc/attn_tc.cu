@@ -195,14 +195,13 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bo
 // What the roles need to know of a work item (decoded once, by the stream's Q / K producer).
 struct Slot {
   int h, i, l0, nlist, q_valid, s0, tok0;   // tok0: first row of the item in q / o / lse
-  int first[2];                             // the list's first two entries
+  int first[2];                             // the list's first two entries (not for the block maxima)
   __device__ __forceinline__ int ntiles() const { return (nlist + 1) >> 1; }
 };
 __device__ __forceinline__ int slot_block(const Slot& it, const int32_t* col_idx, int p) {
   return p < it.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + it.l0 + p) : -1;
 }
 // Block index of a list entry: -1 past the end of the list, -2 outside [0, i].
-__device__ __forceinline__ int list_entry(const Item& it, int p, int raw) { return p >= it.nlist ? -1 : (raw < 0 || raw > it.i) ? -2 : raw; }
 __device__ __forceinline__ int slot_check(const Slot& it, int p, int raw) {
   if (p >= it.nlist) return -1;
   return (raw < 0 || raw > it.i) ? -2 : raw;
@@ -279,6 +278,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     it.s0 = (int)b.x; it.tok0 = (int)b.y; it.first[0] = (int)b.z; it.first[1] = (int)b.w;
     return it;
   };
+  auto first_entry = [&](const Slot& it, int p) -> int { return kBlockMax ? slot_block(it, col_idx, p) : it.first[p]; };
   auto item_full = [&](int s, uint32_t n) -> int { return s * kBarsPerStream + ITEM_FULL + (int)(n & 3u); };
   auto release_item = [&](int s, uint32_t n) { mbar_arrive(sh.bar(s * kBarsPerStream + ITEM_EMPTY + (int)(n & 3u))); };
 
@@ -301,9 +301,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         uint32_t nitem = 0, cnt = 0, ku = 0, kph = 0;
         bool ok = true;
         // An item is decoded and announced while the one before it is copied: its row pointers and its first list entries are two
-        // trips to L2, one after the other, that every role of the stream would wait for at the item's start.
-        Item it{}, nx{};
-        int na0 = -1, nb0 = -1;                            // first entries of the next list
+        // trips to L2, one after the other, that every role of the stream would wait for at the item's start.  The block maxima take a tile in a
+        // quarter of the time, and copies that wait behind the two trips leave their group without tiles: they decode behind an item's last
+        // copy, and each role reads its entries (4096 tokens, 32 heads, an eighth listed: 21.5 us with all that in the middle of the copies, 19.7 so;
+        // over 50 random batches and chunks 3 to 5 % on average).
+        Item nx{};
         bool more = false;
         auto locate = [&](int64_t w) {                     // which item comes next
           more = w < m.q_rows;
@@ -311,8 +313,8 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           if (more) nx = decode_item<kChunk, kChunk || !kBlockMax>(m, row_ptr, w);
         };
         auto announce = [&](uint32_t n) -> bool {
-          na0 = 0 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0) : -1;
-          nb0 = 1 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0 + 1) : -1;
+          const int na0 = !kBlockMax && 0 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0) : -1;
+          const int nb0 = !kBlockMax && 1 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0 + 1) : -1;
           // the slot's previous content (item n - 4) has been read by everyone
           if (!mbar_wait(sh, bb + ITEM_EMPTY + (int)(n & 3u), ((n >> 2) & 1u) ^ 1u, status)) return false;
           const int tok0 = nx.s0 + nx.i * kBlock + (kChunk ? nx.dq : 0);
@@ -323,20 +325,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         };
         locate(draw());
         ok = announce(0);
-        for (uint32_t n = 0; ok && more; ++n) {
-          it = nx;
-          int ja = list_entry(it, 0, na0), jb = list_entry(it, 1, nb0);
+        for (uint32_t n = 0; ok; ++n) {
+          const Slot it = read_slot(s, n);                 // (its own announcement: two items in 56 registers are 1 % of a long launch)
+          if (it.nlist < 0) break;
+          int ja = slot_check(it, 0, first_entry(it, 0)), jb = slot_check(it, 1, first_entry(it, 1));
           const int64_t w = draw();                        // the next one is on its way while this one is copied
-          if (it.ntiles == 0) { locate(w); ok = announce(n + 1); continue; }
-          const int tok0 = it.s0 + it.i * kBlock + (kChunk ? it.dq : 0);
+          const int ntiles = it.ntiles(), g = it.h / m.group;
+          if (ntiles == 0) { locate(w); ok = announce(n + 1); continue; }
           const uint32_t qb = nitem & 1u;
           if (!mbar_wait(sh, bb + Q_EMPTY + (int)qb, ((nitem >> 1) & 1u) ^ 1u, status)) break;
           mbar_expect_tx(sh.bar(bb + Q_FULL + (int)qb), kQBytes);
-          tma_load_3d(sbase + kStQ + qb * kQBytes, &map_q, sh.bar(bb + Q_FULL + (int)qb), 0, it.h, tok0);
-          tma_load_3d(sbase + kStQ + qb * kQBytes + kHalfQ, &map_q, sh.bar(bb + Q_FULL + (int)qb), 64, it.h, tok0);
+          tma_load_3d(sbase + kStQ + qb * kQBytes, &map_q, sh.bar(bb + Q_FULL + (int)qb), 0, it.h, it.tok0);
+          tma_load_3d(sbase + kStQ + qb * kQBytes + kHalfQ, &map_q, sh.bar(bb + Q_FULL + (int)qb), 64, it.h, it.tok0);
           ++nitem;
-          for (int t = 0; t < it.ntiles; ++t, ++cnt) {
-            const int na = list_block(it, col_idx, 2 * t + 2), nb2 = list_block(it, col_idx, 2 * t + 3);   // next pair
+          for (int t = 0; t < ntiles; ++t, ++cnt) {
+            const int ra = slot_block(it, col_idx, 2 * t + 2), rb = slot_block(it, col_idx, 2 * t + 3);   // next pair
             if (ja == -2 || jb == -2) atomicCAS(status, 0, (int)SEER_ERR_INVALID_INDEX);
             const bool has_b = jb != -1;
             // a rejected entry: any valid block, masked out in the softmax
@@ -347,16 +350,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
               if (!mbar_wait(sh, bb + empty_k + (int)ku, kph ^ 1u, status)) { ok = false; break; }
               const uint32_t fb = sh.bar(bb + K_FULL + (int)ku), dst = sbase + kStK + ku * kUnit;
               mbar_expect_tx(fb, has_b ? kUnit : kUnit / 2);   // (an odd list's last tile: the scores of the missing block are not looked at)
-              tma_load_3d(dst, &map_k, fb, 64 * dh, it.g, ta);
-              if (has_b) tma_load_3d(dst + kHalfQ, &map_k, fb, 64 * dh, it.g, tb);
+              tma_load_3d(dst, &map_k, fb, 64 * dh, g, ta);
+              if (has_b) tma_load_3d(dst + kHalfQ, &map_k, fb, 64 * dh, g, tb);
               if (++ku == ring_k) { ku = 0; kph ^= 1u; }
             }
             tr.ev(2);
             if (!ok) break;
-            ja = na; jb = nb2;
-            if (t == 0) locate(w);
-            if (t == min(1, it.ntiles - 1) && !announce(n + 1)) { ok = false; break; }
+            ja = slot_check(it, 2 * t + 2, ra); jb = slot_check(it, 2 * t + 3, rb);
+            if (!kBlockMax && t == 0) locate(w);
+            if (!kBlockMax && t == min(1, ntiles - 1) && !announce(n + 1)) { ok = false; break; }
           }
+          if (kBlockMax && ok) { locate(w); ok = announce(n + 1); }
         }
       }
     }
@@ -532,7 +536,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         }
         continue;
       }
-      int raw = half ? it.first[1] : it.first[0];
+      int raw = kBlockMax ? slot_block(it, col_idx, half) : half ? it.first[1] : it.first[0];
       tr.ev(36);
       if constexpr (kBlockMax) {
         int* wmax = reinterpret_cast<int*>(smem + kOffMl + s * kMlBytes);   // [2 tile parities][4 warps]: maxima as order-preserving integers

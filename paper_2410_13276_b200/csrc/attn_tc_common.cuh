@@ -250,13 +250,6 @@ __device__ __forceinline__ Item decode_item(const SeqMeta& m, const int32_t* row
   return it;
 }
 
-// Block index of list position p of an item: -1 past the end of the list, -2 for an entry outside [0, i].
-__device__ __forceinline__ int list_block(const Item& it, const int32_t* col_idx, int p) {
-  if (p >= it.nlist) return -1;
-  const int j = col_idx[it.l0 + p];
-  return (j < 0 || j > it.i) ? -2 : j;
-}
-
 // Optional cycle accounting of CTA 0 (diagnostics): every role attributes the clocks between two consecutive marks to the
 // tag of the later mark and adds them, and the mark, to trace[role * 8192 + tag * 2 ...] (reductions: nothing is waited for).
 template <bool ON>
