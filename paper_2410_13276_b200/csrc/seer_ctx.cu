@@ -18,6 +18,24 @@ struct SlotLayout {
 };
 constexpr size_t kSlotBytes = (SlotLayout(kMaxBatch).bytes + 255) / 256 * 256;
 
+// Uploads are staged one behind the other in a page-locked ring of two slots of the largest batch: page-locking is what creating a
+// context is bound by (by the megabyte), and a batch of 64 needs 3 KB of it.
+constexpr size_t kStageBytes = 2 * kSlotBytes;
+
+// Room for `bytes` in the ring, for the upload of slot `slot`; waits for uploads still in flight that lie there.
+static char* stage_room(seer_ctx* ctx, int slot, size_t bytes) {
+  size_t at = ctx->stage_pos;
+  if (at + bytes > kStageBytes) at = 0;
+  for (int i = 0; i < kMetaSlots; ++i) {
+    const MetaSlot& o = ctx->slots[i];
+    if (i != slot && o.stage_lo < at + bytes && at < o.stage_hi && cudaEventSynchronize(o.ready) != cudaSuccess) return nullptr;
+  }
+  ctx->slots[slot].stage_lo = at;
+  ctx->slots[slot].stage_hi = at + bytes;
+  ctx->stage_pos = align_up(at + bytes, 256);
+  return (char*)ctx->stage + at;
+}
+
 seer_status shape_totals(const seer_shape* s, ShapeTotals* t) {
   if (!s || !s->cu_seqlens_host || s->batch < 1) return SEER_ERR_INVALID_ARG;
   if (s->num_q_heads < 1 || s->num_kv_heads < 1) return SEER_ERR_INVALID_ARG;
@@ -106,7 +124,8 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
       if (cudaEventSynchronize(ctx->slots[slot].ready) != cudaSuccess) return SEER_ERR_CUDA;
     }
     MetaSlot& s = ctx->slots[slot];
-    char* h = (char*)s.pinned;
+    char* h = stage_room(ctx, slot, at.bytes);
+    if (h == nullptr) return SEER_ERR_CUDA;
     int32_t* cu = (int32_t*)(h + at.cu);
     int32_t* blk = (int32_t*)(h + at.blk);
     int64_t* sc = (int64_t*)(h + at.score);
@@ -142,7 +161,7 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
       place[p] = make_int4(cu[b], cu[b + 1] - cu[b], blk[b], qd[b]);
       qb[p + 1] = qb[p] + blk[b + 1] - blk[b] - qo[b];
     }
-    if (cudaMemcpyAsync(s.dev, s.pinned, at.bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SEER_ERR_CUDA;
+    if (cudaMemcpyAsync(s.dev, h, at.bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SEER_ERR_CUDA;
     if (cudaEventRecord(s.ready, stream) != cudaSuccess) return SEER_ERR_CUDA;
     s.key = key;
   } else {
@@ -300,17 +319,18 @@ seer_status seer_create(seer_ctx** out, int device) {
   int count = 0;
   if (cudaGetDeviceCount(&count) != cudaSuccess || device < 0 || device >= count) return SEER_ERR_CUDA;
   if (cudaSetDevice(device) != cudaSuccess) return SEER_ERR_CUDA;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) return SEER_ERR_CUDA;
-  if (prop.major != 10) return SEER_ERR_CUDA;  // kernels are built for sm_100a only
+  int major = 0, sms = 0;                            // (all of a device's properties take 2.5 ms)
+  if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return SEER_ERR_CUDA;
+  if (major != 10) return SEER_ERR_CUDA;  // kernels are built for sm_100a only
   seer_ctx* ctx = new seer_ctx();
   ctx->device = device;
-  ctx->num_sms = prop.multiProcessorCount;
+  ctx->num_sms = sms;
   bool ok = cudaMalloc(&ctx->d_status, sizeof(int)) == cudaSuccess &&
-            cudaMemset(ctx->d_status, 0, sizeof(int)) == cudaSuccess;
+            cudaMemset(ctx->d_status, 0, sizeof(int)) == cudaSuccess && cudaMallocHost(&ctx->stage, kStageBytes) == cudaSuccess;
   for (int i = 0; ok && i < kMetaSlots; ++i) {
     MetaSlot& s = ctx->slots[i];
-    ok = cudaMalloc(&s.dev, kSlotBytes) == cudaSuccess && cudaMallocHost(&s.pinned, kSlotBytes) == cudaSuccess &&
+    ok = cudaMalloc(&s.dev, kSlotBytes) == cudaSuccess &&
          cudaEventCreateWithFlags(&s.ready, cudaEventDisableTiming) == cudaSuccess &&
          cudaEventCreateWithFlags(&s.last_use, cudaEventDisableTiming) == cudaSuccess;
   }
@@ -335,11 +355,11 @@ void seer_destroy(seer_ctx* ctx) {
   for (int i = 0; i < kMetaSlots; ++i) {
     MetaSlot& s = ctx->slots[i];
     if (s.dev) cudaFree(s.dev);
-    if (s.pinned) cudaFreeHost(s.pinned);
     if (s.ready) cudaEventDestroy(s.ready);
     if (s.last_use) cudaEventDestroy(s.last_use);
   }
   if (ctx->d_status) cudaFree(ctx->d_status);
+  if (ctx->stage) cudaFreeHost(ctx->stage);
   if (ctx->h2d_stream) cudaStreamDestroy(ctx->h2d_stream);
   if (ctx->d2h_stream) cudaStreamDestroy(ctx->d2h_stream);
   if (ctx->ev_start) cudaEventDestroy(ctx->ev_start);

@@ -94,7 +94,7 @@ __device__ __forceinline__ int64_t score_row_offset(const SeqMeta& m, const Scor
 struct MetaSlot {
   std::vector<int32_t> key;    // cu_seqlens + Hq: what the slot currently describes
   void* dev = nullptr;
-  void* pinned = nullptr;
+  size_t stage_lo = 0, stage_hi = 0;   // where the staging ring holds what was uploaded last
   cudaEvent_t ready = nullptr;     // upload finished
   cudaEvent_t last_use = nullptr;  // last library call that read the slot
   uint64_t stamp = 0;
@@ -110,6 +110,8 @@ struct seer_ctx {
   int64_t launches = 0;
   uint64_t clock = 0;
   seer::MetaSlot slots[seer::kMetaSlots];
+  void* stage = nullptr;           // page-locked ring the slots' uploads start from
+  size_t stage_pos = 0;
   void* tmap_encode = nullptr;   // cuTensorMapEncodeTiled, resolved at run time
   void* trace = nullptr;         // optional device buffer for the attention kernel's timeline (diagnostics)
   uint32_t wait_limit_us = 2000000u;   // seer_debug_lost_wait
