@@ -89,7 +89,7 @@ size_t gate_stats_bytes(const ShapeTotals& t, const seer_shape* s) {
   return align_up((size_t)s->num_q_heads * t.total_blocks * gate_stat_segs(t.max_nb) * sizeof(float2), 256);
 }
 
-seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream, SeqMeta* m, int* slot_out) {
+seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream, SeqMeta* m, int* slot_out, int keep) {
   if (!ctx) return SEER_ERR_INVALID_ARG;
   ShapeTotals t;
   seer_status st = shape_totals(shape, &t);
@@ -110,8 +110,9 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
     // in flight (more than kMetaSlots shapes cycling faster than the GPU works through them) does the call wait
     // for the oldest one
     slot = -1;
-    int oldest = 0;
+    int oldest = keep == 0 ? 1 : 0;
     for (int i = 0; i < kMetaSlots; ++i) {
+      if (i == keep) continue;
       if (ctx->slots[i].stamp < ctx->slots[oldest].stamp) oldest = i;
       if (cudaEventQuery(ctx->slots[i].last_use) == cudaSuccess && cudaEventQuery(ctx->slots[i].ready) == cudaSuccess &&
           (slot < 0 || ctx->slots[i].stamp < ctx->slots[slot].stamp))
@@ -655,7 +656,7 @@ seer_status seer_expand_block_lists(seer_ctx* ctx, const seer_shape* shape, cons
   SeqMeta m128, m64; int slot128, slot64;
   st = prepare(ctx, shape, stream, &m128, &slot128);
   if (st != SEER_OK) return st;
-  st = prepare(ctx, &fine, stream, &m64, &slot64);
+  st = prepare(ctx, &fine, stream, &m64, &slot64, slot128);
   if (st != SEER_OK) { finish_call(ctx, slot128, stream); return st; }
   int n = launch_expand_lists(ctx, m128, m64, row_ptr, col_idx, row_ptr64, col_idx64, col_capacity64, nnz_out, stream);
   finish_call(ctx, slot128, stream);

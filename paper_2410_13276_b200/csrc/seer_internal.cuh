@@ -125,8 +125,9 @@ struct seer_ctx {
 namespace seer {
 
 // Validates the shape, makes its metadata resident on the device (ordered before later work on `stream`)
-// and fills `m`.  `slot_out` identifies the slot to pass to finish_call.
-seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream, SeqMeta* m, int* slot_out);
+// and fills `m`.  `slot_out` identifies the slot to pass to finish_call.  `keep`: a slot that the same call has prepared before, which
+// is not taken for this shape though nothing in flight reads it yet.
+seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream, SeqMeta* m, int* slot_out, int keep = -1);
 void finish_call(seer_ctx* ctx, int slot, cudaStream_t stream);
 // Whether tensors that the kernels copy 16 bytes at a time begin on 16 bytes (a misaligned access would end the context).
 bool on_16(const void* a, const void* b, const void* c = nullptr, const void* d = nullptr);

@@ -35,3 +35,39 @@ def test_calls_of_many_shapes_in_flight(batches):
         assert B.seer_poll_device_status(ctx) == 0
         for shape, scores, ((rp, col), (rp1, col1)) in calls:
             assert torch.equal(rp, rp1) and torch.equal(col, col1)
+
+
+def test_the_two_shapes_of_an_expansion_have_a_slot_each():
+    """seer_expand_block_lists reads the offsets of the 128-token and of the 64-token blocks.  With every other slot in flight on a busy stream the
+    second shape must not take the slot of the first."""
+    import torch
+    from paper_2410_13276_b200 import binding as B
+    ctx = B.Context(0)
+    params = B.make_mask_params(B.SEER_TOPK_COUNT, k=2, flags=1)
+    cu = np.array([0, 700, 1000], np.int32)
+    shape = B.make_shape(cu, 2, 1, block=128)
+    rows, rows64 = B.seer_mask_rows(shape), 2 * (11 + 5)
+    scores = torch.rand(B.seer_scores_elems(shape), device="cuda")
+    lists = lambda n, m: (torch.full((n + 1,), -7, dtype=torch.int32, device="cuda"), torch.full((m,), -7, dtype=torch.int32, device="cuda"))
+    rp, col = lists(rows, B.seer_causal_blocks(shape))
+    B.seer_block_mask(ctx, shape, scores, params, rp, col)
+    assert B.seer_poll_device_status(ctx) == 0
+    ref, out = lists(rows64, 4 * col.numel()), lists(rows64, 4 * col.numel())
+    alone = B.Context(0)
+    B.seer_expand_block_lists(alone, shape, rp, col, *ref)
+    assert B.seer_poll_device_status(alone) == 0
+    busy, side = torch.randn(4096, 4096, device="cuda"), torch.cuda.Stream()
+    others = []
+    for n in range(7):                                    # eight slots in all
+        s = B.make_shape([0, 640 + 64 * n], 1, 1)
+        others.append((s, torch.rand(B.seer_scores_elems(s), device="cuda"), *lists(B.seer_mask_rows(s), B.seer_causal_blocks(s))))
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        for _ in range(30):
+            busy = busy @ busy * 1e-3
+        for s, x, r, c in others:
+            B.seer_block_mask(ctx, s, x, params, r, c)
+    B.seer_expand_block_lists(ctx, shape, rp, col, *out)
+    torch.cuda.synchronize()
+    assert B.seer_poll_device_status(ctx) == 0
+    assert torch.equal(out[0], ref[0]) and torch.equal(out[1], ref[1])
