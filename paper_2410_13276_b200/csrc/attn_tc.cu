@@ -3,10 +3,12 @@
 // What bounds it.  Long lists: the copies of K and V into shared memory (64 KB per pair of listed 64 x 64 blocks, about 885 clocks
 // at the 74 bytes a clock that an SM takes from L2, of 917 to 1060 that a pair takes), close before the MMA pipe (8 x 48 + 4 x 76 =
 // 688 clocks: 75 % active on dense lists of 16k tokens), and in launches of more than a few milliseconds the board's power limit.
-// Short lists: an item's start and end, about 4800 clocks beside 2000 for a stream's tile.  Of them the wait for the last P V 1300, merge and
-// stores 2700; everything that needs no O is done during the wait, and an item's row pointers and first list entries are fetched
-// while the item before it is copied.  With those after the wait, the entries fetched at the item's start, and producers that slept between
-// their polls: 6000 clocks; 24 prompts of 16 900 tokens 173 us where this takes 163, 32k tokens 1384 and 1335, 128k 16.7 and 16.1 ms.
+// Short lists: an item's start and end, about 5000 clocks beside 1900 for a stream's tile.  Of them the wait for the last P V 1400, merge and
+// stores 3000 (2700 without instrumentation); everything that needs no O is done during the wait, and an item's row pointers and first list
+// entries are fetched while the item before it is copied.  With those after the wait, the entries fetched at the item's start, and
+// producers that slept between their polls: 6000 clocks; the launch by itself, both in turn: 24 prompts of 16 900 tokens 174 us where this
+// takes 166, 32k tokens 1232 and 1174, 48k 2557 and 2480, 128k 16.7 and 16.1 ms; dense 2000-token prompts 435 and 432.  (A whole pass, which runs
+// hotter: 3 % on short prompts, 1 to 2 on long ones.)
 //
 // Tiles.  A query block is 64 rows and every (head, query block) has its own list, so no two items share their keys.
 // The MMAs are the weight-stationary form (tcgen05.mma.ws) with M = 64: the 128 lanes of tensor memory hold two 64-row
@@ -61,8 +63,8 @@ constexpr int kPolyPairsOf8 = 2;
 constexpr uint32_t kHalfQ = 64 * 128;            // bytes of one d half of a 64-row tile (8 KB)
 constexpr uint32_t kQBytes = 2 * kHalfQ;         // 16 KB
 constexpr uint32_t kUnit = 16384;                // a K or V unit
-// Ring depths per stream: three K units and two V units (two and three: 128k tokens 16.3 ms where this takes 16.1, 32k 1379 and 1355 us, dense 16k
-// 2505 and 2464).
+// Ring depths per stream: three K units and two V units (two and three: 128k tokens 16.33 ms where this takes 16.15 to 16.25, 32k 1201 and 1174 us,
+// dense 16k 2481 and 2450, short prompts 0.5 % slower; the launch by itself).
 constexpr uint32_t kKUnits = 3, kVUnits = 2;
 // shared memory map (offsets from a 1024-byte aligned base); the big buffers of a stream are contiguous
 constexpr uint32_t kStQ = 0, kStK = 2 * kQBytes, kStV = kStK + kKUnits * kUnit;
@@ -212,7 +214,8 @@ __device__ __forceinline__ int slot_check(const Slot& it, int p, int raw) {
 // probability exp(scale * s - lse) of its 64 x 64 tile (Sec. 3.2, Eq. 2 on the listed blocks), `lse` being an input: a
 // thread takes the maximum of its row, a block's maximum is one redux per warp and a word from its neighbour.
 // Without V and O a stream has five K units and four S buffers: with two of each it waits for copies and MMAs in turn (16k tokens, 32
-// heads, all causal blocks: 1277 us and 1060 so, 520 clocks a tile; 440 are its 32 KB from L2, 384 its MMAs).
+// heads, all causal blocks: 1277 us and 1060 so when both were timed on a cool board, 520 clocks a tile; 440 are its 32 KB from L2, 384 its
+// MMAs; 1160 to 1210 us behind an attention launch).
 // kO32: o begins on 32 bytes.  (A test of the address in the kernel instead: 32k tokens 1392 -> 1404 us.)
 template <bool kTrace, bool kChunk, bool kBlockMax = false, bool kO32 = true>
 __global__ void __launch_bounds__(kThreads, 1)
