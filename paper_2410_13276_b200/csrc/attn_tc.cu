@@ -49,17 +49,11 @@ namespace tc {
 using namespace tcc;
 
 constexpr int kThreads = 512;
-constexpr float kNoRef = -1e30f;   // reference of a row that has not seen a live block
-// A tile whose row sum reaches this moves the row's reference: 2^60 above the first block's maximum, far from the 2^127 at
-// which P or the sums would overflow, and far above what a prompt's sink or stripes rise (a move costs about two tiles).
-constexpr float kRise = 1.152921504606847e18f;   // 2^60
 // Registers of the helpers' and the softmax warpgroups, two each: 2 * (helper + softmax) * 128 = 65536.  (The softmax pass wants 200; the
 // block maxima want less, and their producer spills with 56.)
 template <bool kBlockMax> constexpr int kHelperRegs = kBlockMax ? 64 : 56;
 template <bool kBlockMax> constexpr int kSoftmaxRegs = 256 - kHelperRegs<kBlockMax>;
 constexpr int kGroupThreads = 128;
-// of every eight pairs of a pass this many take their exponentials on the FMA pipe (0, 1 and 3 measured within 2 % of it)
-constexpr int kPolyPairsOf8 = 2;
 constexpr uint32_t kHalfQ = 64 * 128;            // bytes of one d half of a 64-row tile (8 KB)
 constexpr uint32_t kQBytes = 2 * kHalfQ;         // 16 KB
 constexpr uint32_t kUnit = 16384;                // a K or V unit
@@ -91,108 +85,6 @@ __device__ __forceinline__ uint32_t col_o(int s) { return (uint32_t)s * 256u + 1
 
 constexpr uint32_t kIdescS = make_idesc(false, false, 128u, 64u);
 constexpr uint32_t kIdescPV = make_idesc(false, true, 256u, 64u);
-
-__device__ __forceinline__ bool mbar_test(uint32_t addr, uint32_t parity) {
-  uint32_t done;
-  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-               : "=r"(done) : "r"(addr), "r"(parity) : "memory");
-  return done != 0;
-}
-
-// 2^x for two values at once on the FMA pipe (the special-function unit does 16 exponentials per clock and SM): x = n + f
-// with n = round(x), 2^f by a cubic (relative error 7.5e-5, far below the bf16 rounding of P), 2^n by adding n to the
-// exponent field.  x is clamped to [-125, 128] so that the exponent field stays in 1..255: below gives ~2^-125, above
-// something no smaller than 2^127, which the caller's test of the sum sees; so does a NaN, which the clamp lets through.
-__device__ __forceinline__ float clamp_nan(float x) {
-  float y;
-  asm("max.NaN.f32 %0, %1, 0fC2FA0000;" : "=f"(y) : "f"(x));   // -125
-  asm("min.NaN.f32 %0, %1, 0f43000000;" : "=f"(x) : "f"(y));   // 128
-  return x;
-}
-__device__ __forceinline__ float2 exp2_poly2(float2 x) {
-  x.x = clamp_nan(x.x); x.y = clamp_nan(x.y);
-  const float2 magic = make_float2(12582912.f, 12582912.f);        // 1.5 * 2^23: the sum's low mantissa bits are round(x)
-  const float2 t = __fadd2_rn(x, magic);
-  const float2 n = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
-  const float2 f = __fadd2_rn(x, make_float2(-n.x, -n.y));         // in [-0.5, 0.5]
-  float2 r = __ffma2_rn(make_float2(0.05517168343067169f, 0.05517168343067169f), f, make_float2(0.2426111251115799f, 0.2426111251115799f));
-  r = __ffma2_rn(r, f, make_float2(0.6932609677314758f, 0.6932609677314758f));
-  r = __ffma2_rn(r, f, make_float2(0.9999280571937561f, 0.9999280571937561f));
-  r.x = __int_as_float(__float_as_int(r.x) + (__float_as_int(t.x) << 23));
-  r.y = __int_as_float(__float_as_int(r.y) + (__float_as_int(t.y) << 23));
-  return r;
-}
-
-// One pass over this thread's row of a 64 x 64 block of scores: p = 2^(sl2 * s - R), packed to bf16 pairs in pk; returns the
-// sum of the row.  kPolyPairsOf8 of every eight pairs take their exponentials on the FMA pipe, the others on the
-// special-function unit.  MASKED: the causal mask of the diagonal block (keys after `row` are dropped).
-template <bool MASKED>
-__device__ __forceinline__ float row_pass(uint32_t s_addr, float sl2, float R, int row, uint32_t (&pk)[32]) {
-  const float2 sl22 = make_float2(sl2, sl2), nr = make_float2(-R, -R);
-  float2 acc[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.f, 0.f);
-  // two TMEM round trips: the second half is requested before the first is worked on
-  uint32_t sv[2][32];
-  tc_ld32(s_addr, sv[0]);
-#pragma unroll
-  for (int ch = 0; ch < 2; ++ch) {
-    tc_wait_ld32(sv[ch]);
-    if (ch == 0) tc_ld32(s_addr + 32, sv[1]);
-    // stage by stage over the 32 keys, each stage a run of independent instructions, in place
-    float2 v[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __ffma2_rn(make_float2(__uint_as_float(sv[ch][2 * i]), __uint_as_float(sv[ch][2 * i + 1])), sl22, nr);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      if ((i & 7) < kPolyPairsOf8) v[i] = exp2_poly2(v[i]);
-      else v[i] = make_float2(ex2f(v[i].x), ex2f(v[i].y));
-    }
-    if (MASKED) {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int c = ch * 32 + 2 * i;
-        if (c > row) v[i].x = 0.f;
-        if (c + 1 > row) v[i].y = 0.f;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) pk[ch * 16 + i] = pack_bf16(v[i].x, v[i].y);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i & 3] = __fadd2_rn(acc[i & 3], v[i]);
-  }
-  const float2 a = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
-  return a.x + a.y;
-}
-
-// The largest raw score of this thread's row (MASKED: among the keys it sees, key <= last; -inf if there is none).
-// Off the diagonal the 64 predicates are left out (with them a 128k prompt takes 2 % longer).
-template <bool MASKED>
-__device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
-  float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
-  uint32_t sv[2][32];
-  tc_ld32(s_addr, sv[0]);
-  tc_ld32(s_addr + 32, sv[1]);
-  tc_wait_ld32(sv[0]);
-  tc_wait_ld32(sv[1]);
-#pragma unroll
-  for (int ch = 0; ch < 2; ++ch)
-#pragma unroll
-    for (int e = 0; e < 32; ++e)
-      if (!MASKED || ch * 32 + e <= last) mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(sv[ch][e]));
-  return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
-}
-
-// 32 bytes, at once where the address allows it (the host asks for 16)
-__device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bool aligned) {
-  if (!aligned) {
-    reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    return;
-  }
-  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]),
-               "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-}
 
 // What the roles need to know of a work item (decoded once, by the stream's Q / K producer).
 struct Slot {
@@ -583,62 +475,40 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
       for (int t = 0; t < ntiles; ++t, ++cnt) {
         const uint32_t buf = cnt & 1u;
         tr.sample(cnt);
-        const int j = slot_check(it, 2 * t + half, raw);    // (uniform in the warp)
+        const int here = raw;                               // (uniform in the warp; -1 past the list's end)
         raw = slot_block(it, col_idx, 2 * t + 2 + half);    // the next tile's list entry: looked at when its turn comes
         tr.ev(31);
-        fail = !mbar_wait(sh, bb + S_FULL + (int)buf, (cnt >> 1) & 1u, status);
-        if (__any_sync(0xffffffffu, fail)) { fail = true; break; }
+        fail = !mbar_wait_warp(sh, bb + S_FULL + (int)buf, (cnt >> 1) & 1u, status);
+        if (fail) break;
         tr.ev(32);
         tc_fence_after();
         const uint32_t s_addr = tmem + lane_addr + col_s(s, buf);
-        uint32_t pk[32];
-        if (j < 0) {                                        // absent or rejected: contributes nothing
-#pragma unroll
-          for (int i = 0; i < 32; ++i) pk[i] = 0u;
-        } else {
-          const bool diag = j == it.i;
+        if ((uint32_t)here < (uint32_t)it.i) {              // the plain pass: a block before the diagonal
           if (t == 0) {
-            const float mx = diag ? row_max<true>(s_addr, row) : row_max<false>(s_addr, 63);
+            const float mx = row_max<false>(s_addr, 63);
             if (fabsf(mx) < 3.0e38f) R = mx * sl2;
           }
-          float sum = diag ? row_pass<true>(s_addr, sl2, R, row, pk) : row_pass<false>(s_addr, sl2, R, row, pk);
-          const bool over = !(sum < kRise);
-          if (__any_sync(0xffffffffu, over)) {
-            // ---- some row's reference has to move (or its scores are not finite): O at rest, rows rescaled, tile taken again
-            if (t > 0) {
-              fail = !mbar_wait(sh, bb + PV_DONE + (int)(buf ^ 1u), ((cnt - 1) >> 1) & 1u, status);
-              if (__any_sync(0xffffffffu, fail)) { fail = true; break; }
-              tc_fence_after();
-            }
-            const float mx = row_max<true>(s_addr, diag ? row : 63) * sl2;
-            const float nr = over && fabsf(mx) < 3.0e38f ? fmaxf(R, mx) : R;
-            const float alpha = nr == R ? 1.f : exp2f(R - nr);
-            R = nr;
-            l = alpha == 0.f ? 0.f : __fmul_rn(l, alpha);
-            if (t > 0) {
-#pragma unroll 1
-              for (int ch = 0; ch < 8; ++ch) {
-                uint32_t ov[16];
-                tc_ld16(o_addr + ch * 16, ov);
-                tc_wait_ld(ov);
-#pragma unroll
-                for (int e = 0; e < 16; ++e) ov[e] = alpha == 0.f ? 0u : __float_as_uint(__uint_as_float(ov[e]) * alpha);
-                tc_st16(o_addr + ch * 16, ov);
-              }
-            }
-            sum = diag ? row_pass<true>(s_addr, sl2, R, row, pk) : row_pass<false>(s_addr, sl2, R, row, pk);
-            if (!(sum < kRise)) sum = CUDART_NAN_F;         // an infinite score or a NaN: so is the row
-            tr.ev(40);
+          uint32_t pk[32];
+          const float sum = row_pass<false>(s_addr, sl2, R, 63, pk);
+          if (!__any_sync(0xffffffffu, !(sum < kRise))) {
+            l = __fadd_rn(l, sum);
+            tr.ev(33);
+            tc_st32(s_addr, pk);                            // P over the scores this thread has read
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sh.bar(bb + P_FULL + (int)buf));
+            tr.ev(34);
+            continue;
           }
-          l = __fadd_rn(l, sum);
         }
-        tr.ev(33);
-        tc_st32(s_addr, pk);                                // P over the scores this thread has read
-        tc_wait_st();
-        tc_fence_before();
+        const float4 x = other_tile(sh, s_addr, o_addr, sl2, R, l, (uint32_t)here > (uint32_t)it.i ? -1 : here == it.i ? row : 63, t == 0 && here == it.i, t,
+                                    bb + PV_DONE + (int)(buf ^ 1u), ((cnt - 1) >> 1) & 1u, status);
+        R = x.x; l = x.y; fail = x.z != 0.f;
+        if (fail) break;
         __syncwarp();
         if (lane == 0) mbar_arrive(sh.bar(bb + P_FULL + (int)buf));
-        tr.ev(34);
+        tr.ev(40);
       }
       if constexpr (!kBlockMax) {
         // ---------------------------------------------------------------------------------------- epilogue: merge, store

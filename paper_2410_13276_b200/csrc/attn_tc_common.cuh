@@ -95,6 +95,15 @@ __device__ __forceinline__ bool mbar_wait(const Shared& sh, int bar, uint32_t pa
   return false;
 }
 
+// The same by a converged warp; the outcome is the warp's, from one vote where the phase is complete.
+__device__ __forceinline__ bool mbar_wait_warp(const Shared& sh, int bar, uint32_t parity, int* status) {
+  uint32_t done;
+  asm volatile("{\n\t.reg .pred p, q;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tvote.sync.all.pred q, p, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(done) : "r"(sh.bar(bar)), "r"(parity) : "memory");
+  if (done) return true;
+  return __all_sync(0xffffffffu, mbar_wait(sh, bar, parity, status));
+}
+
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
   asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
                ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
@@ -290,6 +299,171 @@ constexpr uint32_t make_idesc(bool a_mn_major, bool b_mn_major, uint32_t n = 64u
          ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 
+// ------------------------------------------------------------------------------------------------ softmax of the attention
+constexpr float kNoRef = -1e30f;   // reference of a row that has not seen a live block
+// A tile whose row sum reaches this moves the row's reference: 2^60 above the first block's maximum, far from the 2^127 at
+// which P or the sums would overflow, and far above what a prompt's sink or stripes rise (a move costs about two tiles).
+constexpr float kRise = 1.152921504606847e18f;   // 2^60
+// of every eight pairs of a pass this many take their exponentials on the FMA pipe (0, 1 and 3 measured within 2 % of it)
+constexpr int kPolyPairsOf8 = 2;
+
+__device__ __forceinline__ bool mbar_test(uint32_t addr, uint32_t parity) {
+  uint32_t done;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(done) : "r"(addr), "r"(parity) : "memory");
+  return done != 0;
+}
+
+// 2^x for two values at once on the FMA pipe (the special-function unit does 16 exponentials per clock and SM): x = n + f
+// with n = round(x), 2^f by a cubic (relative error 7.5e-5, far below the bf16 rounding of P), 2^n by adding n to the
+// exponent field.  x is clamped to [-125, 128] so that the exponent field stays in 1..255: below gives ~2^-125, above
+// something no smaller than 2^127, which the caller's test of the sum sees; so does a NaN, which the clamp lets through.
+__device__ __forceinline__ float clamp_nan(float x) {
+  float y;
+  asm("max.NaN.f32 %0, %1, 0fC2FA0000;" : "=f"(y) : "f"(x));   // -125
+  asm("min.NaN.f32 %0, %1, 0f43000000;" : "=f"(x) : "f"(y));   // 128
+  return x;
+}
+__device__ __forceinline__ float2 exp2_poly2(float2 x) {
+  x.x = clamp_nan(x.x); x.y = clamp_nan(x.y);
+  const float2 magic = make_float2(12582912.f, 12582912.f);        // 1.5 * 2^23: the sum's low mantissa bits are round(x)
+  const float2 t = __fadd2_rn(x, magic);
+  const float2 n = __fadd2_rn(t, make_float2(-12582912.f, -12582912.f));
+  const float2 f = __fadd2_rn(x, make_float2(-n.x, -n.y));         // in [-0.5, 0.5]
+  float2 r = __ffma2_rn(make_float2(0.05517168343067169f, 0.05517168343067169f), f, make_float2(0.2426111251115799f, 0.2426111251115799f));
+  r = __ffma2_rn(r, f, make_float2(0.6932609677314758f, 0.6932609677314758f));
+  r = __ffma2_rn(r, f, make_float2(0.9999280571937561f, 0.9999280571937561f));
+  r.x = __int_as_float(__float_as_int(r.x) + (__float_as_int(t.x) << 23));
+  r.y = __int_as_float(__float_as_int(r.y) + (__float_as_int(t.y) << 23));
+  return r;
+}
+
+// One pass over this thread's row of a 64 x 64 block of scores: p = 2^(sl2 * s - R), packed to bf16 pairs in pk; returns the
+// sum of the row.  kPolyPairsOf8 of every eight pairs take their exponentials on the FMA pipe, the others on the
+// special-function unit.  MASKED: the causal mask of the diagonal block (keys after `row` are dropped).
+template <bool MASKED>
+__device__ __forceinline__ float row_pass(uint32_t s_addr, float sl2, float R, int row, uint32_t (&pk)[32]) {
+  const float2 sl22 = make_float2(sl2, sl2), nr = make_float2(-R, -R);
+  float2 acc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.f, 0.f);
+  // two TMEM round trips: the second half is requested before the first is worked on
+  uint32_t sv[2][32];
+  tc_ld32(s_addr, sv[0]);
+#pragma unroll
+  for (int ch = 0; ch < 2; ++ch) {
+    tc_wait_ld32(sv[ch]);
+    if (ch == 0) tc_ld32(s_addr + 32, sv[1]);
+    // stage by stage over the 32 keys, each stage a run of independent instructions, in place
+    float2 v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __ffma2_rn(make_float2(__uint_as_float(sv[ch][2 * i]), __uint_as_float(sv[ch][2 * i + 1])), sl22, nr);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if ((i & 7) < kPolyPairsOf8) v[i] = exp2_poly2(v[i]);
+      else v[i] = make_float2(ex2f(v[i].x), ex2f(v[i].y));
+    }
+    if (MASKED) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int c = ch * 32 + 2 * i;
+        if (c > row) v[i].x = 0.f;
+        if (c + 1 > row) v[i].y = 0.f;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) pk[ch * 16 + i] = pack_bf16(v[i].x, v[i].y);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i & 3] = __fadd2_rn(acc[i & 3], v[i]);
+  }
+  const float2 a = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
+  return a.x + a.y;
+}
+
+// The largest raw score of this thread's row (MASKED: among the keys it sees, key <= last; -inf if there is none).
+// Off the diagonal the 64 predicates are left out (with them a 128k prompt takes 2 % longer).
+template <bool MASKED>
+__device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
+  float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+  uint32_t sv[2][32];
+  tc_ld32(s_addr, sv[0]);
+  tc_ld32(s_addr + 32, sv[1]);
+  tc_wait_ld32(sv[0]);
+  tc_wait_ld32(sv[1]);
+#pragma unroll
+  for (int ch = 0; ch < 2; ++ch)
+#pragma unroll
+    for (int e = 0; e < 32; ++e)
+      if (!MASKED || ch * 32 + e <= last) mx[e & 3] = fmaxf(mx[e & 3], __uint_as_float(sv[ch][e]));
+  return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+}
+
+// A tile that is not for the plain pass: the diagonal block (last = row), one that is absent or rejected (last < 0), or one where some row's
+// reference has to move; from the scores to P in their place.  `fresh`: the row has no reference yet.  Returns the row's (reference, sum) and whether a wait was lost.
+// A function of its own, not inlined: where these paths join the plain pass's results, or share its registers, every tile pays for them.  The
+// attention launch by itself, 32k tokens 1285 us inline and 1250 so, 24 short prompts 164.6 and 161.6, 48k 2722 and 2690, dense 16k 2410 and 2367;
+// all paths in one inlined loop beside the plain pass: 1426, 208.7, 2950, 2534.  (The diagonal of short lists inlined as a third copy: 1321, 174.)
+static __device__ __noinline__ float4 other_tile(Shared sh, uint32_t s_addr, uint32_t o_addr, float sl2, float R, float l, int last, bool fresh, int t, int pv_bar, uint32_t pv_par, int* status) {
+  uint32_t pk[32];
+  if (last < 0) {                                           // absent or rejected: contributes nothing
+#pragma unroll
+    for (int i = 0; i < 32; ++i) pk[i] = 0u;
+  } else {
+    float sum;
+    if (fresh) {                                            // (the same for the whole warp: tensor memory is read by all its lanes)
+      const float mx = row_max<true>(s_addr, last);
+      if (fabsf(mx) < 3.0e38f) R = mx * sl2;
+    }
+    for (int taken = 0;; taken = 1) {
+      sum = row_pass<true>(s_addr, sl2, R, last, pk);
+      const bool over = !(sum < kRise);
+      if (taken) {
+        if (over) sum = CUDART_NAN_F;                       // an infinite score or a NaN: so is the row
+        break;
+      }
+      if (!__any_sync(0xffffffffu, over)) break;
+      // ---- some row's reference has to move (or its scores are not finite): O at rest, rows rescaled, tile taken again
+      if (t > 0) {
+        const bool fail = !mbar_wait(sh, pv_bar, pv_par, status);
+        if (__any_sync(0xffffffffu, fail)) return make_float4(R, l, 1.f, 0.f);
+        tc_fence_after();
+      }
+      const float mx = row_max<true>(s_addr, last) * sl2;
+      const float nr = over && fabsf(mx) < 3.0e38f ? fmaxf(R, mx) : R;
+      const float alpha = nr == R ? 1.f : exp2f(R - nr);
+      R = nr;
+      l = alpha == 0.f ? 0.f : __fmul_rn(l, alpha);
+      if (t > 0) {
+#pragma unroll 1
+        for (int ch = 0; ch < 8; ++ch) {
+          uint32_t ov[16];
+          tc_ld16(o_addr + ch * 16, ov);
+          tc_wait_ld(ov);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) ov[e] = alpha == 0.f ? 0u : __float_as_uint(__uint_as_float(ov[e]) * alpha);
+          tc_st16(o_addr + ch * 16, ov);
+        }
+      }
+    }
+    l = __fadd_rn(l, sum);
+  }
+  tc_st32(s_addr, pk);                                      // P over the scores this thread has read
+  tc_wait_st();
+  tc_fence_before();
+  return make_float4(R, l, 0.f, 0.f);
+}
+
+// 32 bytes, at once where the address allows it (the host asks for 16)
+__device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bool aligned) {
+  if (!aligned) {
+    reinterpret_cast<uint4*>(p)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    reinterpret_cast<uint4*>(p)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    return;
+  }
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]),
+               "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+}
 
 }  // namespace tcc
+
 }  // namespace seer
