@@ -380,6 +380,39 @@ __device__ __forceinline__ float row_pass(uint32_t s_addr, float sl2, float R, i
   return a.x + a.y;
 }
 
+// The same, of a row that is in registers.
+template <bool MASKED>
+__device__ __forceinline__ float row_pass_of(const uint32_t (&sv)[2][32], float sl2, float R, int last, uint32_t (&pk)[32]) {
+  const float2 sl22 = make_float2(sl2, sl2), nr = make_float2(-R, -R);
+  float2 acc[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int ch = 0; ch < 2; ++ch) {
+    float2 v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __ffma2_rn(make_float2(__uint_as_float(sv[ch][2 * i]), __uint_as_float(sv[ch][2 * i + 1])), sl22, nr);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if ((i & 7) < kPolyPairsOf8) v[i] = exp2_poly2(v[i]);
+      else v[i] = make_float2(ex2f(v[i].x), ex2f(v[i].y));
+    }
+    if (MASKED) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int c = ch * 32 + 2 * i;
+        if (c > last) v[i].x = 0.f;
+        if (c + 1 > last) v[i].y = 0.f;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) pk[ch * 16 + i] = pack_bf16(v[i].x, v[i].y);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i & 3] = __fadd2_rn(acc[i & 3], v[i]);
+  }
+  const float2 a = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
+  return a.x + a.y;
+}
 // The largest raw score of this thread's row (MASKED: among the keys it sees, key <= last; -inf if there is none).
 // Off the diagonal the 64 predicates are left out (with them a 128k prompt takes 2 % longer).
 template <bool MASKED>
@@ -399,50 +432,65 @@ __device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
 }
 
 // A tile that is not for the plain pass: the diagonal block (last = row), one that is absent or rejected (last < 0), or one where some row's
-// reference has to move; from the scores to P in their place.  `fresh`: the row has no reference yet.  Returns the row's (reference, sum) and whether a wait was lost.
+// reference has to move; from the scores to P in their place.  `fresh`: the row has no reference yet.  Returns the row's (reference,
+// sum) and whether a wait was lost.  Conditions around tensor memory loads are the same for a whole warp: all its lanes take part in them.
 // A function of its own, not inlined: where these paths join the plain pass's results, or share its registers, every tile pays for them.  The
-// attention launch by itself, 32k tokens 1285 us inline and 1250 so, 24 short prompts 164.6 and 161.6, 48k 2722 and 2690, dense 16k 2410 and 2367;
-// all paths in one inlined loop beside the plain pass: 1426, 208.7, 2950, 2534.  (The diagonal of short lists inlined as a third copy: 1321, 174.)
+// attention launch by itself, 32k tokens 1285 us inline and 1240 so, 24 short prompts 165.6 and 164.2, 48k 2722 and 2690, dense 16k 2410 and 2360;
+// all paths in one inlined loop beside the plain pass: 1426, 208.7, 2950, 2534.  (The scores are taken to registers once: read again for the
+// maximum and for the pass, 32k tokens take 1250.)
 static __device__ __noinline__ float4 other_tile(Shared sh, uint32_t s_addr, uint32_t o_addr, float sl2, float R, float l, int last, bool fresh, int t, int pv_bar, uint32_t pv_par, int* status) {
   uint32_t pk[32];
   if (last < 0) {                                           // absent or rejected: contributes nothing
 #pragma unroll
     for (int i = 0; i < 32; ++i) pk[i] = 0u;
   } else {
-    float sum;
-    if (fresh) {                                            // (the same for the whole warp: tensor memory is read by all its lanes)
-      const float mx = row_max<true>(s_addr, last);
-      if (fabsf(mx) < 3.0e38f) R = mx * sl2;
-    }
+    float sum = 0.f;
+    bool over = false;
     for (int taken = 0;; taken = 1) {
-      sum = row_pass<true>(s_addr, sl2, R, last, pk);
-      const bool over = !(sum < kRise);
+      uint32_t sv[2][32];
+      tc_ld32(s_addr, sv[0]);
+      tc_ld32(s_addr + 32, sv[1]);
+      tc_wait_ld32(sv[0]);
+      tc_wait_ld32(sv[1]);
+      if (taken || fresh) {                                 // (the same for the whole warp)
+        float mx4[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll
+        for (int c = 0; c < 64; ++c)
+          if (c <= last) mx4[c & 3] = fmaxf(mx4[c & 3], __uint_as_float(sv[c >> 5][c & 31]));
+        const float raw = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+        if (!taken) {
+          if (fabsf(raw) < 3.0e38f) R = raw * sl2;
+        } else {
+          const float mx = raw * sl2;
+          const float nr = over && fabsf(mx) < 3.0e38f ? fmaxf(R, mx) : R;
+          const float alpha = nr == R ? 1.f : exp2f(R - nr);
+          R = nr;
+          l = alpha == 0.f ? 0.f : __fmul_rn(l, alpha);
+          if (t > 0) {
+#pragma unroll 1
+            for (int ch = 0; ch < 8; ++ch) {
+              uint32_t ov[16];
+              tc_ld16(o_addr + ch * 16, ov);
+              tc_wait_ld(ov);
+#pragma unroll
+              for (int e = 0; e < 16; ++e) ov[e] = alpha == 0.f ? 0u : __float_as_uint(__uint_as_float(ov[e]) * alpha);
+              tc_st16(o_addr + ch * 16, ov);
+            }
+          }
+        }
+      }
+      sum = row_pass_of<true>(sv, sl2, R, last, pk);
       if (taken) {
-        if (over) sum = CUDART_NAN_F;                       // an infinite score or a NaN: so is the row
+        if (!(sum < kRise)) sum = CUDART_NAN_F;             // an infinite score or a NaN: so is the row
         break;
       }
+      over = !(sum < kRise);
       if (!__any_sync(0xffffffffu, over)) break;
       // ---- some row's reference has to move (or its scores are not finite): O at rest, rows rescaled, tile taken again
       if (t > 0) {
         const bool fail = !mbar_wait(sh, pv_bar, pv_par, status);
         if (__any_sync(0xffffffffu, fail)) return make_float4(R, l, 1.f, 0.f);
         tc_fence_after();
-      }
-      const float mx = row_max<true>(s_addr, last) * sl2;
-      const float nr = over && fabsf(mx) < 3.0e38f ? fmaxf(R, mx) : R;
-      const float alpha = nr == R ? 1.f : exp2f(R - nr);
-      R = nr;
-      l = alpha == 0.f ? 0.f : __fmul_rn(l, alpha);
-      if (t > 0) {
-#pragma unroll 1
-        for (int ch = 0; ch < 8; ++ch) {
-          uint32_t ov[16];
-          tc_ld16(o_addr + ch * 16, ov);
-          tc_wait_ld(ov);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) ov[e] = alpha == 0.f ? 0u : __float_as_uint(__uint_as_float(ov[e]) * alpha);
-          tc_st16(o_addr + ch * 16, ov);
-        }
       }
     }
     l = __fadd_rn(l, sum);
