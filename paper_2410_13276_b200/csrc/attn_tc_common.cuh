@@ -132,6 +132,12 @@ __device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint
                "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
                ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
+// A from shared memory
+__device__ __forceinline__ void tc_mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+               "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+               ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
 // Weight-stationary form, A from shared memory / from tensor memory (M = 64: see attn_tc.cu)
 __device__ __forceinline__ void tc_mma_ws(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -513,5 +519,12 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bo
 }
 
 }  // namespace tcc
+
+// Attention where pairs of query blocks list the same blocks (attn_pair.cu).  The check zeroes the work counter and writes `epoch` to the
+// word behind it where some pair's lists differ; attn_tc_kernel returns at once where none do, attn_pair_kernel where some do.
+seer_status init_attn_pair();
+int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, int epoch, cudaStream_t stream);
+int launch_attn_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mv32, const int32_t* row_ptr,
+                     const int32_t* col_idx, void* o, float* lse, int* counter, int epoch, cudaStream_t stream);
 
 }  // namespace seer

@@ -10,11 +10,11 @@ static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Byte offsets of the arrays inside a metadata slot: as long as the batch, so that a new shape's upload is.
 struct SlotLayout {
-  size_t place, score, cu, blk, qoff, qdelta, qblk, bytes;
+  size_t place, score, cu, blk, qoff, qdelta, qblk, pair, bytes;
   explicit constexpr SlotLayout(int batch)
       : place(0), score(place + sizeof(int4) * batch), cu(score + sizeof(int64_t) * (batch + 1)), blk(cu + sizeof(int32_t) * (batch + 1)),
         qoff(blk + sizeof(int32_t) * (batch + 1)), qdelta(qoff + sizeof(int32_t) * batch), qblk(qdelta + sizeof(int32_t) * batch),
-        bytes(qblk + sizeof(int32_t) * (batch + 1)) {}
+        pair(qblk + sizeof(int32_t) * (batch + 1)), bytes(pair + sizeof(int32_t) * (batch + 1)) {}
 };
 constexpr size_t kSlotBytes = (SlotLayout(kMaxBatch).bytes + 255) / 256 * 256;
 
@@ -135,7 +135,8 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
     int32_t* qb = (int32_t*)(h + at.qblk);
     int4* place = (int4*)(h + at.place);
     int32_t* order = qb + 1;                           // (its places are read before they become block counts)
-    blk[0] = 0; sc[0] = 0; qb[0] = 0;
+    int32_t* pairs = (int32_t*)(h + at.pair);
+    blk[0] = 0; sc[0] = 0; qb[0] = 0; pairs[0] = 0;
     for (int b = 0; b < shape->batch; ++b) {
       cu[b] = shape->cu_seqlens_host[b];
       int32_t nb = (shape->cu_seqlens_host[b + 1] - shape->cu_seqlens_host[b] + shape->block - 1) / shape->block;
@@ -161,6 +162,7 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
       const int b = order[p];
       place[p] = make_int4(cu[b], cu[b + 1] - cu[b], blk[b], qd[b]);
       qb[p + 1] = qb[p] + blk[b + 1] - blk[b] - qo[b];
+      pairs[p + 1] = pairs[p] + (qo[b] < blk[b + 1] - blk[b] ? (blk[b + 1] - blk[b] + 1) / 2 - qo[b] / 2 : 0);
     }
     if (cudaMemcpyAsync(s.dev, h, at.bytes, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SEER_ERR_CUDA;
     if (cudaEventRecord(s.ready, stream) != cudaSuccess) return SEER_ERR_CUDA;
@@ -193,7 +195,7 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
   m->total_q_tokens = (int32_t)t.total_q_tokens;
   m->chunked = shape->cu_seqlens_q_host ? 1 : 0;
   double tiles = 0;
-  int64_t q_blocks = 0;
+  int64_t q_blocks = 0, pair_blocks = 0;
   for (int b = 0; b < shape->batch; ++b) {
     const double nb = (shape->cu_seqlens_host[b + 1] - shape->cu_seqlens_host[b] + shape->block - 1) / shape->block;
     double before = 0;                                 // blocks before the chunk
@@ -201,11 +203,16 @@ seer_status prepare(seer_ctx* ctx, const seer_shape* shape, cudaStream_t stream,
       before = ((shape->cu_seqlens_host[b + 1] - shape->cu_seqlens_host[b]) - (cq[b + 1] - cq[b])) / shape->block;
     tiles += (nb * nb - before * before) / 2 / (128.0 * kScoreTile);
     const int32_t* cq = shape->cu_seqlens_q_host;
-    if (!cq || cq[b + 1] > cq[b]) q_blocks += (int64_t)(nb - before);   // (a chunk starts on a block)
+    if (!cq || cq[b + 1] > cq[b]) {                       // (a chunk starts on a block)
+      q_blocks += (int64_t)(nb - before);
+      if (nb > before) pair_blocks += ((int64_t)nb + 1) / 2 - (int64_t)before / 2;
+    }
     if (shape->batch == 1) m->first_q_block = (int32_t)before;
   }
   if (shape->batch != 1) m->first_q_block = 0;
   m->q_rows = q_blocks * shape->num_q_heads;
+  m->pair_off = (const int32_t*)(d + at.pair);
+  m->pair_units = pair_blocks * shape->num_q_heads;
   m->score_tiles = (int64_t)(tiles * shape->num_q_heads);
   m->wait_limit_us = ctx->wait_limit_us;
   m->lose_v_copy = ctx->lose_v_copy;

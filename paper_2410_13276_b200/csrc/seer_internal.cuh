@@ -39,6 +39,8 @@ struct SeqMeta {
   // the attention's order of the sequences
   const int4* place;           // [batch] (first token, tokens, first block, qdelta) of the sequence at each place
   const int32_t* qblk_off;     // [batch + 1] blocks with queries at the places before
+  const int32_t* pair_off;     // [batch + 1] pairs of blocks (2u, 2u + 1) with queries at the places before
+  int64_t pair_units;          // such pairs, all heads
   int32_t total_q_tokens;      // tokens in q / o / lse
   int32_t chunked;             // 1 if the shape carries cu_seqlens_q
   // bounded waits of the tcgen05 attention kernel, and the test hook that makes one of them run out

@@ -1,0 +1,111 @@
+"""Attention where query blocks 2u and 2u + 1 list the same blocks: o and lse equal those of the launch without a work counter, which takes every
+query block by itself, bit for bit (the same rows, sums in the same order).  The second word of the workspace says which kernel ran: the
+check of the lists writes it where some pair differs."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def problem(lens, hq, hkv, block=64, qlens=None, seed=0):
+    import torch
+    from paper_2410_13276_b200.prefill import Prefill
+    cu = lambda x: np.concatenate([[0], np.cumsum(x)]).astype(np.int32)
+    p = Prefill(cu(lens), hq, hkv, block=block, cu_seqlens_q=None if qlens is None else cu(qlens))
+    g = torch.Generator(device="cuda"); g.manual_seed(seed + sum(lens))
+    draw = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    p.q, p.k, p.v = (2 * draw(p.Tq, hq, 128)).bfloat16(), draw(p.T, hkv, 128).bfloat16(), draw(p.T, hkv, 128).bfloat16()
+    p.wq, p.wk = draw(hq, 128, 128) / 11.3, draw(hkv, 128, 128) / 11.3
+    p.scores.zero_()
+    return p
+
+
+def both_ways(p, by_pairs):
+    import torch
+    outs = []
+    for dynamic in (False, True):
+        p.o.fill_(7.0); p.lse.fill_(7.0)
+        p.ws[4:8] = 0
+        p.attn(dynamic=dynamic)
+        torch.cuda.synchronize()
+        assert p.status() == 0
+        outs.append((p.o.clone().view(torch.int16), p.lse.clone().view(torch.int32)))
+    assert (int(p.ws[4:8].view(torch.int32)) == 0) == by_pairs
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+# every causal block: odd and even block counts, ragged ends, batches in any order with sequences of one block, chunks from odd and even blocks
+@pytest.mark.parametrize("lens,qlens,hq,hkv", [([16421], None, 32, 8), ([700, 1, 12032, 64, 4100], None, 64, 16), ([16500, 9000], [16500 - 64 * 33, 9000 - 64 * 58], 40, 8)])
+def test_dense_lists(lens, qlens, hq, hkv):
+    from paper_2410_13276_b200 import binding as B
+    p = problem(lens, hq, hkv, qlens=qlens)
+    p.mask(B.make_mask_params(B.SEER_TOPK_COUNT, k=1 << 20, flags=B.SEER_FORCE_DIAG))
+    both_ways(p, True)
+
+
+@pytest.mark.parametrize("lens,qlens", [([23500], None), ([16400, 127, 11000], None), ([23500, 2000], [23500 - 128 * 57, 2000 - 128])])
+def test_lists_of_128_token_blocks(lens, qlens):
+    from paper_2410_13276_b200 import binding as B
+    p = problem(lens, 32, 8, block=128, qlens=qlens)
+    p.gate()
+    p.mask(B.make_mask_params(B.SEER_TOPK_RATIO, keep_num=1, keep_den=5, flags=B.SEER_FORCE_DIAG | B.SEER_FORCE_SINK))
+    both_ways(p, True)
+
+
+# lists in any order, of no block to all, the second block with one more (its own, or an earlier one) or not; values and keys that are not finite
+@pytest.mark.parametrize("spoilt", [False, True])
+def test_hand_made_lists(spoilt):
+    import torch
+    lens, hq = [16400, 3000], 32
+    p = problem(lens, hq, 8)
+    r = np.random.default_rng(11)
+    rows, at = [], 0
+    for n in lens:
+        nb = (n + 63) // 64
+        for h in range(hq):
+            for i in range(0, nb, 2):
+                shared = r.permutation(i)[:r.choice([0, 0, 1, 2, 3, 5, 30, i])].tolist()
+                if r.random() < 0.7:
+                    shared.append(i)
+                more = r.choice(3)
+                rows.append(shared)
+                if i + 1 < nb:
+                    at = max(at, len(rows) - 1, key=lambda k: len(rows[k]))
+                    rows.append(shared + ([] if more == 0 else [i + 1] if more == 1 else [int(r.integers(0, i + 2))]))
+    if spoilt:
+        p.v[64 * 101 + 5, 0, 3] = float("inf"); p.v[64 * 40, 2, 100] = float("nan"); p.v[16400 + 64 * 7 + 63, 5, 0] = float("-inf")
+        p.k[64 * 77 + 9, 1, 4] = float("inf"); p.k[64 * 30 + 2, 3] *= 60; p.q[64 * 90:64 * 96] *= 20
+    p.set_lists(np.concatenate([[0], np.cumsum([len(x) for x in rows])]).astype(np.int32), np.array([j for x in rows for j in x], np.int32))
+    both_ways(p, True)
+    # a single pair that differs, by an entry or by a length, or whose own block is not its last entry: each query block by itself
+    for change in (lambda x: x[1:], lambda x: [x[1], x[0]] + x[2:], lambda x: x + x[:2]):
+        other = [change(x) if k == at else x for k, x in enumerate(rows)]
+        p.set_lists(np.concatenate([[0], np.cumsum([len(x) for x in other])]).astype(np.int32), np.array([j for x in other for j in x], np.int32))
+        both_ways(p, False)
+
+
+@pytest.mark.parametrize("lost_tile", [0, 130, 300])
+def test_a_lost_copy(lost_tile):
+    """A V copy that CTA 0 never issues: the call returns with the status, the rows of the items it had in hand stay as they were, all others are
+    right, and the next call is normal."""
+    import torch
+    from paper_2410_13276_b200 import binding as B
+    p = problem([16384], 32, 8)
+    p.mask(B.make_mask_params(B.SEER_TOPK_COUNT, k=1 << 20, flags=B.SEER_FORCE_DIAG))
+    both_ways(p, True)
+    o, lse = p.o.clone(), p.lse.clone()
+    B.seer_debug_lost_wait(p.ctx, 5_000, lost_tile)
+    try:
+        p.o.fill_(float("nan")); p.lse.fill_(float("nan"))
+        p.attn()
+        status = B.seer_poll_device_status(p.ctx)
+    finally:
+        B.seer_debug_lost_wait(p.ctx, 2_000_000, -1)
+    assert B.STATUS_NAMES[status] == "SEER_ERR_TIMEOUT"
+    missing = torch.isnan(p.lse)                                   # [heads, tokens]: whole items of 128 rows
+    assert torch.equal(torch.isnan(p.o.float()).all(-1).T, missing) and torch.equal(torch.isnan(p.o.float()).any(-1).T, missing)
+    items = missing.view(32, -1, 128)
+    assert torch.equal(items.all(-1), items.any(-1)) and 1 <= int(items.any(-1).sum()) <= 5
+    assert torch.equal(p.lse[~missing], lse[~missing]) and torch.equal(p.o.permute(1, 0, 2)[~missing], o.permute(1, 0, 2)[~missing])
+    both_ways(p, True)
+    assert torch.equal(p.o, o) and torch.equal(p.lse, lse)
