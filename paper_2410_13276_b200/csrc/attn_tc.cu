@@ -41,7 +41,7 @@
 #include <cuda.h>
 #include <math_constants.h>
 
-#include "attn_tc_common.cuh"
+#include "attn_pair.cuh"
 
 namespace seer {
 namespace tc {
@@ -119,7 +119,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
                 const int32_t* row_ptr, const int32_t* col_idx,
                 uint16_t* __restrict__ o, float* lse, int* __restrict__ status,
                 unsigned long long* __restrict__ trace, float* block_max = nullptr,
-                int* __restrict__ work_counter = nullptr, const int* differs = nullptr, int epoch = 0) {
+                int* __restrict__ work_counter = nullptr, const int* differs = nullptr, int epoch = 0, int nwords = 0) {
   extern __shared__ __align__(1024) unsigned char smem[];
   Shared sh;
   sh.base = smem_u32(smem);
@@ -129,6 +129,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   if (!kBlockMax && differs != nullptr) {                  // (a way out from further in costs a launch of 32k tokens 2 %)
     grid_wait();
     if (ld_global(reinterpret_cast<const uint32_t*>(differs)) != (uint32_t)epoch) return;   // attn_pair_kernel does the work
+  }
+  if (kBlockMax && differs != nullptr) {                   // (here: the check's words, `nwords` of them)
+    grid_wait();
+    if (tp::lists_agree(differs, nwords, epoch)) return;    // block_max_pair_kernel has done the work
   }
   if ((sh.base & 1023u) != 0u) {                           // the swizzled tiles need the alignment
     grid_wait();
@@ -680,7 +684,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   }
 }
 
-using Kernel = void(CUtensorMap, CUtensorMap, CUtensorMap, SeqMeta, const int32_t*, const int32_t*, uint16_t*, float*, int*, unsigned long long*, float*, int*, const int*, int);
+using Kernel = void(CUtensorMap, CUtensorMap, CUtensorMap, SeqMeta, const int32_t*, const int32_t*, uint16_t*, float*, int*, unsigned long long*, float*, int*, const int*, int, int);
 
 __global__ void zero_kernel(int* __restrict__ word) {
   grid_wait();
@@ -757,7 +761,7 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
                      : few ? (m.chunked ? tc::attn_tc_kernel<false, true, false, true, true> : tc::attn_tc_kernel<false, false, false, true, true>)
                      : m.chunked ? tc::attn_tc_kernel<false, true> : tc::attn_tc_kernel<false, false>;
   e = launch_next(kernel, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter,
-                  pairs ? (const int*)work_counter + 1 : nullptr, epoch);
+                  pairs ? (const int*)work_counter + 1 : nullptr, epoch, 0);
   if (e != cudaSuccess) return -(int)e;
   ++launched;
   if (pairs) {
@@ -779,10 +783,20 @@ int launch_block_max_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const vo
     return -(int)cudaErrorInvalidValue;
   const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, m.q_rows);
   float* lse_in = const_cast<float*>(lse);   // read only in this mode
-  const cudaError_t e = m.chunked
-      ? launch_next(tc::attn_tc_kernel<false, true, true>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr, nullptr, 0)
-      : launch_next(tc::attn_tc_kernel<false, false, true>, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr, nullptr, 0);
-  return e == cudaSuccess ? 1 : -(int)e;
+  // Pairs of query blocks that share their lists (attn_pair.cu): asked for from 2^18 causal blocks on (8k tokens, 32 heads), sooner than for the
+  // attention, as the map is taken of dense lists above all.  16k tokens: all blocks 1045 -> 770 us, a tenth of them 128 -> 131.
+  int* words = nullptr;
+  int nwords = 0, launched = 0;
+  const int epoch = 1 + (int)(ctx->clock & 0x3fffffff);    // (a word of lists that differ is 0)
+  if (m.score_tiles >= (1 << 18) / (128 * kScoreTile)) {
+    words = ctx->words + (ctx->clock % kWordSets) * tp::kWords;
+    nwords = (int)min((int64_t)tp::kWords, m.pair_units);
+    launched = launch_block_max_pair(ctx, m, mq, mk, row_ptr, col_idx, lse, out, words, nwords, epoch, stream);
+    if (launched < 0) return launched;
+  }
+  const cudaError_t e = launch_next(m.chunked ? tc::attn_tc_kernel<false, true, true> : tc::attn_tc_kernel<false, false, true>, grid, tc::kThreads, tc::kSmemBytes, stream,
+                                    mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr, (const int*)words, epoch, nwords);
+  return e == cudaSuccess ? launched + 1 : -(int)e;
 }
 
 }  // namespace seer

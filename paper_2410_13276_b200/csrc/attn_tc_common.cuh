@@ -526,5 +526,8 @@ seer_status init_attn_pair();
 int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, int epoch, cudaStream_t stream);
 int launch_attn_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mv32, const int32_t* row_ptr,
                      const int32_t* col_idx, void* o, float* lse, int* counter, int epoch, cudaStream_t stream);
+// The block maxima likewise; the answer is `epoch` in all of nwords words (at most tp::kWords) of the context's.
+int launch_block_max_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const int32_t* row_ptr, const int32_t* col_idx, const float* lse,
+                          float* out, int* words, int nwords, int epoch, cudaStream_t stream);
 
 }  // namespace seer

@@ -15,6 +15,7 @@ constexpr int kHeadDim = 128;
 constexpr int kGateDim = 128;
 constexpr int kMaxBatch = 4096;
 constexpr int kMetaSlots = 8;
+constexpr int kWordSets = 16;   // sets of 256 words (block maxima, attn_pair.cu)
 constexpr int kScoreTile = 64;  // column tile of the gate's score kernel, and granularity of the bands of the one-call gate + mask
 
 // Per-batch metadata the kernels read from device memory.
@@ -116,6 +117,7 @@ struct seer_ctx {
   size_t stage_pos = 0;
   void* tmap_encode = nullptr;   // cuTensorMapEncodeTiled, resolved at run time
   void* trace = nullptr;         // optional device buffer for the attention kernel's timeline (diagnostics)
+  int* words = nullptr;          // kWordSets sets of words through which a check of lists answers (block maxima)
   uint32_t wait_limit_us = 2000000u;   // seer_debug_lost_wait
   int32_t lose_v_copy = -1;
   // seer_prefill_host: copy streams and the events of its two-deep pipeline over KV-head slices

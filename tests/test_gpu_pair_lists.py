@@ -34,6 +34,29 @@ def both_ways(p, by_pairs):
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
 
 
+def maxima_of_groups(p):
+    """Block maxima: equal to those of each KV head's problem by itself, which is below the size from which pairs are asked for."""
+    import torch
+    from paper_2410_13276_b200.prefill import Prefill
+    p.attn()
+    p.bmax = torch.full((max(p.col_idx.numel(), 1),), -1.0, device="cuda")
+    got = p.block_max()
+    rp, col = p.lists_host()
+    nbs, group = (np.diff(p.cu) + 63) // 64, p.hq // p.hkv
+    for g in range(p.hkv):
+        part = Prefill(p.cu, group, 1, cu_seqlens_q=p.cu_q, ctx=p.ctx)
+        part.q, part.k, part.lse = p.q[:, g * group:(g + 1) * group].contiguous(), p.k[:, g:g + 1].contiguous(), p.lse[g * group:(g + 1) * group].contiguous()
+        base, spans = 0, []
+        for nb in nbs:
+            spans.append((base + g * group * nb, base + (g + 1) * group * nb))
+            base += p.hq * nb
+        lens = np.concatenate([np.diff(rp[a:b + 1]) for a, b in spans])
+        part.set_lists(np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), np.concatenate([col[rp[a]:rp[b]] for a, b in spans]).astype(np.int32))
+        want = part.block_max()[:int(lens.sum())]
+        assert torch.equal(torch.cat([got[int(rp[a]):int(rp[b])] for a, b in spans]).view(torch.int32), want.view(torch.int32)), g
+    assert p.status() == 0
+
+
 # every causal block: odd and even block counts, ragged ends, batches in any order with sequences of one block, chunks from odd and even blocks
 @pytest.mark.parametrize("lens,qlens,hq,hkv", [([16421], None, 32, 8), ([700, 1, 12032, 64, 4100], None, 64, 16), ([16500, 9000], [16500 - 64 * 33, 9000 - 64 * 58], 40, 8)])
 def test_dense_lists(lens, qlens, hq, hkv):
@@ -41,6 +64,7 @@ def test_dense_lists(lens, qlens, hq, hkv):
     p = problem(lens, hq, hkv, qlens=qlens)
     p.mask(B.make_mask_params(B.SEER_TOPK_COUNT, k=1 << 20, flags=B.SEER_FORCE_DIAG))
     both_ways(p, True)
+    maxima_of_groups(p)
 
 
 @pytest.mark.parametrize("lens,qlens", [([23500], None), ([16400, 127, 11000], None), ([23500, 2000], [23500 - 128 * 57, 2000 - 128])])
@@ -77,11 +101,13 @@ def test_hand_made_lists(spoilt):
         p.k[64 * 77 + 9, 1, 4] = float("inf"); p.k[64 * 30 + 2, 3] *= 60; p.q[64 * 90:64 * 96] *= 20
     p.set_lists(np.concatenate([[0], np.cumsum([len(x) for x in rows])]).astype(np.int32), np.array([j for x in rows for j in x], np.int32))
     both_ways(p, True)
+    maxima_of_groups(p)
     # a single pair that differs, by an entry or by a length, or whose own block is not its last entry: each query block by itself
     for change in (lambda x: x[1:], lambda x: [x[1], x[0]] + x[2:], lambda x: x + x[:2]):
         other = [change(x) if k == at else x for k, x in enumerate(rows)]
         p.set_lists(np.concatenate([[0], np.cumsum([len(x) for x in other])]).astype(np.int32), np.array([j for x in other for j in x], np.int32))
         both_ways(p, False)
+    maxima_of_groups(p)                                            # (a CTA with that pair takes each block by itself, the others theirs by pairs)
 
 
 @pytest.mark.parametrize("lost_tile", [0, 130, 300])
