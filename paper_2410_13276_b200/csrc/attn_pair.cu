@@ -492,8 +492,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 // ------------------------------------------------------------------------------------------------ block maxima
 // The largest probability of every listed 64 x 64 tile (Sec. 3.2, Eq. 2 on the listed blocks; attn_tc_kernel<.., kBlockMax>) where all pairs have
 // one list each: the pipeline above without V, its tensor memory four S buffers and its K ring five tiles deep.  A tile's K, 32 KB, serves four
-// blocks; the maxima are the same bit for bit.  16 384 tokens, 32 heads, all blocks: 1045 -> 770 us, 800 clocks a tile of which 512 are its MMAs and 442 its
-// copies: a group's chain from scores to maximum is as long.
+// blocks; the maxima are the same bit for bit.  16 384 tokens, 32 heads, all blocks: 1045 -> 755 us, 800 clocks a tile of which 512 are its MMAs and 442 its
+// copies.  (Q from tensor memory, which halves what the MMAs read of shared memory, and two tiles at a time in a group: no gain.)
 //
 // The call has no workspace to pass the check's answer through.  It goes through words of the context, one for each block of the check: `epoch` where the block
 // found its pairs so, else 0.  The context's ring of them is shared by calls on several streams, so a word may be overwritten by a later
@@ -547,7 +547,7 @@ block_max_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         for (uint32_t n = 0; ok; ++n) {
           const int64_t w = dealt_pair(m, n);
           PairItem it{};
-          if (w >= 0) it = decode_pair<kChunk>(m, row_ptr, w);
+          if (w >= 0) it = decode_pair<kChunk, true>(m, row_ptr, w);
           const int tiles = (it.len + 1) >> 1, g = it.h / m.group;
           const int x0 = it.n[0] > 0 ? (int)ld_global(col + it.l0 + it.n[0] - 1) : -1, x1 = it.n[1] > 0 ? (int)ld_global(col + it.l0 + it.n[1] - 1) : -1;
           if (!mbar_wait(sh, M_ITEM_EMPTY + (int)(n & 3u), ((n >> 2) & 1u) ^ 1u, status)) break;
@@ -650,7 +650,7 @@ block_max_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
       if (!(fabsf(L) < 3.0e38f)) L = 0.f;                   // a query without a key has no probabilities to report
       const float L2 = L * 1.4426950408889634f;
       // Lane k holds the warp's maximum of the k-th tile since the block's two warps last met, as an order-preserving integer: they meet every
-      // 32 tiles (every tile: 16k tokens, all blocks, 850 us where this takes 770).
+      // 32 tiles (every tile: 16k tokens, all blocks, 850 us where this takes 755).
       int key = 0, first_p = g;
       for (int p = g; p < len + g; p += 2, ++cnt) {         // (both groups take every tile, the second one without a block in an odd list's last)
         const uint32_t sbuf = cnt & 3u;

@@ -13,7 +13,9 @@ struct PairItem {
   int n[2], valid[2];          // entries and query rows of the two blocks (no rows: not there)
 };
 
-template <bool kChunk>
+// The w-th pair: KV head by KV head of a sequence, from the last pair to the first, a pair's heads side by side.  kZigzag: every other KV head from the
+// first pair to the last, so that the lists' lengths have no jump from one head to the next.
+template <bool kChunk, bool kZigzag = false>
 __device__ __forceinline__ PairItem decode_pair(const SeqMeta& m, const int32_t* row_ptr, int64_t w) {
   PairItem it;
   const int p = find_sequence(m.pair_off, m.batch, (int)(w / m.num_q_heads)), before = m.pair_off[p];
@@ -21,7 +23,9 @@ __device__ __forceinline__ PairItem decode_pair(const SeqMeta& m, const int32_t*
   const int nb = (s.y + kBlock - 1) / kBlock, np = m.pair_off[p + 1] - before;
   const int first = kChunk ? nb - (m.qblk_off[p + 1] - m.qblk_off[p]) : 0;
   const int local = (int)(w - (int64_t)m.num_q_heads * before);
-  const int g = local / (np * m.group), rem = local - g * np * m.group;
+  const int g = local / (np * m.group);
+  int rem = local - g * np * m.group;
+  if (kZigzag && ((m.num_kv_heads - 1 - g) & 1)) rem = np * m.group - 1 - rem;
   it.i0 = 2 * ((nb + 1) / 2 - 1 - rem / m.group);
   it.h = g * m.group + rem % m.group;
   it.s0 = s.x;
@@ -69,8 +73,9 @@ __device__ __forceinline__ bool pair_ok(const SeqMeta& m, const int32_t* row_ptr
   return ok;
 }
 
-// The static deal of the block maxima: CTA c takes the pairs of every grid-sized round, from either end in turn, so that no CTA has the longest
-// list of every round.  -1: past the last one.
+// The static deal of the block maxima: CTA c takes the pairs of every grid-sized round, from either end in turn.  In the zigzag order the longest
+// share is 0.7 % above the mean for 16k tokens and 32 heads, all blocks (6 % with every head from its last pair on, 64 % for 9000 tokens).  -1: past the
+// last one.
 __device__ __forceinline__ int64_t dealt_pair(const SeqMeta& m, uint32_t k) {
   const int64_t w = (int64_t)k * gridDim.x + ((k & 1u) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
   return w < m.pair_units ? w : -1;

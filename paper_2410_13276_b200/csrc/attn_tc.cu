@@ -784,7 +784,7 @@ int launch_block_max_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const vo
   const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, m.q_rows);
   float* lse_in = const_cast<float*>(lse);   // read only in this mode
   // Pairs of query blocks that share their lists (attn_pair.cu): asked for from 2^18 causal blocks on (8k tokens, 32 heads), sooner than for the
-  // attention, as the map is taken of dense lists above all.  16k tokens: all blocks 1045 -> 770 us, a tenth of them 128 -> 131.
+  // attention, as the map is taken of dense lists above all.  16k tokens: all blocks 1045 -> 755 us, a tenth of them 128 -> 131.
   int* words = nullptr;
   int nwords = 0, launched = 0;
   const int epoch = 1 + (int)(ctx->clock & 0x3fffffff);    // (a word of lists that differ is 0)
