@@ -703,17 +703,22 @@ using Kernel = void(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, SeqMeta,
 
 }  // namespace tp
 
-seer_status init_attn_pair() {
+static cudaError_t ready(seer_ctx* ctx) {
+  if (ctx->pair_kernels) return cudaSuccess;
+  cudaError_t e = cudaSuccess;
   for (tp::Kernel* k : {tp::attn_pair_kernel<false, false>, tp::attn_pair_kernel<false, true>, tp::attn_pair_kernel<true, false>, tp::attn_pair_kernel<true, true>})
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp::kSmemBytes) != cudaSuccess) return SEER_ERR_CUDA;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp::kSmemBytes);
   for (auto* k : {tp::block_max_pair_kernel<false>, tp::block_max_pair_kernel<true>})
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp::kSmemBytes) != cudaSuccess) return SEER_ERR_CUDA;
-  return SEER_OK;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tp::kSmemBytes);
+  ctx->pair_kernels = e == cudaSuccess;
+  return e;
 }
 
 int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, int epoch, cudaStream_t stream) {
   const unsigned blocks = (unsigned)min((int64_t)ctx->num_sms * 2, (m.pair_units + tp::kCheckWarps - 1) / tp::kCheckWarps);
-  const cudaError_t e = launch_next(m.chunked ? tp::check_kernel<true> : tp::check_kernel<false>, blocks, tp::kCheckWarps * 32, 0, stream, m, row_ptr, col_idx, counter, counter + 1, epoch);
+  cudaError_t e = ready(ctx);
+  if (e != cudaSuccess) return -(int)e;
+  e = launch_next(m.chunked ? tp::check_kernel<true> : tp::check_kernel<false>, blocks, tp::kCheckWarps * 32, 0, stream, m, row_ptr, col_idx, counter, counter + 1, epoch);
   return e == cudaSuccess ? 1 : -(int)e;
 }
 
@@ -729,7 +734,9 @@ int launch_attn_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, con
 
 int launch_block_max_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const int32_t* row_ptr, const int32_t* col_idx, const float* lse,
                           float* out, int* words, int nwords, int epoch, cudaStream_t stream) {
-  cudaError_t e = launch_next(m.chunked ? tp::check_words_kernel<true> : tp::check_words_kernel<false>, (unsigned)nwords, tp::kCheckWarps * 32, 0, stream, m, row_ptr, col_idx,
+  cudaError_t e = ready(ctx);
+  if (e != cudaSuccess) return -(int)e;
+  e = launch_next(m.chunked ? tp::check_words_kernel<true> : tp::check_words_kernel<false>, (unsigned)nwords, tp::kCheckWarps * 32, 0, stream, m, row_ptr, col_idx,
                               words, epoch);
   if (e != cudaSuccess) return -(int)e;
   e = launch_next(m.chunked ? tp::block_max_pair_kernel<true> : tp::block_max_pair_kernel<false>, (unsigned)min((int64_t)ctx->num_sms, m.pair_units), tp::kThreads,

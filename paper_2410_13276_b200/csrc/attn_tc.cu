@@ -717,7 +717,6 @@ seer_status init_attn_tc(seer_ctx* ctx) {
       qres != cudaDriverEntryPointSuccess)
     return SEER_ERR_CUDA;
   ctx->tmap_encode = fn;
-  if (init_attn_pair() != SEER_OK) return SEER_ERR_CUDA;
   for (tc::Kernel* k : {tc::attn_tc_kernel<false, false>, tc::attn_tc_kernel<false, true>, tc::attn_tc_kernel<true, false>,
                         tc::attn_tc_kernel<false, false, false, false>, tc::attn_tc_kernel<false, true, false, false>,
                         tc::attn_tc_kernel<false, false, true>, tc::attn_tc_kernel<false, true, true>,

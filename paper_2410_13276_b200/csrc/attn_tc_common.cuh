@@ -522,7 +522,6 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bo
 
 // Attention where pairs of query blocks list the same blocks (attn_pair.cu).  The check zeroes the work counter and writes `epoch` to the
 // word behind it where some pair's lists differ; attn_tc_kernel returns at once where none do, attn_pair_kernel where some do.
-seer_status init_attn_pair();
 int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, int epoch, cudaStream_t stream);
 int launch_attn_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mv32, const int32_t* row_ptr,
                      const int32_t* col_idx, void* o, float* lse, int* counter, int epoch, cudaStream_t stream);

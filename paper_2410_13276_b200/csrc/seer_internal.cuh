@@ -117,6 +117,7 @@ struct seer_ctx {
   size_t stage_pos = 0;
   void* tmap_encode = nullptr;   // cuTensorMapEncodeTiled, resolved at run time
   void* trace = nullptr;         // optional device buffer for the attention kernel's timeline (diagnostics)
+  bool pair_kernels = false;     // their shared-memory limits are set (by the first call that may use them: 0.1 ms of creating a context)
   int* words = nullptr;          // kWordSets sets of words through which a check of lists answers (block maxima)
   uint32_t wait_limit_us = 2000000u;   // seer_debug_lost_wait
   int32_t lose_v_copy = -1;
