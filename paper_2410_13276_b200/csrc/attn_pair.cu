@@ -492,8 +492,9 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 // ------------------------------------------------------------------------------------------------ block maxima
 // The largest probability of every listed 64 x 64 tile (Sec. 3.2, Eq. 2 on the listed blocks; attn_tc_kernel<.., kBlockMax>) where all pairs have
 // one list each: the pipeline above without V, its tensor memory four S buffers and its K ring five tiles deep.  A tile's K, 32 KB, serves four
-// blocks; the maxima are the same bit for bit.  16 384 tokens, 32 heads, all blocks: 1045 -> 755 us, 800 clocks a tile of which 512 are its MMAs and 442 its
-// copies.  (Q from tensor memory, which halves what the MMAs read of shared memory, and two tiles at a time in a group: no gain.)
+// blocks; the maxima are the same bit for bit.  16 384 tokens, 32 heads, all blocks: 1045 -> 755 us, the
+// tensor pipe 94 % active with its operands' reads.  (Q from tensor memory, which halves what the MMAs read of shared memory, and two tiles
+// at a time in a group: no gain.)
 //
 // The call has no workspace to pass the check's answer through.  It goes through words of the context, one for each block of the check: `epoch` where the block
 // found its pairs so, else 0.  The context's ring of them is shared by calls on several streams, so a word may be overwritten by a later
