@@ -333,6 +333,9 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 if (++vu == kVUnits) { vu = 0; vph ^= 1u; }
               }
               if (!mbar_wait(sh, V_FULL + (int)vu, vph, status)) { ok = false; break; }
+              // The tile before (lone() sees that there is one) has accumulated on the same O in another form and shape: MMAs of one
+              // accumulator keep their order by themselves only within a shape.
+              if (!mbar_wait(sh, PV_DONE + (int)(pbuf ^ 1u), ((cp - 1u) >> 1) & 1u, status)) { ok = false; break; }
               tc_fence_after();
               const uint32_t v4lo = vd4_lo + vu * (kUnit >> 4);
 #pragma unroll

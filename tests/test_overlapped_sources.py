@@ -1,4 +1,6 @@
-"""Kernels that start while the kernel before them runs must not promise the compiler that what that kernel writes is constant: no
+"""Properties of the kernels' sources that no run shows reliably.
+
+Kernels that start while the kernel before them runs must not promise the compiler that what that kernel writes is constant: no
 __restrict__ and no __ldg on the buffers that the calls hand from one kernel to the next."""
 import os
 import re
@@ -13,3 +15,19 @@ def test_buffers_between_kernels_are_not_promised_constant():
         text = re.sub(r"//[^\n]*", "", open(os.path.join(build.CSRC, name)).read())
         assert not re.findall(r"__restrict__\s+" + HANDED_ON + r"\b", text), name
         assert not re.findall(r"__ldg\([^;]*\b" + HANDED_ON + r"\b", text), name
+
+
+def code(name):
+    return re.sub(r"//[^\n]*", "", open(os.path.join(build.CSRC, name)).read())
+
+
+def test_a_product_of_another_shape_waits_for_the_ones_before_it():
+    """The pair kernel's product for the second block alone goes to an accumulator that products of another form and shape write: MMAs of one
+    accumulator keep their order by themselves only within a shape, so a wait for the commit of the tile before stands between them."""
+    text = code("attn_pair.cu")
+    lone = [m.start() for m in re.finditer(r"\btc_mma_ws_ts\(", text)]
+    assert len(lone) == 1
+    before = text[:lone[0]]
+    wait = before.rfind("mbar_wait(sh, PV_DONE")
+    assert wait > max(before.rfind("tc_mma_ts("), before.rfind("tc_mma_ss(")), "no wait between the two forms"
+    assert "tc_fence_after()" in before[wait:]
