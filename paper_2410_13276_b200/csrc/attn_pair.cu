@@ -448,7 +448,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         sco = lo > 0.f ? 1.f / lo : 0.f;
         lse_row = l > 0.f ? (R + log2f(l)) * 0.6931471805599453f : -CUDART_INF_F;
       }
-      fail = !mbar_wait(sh, PV_DONE + (int)((cnt - 1) & 1u), ((cnt - 1) >> 1) & 1u, status);
+      fail = !mbar_wait_warp(sh, PV_DONE + (int)((cnt - 1) & 1u), ((cnt - 1) >> 1) & 1u, status);
       fail = named_bar_or(bar_vote, kBoth, fail);           // no row is stored by halves
       if (fail) break;
       tc_fence_after();

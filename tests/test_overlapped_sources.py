@@ -31,3 +31,17 @@ def test_a_product_of_another_shape_waits_for_the_ones_before_it():
     wait = before.rfind("mbar_wait(sh, PV_DONE")
     assert wait > max(before.rfind("tc_mma_ts("), before.rfind("tc_mma_ss(")), "no wait between the two forms"
     assert "tc_fence_after()" in before[wait:]
+
+
+def test_lanes_agree_before_an_aligned_barrier():
+    """named_bar_or is an aligned barrier: all lanes of a warp come to it together.  A bounded wait returns lane by lane, so where a softmax or maxima
+    warp keeps its outcome, the warp votes before it goes on to a barrier."""
+    for name in ("attn_tc.cu", "attn_pair.cu"):
+        text = code(name)
+        assert "bar.red.or.pred" in code("attn_tc_common.cuh")
+        kept = list(re.finditer(r"\bfail = (?:[^;]*\|\| )?!mbar_wait\(", text))
+        assert kept, name
+        for m in kept:
+            after = text[m.end():]
+            vote, bar = after.find("__any_sync("), after.find("named_bar_or(")
+            assert 0 <= vote < (bar if bar >= 0 else len(after)), (name, text[m.start():m.start() + 90])
