@@ -195,8 +195,9 @@ seer_status seer_set_attn_impl(seer_ctx* ctx, int impl);
  * SEER_ERR_TIMEOUT on the device status, sets a flag that every other role of its CTA polls, the CTA lets the copies
  * and MMAs in flight land, frees its tensor memory and returns; rows it had not finished are not written.
  * lose_v_copy_of_tile >= 0 makes exactly one wait run out: the first stream of CTA 0 never issues the V copy of its
- * tile with that ordinal (counted over the CTA's work items from 0), so the MMA issuer's wait for it expires;
- * (where pairs of query blocks are done together, CTA 0 does not issue the V copy of its tile with that ordinal);
+ * tile with that ordinal (counted over the CTA's work items from 0), so the MMA issuer's wait for it expires
+ * (where pairs of query blocks are done together, CTA 0 does not issue the V copy of its tile with that ordinal; the
+ * block maxima, which read no V, lose the K copy of that tile);
  * nothing faults and the context stays usable.  -1 switches the hook off.  wait_limit_us = 0 is rejected. */
 seer_status seer_debug_lost_wait(seer_ctx* ctx, uint32_t wait_limit_us, int32_t lose_v_copy_of_tile);
 

@@ -546,7 +546,7 @@ block_max_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     if (warp == 0) {
       if (elect_one()) {
         const uint32_t* col = reinterpret_cast<const uint32_t*>(col_idx);
-        uint32_t nitem = 0, ku = 0, kph = 0;
+        uint32_t nitem = 0, ku = 0, kph = 0, cnt = 0;
         bool ok = true;
         for (uint32_t n = 0; ok; ++n) {
           const int64_t w = dealt_pair(m, n);
@@ -572,18 +572,21 @@ block_max_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
               for (int dh = 0; dh < 2; ++dh)
                 tma_load_3d(sh.base + kOffQ + qb * kQBytes + (uint32_t)(2 * dh + half) * kHalfTile, &map_q, qf, 64 * dh, it.h, it.tok0 + 64 * half);
           ++nitem;
-          for (int t = 0; t < tiles; ++t) {
+          for (int t = 0; t < tiles; ++t, ++cnt) {
             const int p = 2 * t + 2;
             const int ra = p < it.len ? (int)ld_global(col + it.l0 + p) : -1, rb = p + 1 < it.len ? (int)ld_global(col + it.l0 + p + 1) : -1;   // next pair
             const bool has_b = jb >= 0;
             const int ta = it.s0 + ja * kBlock, tb = it.s0 + jb * kBlock;
             if (!mbar_wait(sh, M_K_EMPTY + (int)ku, kph ^ 1u, status)) { ok = false; break; }
             const uint32_t fb = sh.bar(M_K_FULL + (int)ku), dst = sh.base + kOffK + ku * kUnit;
-            mbar_expect_tx(fb, has_b ? kUnit : kUnit / 2);
+            // test hook: one K copy that is never issued, so that the issuer's wait for it runs out
+            if (blockIdx.x != 0 || m.lose_v_copy < 0 || cnt != (uint32_t)m.lose_v_copy) {
+              mbar_expect_tx(fb, has_b ? kUnit : kUnit / 2);
 #pragma unroll
-            for (int dh = 0; dh < 2; ++dh) {
-              tma_load_3d(dst + (uint32_t)dh * 2 * kHalfTile, &map_k, fb, 64 * dh, g, ta);
-              if (has_b) tma_load_3d(dst + (uint32_t)dh * 2 * kHalfTile + kHalfTile, &map_k, fb, 64 * dh, g, tb);
+              for (int dh = 0; dh < 2; ++dh) {
+                tma_load_3d(dst + (uint32_t)dh * 2 * kHalfTile, &map_k, fb, 64 * dh, g, ta);
+                if (has_b) tma_load_3d(dst + (uint32_t)dh * 2 * kHalfTile + kHalfTile, &map_k, fb, 64 * dh, g, tb);
+              }
             }
             if (++ku == kMaxKUnits) { ku = 0; kph ^= 1u; }
             ja = ra; jb = rb;
@@ -640,14 +643,16 @@ block_max_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const int bar_block = 1 + 2 * g + half;                 // the two warps of a query block
     constexpr int bar_vote = 5, kBoth = 256;
     uint32_t cnt = 0, flushes = 0;
+    bool lost = false;                                      // this warp, or its neighbour, has given up
     for (uint32_t n = 0;; ++n) {
-      bool fail = !mbar_wait_warp(sh, M_ITEM_FULL + (int)(n & 3u), (n >> 2) & 1u, status);
+      bool fail = lost || !mbar_wait_warp(sh, M_ITEM_FULL + (int)(n & 3u), (n >> 2) & 1u, status);
       uint4 a{}, b{}, c{};
       if (!fail) { a = ld_shared_v4(ring_addr(n)); b = ld_shared_v4(ring_addr(n) + 16u); c = ld_shared_v4(ring_addr(n) + 32u); }
       __syncwarp();
       if (lane == 0 && !fail) mbar_arrive(sh.bar(M_ITEM_EMPTY + (int)(n & 3u)));
       const int len = (int)a.w;
-      if (fail || len < 0) { named_bar_or(bar_vote, kBoth, fail); break; }
+      // A warp with an item waits in it for its neighbour: so either all warps have the item, or none goes on.
+      if (named_bar_or(bar_vote, kBoth, fail) || len < 0) break;
       const int mine_n = (int)(half ? b.z : b.y), plain = (int)(half ? c.y : c.x), l0 = (int)(half ? b.x : a.z);
       const int valid = (int)(half ? b.w >> 16 : b.w & 0xffffu);
       float L = row < valid ? lse[(int64_t)a.x * lse_stride + (int)a.y + 64 * half + row] : 0.f;
@@ -677,7 +682,7 @@ block_max_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         if (at == 31 || p + 2 >= len + g) {
           int* there = other + (flushes++ & 1u) * 32;
           if ((quad & 1) != 0) there[lane] = key;
-          if (named_bar_or(bar_block, 64, false)) break;
+          if (named_bar_or(bar_block, 64, false)) { lost = true; break; }
           const int mine = first_p + 2 * lane;
           if ((quad & 1) == 0 && lane <= at && mine < mine_n) {
             int kx = max(key, there[lane]);
@@ -687,8 +692,7 @@ block_max_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
           first_p = p + 2;
         }
       }
-      if (fail) named_bar_or(bar_block, 64, true);          // (the neighbour may be waiting there)
-      if (named_bar_or(bar_vote, kBoth, fail)) break;
+      if (fail) { named_bar_or(bar_block, 64, true); lost = true; }   // (the neighbour is waiting there, or will)
     }
   }
 

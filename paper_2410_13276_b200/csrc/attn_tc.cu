@@ -251,13 +251,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             // a rejected entry: any valid block, masked out in the softmax
             const int ta = it.s0 + (ja < 0 ? 0 : ja) * kBlock, tb = it.s0 + (jb < 0 ? 0 : jb) * kBlock;
             tr.sample(cnt); tr.ev(1);
+            // test hook of the block maxima: one K copy that is never issued, so that the issuer's wait for it runs out
+            const bool lost = kBlockMax && s == 0 && blockIdx.x == 0 && m.lose_v_copy >= 0 && cnt == (uint32_t)m.lose_v_copy;
 #pragma unroll
             for (int dh = 0; dh < 2; ++dh) {
               if (!mbar_wait(sh, bb + empty_k + (int)ku, kph ^ 1u, status)) { ok = false; break; }
               const uint32_t fb = sh.bar(bb + K_FULL + (int)ku), dst = sbase + kStK + ku * kUnit;
-              mbar_expect_tx(fb, has_b ? kUnit : kUnit / 2);   // (an odd list's last tile: the scores of the missing block are not looked at)
-              tma_load_3d(dst, &map_k, fb, 64 * dh, g, ta);
-              if (has_b) tma_load_3d(dst + kHalfQ, &map_k, fb, 64 * dh, g, tb);
+              if (!lost) {
+                mbar_expect_tx(fb, has_b ? kUnit : kUnit / 2);   // (an odd list's last tile: the scores of the missing block are not looked at)
+                tma_load_3d(dst, &map_k, fb, 64 * dh, g, ta);
+                if (has_b) tma_load_3d(dst + kHalfQ, &map_k, fb, 64 * dh, g, tb);
+              }
               if (++ku == ring_k) { ku = 0; kph ^= 1u; }
             }
             tr.ev(2);
@@ -419,17 +423,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     const bool o32 = kTrace ? (reinterpret_cast<uintptr_t>(o) & 31) == 0 : kO32;
     Tracer<kTrace> tr; tr.init(r == 0 ? trace : nullptr, 4 + s);
     uint32_t cnt = 0, nitem = 0;                            // tiles and items with tiles this stream has processed
+    bool lost = false;                                      // block maxima: this warp, or its neighbour, has given up
     for (uint32_t n = 0;; ++n) {
       tr.sample(0);
-      // a lost wait does not simply leave: the warps of a group meet once per item with tiles, and all of them have to get
-      // there; a warp that gives up votes early, the others find its vote at their next meeting
-      bool fail = !mbar_wait(sh, item_full(s, n), (n >> 2) & 1u, status);
+      // a lost wait does not simply leave: the warps of a group meet once per item with tiles (block maxima: before every item), and all of
+      // them have to get there; a warp that gives up votes early, the others find its vote at their next meeting
+      bool fail = (kBlockMax && lost) || !mbar_wait(sh, item_full(s, n), (n >> 2) & 1u, status);
       Slot it{};
       if (!fail) it = read_slot(s, n);
       __syncwarp();
       if (lane == 0 && !fail) release_item(s, n);
       fail = __any_sync(0xffffffffu, fail);
-      if (fail || it.nlist < 0) { named_bar_or(bar_vote, kGroupThreads, fail); break; }
+      if constexpr (kBlockMax) {
+        // a warp with an item waits in it for its neighbour: so either all warps of the group have the item, or none goes on
+        if (named_bar_or(bar_vote, kGroupThreads, fail) || it.nlist < 0) break;
+      } else if (fail || it.nlist < 0) { named_bar_or(bar_vote, kGroupThreads, fail); break; }
       const int ntiles = it.ntiles();
       if (ntiles == 0) {                                    // no visible key: o = 0, lse = -inf
         if constexpr (!kBlockMax) {
@@ -469,15 +477,15 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(sh.bar(bb + M_TAKEN + (int)sbuf));
-          if (named_bar_or(5 + 2 * s + half, 64, false)) break;
+          if (named_bar_or(5 + 2 * s + half, 64, false)) { lost = true; break; }
           if ((quad & 1) == 0 && lane == 0 && p < it.nlist) {
             int kx = max(wmax[buf * 4 + quad], wmax[buf * 4 + quad + 1]);
             kx ^= (kx >> 31) & 0x7fffffff;
             block_max[it.l0 + p] = exp2f(__int_as_float(kx));   // 2^(-inf) = 0: no causal pair, or a rejected entry
           }
         }
-        if (fail) named_bar_or(5 + 2 * s + half, 64, true); // (the neighbour may be waiting there)
-        if (named_bar_or(bar_vote, kGroupThreads, fail)) break;
+        if (fail) { named_bar_or(5 + 2 * s + half, 64, true); lost = true; }   // (the neighbour is waiting there, or will)
+        if (lost) continue;
         if (lane == 0) mbar_arrive(sh.bar(bb + Q_EMPTY + (int)(nitem & 1u)));
         ++nitem;
         continue;

@@ -1,7 +1,7 @@
 """The bounded waits of the tcgen05 attention kernel, exercised without faulting anything (needs a B200).
 
 seer_debug_lost_wait makes exactly one wait run out: the first stream of CTA 0 never issues the V copy of one of its
-tiles, so the MMA issuer's wait for that copy expires after the (shortened) limit.  What must then hold: the device
+tiles (the block maxima: the K copy), so the MMA issuer's wait for that copy expires after the (shortened) limit.  What must then hold: the device
 status is SEER_ERR_TIMEOUT, the kernel has returned (the call and the poll come back), every row that does not belong
 to the stream that lost its copy equals the normal run bit for bit, and the context goes on working: the next call
 without the hook gives the normal result (so the tensor memory of the aborted CTA was freed and no barrier is left
@@ -122,6 +122,38 @@ def test_a_lost_last_copy_leaves_the_items_rows_unwritten(rt, keep, lost_tile, l
     p.o.fill_(float("nan")); p.lse.fill_(float("nan"))
     p.attn(); torch.cuda.synchronize()
     assert p.status() == 0 and torch.equal(p.o, o_ref) and torch.equal(p.lse, lse_ref)
+
+
+@pytest.mark.parametrize("S,hq,hkv,lost_tile", [(4096, 8, 2, 0), (4096, 8, 2, 37), (8192, 32, 8, 0), (8192, 32, 8, 31), (8192, 32, 8, 32), (8192, 32, 8, 333)])
+def test_a_lost_copy_of_the_block_maxima(rt, S, hq, hkv, lost_tile):
+    """A K copy that CTA 0 never issues, query block by query block (4096 tokens) and by pairs (8192: 2^18 causal blocks): the call returns with the
+    status, entries of CTA 0's share are right or as they were, all others are right, and the next call is normal."""
+    import torch
+    B, Prefill, ctx = rt
+    w = W.make_small(seed=4244, seqlens=[S], hq=hq, hkv=hkv)
+    p = Prefill(w.cu_seqlens, hq, hkv, ctx=ctx, want_lse=True)
+    p.set_inputs(w.q, w.k, w.v, w.wq, w.wk)
+    p.scores.zero_()
+    p.mask(B.make_mask_params(B.SEER_TOPK_COUNT, k=1 << 20, flags=B.SEER_FORCE_DIAG))
+    p.attn()
+    want = p.block_max().clone()
+    assert p.status() == 0
+    B.seer_debug_lost_wait(ctx, 5_000, lost_tile)
+    try:
+        p.bmax.fill_(-1.0)
+        p.block_max()
+        status = B.seer_poll_device_status(ctx)
+    finally:
+        B.seer_debug_lost_wait(ctx, 2_000_000, -1)
+    assert B.STATUS_NAMES[status] == "SEER_ERR_TIMEOUT"
+    missing = p.bmax == -1.0
+    assert torch.equal(p.bmax[~missing], want[~missing])
+    rows = torch.searchsorted(p.row_ptr.long(), torch.nonzero(missing)[:, 0], right=True).unique().numel()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert 1 <= rows <= 2 * (-(-hq * (S // 64) // (2 * sms)) + 1)
+    p.bmax.fill_(-1.0)
+    p.block_max()
+    assert p.status() == 0 and torch.equal(p.bmax, want)
 
 
 def test_lost_wait_hook_rejects_a_zero_limit(rt):
