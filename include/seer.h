@@ -164,8 +164,8 @@ seer_status seer_block_mask(seer_ctx* ctx, const seer_shape* shape, const float*
  *    overflow where a row's scores rise far (by up to 2^60 in probability) above those of the first block of its list.
  *    ws (optional): with a workspace of at least 256 bytes (256-byte aligned, as for the other calls) the first word
  *    becomes the counter from which the tcgen05 kernel's persistent CTAs draw their (head, query block) work items,
- *    so that a CTA that finishes early takes more of them, and the second word says whether pairs of query blocks list the same
- *    blocks (large problems, which are then done by pairs); without a workspace (NULL), and where there are no more than two items
+ *    so that a CTA that finishes early takes more of them, and the others of these 256 bytes say whether pairs of query blocks list
+ *    the same blocks (large problems, which are then done by pairs); without a workspace (NULL), and where there are no more than two items
  *    a CTA, the items are dealt statically.  The results are identical bit for bit.  Calls that may run at the same time must not share the workspace. */
 seer_status seer_sparse_attn(seer_ctx* ctx, const seer_shape* shape, const void* q, const void* k, const void* v,
                              const int32_t* row_ptr, const int32_t* col_idx, void* o, float* lse, void* ws,

@@ -55,44 +55,31 @@ constexpr uint32_t kIdescS = make_idesc(false, false, 128u, 128u);
 constexpr uint32_t kIdescPV = make_idesc(false, true, 128u, 128u);
 constexpr uint32_t kIdescLone = make_idesc(false, true, 256u, 64u);
 
-// Zeroes the work counter and writes `epoch` to *differs unless every pair of query blocks has one list (pair_ok).
-// Where lists differ a block finds out with its first items, after three trips to L2.  (One write a block: as many as there are warps, to one
-// word, take 5 us.)
-constexpr int kCheckWarps = 8;
+// Whether every pair of query blocks has one list (pair_ok), answered block by block: words[block] becomes `epoch` where the block found its pairs
+// so, else 0.  Also zeroes the attention's work counter.  A warp goes through its pairs by itself and leaves where one of its block's differs: where lists
+// differ it finds out with the first, after three trips to L2.
+constexpr int kCheckWarps = 32;
 template <bool kChunk>
-__global__ void __launch_bounds__(kCheckWarps * 32) check_kernel(SeqMeta m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, int* differs, int epoch) {
+__global__ void __launch_bounds__(kCheckWarps * 32) check_kernel(SeqMeta m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, int* words, int epoch) {
+  __shared__ int differs;
+  if (threadIdx.x == 0) differs = 0;
+  __syncthreads();
   grid_wait();
-  if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
+  if (counter != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
   const int lane = threadIdx.x & 31;
-  const uint32_t* col = reinterpret_cast<const uint32_t*>(col_idx);
-  for (int64_t w0 = (int64_t)blockIdx.x * kCheckWarps; w0 < m.pair_units; w0 += (int64_t)gridDim.x * kCheckWarps) {
-    const int64_t w = w0 + (threadIdx.x >> 5);
-    const bool ok = w >= m.pair_units || pair_ok<kChunk>(m, row_ptr, col, w, lane);
-    const bool others = w0 >= (int64_t)gridDim.x * kCheckWarps && threadIdx.x == 0 && *(volatile int*)differs == epoch;   // (not for the first items)
-    if (__syncthreads_or(!ok || others)) {
-      if (threadIdx.x == 0) *(volatile int*)differs = epoch;
-      return;
-    }
+  for (int64_t w = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < m.pair_units; w += (int64_t)gridDim.x * kCheckWarps) {
+    if (__any_sync(0xffffffffu, *(volatile int*)&differs != 0)) break;
+    if (!pair_ok<kChunk>(m, row_ptr, reinterpret_cast<const uint32_t*>(col_idx), w, lane) && lane == 0) *(volatile int*)&differs = 1;
   }
-}
-
-// The same question for the block maxima, answered block by block in words[].
-template <bool kChunk>
-__global__ void __launch_bounds__(kCheckWarps * 32) check_words_kernel(SeqMeta m, const int32_t* row_ptr, const int32_t* col_idx, int* words, int epoch) {
-  grid_wait();
-  bool ok = true;
-  for (int64_t w0 = (int64_t)blockIdx.x * kCheckWarps; ok && w0 < m.pair_units; w0 += (int64_t)gridDim.x * kCheckWarps) {
-    const int64_t w = w0 + (threadIdx.x >> 5);
-    ok = !__syncthreads_or(w < m.pair_units && !pair_ok<kChunk>(m, row_ptr, reinterpret_cast<const uint32_t*>(col_idx), w, threadIdx.x & 31));
-  }
-  if (threadIdx.x == 0) *(volatile int*)(words + blockIdx.x) = ok ? epoch : 0;
+  __syncthreads();
+  if (threadIdx.x == 0) *(volatile int*)(words + blockIdx.x) = differs == 0 ? epoch : 0;
 }
 
 template <bool kChunk, bool kO32>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
                  const __grid_constant__ CUtensorMap map_v32, SeqMeta m, const int32_t* row_ptr, const int32_t* col_idx, uint16_t* __restrict__ o, float* lse, int* __restrict__ status,
-                 int* __restrict__ work_counter, const int* differs, int epoch) {
+                 int* __restrict__ work_counter, const int* words, int nwords, int epoch) {
   extern __shared__ __align__(1024) unsigned char smem[];
   Shared sh;
   sh.base = smem_u32(smem);
@@ -105,7 +92,7 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     return;
   }
   grid_wait();
-  if (ld_global(reinterpret_cast<const uint32_t*>(differs)) == (uint32_t)epoch) return;   // attn_tc_kernel has done it
+  if (!lists_agree(words, nwords, epoch)) return;           // attn_tc_kernel has done it
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kOffMisc);
   if (threadIdx.x == 0) {
@@ -499,8 +486,8 @@ attn_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 // tensor pipe 94 % active with its operands' reads.  (Q from tensor memory, which halves what the MMAs read of shared memory, and two tiles
 // at a time in a group: no gain.)
 //
-// The call has no workspace to pass the check's answer through.  It goes through words of the context, one for each block of the check: `epoch` where the block
-// found its pairs so, else 0.  The context's ring of them is shared by calls on several streams, so a word may be overwritten by a later
+// The call has no workspace to pass the check's answer through.  It goes through words of the context.
+// The context's ring of them is shared by calls on several streams, so a word may be overwritten by a later
 // call's; it never gets this call's number again.  So a CTA that does not find all words takes the lists to differ, and as this
 // kernel runs before attn_tc_kernel, no row is left out by both: at worst it is done twice, with the same result.
 constexpr uint32_t kMaxKUnits = 5, kMaxS = 4;
@@ -707,7 +694,7 @@ block_max_pair_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
   }
 }
 
-using Kernel = void(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, SeqMeta, const int32_t*, const int32_t*, uint16_t*, float*, int*, int*, const int*, int);
+using Kernel = void(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, SeqMeta, const int32_t*, const int32_t*, uint16_t*, float*, int*, int*, const int*, int, int);
 
 }  // namespace tp
 
@@ -722,34 +709,28 @@ static cudaError_t ready(seer_ctx* ctx) {
   return e;
 }
 
-int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, int epoch, cudaStream_t stream) {
-  const unsigned blocks = (unsigned)min((int64_t)ctx->num_sms * 2, (m.pair_units + tp::kCheckWarps - 1) / tp::kCheckWarps);
+int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, const PairAnswer& a, cudaStream_t stream) {
   cudaError_t e = ready(ctx);
   if (e != cudaSuccess) return -(int)e;
-  e = launch_next(m.chunked ? tp::check_kernel<true> : tp::check_kernel<false>, blocks, tp::kCheckWarps * 32, 0, stream, m, row_ptr, col_idx, counter, counter + 1, epoch);
+  e = launch_next(m.chunked ? tp::check_kernel<true> : tp::check_kernel<false>, (unsigned)a.nwords, tp::kCheckWarps * 32, 0, stream, m, row_ptr, col_idx, counter, a.words, a.epoch);
   return e == cudaSuccess ? 1 : -(int)e;
 }
 
 int launch_attn_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mv32, const int32_t* row_ptr,
-                     const int32_t* col_idx, void* o, float* lse, int* counter, int epoch, cudaStream_t stream) {
+                     const int32_t* col_idx, void* o, float* lse, int* counter, const PairAnswer& a, cudaStream_t stream) {
   const bool o32 = ((uintptr_t)o & 31) == 0;
   tp::Kernel* kernel = m.chunked ? (o32 ? tp::attn_pair_kernel<true, true> : tp::attn_pair_kernel<true, false>)
                                  : (o32 ? tp::attn_pair_kernel<false, true> : tp::attn_pair_kernel<false, false>);
   const cudaError_t e = launch_next(kernel, (unsigned)min((int64_t)ctx->num_sms, m.pair_units), tp::kThreads, tp::kSmemBytes, stream, mq, mk, mv, mv32, m, row_ptr,
-                                    col_idx, (uint16_t*)o, lse, ctx->d_status, counter, (const int*)(counter + 1), epoch);
+                                    col_idx, (uint16_t*)o, lse, ctx->d_status, counter, (const int*)a.words, a.nwords, a.epoch);
   return e == cudaSuccess ? 1 : -(int)e;
 }
 
 int launch_block_max_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const int32_t* row_ptr, const int32_t* col_idx, const float* lse,
-                          float* out, int* words, int nwords, int epoch, cudaStream_t stream) {
-  cudaError_t e = ready(ctx);
-  if (e != cudaSuccess) return -(int)e;
-  e = launch_next(m.chunked ? tp::check_words_kernel<true> : tp::check_words_kernel<false>, (unsigned)nwords, tp::kCheckWarps * 32, 0, stream, m, row_ptr, col_idx,
-                              words, epoch);
-  if (e != cudaSuccess) return -(int)e;
-  e = launch_next(m.chunked ? tp::block_max_pair_kernel<true> : tp::block_max_pair_kernel<false>, (unsigned)min((int64_t)ctx->num_sms, m.pair_units), tp::kThreads,
-                  tp::kSmemBytes, stream, mq, mk, m, row_ptr, col_idx, lse, ctx->d_status, out, (const int*)words, nwords, epoch);
-  return e == cudaSuccess ? 2 : -(int)e;
+                          float* out, const PairAnswer& a, cudaStream_t stream) {
+  const cudaError_t e = launch_next(m.chunked ? tp::block_max_pair_kernel<true> : tp::block_max_pair_kernel<false>, (unsigned)min((int64_t)ctx->num_sms, m.pair_units), tp::kThreads,
+                                    tp::kSmemBytes, stream, mq, mk, m, row_ptr, col_idx, lse, ctx->d_status, out, (const int*)a.words, a.nwords, a.epoch);
+  return e == cudaSuccess ? 1 : -(int)e;
 }
 
 }  // namespace seer

@@ -80,8 +80,7 @@ __device__ __forceinline__ int64_t dealt_pair(const SeqMeta& m, uint32_t k) {
   const int64_t w = (int64_t)k * gridDim.x + ((k & 1u) ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
   return w < m.pair_units ? w : -1;
 }
-// Whether all of a check's words are this call's (kWords of them at most, as many threads or more).
-constexpr int kWords = 256;
+// Whether all of a check's words are this call's (kPairWords of them at most, as many threads or more).
 __device__ __forceinline__ bool lists_agree(const int* words, int nwords, int epoch) {
   return !__syncthreads_or((int)threadIdx.x < nwords && *(const volatile int*)(words + threadIdx.x) != epoch);
 }

@@ -119,20 +119,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
                 const int32_t* row_ptr, const int32_t* col_idx,
                 uint16_t* __restrict__ o, float* lse, int* __restrict__ status,
                 unsigned long long* __restrict__ trace, float* block_max = nullptr,
-                int* __restrict__ work_counter = nullptr, const int* differs = nullptr, int epoch = 0, int nwords = 0) {
+                int* __restrict__ work_counter = nullptr, const int* words = nullptr, int nwords = 0, int epoch = 0) {
   extern __shared__ __align__(1024) unsigned char smem[];
   Shared sh;
   sh.base = smem_u32(smem);
   sh.bar0 = sh.base + kOffBar;
   sh.abort_addr = sh.base + kOffMisc + 8;
   sh.limit_us = m.wait_limit_us;
-  if (!kBlockMax && differs != nullptr) {                  // (a way out from further in costs a launch of 32k tokens 2 %)
+  if (words != nullptr) {                                  // (a way out from further in costs a launch of 32k tokens 2 %)
     grid_wait();
-    if (ld_global(reinterpret_cast<const uint32_t*>(differs)) != (uint32_t)epoch) return;   // attn_pair_kernel does the work
-  }
-  if (kBlockMax && differs != nullptr) {                   // (here: the check's words, `nwords` of them)
-    grid_wait();
-    if (tp::lists_agree(differs, nwords, epoch)) return;    // block_max_pair_kernel has done the work
+    if (tp::lists_agree(words, nwords, epoch)) return;      // attn_pair_kernel does the work, block_max_pair_kernel has done it
   }
   if ((sh.base & 1023u) != 0u) {                           // the swizzled tiles need the alignment
     grid_wait();
@@ -751,9 +747,9 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
   // nothing to do; where they do share them it saves a sixth of the launch.  Asked from 2^20 causal blocks on (16k tokens, 32 heads: a tenth of
   // them takes 240 us, all of them 2400).
   const bool pairs = work_counter != nullptr && ctx->trace == nullptr && m.score_tiles >= (1 << 20) / (128 * kScoreTile);
-  const int epoch = (int)ctx->clock;
+  const PairAnswer answer(ctx, m, pairs ? work_counter + 1 : nullptr);
   if (pairs) {
-    launched = launch_pair_check(ctx, m, row_ptr, col_idx, work_counter, epoch, stream);
+    launched = launch_pair_check(ctx, m, row_ptr, col_idx, work_counter, answer, stream);
     if (launched < 0) return launched;
   } else if (work_counter != nullptr) {
     e = launch_next(tc::zero_kernel, 1, 32, 0, stream, work_counter);
@@ -768,13 +764,13 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
                      : few ? (m.chunked ? tc::attn_tc_kernel<false, true, false, true, true> : tc::attn_tc_kernel<false, false, false, true, true>)
                      : m.chunked ? tc::attn_tc_kernel<false, true> : tc::attn_tc_kernel<false, false>;
   e = launch_next(kernel, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter,
-                  pairs ? (const int*)work_counter + 1 : nullptr, epoch, 0);
+                  (const int*)answer.words, answer.nwords, answer.epoch);
   if (e != cudaSuccess) return -(int)e;
   ++launched;
   if (pairs) {
     CUtensorMap mv64;
     if (!tc::make_map(ctx, &mv64, v, m.total_tokens, m.num_kv_heads, 64)) return -(int)cudaErrorInvalidValue;
-    const int n = launch_attn_pair(ctx, m, mq, mk, mv64, mv, row_ptr, col_idx, o, lse, work_counter, epoch, stream);
+    const int n = launch_attn_pair(ctx, m, mq, mk, mv64, mv, row_ptr, col_idx, o, lse, work_counter, answer, stream);
     if (n < 0) return n;
     launched += n;
   }
@@ -792,17 +788,18 @@ int launch_block_max_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const vo
   float* lse_in = const_cast<float*>(lse);   // read only in this mode
   // Pairs of query blocks that share their lists (attn_pair.cu): asked for from 2^18 causal blocks on (8k tokens, 32 heads), sooner than for the
   // attention, as the map is taken of dense lists above all.  16k tokens: all blocks 1045 -> 755 us, a tenth of them 128 -> 131.
-  int* words = nullptr;
-  int nwords = 0, launched = 0;
-  const int epoch = 1 + (int)(ctx->clock & 0x3fffffff);    // (a word of lists that differ is 0)
-  if (m.score_tiles >= (1 << 18) / (128 * kScoreTile)) {
-    words = ctx->words + (ctx->clock % kWordSets) * tp::kWords;
-    nwords = (int)min((int64_t)tp::kWords, m.pair_units);
-    launched = launch_block_max_pair(ctx, m, mq, mk, row_ptr, col_idx, lse, out, words, nwords, epoch, stream);
+  const bool pairs = m.score_tiles >= (1 << 18) / (128 * kScoreTile);
+  const PairAnswer answer(ctx, m, pairs ? ctx->words + (ctx->clock % kWordSets) * kPairWords : nullptr);
+  int launched = 0;
+  if (pairs) {
+    launched = launch_pair_check(ctx, m, row_ptr, col_idx, nullptr, answer, stream);
     if (launched < 0) return launched;
+    const int n = launch_block_max_pair(ctx, m, mq, mk, row_ptr, col_idx, lse, out, answer, stream);
+    if (n < 0) return n;
+    launched += n;
   }
   const cudaError_t e = launch_next(m.chunked ? tc::attn_tc_kernel<false, true, true> : tc::attn_tc_kernel<false, false, true>, grid, tc::kThreads, tc::kSmemBytes, stream,
-                                    mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr, (const int*)words, epoch, nwords);
+                                    mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr, (const int*)answer.words, answer.nwords, answer.epoch);
   return e == cudaSuccess ? launched + 1 : -(int)e;
 }
 

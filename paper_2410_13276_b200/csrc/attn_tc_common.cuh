@@ -520,13 +520,18 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bo
 
 }  // namespace tcc
 
-// Attention where pairs of query blocks list the same blocks (attn_pair.cu).  The check zeroes the work counter and writes `epoch` to the
-// word behind it where some pair's lists differ; attn_tc_kernel returns at once where none do, attn_pair_kernel where some do.
-int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, int epoch, cudaStream_t stream);
+// Attention where pairs of query blocks list the same blocks (attn_pair.cu).  The check answers in `nwords` words, all of them written by every call: `epoch`
+// in all of them where all pairs do.  attn_tc_kernel then returns at once, otherwise attn_pair_kernel.  (The attention's words lie behind the counter in a workspace
+// of 256 bytes or more, those of the block maxima in the context.)
+struct PairAnswer {
+  int* words;
+  int nwords, epoch;
+  PairAnswer(const seer_ctx* ctx, const SeqMeta& m, int* at) : words(at), nwords((int)min((int64_t)kPairWords, m.pair_units)), epoch(1 + (int)(ctx->clock & 0x3fffffff)) {}
+};
+int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, const PairAnswer& a, cudaStream_t stream);
 int launch_attn_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mv32, const int32_t* row_ptr,
-                     const int32_t* col_idx, void* o, float* lse, int* counter, int epoch, cudaStream_t stream);
-// The block maxima likewise; the answer is `epoch` in all of nwords words (at most tp::kWords) of the context's.
+                     const int32_t* col_idx, void* o, float* lse, int* counter, const PairAnswer& a, cudaStream_t stream);
 int launch_block_max_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const int32_t* row_ptr, const int32_t* col_idx, const float* lse,
-                          float* out, int* words, int nwords, int epoch, cudaStream_t stream);
+                          float* out, const PairAnswer& a, cudaStream_t stream);
 
 }  // namespace seer

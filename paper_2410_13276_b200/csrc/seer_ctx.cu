@@ -335,7 +335,7 @@ seer_status seer_create(seer_ctx** out, int device) {
   ctx->device = device;
   ctx->num_sms = sms;
   // (the status word, and behind it the sets of words of the block maxima)
-  constexpr size_t kStatusBytes = 256 + (size_t)kWordSets * 256 * sizeof(int);
+  constexpr size_t kStatusBytes = 256 + (size_t)kWordSets * kPairWords * sizeof(int);
   bool ok = cudaMalloc(&ctx->d_status, kStatusBytes) == cudaSuccess &&
             cudaMemset(ctx->d_status, 0, kStatusBytes) == cudaSuccess && cudaMallocHost(&ctx->stage, kStageBytes) == cudaSuccess;
   if (ok) ctx->words = ctx->d_status + 64;

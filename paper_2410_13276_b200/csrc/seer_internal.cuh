@@ -15,7 +15,8 @@ constexpr int kHeadDim = 128;
 constexpr int kGateDim = 128;
 constexpr int kMaxBatch = 4096;
 constexpr int kMetaSlots = 8;
-constexpr int kWordSets = 16;   // sets of 256 words (block maxima, attn_pair.cu)
+constexpr int kPairWords = 63;  // words of the answer whether pairs of query blocks share their lists (attn_pair.cu)
+constexpr int kWordSets = 16;   // sets of them in a context (block maxima)
 constexpr int kScoreTile = 64;  // column tile of the gate's score kernel, and granularity of the bands of the one-call gate + mask
 
 // Per-batch metadata the kernels read from device memory.

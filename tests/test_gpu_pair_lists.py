@@ -1,6 +1,6 @@
 """Attention where query blocks 2u and 2u + 1 list the same blocks: o and lse equal those of the launch without a work counter, which takes every
-query block by itself, bit for bit (the same rows, sums in the same order).  The second word of the workspace says which kernel ran: the
-check of the lists writes it where some pair differs."""
+query block by itself, bit for bit (the same rows, sums in the same order).  The words behind the counter say which kernel ran: the
+check of the lists answers there."""
 import numpy as np
 import pytest
 
@@ -22,24 +22,66 @@ def problem(lens, hq, hkv, block=64, qlens=None, seed=0):
 
 def both_ways(p, by_pairs):
     import torch
+    from paper_2410_13276_b200 import binding as B
     outs = []
-    for dynamic in (False, True):
+    answer = p.ws[4:256].view(torch.int32)                         # behind the work counter: one word for each block of the check
+    for left in (None, 0, 0x7f7f7f7f):                             # without a workspace; with one that something has been left in
         p.o.fill_(7.0); p.lse.fill_(7.0)
-        p.ws[4:8] = 0
-        p.attn(dynamic=dynamic)
+        if left is not None:
+            answer.fill_(left)
+        before = B.seer_launch_count(p.ctx)
+        p.attn(dynamic=left is not None)
         torch.cuda.synchronize()
         assert p.status() == 0
+        if left is not None:
+            # the check, the kernel for single blocks and the one for pairs, of which one returns at once; every word is this call's
+            assert B.seer_launch_count(p.ctx) - before == 3
+            said = set(answer.tolist())
+            assert 0x7f7f7f7f not in said and (0 not in said) == by_pairs and (len(said) == 1 or not by_pairs)
         outs.append((p.o.clone().view(torch.int16), p.lse.clone().view(torch.int32)))
-    assert (int(p.ws[4:8].view(torch.int32)) == 0) == by_pairs
-    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    for o, lse in outs[1:]:
+        assert torch.equal(outs[0][0], o) and torch.equal(outs[0][1], lse)
 
 
-def maxima_of_groups(p):
+def maxima_by_pairs(p):
+    """Which kernel gives the block maxima: CTA 0 loses its first copy, so the entries of its items stay as they were.  By pairs those are both lists
+    of a pair of query blocks; otherwise the items of a CTA are blocks of several heads, and none has its neighbour among them."""
+    import torch
+    from paper_2410_13276_b200 import binding as B
+    p.bmax = torch.full((max(p.col_idx.numel(), 1),), -1.0, device="cuda")
+    B.seer_debug_lost_wait(p.ctx, 5_000, 0)
+    try:
+        before = B.seer_launch_count(p.ctx)
+        p.block_max()
+        assert B.seer_launch_count(p.ctx) - before == 3            # the check and both kernels
+        assert B.STATUS_NAMES[B.seer_poll_device_status(p.ctx)] == "SEER_ERR_TIMEOUT"
+    finally:
+        B.seer_debug_lost_wait(p.ctx, 2_000_000, -1)
+    rp, _ = p.lists_host()
+    left = (p.bmax[:int(rp[-1])] == -1.0).cpu().numpy()
+    rows = set(np.unique(np.searchsorted(rp, np.flatnonzero(left), side="right") - 1).tolist())
+    nbs = (np.diff(p.cu) + 63) // 64
+    base, both, lone = 0, 0, 0
+    for n, nq in zip(nbs, nbs if p.cu_q is None else np.diff(p.cu_q)):
+        first = n - ((nq + 63) // 64 if p.cu_q is not None else n)
+        for h in range(p.hq):
+            for i in range(0, n, 2):
+                here = [r in rows for r, j in ((base + h * n + i, i), (base + h * n + i + 1, i + 1)) if first <= j < n and rp[r + 1] > rp[r]]
+                if len(here) == 2:
+                    both, lone = both + all(here), lone + (sum(here) == 1)
+        base += p.hq * n
+    assert both + lone > 0 and (both == 0 or lone == 0)
+    return both > 0
+
+
+def maxima_of_groups(p, by_pairs):
     """Block maxima: equal to those of each KV head's problem by itself, which is below the size from which pairs are asked for."""
     import torch
+    from paper_2410_13276_b200 import binding as B
     from paper_2410_13276_b200.prefill import Prefill
     p.attn()
-    p.bmax = torch.full((max(p.col_idx.numel(), 1),), -1.0, device="cuda")
+    assert maxima_by_pairs(p) == by_pairs
+    p.bmax.fill_(-1.0)
     got = p.block_max()
     rp, col = p.lists_host()
     nbs, group = (np.diff(p.cu) + 63) // 64, p.hq // p.hkv
@@ -52,7 +94,9 @@ def maxima_of_groups(p):
             base += p.hq * nb
         lens = np.concatenate([np.diff(rp[a:b + 1]) for a, b in spans])
         part.set_lists(np.concatenate([[0], np.cumsum(lens)]).astype(np.int32), np.concatenate([col[rp[a]:rp[b]] for a, b in spans]).astype(np.int32))
+        before = B.seer_launch_count(p.ctx)
         want = part.block_max()[:int(lens.sum())]
+        assert B.seer_launch_count(p.ctx) - before == 1            # (not asked)
         assert torch.equal(torch.cat([got[int(rp[a]):int(rp[b])] for a, b in spans]).view(torch.int32), want.view(torch.int32)), g
     assert p.status() == 0
 
@@ -64,7 +108,7 @@ def test_dense_lists(lens, qlens, hq, hkv):
     p = problem(lens, hq, hkv, qlens=qlens)
     p.mask(B.make_mask_params(B.SEER_TOPK_COUNT, k=1 << 20, flags=B.SEER_FORCE_DIAG))
     both_ways(p, True)
-    maxima_of_groups(p)
+    maxima_of_groups(p, True)
 
 
 @pytest.mark.parametrize("lens,qlens", [([23500], None), ([16400, 127, 11000], None), ([23500, 2000], [23500 - 128 * 57, 2000 - 128])])
@@ -101,13 +145,13 @@ def test_hand_made_lists(spoilt):
         p.k[64 * 77 + 9, 1, 4] = float("inf"); p.k[64 * 30 + 2, 3] *= 60; p.q[64 * 90:64 * 96] *= 20
     p.set_lists(np.concatenate([[0], np.cumsum([len(x) for x in rows])]).astype(np.int32), np.array([j for x in rows for j in x], np.int32))
     both_ways(p, True)
-    maxima_of_groups(p)
+    maxima_of_groups(p, True)
     # a single pair that differs, by an entry or by a length, or whose own block is not its last entry: each query block by itself
     for change in (lambda x: x[1:], lambda x: [x[1], x[0]] + x[2:], lambda x: x + x[:2]):
         other = [change(x) if k == at else x for k, x in enumerate(rows)]
         p.set_lists(np.concatenate([[0], np.cumsum([len(x) for x in other])]).astype(np.int32), np.array([j for x in other for j in x], np.int32))
         both_ways(p, False)
-    maxima_of_groups(p)                                            # (a CTA with that pair takes each block by itself, the others theirs by pairs)
+    maxima_of_groups(p, False)                                     # (one pair that differs: the whole call)
 
 
 @pytest.mark.parametrize("lost_tile", [0, 130, 300])
