@@ -566,7 +566,23 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             continue;
           }
         }
-        const float4 x = other_tile(sh, s_addr, o_addr, sl2, R, l, (uint32_t)here > (uint32_t)it.i ? -1 : here == it.i ? row : 63, t == 0 && here == it.i, t,
+        // Absent (every odd list ends with one) or rejected: contributes nothing.  Here and not in other_tile: lists of a few blocks have one such tile
+        // in six, and the call for it made them slower than they were with every path in the loop (the launch by itself, 32 heads, one in twenty, with
+        // every path in the loop, with the call, and so: 11 584 tokens 142.5, 146.3 and 140.3 us, 16 384 236.1, 238.1 and 232.6; one in ten, 65 536
+        // tokens 4291, 4175 and 4115).
+        if ((uint32_t)here > (uint32_t)it.i) {
+          uint32_t pk[32];
+#pragma unroll
+          for (int i = 0; i < 32; ++i) pk[i] = 0u;
+          tc_st32(s_addr, pk);
+          tc_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(sh.bar(bb + P_FULL + (int)buf));
+          tr.ev(34);
+          continue;
+        }
+        const float4 x = other_tile(sh, s_addr, o_addr, sl2, R, l, here == it.i ? row : 63, t == 0 && here == it.i, t,
                                     bb + PV_DONE + (int)(buf ^ 1u), ((cnt - 1) >> 1) & 1u, status);
         R = x.x; l = x.y; fail = x.z != 0.f;
         if (fail) break;

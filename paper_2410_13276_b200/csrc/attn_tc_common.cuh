@@ -437,7 +437,7 @@ __device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
   return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
 }
 
-// A tile that is not for the plain pass: the diagonal block (last = row), one that is absent or rejected (last < 0), or one where some row's
+// A tile that is not for the plain pass: the diagonal block (last = row), one that is not this row's (last < 0; by pairs), or one where some row's
 // reference has to move; from the scores to P in their place.  `fresh`: the row has no reference yet.  Returns the row's (reference,
 // sum) and whether a wait was lost.  Conditions around tensor memory loads are the same for a whole warp: all its lanes take part in them.
 // A function of its own, not inlined: where these paths join the plain pass's results, or share its registers, every tile pays for them.  The
@@ -446,7 +446,7 @@ __device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
 // maximum and for the pass, 32k tokens take 1250.)
 static __device__ __noinline__ float4 other_tile(Shared sh, uint32_t s_addr, uint32_t o_addr, float sl2, float R, float l, int last, bool fresh, int t, int pv_bar, uint32_t pv_par, int* status) {
   uint32_t pk[32];
-  if (last < 0) {                                           // absent or rejected: contributes nothing
+  if (last < 0) {                                           // contributes nothing
 #pragma unroll
     for (int i = 0; i < 32; ++i) pk[i] = 0u;
   } else {
