@@ -195,6 +195,7 @@ def cpu_oracle_sample(w, spec, rp, col, budget_rows=None):
 TIMELINE_TAGS = {1: "loop", 2: "copies of a tile (waits for empty units)", 10: "to the next S", 12: "S: wait K units, MMAs, commits",
                  13: "to the next P V", 15: "wait P_FULL", 16: "P V: wait V units, MMAs, commits", 31: "list entry",
                  32: "wait S_FULL", 33: "softmax pass (incl. first-tile reference)", 34: "store P, arrive P_FULL",
+                 35: "softmax pass of the diagonal",
                  36: "item start / end of the tile loop", 37: "epilogue: wait the last P V", 38: "epilogue: merge and store",
                  40: "pass with a moved reference"}
 TIMELINE_ROLES = ["producer K+Q, stream 0", "issuer, stream 0", "producer V, stream 0", "issuer, stream 1",

@@ -109,10 +109,7 @@ __device__ __forceinline__ int slot_check(const Slot& it, int p, int raw) {
 // heads, all causal blocks: 1277 us and 1060 so when both were timed on a cool board, 520 clocks a tile; 440 are its 32 KB from L2, 384 its
 // MMAs; 1160 to 1210 us behind an attention launch).
 // kO32: o begins on 32 bytes.  (A test of the address in the kernel instead: 32k tokens 1392 -> 1404 us.)
-// kShort: every path of a tile in the loop.  Where lists are of one to three blocks most tiles are diagonal or a row's first, and each CTA has few:
-// the jump to other_tile costs more than it saves (sequences of 343 and 270 tokens, 40 heads, the whole pass 32.0 and 32.5 us; 24 of 1 to 56
-// tokens 38.1 and 39.0; from 32 blocks on other_tile is the faster one: 2048 tokens 29.3 and 29.0, a batch of up to 2000 243.6 and 241.7).
-template <bool kTrace, bool kChunk, bool kBlockMax = false, bool kO32 = true, bool kShort = false>
+template <bool kTrace, bool kChunk, bool kBlockMax = false, bool kO32 = true>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, SeqMeta m,
@@ -498,55 +495,12 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         tr.ev(32);
         tc_fence_after();
         const uint32_t s_addr = tmem + lane_addr + col_s(s, buf);
-        if constexpr (kShort) {
-          uint32_t pk[32];
-          const int j = (uint32_t)here > (uint32_t)it.i ? -1 : here;
-          if (j < 0) {                                        // absent or rejected: contributes nothing
-#pragma unroll
-            for (int i = 0; i < 32; ++i) pk[i] = 0u;
-          } else {
-            const bool diag = j == it.i;
-            if (t == 0) {
-              const float mx = diag ? row_max<true>(s_addr, row) : row_max<false>(s_addr, 63);
-              if (fabsf(mx) < 3.0e38f) R = mx * sl2;
-            }
-            float sum = diag ? row_pass<true>(s_addr, sl2, R, row, pk) : row_pass<false>(s_addr, sl2, R, row, pk);
-            const bool over = !(sum < kRise);
-            if (__any_sync(0xffffffffu, over)) {
-              // ---- some row's reference has to move (or its scores are not finite): O at rest, rows rescaled, tile taken again
-              if (t > 0) {
-                fail = !mbar_wait(sh, bb + PV_DONE + (int)(buf ^ 1u), ((cnt - 1) >> 1) & 1u, status);
-                if (__any_sync(0xffffffffu, fail)) { fail = true; break; }
-                tc_fence_after();
-              }
-              const float mx = row_max<true>(s_addr, diag ? row : 63) * sl2;
-              const float nr = over && fabsf(mx) < 3.0e38f ? fmaxf(R, mx) : R;
-              const float alpha = nr == R ? 1.f : exp2f(R - nr);
-              R = nr;
-              l = alpha == 0.f ? 0.f : __fmul_rn(l, alpha);
-              if (t > 0) {
-#pragma unroll 1
-                for (int ch = 0; ch < 8; ++ch) {
-                  uint32_t ov[16];
-                  tc_ld16(o_addr + ch * 16, ov);
-                  tc_wait_ld(ov);
-#pragma unroll
-                  for (int e = 0; e < 16; ++e) ov[e] = alpha == 0.f ? 0u : __float_as_uint(__uint_as_float(ov[e]) * alpha);
-                  tc_st16(o_addr + ch * 16, ov);
-                }
-              }
-              sum = diag ? row_pass<true>(s_addr, sl2, R, row, pk) : row_pass<false>(s_addr, sl2, R, row, pk);
-              if (!(sum < kRise)) sum = CUDART_NAN_F;         // an infinite score or a NaN: so is the row
-            }
-            l = __fadd_rn(l, sum);
-          }
-          tc_st32(s_addr, pk);                                // P over the scores this thread has read
-          tc_wait_st();
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(sh.bar(bb + P_FULL + (int)buf));
-          continue;
-        }
+        // Each kind of tile to its own end: where the paths join the plain pass's results, or share its registers, every tile pays for them (a
+        // launch of 32k tokens 1426 us with all in one, 1240 with the plain pass alone and a call for everything else).  The call is for tiles
+        // whose reference moves, which are few.  With it for absent tiles and the diagonal too, lists of a few blocks, which have one in six
+        // of these, were slower than with all in one.  The launch by itself, 32 heads, all in one, call for all but the plain pass, and so:
+        // one in twenty, 11 584 tokens 142.5, 146.3 and 139.8 us, 16 384 236.1, 238.1 and 235.2; one in ten, 65 536 4291, 4175 and 4134.  48
+        // sequences of up to 4, 8, 16 and 30 blocks, one in ten, the whole pass: all in one 109.7, 184.9, 305.1 and 535.6 us, so 108.3, 182.9, 299.8 and 524.6.
         if ((uint32_t)here < (uint32_t)it.i) {              // the plain pass: a block before the diagonal
           if (t == 0) {
             const float mx = row_max<false>(s_addr, 63);
@@ -566,11 +520,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             continue;
           }
         }
-        // Absent (every odd list ends with one) or rejected: contributes nothing.  Here and not in other_tile: lists of a few blocks have one such tile
-        // in six, and the call for it made them slower than they were with every path in the loop (the launch by itself, 32 heads, one in twenty, with
-        // every path in the loop, with the call, and so: 11 584 tokens 142.5, 146.3 and 140.3 us, 16 384 236.1, 238.1 and 232.6; one in ten, 65 536
-        // tokens 4291, 4175 and 4115).
-        if ((uint32_t)here > (uint32_t)it.i) {
+        if ((uint32_t)here > (uint32_t)it.i) {              // absent (every odd list ends with one) or rejected: contributes nothing
           uint32_t pk[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) pk[i] = 0u;
@@ -582,13 +532,32 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
           tr.ev(34);
           continue;
         }
-        const float4 x = other_tile(sh, s_addr, o_addr, sl2, R, l, here == it.i ? row : 63, t == 0 && here == it.i, t,
-                                    bb + PV_DONE + (int)(buf ^ 1u), ((cnt - 1) >> 1) & 1u, status);
+        if (here == it.i) {
+          if (t == 0) {
+            const float mx = row_max<true>(s_addr, row);
+            if (fabsf(mx) < 3.0e38f) R = mx * sl2;
+          }
+          uint32_t pk[32];
+          const float sum = row_pass<true>(s_addr, sl2, R, row, pk);
+          if (!__any_sync(0xffffffffu, !(sum < kRise))) {
+            l = __fadd_rn(l, sum);
+            tr.ev(35);
+            tc_st32(s_addr, pk);
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sh.bar(bb + P_FULL + (int)buf));
+            tr.ev(34);
+            continue;
+          }
+        }
+        // some row's reference has to move
+        const float4 x = other_tile(sh, s_addr, o_addr, sl2, R, l, here == it.i ? row : 63, false, t, bb + PV_DONE + (int)(buf ^ 1u), ((cnt - 1) >> 1) & 1u, status);
         R = x.x; l = x.y; fail = x.z != 0.f;
         if (fail) break;
         __syncwarp();
         if (lane == 0) mbar_arrive(sh.bar(bb + P_FULL + (int)buf));
-        tr.ev(40);
+        tr.ev(40);                                          // (a moved reference)
       }
       if constexpr (!kBlockMax) {
         // ---------------------------------------------------------------------------------------- epilogue: merge, store
@@ -739,8 +708,7 @@ seer_status init_attn_tc(seer_ctx* ctx) {
   ctx->tmap_encode = fn;
   for (tc::Kernel* k : {tc::attn_tc_kernel<false, false>, tc::attn_tc_kernel<false, true>, tc::attn_tc_kernel<true, false>,
                         tc::attn_tc_kernel<false, false, false, false>, tc::attn_tc_kernel<false, true, false, false>,
-                        tc::attn_tc_kernel<false, false, true>, tc::attn_tc_kernel<false, true, true>,
-                        tc::attn_tc_kernel<false, false, false, true, true>, tc::attn_tc_kernel<false, true, false, true, true>})
+                        tc::attn_tc_kernel<false, false, true>, tc::attn_tc_kernel<false, true, true>})
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kSmemBytes) != cudaSuccess) return SEER_ERR_CUDA;
   return SEER_OK;
 }
@@ -774,11 +742,9 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
   }
   unsigned long long* tb = (unsigned long long*)ctx->trace;
   const bool o32 = ((uintptr_t)o & 31) == 0;
-  const bool few = m.max_nb < 32;                          // (kShort)
-  tc::Kernel* kernel = tb != nullptr && !m.chunked ? tc::attn_tc_kernel<true, false>   // (chunks are never instrumented)
-                     : !o32 ? (m.chunked ? tc::attn_tc_kernel<false, true, false, false> : tc::attn_tc_kernel<false, false, false, false>)
-                     : few ? (m.chunked ? tc::attn_tc_kernel<false, true, false, true, true> : tc::attn_tc_kernel<false, false, false, true, true>)
-                     : m.chunked ? tc::attn_tc_kernel<false, true> : tc::attn_tc_kernel<false, false>;
+  tc::Kernel* kernel = m.chunked ? (o32 ? tc::attn_tc_kernel<false, true> : tc::attn_tc_kernel<false, true, false, false>)   // (never instrumented)
+                     : tb != nullptr ? tc::attn_tc_kernel<true, false>
+                     : o32 ? tc::attn_tc_kernel<false, false> : tc::attn_tc_kernel<false, false, false, false>;
   e = launch_next(kernel, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter,
                   (const int*)answer.words, answer.nwords, answer.epoch);
   if (e != cudaSuccess) return -(int)e;

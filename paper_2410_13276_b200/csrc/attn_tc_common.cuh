@@ -437,13 +437,10 @@ __device__ __forceinline__ float row_max(uint32_t s_addr, int last) {
   return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
 }
 
-// A tile that is not for the plain pass: the diagonal block (last = row), one that is not this row's (last < 0; by pairs), or one where some row's
-// reference has to move; from the scores to P in their place.  `fresh`: the row has no reference yet.  Returns the row's (reference,
-// sum) and whether a wait was lost.  Conditions around tensor memory loads are the same for a whole warp: all its lanes take part in them.
-// A function of its own, not inlined: where these paths join the plain pass's results, or share its registers, every tile pays for them.  The
-// attention launch by itself, 32k tokens 1285 us inline and 1240 so, 24 short prompts 165.6 and 164.2, 48k 2722 and 2690, dense 16k 2410 and 2360;
-// all paths in one inlined loop beside the plain pass: 1426, 208.7, 2950, 2534.  (The scores are taken to registers once: read again for the
-// maximum and for the pass, 32k tokens take 1250.)
+// A tile where some row's reference has to move; by pairs also the diagonal block (last = row) and one that is not this row's (last < 0); from the scores
+// to P in their place.  `fresh`: the row has no reference yet.  Returns the row's (reference, sum) and whether a wait was lost.  Conditions around
+// tensor memory loads are the same for a whole warp: all its lanes take part in them.
+// A function of its own, not inlined: the plain pass would pay for sharing its registers (attn_tc.cu).
 static __device__ __noinline__ float4 other_tile(Shared sh, uint32_t s_addr, uint32_t o_addr, float sl2, float R, float l, int last, bool fresh, int t, int pv_bar, uint32_t pv_par, int* status) {
   uint32_t pk[32];
   if (last < 0) {                                           // contributes nothing
