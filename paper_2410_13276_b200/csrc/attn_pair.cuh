@@ -6,18 +6,29 @@
 namespace seer {
 namespace tp {
 
-struct PairItem {
+using namespace tcc;
+
+constexpr uint32_t kHalfTile = 64 * 128;         // bytes of one d half of a 64-row tile (8 KB)
+constexpr uint32_t kQBytes = 4 * kHalfTile;      // 32 KB: [d half][query block]
+constexpr uint32_t kUnit = 4 * kHalfTile;        // a tile's K, [d half][block], or its V, [block][d half]
+constexpr uint32_t kOffQ = 0, kOffK = 2 * kQBytes;   // two buffers of Q, then the rings
+constexpr uint32_t kIdescS = make_idesc(false, false, 128u, 128u);
+
+struct PairPlace {
   int h, i0, s0, tok0;         // first query block; first key token of the sequence; first row of block i0 in q / o / lse
+  int valid[2];                // query rows of the two blocks (none: not there)
+  int64_t row;                 // of block i0 in row_ptr
+};
+struct PairItem : PairPlace {
   int l0, len;                 // the longer list
-  int l[2];                    // both lists' starts
-  int n[2], valid[2];          // entries and query rows of the two blocks (no rows: not there)
+  int l[2], n[2];              // both lists' starts and lengths
 };
 
 // The w-th pair: KV head by KV head of a sequence, from the last pair to the first, a pair's heads side by side.  kZigzag: every other KV head from the
 // first pair to the last, so that the lists' lengths have no jump from one head to the next.
 template <bool kChunk, bool kZigzag = false>
-__device__ __forceinline__ PairItem decode_pair(const SeqMeta& m, const int32_t* row_ptr, int64_t w) {
-  PairItem it;
+__device__ __forceinline__ PairPlace place_pair(const SeqMeta& m, int64_t w) {
+  PairPlace it;
   const int p = find_sequence(m.pair_off, m.batch, (int)(w / m.num_q_heads)), before = m.pair_off[p];
   const int4 s = m.place[p];
   const int nb = (s.y + kBlock - 1) / kBlock, np = m.pair_off[p + 1] - before;
@@ -30,13 +41,18 @@ __device__ __forceinline__ PairItem decode_pair(const SeqMeta& m, const int32_t*
   it.h = g * m.group + rem % m.group;
   it.s0 = s.x;
   it.tok0 = s.x + it.i0 * kBlock + (kChunk ? s.w : 0);
-  const int64_t row = (int64_t)m.num_q_heads * s.z + (int64_t)it.h * nb + it.i0;
-  const bool a = it.i0 >= first, b = it.i0 + 1 < nb;
-  const int l0 = row_ptr[row], l1 = row_ptr[row + 1], l2 = b ? row_ptr[row + 2] : l1;
-  it.n[0] = a ? l1 - l0 : 0;
-  it.n[1] = b ? l2 - l1 : 0;
-  it.valid[0] = a ? min(kBlock, s.y - it.i0 * kBlock) : 0;
-  it.valid[1] = b ? min(kBlock, s.y - (it.i0 + 1) * kBlock) : 0;
+  it.row = (int64_t)m.num_q_heads * s.z + (int64_t)it.h * nb + it.i0;
+  it.valid[0] = it.i0 >= first ? min(kBlock, s.y - it.i0 * kBlock) : 0;
+  it.valid[1] = it.i0 + 1 < nb ? min(kBlock, s.y - (it.i0 + 1) * kBlock) : 0;
+  return it;
+}
+template <bool kChunk, bool kZigzag = false>
+__device__ __forceinline__ PairItem decode_pair(const SeqMeta& m, const int32_t* row_ptr, int64_t w) {
+  PairItem it;
+  static_cast<PairPlace&>(it) = place_pair<kChunk, kZigzag>(m, w);
+  const int l0 = row_ptr[it.row], l1 = row_ptr[it.row + 1], l2 = it.valid[1] > 0 ? row_ptr[it.row + 2] : l1;
+  it.n[0] = it.valid[0] > 0 ? l1 - l0 : 0;
+  it.n[1] = it.valid[1] > 0 ? l2 - l1 : 0;
   const bool second = it.n[1] >= it.n[0];
   it.l0 = second ? l1 : l0;
   it.len = second ? it.n[1] : it.n[0];
@@ -47,9 +63,9 @@ __device__ __forceinline__ PairItem decode_pair(const SeqMeta& m, const int32_t*
 // Whether the pair has one list: the same entries, all before the first block or, at the end of that block's list, the block itself; the second
 // block may list one more, up to itself.  A pair's second block alone, or the first, where the other has no queries: entries before the
 // block, the last one up to it.  (By a converged warp.)
-template <bool kChunk>
+template <bool kChunk, bool kZigzag = false>
 __device__ __forceinline__ bool pair_ok(const SeqMeta& m, const int32_t* row_ptr, const uint32_t* col, int64_t w, int lane) {
-  const PairItem it = decode_pair<kChunk>(m, row_ptr, w);
+  const PairItem it = decode_pair<kChunk, kZigzag>(m, row_ptr, w);
   const int l2 = it.n[1] >= it.n[0] ? it.l[0] : it.l[1];
   const bool both = it.valid[0] > 0 && it.valid[1] > 0;
   const int n = both ? min(it.n[0], it.n[1]) : 0;         // entries that both list

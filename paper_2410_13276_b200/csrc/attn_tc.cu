@@ -41,7 +41,7 @@
 #include <cuda.h>
 #include <math_constants.h>
 
-#include "attn_pair.cuh"
+#include "block_max_pair.cuh"
 
 namespace seer {
 namespace tc {
@@ -77,6 +77,7 @@ enum Bar { Q_FULL = 0 /* + buf */, Q_EMPTY = 2, K_FULL = 4 /* + unit */, K_EMPTY
            // the block maxima have no V, no P and no O: five K units, four S buffers (M_TAKEN: the group has its maxima)
            M_KEMPTY = 30, M_TAKEN = 10, kBarsMax = 35 };
 static_assert(kBarsMax <= kBarsPerStream && kKUnits <= 3 && kVUnits <= 3, "barrier map");
+static_assert(tp::kMaxEnd <= kOffBar, "the maxima by pairs have barriers of their own");
 
 constexpr uint32_t kTmemCols = 512;
 // TMEM columns of a stream: two S buffers (P in their first 32 columns), O
@@ -116,16 +117,16 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
                 const int32_t* row_ptr, const int32_t* col_idx,
                 uint16_t* __restrict__ o, float* lse, int* __restrict__ status,
                 unsigned long long* __restrict__ trace, float* block_max = nullptr,
-                int* __restrict__ work_counter = nullptr, const int* words = nullptr, int nwords = 0, int epoch = 0) {
+                int* __restrict__ work_counter = nullptr, const int* words = nullptr, int nwords = 0, int epoch = 0, bool pairs = false) {
   extern __shared__ __align__(1024) unsigned char smem[];
   Shared sh;
   sh.base = smem_u32(smem);
   sh.bar0 = sh.base + kOffBar;
   sh.abort_addr = sh.base + kOffMisc + 8;
   sh.limit_us = m.wait_limit_us;
-  if (words != nullptr) {                                  // (a way out from further in costs a launch of 32k tokens 2 %)
+  if (!kBlockMax && words != nullptr) {                    // (a way out from further in costs a launch of 32k tokens 2 %)
     grid_wait();
-    if (tp::lists_agree(words, nwords, epoch)) return;      // attn_pair_kernel does the work, block_max_pair_kernel has done it
+    if (tp::lists_agree(words, nwords, epoch)) return;      // attn_pair_kernel does the work
   }
   if ((sh.base & 1023u) != 0u) {                           // the swizzled tiles need the alignment
     grid_wait();
@@ -139,9 +140,9 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     for (int s = 0; s < 2; ++s) {
       const int b = s * kBarsPerStream;
       for (int i = 0; i < (kBlockMax ? kBarsMax : kBars); ++i) {
-        // Q_EMPTY, P_FULL: one arrival per warp of the softmax group; ITEM_EMPTY: those, the V producer and the issuer
+        // Q_EMPTY, P_FULL: one arrival per warp of the softmax group; ITEM_EMPTY: those, the V producer (block maxima: the K producer) and the issuer
         const bool group = (i >= Q_EMPTY && i < Q_EMPTY + 2) || (kBlockMax ? i >= M_TAKEN && i < M_TAKEN + 4 : i >= P_FULL && i < P_FULL + 2);
-        mbar_init(sh.bar(b + i), i >= ITEM_EMPTY && i < ITEM_EMPTY + 4 ? (kBlockMax ? 5 : 6) : group ? 4 : 1);
+        mbar_init(sh.bar(b + i), i >= ITEM_EMPTY && i < ITEM_EMPTY + 4 ? 6 : group ? 4 : 1);
       }
     }
     st_shared_u32(sh.abort_flag(), 0u);
@@ -151,8 +152,17 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sh.base + kOffMisc), "r"(kTmemCols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  if (kBlockMax && pairs && warp == 2) tp::max_init(sh.base, lane);
   tc_fence_before();
-  __syncthreads();
+  bool by_pairs = false;
+  if constexpr (kBlockMax) {
+    if (pairs) {
+      __syncwarp();                                        // (thread 0 has set up the barriers)
+      grid_wait();
+      by_pairs = tp::share_agrees<kChunk>(m, row_ptr, col_idx, warp, lane);   // (meets as below)
+    }
+  }
+  if (!(kBlockMax && pairs)) __syncthreads();
   tc_fence_after();
   grid_wait();
   const uint32_t tmem = *tmem_slot;
@@ -179,9 +189,21 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   };
   auto first_entry = [&](const Slot& it, int p) -> int { return kBlockMax ? slot_block(it, col_idx, p) : it.first[p]; };
   auto item_full = [&](int s, uint32_t n) -> int { return s * kBarsPerStream + ITEM_FULL + (int)(n & 3u); };
+  auto put_item = [&](int s, uint32_t n, const Item& nx, bool more, int e0, int e1) -> bool {
+    // the slot's previous content (item n - 4) has been read by everyone
+    if (!mbar_wait(sh, s * kBarsPerStream + ITEM_EMPTY + (int)(n & 3u), ((n >> 2) & 1u) ^ 1u, status)) return false;
+    const int tok0 = nx.s0 + nx.i * kBlock + (kChunk ? nx.dq : 0);
+    st_shared_v4(ring_addr(s, n), (uint32_t)nx.h, (uint32_t)nx.i << 7 | (uint32_t)nx.q_valid, (uint32_t)nx.l0, more ? (uint32_t)nx.nlist : 0xffffffffu);
+    st_shared_v4(ring_addr(s, n) + 16u, (uint32_t)nx.s0, (uint32_t)tok0, (uint32_t)e0, (uint32_t)e1);
+    mbar_arrive(sh.bar(item_full(s, n)));
+    return true;
+  };
   auto release_item = [&](int s, uint32_t n) { mbar_arrive(sh.bar(s * kBarsPerStream + ITEM_EMPTY + (int)(n & 3u))); };
 
-  if (warp < 4 || warp >= 12) {
+  if (by_pairs) {
+    if constexpr (kBlockMax)
+      tp::block_max_pairs<kChunk, kHelperRegs<true>, kSoftmaxRegs<true>>(map_q, map_k, m, sh, smem, tmem, warp, lane, row_ptr, col_idx, lse, status, block_max);
+  } else if (warp < 4 || warp >= 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kHelperRegs<kBlockMax>));
     // ========================================================================================== producer of Q and K (TMA)
     if (warp == 0 || warp == 2) {
@@ -200,37 +222,35 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
         uint32_t nitem = 0, cnt = 0, ku = 0, kph = 0;
         bool ok = true;
         // An item is decoded and announced while the one before it is copied: its row pointers and its first list entries are two
-        // trips to L2, one after the other, that every role of the stream would wait for at the item's start.  The block maxima take a tile in a
-        // quarter of the time, and copies that wait behind the two trips leave their group without tiles: they decode behind an item's last
-        // copy, and each role reads its entries (4096 tokens, 32 heads, an eighth listed: 21.5 us with all that in the middle of the copies, 19.7 so;
-        // over 50 random batches and chunks 3 to 5 % on average).
+        // trips to L2, one after the other, that every role of the stream would wait for at the item's start.  (The block maxima have warps to spare for it.)
         Item nx{};
         bool more = false;
         auto locate = [&](int64_t w) {                     // which item comes next
           more = w < m.q_rows;
           nx = Item{};
-          if (more) nx = decode_item<kChunk, kChunk || !kBlockMax>(m, row_ptr, w);
+          if (more) nx = decode_item<kChunk, true>(m, row_ptr, w);
         };
         auto announce = [&](uint32_t n) -> bool {
-          const int na0 = !kBlockMax && 0 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0) : -1;
-          const int nb0 = !kBlockMax && 1 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0 + 1) : -1;
-          // the slot's previous content (item n - 4) has been read by everyone
-          if (!mbar_wait(sh, bb + ITEM_EMPTY + (int)(n & 3u), ((n >> 2) & 1u) ^ 1u, status)) return false;
-          const int tok0 = nx.s0 + nx.i * kBlock + (kChunk ? nx.dq : 0);
-          st_shared_v4(ring_addr(s, n), (uint32_t)nx.h, (uint32_t)nx.i << 7 | (uint32_t)nx.q_valid, (uint32_t)nx.l0, more ? (uint32_t)nx.nlist : 0xffffffffu);
-          st_shared_v4(ring_addr(s, n) + 16u, (uint32_t)nx.s0, (uint32_t)tok0, (uint32_t)na0, (uint32_t)nb0);
-          mbar_arrive(sh.bar(item_full(s, n)));
-          return true;
+          const int na0 = 0 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0) : -1;
+          const int nb0 = 1 < nx.nlist ? (int)ld_global(reinterpret_cast<const uint32_t*>(col_idx) + nx.l0 + 1) : -1;
+          return put_item(s, n, nx, more, na0, nb0);
         };
-        locate(draw());
-        ok = announce(0);
+        if (!kBlockMax) {
+          locate(draw());
+          ok = announce(0);
+        }
         for (uint32_t n = 0; ok; ++n) {
+          if (kBlockMax && !mbar_wait(sh, item_full(s, n), (n >> 2) & 1u, status)) break;
           const Slot it = read_slot(s, n);                 // (its own announcement: two items in 56 registers are 1 % of a long launch)
+          if (kBlockMax) release_item(s, n);
           if (it.nlist < 0) break;
           int ja = slot_check(it, 0, first_entry(it, 0)), jb = slot_check(it, 1, first_entry(it, 1));
-          const int64_t w = draw();                        // the next one is on its way while this one is copied
+          const int64_t w = kBlockMax ? 0 : draw();        // the next one is on its way while this one is copied
           const int ntiles = it.ntiles(), g = it.h / m.group;
-          if (ntiles == 0) { locate(w); ok = announce(n + 1); continue; }
+          if (ntiles == 0) {
+            if (!kBlockMax) { locate(w); ok = announce(n + 1); }
+            continue;
+          }
           const uint32_t qb = nitem & 1u;
           if (!mbar_wait(sh, bb + Q_EMPTY + (int)qb, ((nitem >> 1) & 1u) ^ 1u, status)) break;
           mbar_expect_tx(sh.bar(bb + Q_FULL + (int)qb), kQBytes);
@@ -263,13 +283,36 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
             if (!kBlockMax && t == 0) locate(w);
             if (!kBlockMax && t == min(1, ntiles - 1) && !announce(n + 1)) { ok = false; break; }
           }
-          if (kBlockMax && ok) { locate(w); ok = announce(n + 1); }
         }
       }
     }
     // ========================================================================================== producer of V (TMA)
     else if (warp == 12 || warp == 13) {
-      if (!kBlockMax) if (elect_one()) {
+      if (kBlockMax) {
+        // The block maxima: items are decoded and announced ahead of the copies.  Where lists have a few blocks the producer has no time for it
+        // (24 sequences of 2048 tokens, 64 heads, one in twenty: 273 us behind an item's last copy, 257 so).
+        if (elect_one()) {
+          const int s = warp - 12;
+          bool more = true;
+          for (uint32_t n = 0; more; ++n) {
+            Item nx{};
+            if (pairs) {                                   // the blocks of the pairs dealt to this CTA (share_agrees), a stream each
+              const int64_t w = tp::dealt_pair(m, n);
+              more = w >= 0;
+              if (more) {
+                const tp::PairItem u = tp::decode_pair<kChunk, true>(m, row_ptr, w);
+                nx.h = u.h; nx.i = u.i0 + s; nx.s0 = u.s0; nx.dq = u.tok0 - u.s0 - u.i0 * kBlock;
+                nx.l0 = s ? u.l[1] : u.l[0]; nx.nlist = s ? u.n[1] : u.n[0]; nx.q_valid = s ? u.valid[1] : u.valid[0];
+              }
+            } else {
+              const int64_t w = (int64_t)blockIdx.x + (2 * (int64_t)n + s) * gridDim.x;
+              more = w < m.q_rows;
+              if (more) nx = decode_item<kChunk, kChunk>(m, row_ptr, w);
+            }
+            if (!put_item(s, n, nx, more, -1, -1)) break;
+          }
+        }
+      } else if (elect_one()) {
         const int s = warp - 12, bb = s * kBarsPerStream;
         const uint32_t sbase = sh.base + (uint32_t)s * kStreamBytes;
         Tracer<kTrace> tr; tr.init(s == 0 ? trace : nullptr, 2);
@@ -673,7 +716,7 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant_
   }
 }
 
-using Kernel = void(CUtensorMap, CUtensorMap, CUtensorMap, SeqMeta, const int32_t*, const int32_t*, uint16_t*, float*, int*, unsigned long long*, float*, int*, const int*, int, int);
+using Kernel = void(CUtensorMap, CUtensorMap, CUtensorMap, SeqMeta, const int32_t*, const int32_t*, uint16_t*, float*, int*, unsigned long long*, float*, int*, const int*, int, int, bool);
 
 __global__ void zero_kernel(int* __restrict__ word) {
   grid_wait();
@@ -746,7 +789,7 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
                      : tb != nullptr ? tc::attn_tc_kernel<true, false>
                      : o32 ? tc::attn_tc_kernel<false, false> : tc::attn_tc_kernel<false, false, false, false>;
   e = launch_next(kernel, grid, tc::kThreads, tc::kSmemBytes, stream, mq, mk, mv, m, row_ptr, col_idx, (uint16_t*)o, lse, ctx->d_status, tb, nullptr, work_counter,
-                  (const int*)answer.words, answer.nwords, answer.epoch);
+                  (const int*)answer.words, answer.nwords, answer.epoch, false);
   if (e != cudaSuccess) return -(int)e;
   ++launched;
   if (pairs) {
@@ -768,21 +811,14 @@ int launch_block_max_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const vo
     return -(int)cudaErrorInvalidValue;
   const unsigned grid = (unsigned)min((int64_t)ctx->num_sms, m.q_rows);
   float* lse_in = const_cast<float*>(lse);   // read only in this mode
-  // Pairs of query blocks that share their lists (attn_pair.cu): asked for from 2^18 causal blocks on (8k tokens, 32 heads), sooner than for the
-  // attention, as the map is taken of dense lists above all.  16k tokens: all blocks 1045 -> 755 us, a tenth of them 128 -> 131.
+  // From 2^18 causal blocks on (8k tokens, 32 heads) a CTA's share of the work is pairs of query blocks: it takes them by pairs where all of them list the
+  // same blocks (block_max_pair.cuh), and otherwise as single blocks.  To ask takes 2 us.  Without and with: 8192 tokens, 32 heads, every block 276 and
+  // 197 us, one in eight 45.9 and 46.4, one in twenty 30.6 and 32.7; 16 384 tokens 1146 and 797, one in eight 164 and 160; below, the 2 us weigh more (5824
+  // tokens, one in twenty, 19.3), and the map is taken of dense lists above all.  (As a check and a kernel for pairs of their own: 37.7 for the 32.7, 53.3 for the 46.4.)
   const bool pairs = m.score_tiles >= (1 << 18) / (128 * kScoreTile);
-  const PairAnswer answer(ctx, m, pairs ? ctx->words + (ctx->clock % kWordSets) * kPairWords : nullptr);
-  int launched = 0;
-  if (pairs) {
-    launched = launch_pair_check(ctx, m, row_ptr, col_idx, nullptr, answer, stream);
-    if (launched < 0) return launched;
-    const int n = launch_block_max_pair(ctx, m, mq, mk, row_ptr, col_idx, lse, out, answer, stream);
-    if (n < 0) return n;
-    launched += n;
-  }
   const cudaError_t e = launch_next(m.chunked ? tc::attn_tc_kernel<false, true, true> : tc::attn_tc_kernel<false, false, true>, grid, tc::kThreads, tc::kSmemBytes, stream,
-                                    mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr, (const int*)answer.words, answer.nwords, answer.epoch);
-  return e == cudaSuccess ? launched + 1 : -(int)e;
+                                    mq, mk, mk, m, row_ptr, col_idx, nullptr, lse_in, ctx->d_status, nullptr, out, nullptr, nullptr, 0, 0, pairs);
+  return e == cudaSuccess ? 1 : -(int)e;
 }
 
 }  // namespace seer

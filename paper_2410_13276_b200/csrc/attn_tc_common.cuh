@@ -518,8 +518,7 @@ __device__ __forceinline__ void st_global_32(void* p, const uint32_t (&w)[8], bo
 }  // namespace tcc
 
 // Attention where pairs of query blocks list the same blocks (attn_pair.cu).  The check answers in `nwords` words, all of them written by every call: `epoch`
-// in all of them where all pairs do.  attn_tc_kernel then returns at once, otherwise attn_pair_kernel.  (The attention's words lie behind the counter in a workspace
-// of 256 bytes or more, those of the block maxima in the context.)
+// in all of them where all pairs do.  attn_tc_kernel then returns at once, otherwise attn_pair_kernel.  (The words lie behind the counter in a workspace of 256 bytes or more.)
 struct PairAnswer {
   int* words;
   int nwords, epoch;
@@ -528,7 +527,5 @@ struct PairAnswer {
 int launch_pair_check(seer_ctx* ctx, const SeqMeta& m, const int32_t* row_ptr, const int32_t* col_idx, int* counter, const PairAnswer& a, cudaStream_t stream);
 int launch_attn_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv, const CUtensorMap& mv32, const int32_t* row_ptr,
                      const int32_t* col_idx, void* o, float* lse, int* counter, const PairAnswer& a, cudaStream_t stream);
-int launch_block_max_pair(seer_ctx* ctx, const SeqMeta& m, const CUtensorMap& mq, const CUtensorMap& mk, const int32_t* row_ptr, const int32_t* col_idx, const float* lse,
-                          float* out, const PairAnswer& a, cudaStream_t stream);
 
 }  // namespace seer

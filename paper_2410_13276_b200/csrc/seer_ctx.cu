@@ -334,11 +334,8 @@ seer_status seer_create(seer_ctx** out, int device) {
   seer_ctx* ctx = new seer_ctx();
   ctx->device = device;
   ctx->num_sms = sms;
-  // (the status word, and behind it the sets of words of the block maxima)
-  constexpr size_t kStatusBytes = 256 + (size_t)kWordSets * kPairWords * sizeof(int);
-  bool ok = cudaMalloc(&ctx->d_status, kStatusBytes) == cudaSuccess &&
-            cudaMemset(ctx->d_status, 0, kStatusBytes) == cudaSuccess && cudaMallocHost(&ctx->stage, kStageBytes) == cudaSuccess;
-  if (ok) ctx->words = ctx->d_status + 64;
+  bool ok = cudaMalloc(&ctx->d_status, sizeof(int)) == cudaSuccess &&
+            cudaMemset(ctx->d_status, 0, sizeof(int)) == cudaSuccess && cudaMallocHost(&ctx->stage, kStageBytes) == cudaSuccess;
   for (int i = 0; ok && i < kMetaSlots; ++i) {
     MetaSlot& s = ctx->slots[i];
     ok = cudaMalloc(&s.dev, kSlotBytes) == cudaSuccess &&

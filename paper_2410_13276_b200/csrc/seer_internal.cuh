@@ -16,7 +16,6 @@ constexpr int kGateDim = 128;
 constexpr int kMaxBatch = 4096;
 constexpr int kMetaSlots = 8;
 constexpr int kPairWords = 63;  // words of the answer whether pairs of query blocks share their lists (attn_pair.cu)
-constexpr int kWordSets = 16;   // sets of them in a context (block maxima)
 constexpr int kScoreTile = 64;  // column tile of the gate's score kernel, and granularity of the bands of the one-call gate + mask
 
 // Per-batch metadata the kernels read from device memory.
@@ -119,7 +118,6 @@ struct seer_ctx {
   void* tmap_encode = nullptr;   // cuTensorMapEncodeTiled, resolved at run time
   void* trace = nullptr;         // optional device buffer for the attention kernel's timeline (diagnostics)
   bool pair_kernels = false;     // their shared-memory limits are set (by the first call that may use them: 0.1 ms of creating a context)
-  int* words = nullptr;          // kWordSets sets of words through which a check of lists answers (block maxima)
   uint32_t wait_limit_us = 2000000u;   // seer_debug_lost_wait
   int32_t lose_v_copy = -1;
   // seer_prefill_host: copy streams and the events of its two-deep pipeline over KV-head slices

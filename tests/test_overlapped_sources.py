@@ -51,7 +51,7 @@ def test_warps_of_the_maxima_go_into_an_item_together():
     """The two warps of a block meet inside an item, at a barrier without a limit: a warp that lost its wait for the item must not be the one its
     neighbour waits for.  So behind that wait every warp comes to a vote, whatever its own outcome, before it looks at the item."""
     for name, start, meeting in (("attn_tc.cu", "!mbar_wait(sh, item_full(s, n), (n >> 2) & 1u, status);\n      Slot it{}", "named_bar_or(5 + 2 * s + half"),
-                                 ("attn_pair.cu", "!mbar_wait_warp(sh, M_ITEM_FULL", "named_bar_or(bar_block")):
+                                 ("block_max_pair.cuh", "!mbar_wait_warp(sh, M_ITEM_FULL", "named_bar_or(bar_block")):
         text = code(name)
         between = text[text.index(start):text.index(meeting)]
         assert re.search(r"\n *if \(named_bar_or\(bar_vote, \w+, fail\) \|\| [\w.]+ < 0\) break;", between), name
