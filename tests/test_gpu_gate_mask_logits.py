@@ -49,3 +49,29 @@ def test_lists_equal_those_of_the_two_calls(lens, hq, hkv, tail, spoilt):
                 p.gate_mask(params, band_bytes=band)
                 assert p.status() == 0
                 assert torch.equal(p.row_ptr, rp) and torch.equal(p.col_idx[:n], col) and int(p.nnz.item()) == n, (chunk, band)
+
+
+# rows of several warps whose statistics are finite (from 2049 blocks four warps a row, from 8193 eight), the last block of a row a candidate like the others
+@pytest.mark.parametrize("flags", [0, 2])
+@pytest.mark.parametrize("n,tail", [(2049 * 64, 2049), (2563 * 64 - 9, 700), (8193 * 64, 130), (10241 * 64 - 1, 40)])
+def test_rows_without_a_forced_diagonal(n, tail, flags):
+    import torch
+    from paper_2410_13276_b200 import binding as B
+    from paper_2410_13276_b200.prefill import Prefill
+    gen = torch.Generator(device="cuda").manual_seed(n + flags)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    nq = n - 64 * ((n + 63) // 64 - tail)
+    p = Prefill([0, n], 2, 1, want_lse=False, cu_seqlens_q=[0, nq])
+    p.q, p.k, p.wq, p.wk = (2.0 * rand(nq, 2, 128)).bfloat16(), rand(n, 1, 128).bfloat16(), rand(2, 128, 128) / 2, rand(1, 128, 128) / 2
+    p.gate()
+    for params in (B.make_mask_params(B.SEER_TOPK_RATIO, keep_num=1, keep_den=10, flags=flags), B.make_mask_params(B.SEER_TOPK_COUNT, k=33, flags=flags),
+                   B.make_mask_params(B.SEER_TOPK_COUNT, k=n // 64 - tail // 2, flags=flags)):
+        p.mask(params)
+        assert p.status() == 0
+        rp, nnz = p.row_ptr.clone(), int(p.nnz.item())
+        col = p.col_idx[:nnz].clone()
+        p.row_ptr.fill_(-7)
+        p.col_idx.fill_(-7)
+        p.gate_mask(params)
+        assert p.status() == 0
+        assert torch.equal(p.row_ptr, rp) and torch.equal(p.col_idx[:nnz], col) and int(p.nnz.item()) == nnz
