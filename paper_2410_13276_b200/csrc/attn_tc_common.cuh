@@ -346,24 +346,20 @@ __device__ __forceinline__ float2 exp2_poly2(float2 x) {
 
 // One pass over this thread's row of a 64 x 64 block of scores: p = 2^(sl2 * s - R), packed to bf16 pairs in pk; returns the
 // sum of the row.  kPolyPairsOf8 of every eight pairs take their exponentials on the FMA pipe, the others on the
-// special-function unit.  MASKED: the causal mask of the diagonal block (keys after `row` are dropped).
-template <bool MASKED>
-__device__ __forceinline__ float row_pass(uint32_t s_addr, float sl2, float R, int row, uint32_t (&pk)[32]) {
+// special-function unit.  MASKED: the causal mask of the diagonal block (keys after `row` are dropped).  half(ch): the row's 32 keys from 32 ch on.
+template <bool MASKED, class Half>
+__device__ __forceinline__ float row_pass_of(Half half, float sl2, float R, int row, uint32_t (&pk)[32]) {
   const float2 sl22 = make_float2(sl2, sl2), nr = make_float2(-R, -R);
   float2 acc[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.f, 0.f);
-  // two TMEM round trips: the second half is requested before the first is worked on
-  uint32_t sv[2][32];
-  tc_ld32(s_addr, sv[0]);
 #pragma unroll
   for (int ch = 0; ch < 2; ++ch) {
-    tc_wait_ld32(sv[ch]);
-    if (ch == 0) tc_ld32(s_addr + 32, sv[1]);
+    const uint32_t (&sv)[32] = half(ch);
     // stage by stage over the 32 keys, each stage a run of independent instructions, in place
     float2 v[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __ffma2_rn(make_float2(__uint_as_float(sv[ch][2 * i]), __uint_as_float(sv[ch][2 * i + 1])), sl22, nr);
+    for (int i = 0; i < 16; ++i) v[i] = __ffma2_rn(make_float2(__uint_as_float(sv[2 * i]), __uint_as_float(sv[2 * i + 1])), sl22, nr);
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       if ((i & 7) < kPolyPairsOf8) v[i] = exp2_poly2(v[i]);
@@ -385,39 +381,16 @@ __device__ __forceinline__ float row_pass(uint32_t s_addr, float sl2, float R, i
   const float2 a = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
   return a.x + a.y;
 }
-
-// The same, of a row that is in registers.
+// The row from tensor memory, in two round trips: the second half is requested before the first is worked on
 template <bool MASKED>
-__device__ __forceinline__ float row_pass_of(const uint32_t (&sv)[2][32], float sl2, float R, int last, uint32_t (&pk)[32]) {
-  const float2 sl22 = make_float2(sl2, sl2), nr = make_float2(-R, -R);
-  float2 acc[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) acc[i] = make_float2(0.f, 0.f);
-#pragma unroll
-  for (int ch = 0; ch < 2; ++ch) {
-    float2 v[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __ffma2_rn(make_float2(__uint_as_float(sv[ch][2 * i]), __uint_as_float(sv[ch][2 * i + 1])), sl22, nr);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      if ((i & 7) < kPolyPairsOf8) v[i] = exp2_poly2(v[i]);
-      else v[i] = make_float2(ex2f(v[i].x), ex2f(v[i].y));
-    }
-    if (MASKED) {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int c = ch * 32 + 2 * i;
-        if (c > last) v[i].x = 0.f;
-        if (c + 1 > last) v[i].y = 0.f;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) pk[ch * 16 + i] = pack_bf16(v[i].x, v[i].y);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i & 3] = __fadd2_rn(acc[i & 3], v[i]);
-  }
-  const float2 a = __fadd2_rn(__fadd2_rn(acc[0], acc[1]), __fadd2_rn(acc[2], acc[3]));
-  return a.x + a.y;
+__device__ __forceinline__ float row_pass(uint32_t s_addr, float sl2, float R, int row, uint32_t (&pk)[32]) {
+  uint32_t sv[2][32];
+  tc_ld32(s_addr, sv[0]);
+  return row_pass_of<MASKED>([&](int ch) -> const uint32_t (&)[32] {
+    tc_wait_ld32(sv[ch]);
+    if (ch == 0) tc_ld32(s_addr + 32, sv[1]);
+    return sv[ch];
+  }, sl2, R, row, pk);
 }
 // The largest raw score of this thread's row (MASKED: among the keys it sees, key <= last; -inf if there is none).
 // Off the diagonal the 64 predicates are left out (with them a 128k prompt takes 2 % longer).
@@ -482,7 +455,7 @@ static __device__ __noinline__ float4 other_tile(Shared sh, uint32_t s_addr, uin
           }
         }
       }
-      sum = row_pass_of<true>(sv, sl2, R, last, pk);
+      sum = row_pass_of<true>([&](int ch) -> const uint32_t (&)[32] { return sv[ch]; }, sl2, R, last, pk);
       if (taken) {
         if (!(sum < kRise)) sum = CUDART_NAN_F;             // an infinite score or a NaN: so is the row
         break;
