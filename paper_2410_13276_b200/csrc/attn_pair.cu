@@ -2,14 +2,14 @@
 // gate blocks of 128 tokens, and dense lists.  A work item is the two blocks, 128 query rows that share every K and V tile.
 //
 // attn_tc_kernel has an item's 64 rows on both halves of tensor memory's lanes, the even list positions on one and the odd ones on the
-// other, and 64 KB of K and V come from L2 for each pair of listed blocks: 885 of the 917 clocks that a dense pair takes.  Here the lane
+// other, and 64 KB of K and V come from L2 for each pair of listed blocks: 885 clocks of the 960 that they take.  Here the lane
 // half is the query block, and the even and the odd positions belong to two softmax groups with an S, P and O of their own:
 //     S[128 q x 128 keys] = Q (smem) * [K_a; K_b]^T      M = N = 128: columns 0-63 are the even position's scores, 64-127 the odd one's
 //     O_0 += P_a V_a, O_1 += P_b V_b                     M = N = 128, A = P in tensor memory
 // so a tile's 64 KB serve four 64 x 64 blocks instead of two, and its 16 MMAs run at the full rate (1024 clocks for four blocks; the
 // weight-stationary forms take 1376).  What every row is made of is the same, in the same order: the results equal attn_tc_kernel's bit for
 // bit.  A launch by itself, on a cool board and under its power limit: 65 536 tokens, 32 heads, 128-token blocks, one in ten 3740 -> 3100 and 4180
-// -> 3510 us; 16 384 tokens, every block 2190 -> 1850 and 2400 -> 2050.
+// -> 3510 us; 16 384 tokens, every block 2190 -> 1850 and 2356 -> 2082.
 //
 // What bounds it: the power limit in launches of milliseconds; under it the groups, 1400 to 1500 clocks a tile (the pass 1100, with two warps
 // a scheduler that begin it together), and an item's end, 1000 to 2500 clocks until the last P V and 2300 for merge and stores, which both

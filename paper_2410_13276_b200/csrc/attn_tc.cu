@@ -1,10 +1,10 @@
 // Block-sparse causal GQA attention (Sec. 3.3) on the Blackwell tensor path, two work items in flight per CTA.
 //
 // What bounds it.  Long lists: the copies of K and V into shared memory (64 KB per pair of listed 64 x 64 blocks, about 885 clocks
-// at the 74 bytes a clock that an SM takes from L2, of 917 to 1060 that a pair takes), close before the MMA pipe (8 x 48 + 4 x 76 =
+// at the 74 bytes a clock that an SM takes from L2, of 960 that a pair takes with one in ten of 128k tokens), close before the MMA pipe (8 x 48 + 4 x 76 =
 // 688 clocks: 75 % active on dense lists of 16k tokens), and in launches of more than a few milliseconds the board's power limit.
-// Short lists: an item's start and end, about 5000 clocks beside 1900 for a stream's tile.  Of them the wait for the last P V 1400, merge and
-// stores 3000 (2700 without instrumentation); everything that needs no O is done during the wait, and an item's row pointers and first list
+// Short lists: an item's start and end, about 5300 clocks beside 1730 for a stream's tile (instrumented).  Of them the wait for the last P V 1250, merge and
+// stores 3400; everything that needs no O is done during the wait, and an item's row pointers and first list
 // entries are fetched while the item before it is copied.  With those after the wait, the entries fetched at the item's start, and
 // producers that slept between their polls: 6000 clocks; the launch by itself, both in turn: 24 prompts of 16 900 tokens 174 us where this
 // takes 166, 32k tokens 1232 and 1174, 48k 2557 and 2480, 128k 16.7 and 16.1 ms; dense 2000-token prompts 435 and 432.  (A whole pass, which runs
@@ -770,9 +770,10 @@ int launch_attn_tc(seer_ctx* ctx, const SeqMeta& m, const void* q, const void* k
   cudaError_t e = cudaSuccess;
   int launched = 0;
   if (m.q_rows <= 2 * (int64_t)grid) work_counter = nullptr;
-  // Whether pairs of query blocks share their lists is known on the device only.  Asking takes about 4 us, and 2 for the kernel that then has
-  // nothing to do; where they do share them it saves a sixth of the launch.  Asked from 2^20 causal blocks on (16k tokens, 32 heads: a tenth of
-  // them takes 240 us, all of them 2400).
+  // Whether pairs of query blocks share their lists is known on the device only.  Asking takes 3.5 to 5 us: the check, and the kernel that then has
+  // nothing to do.  The launch without and with it, 32 heads, every block, one in ten, one in twenty: 16 384 tokens 2356 and 2082, 353.5 and 356.3, 226.7
+  // and 231.3 us; 13 760 tokens 1685 and 1502, 265.5 and 270.8, 175.4 and 178.1; 8192 tokens 632 and 569, 118.7 and 120.5, 89.4 and 90.7.  Most
+  // launches are of sparse lists, and this one loses at most 2 % of them: it is asked from 2^20 causal blocks on (16 384 tokens, 32 heads).
   const bool pairs = work_counter != nullptr && ctx->trace == nullptr && m.score_tiles >= (1 << 20) / (128 * kScoreTile);
   const PairAnswer answer(ctx, m, pairs ? work_counter + 1 : nullptr);
   if (pairs) {

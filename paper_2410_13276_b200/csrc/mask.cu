@@ -363,7 +363,7 @@ __device__ __forceinline__ uint32_t lean_key(float sc) {
 // TopK lists, W = 1, 4 or 8 warps per row, the row's keys in shared memory (`cap` of them, a multiple of 128 W).  A warp works on a contiguous
 // run of the row's columns, 128 at a time, a lane four of them.
 //
-// It is bound by instruction issue (3.5 of 4 per clock), so the loops are short and rolled (with the keys in registers and the
+// It is bound by instruction issue (three of four per clock on average, four warps a row), so the loops are short and rolled (with the keys in registers and the
 // loops unrolled it waited for instructions), what a row needs once is done by one of its warps and passed on, and the
 // counts that order the warps' parts of the list are taken in the pass that gathers the threshold's class.
 // A row gets one warp up to 2048 blocks, and as many as keep it at 2048 keys per warp beyond.  Measured: 65 536 rows of up to
